@@ -1145,7 +1145,7 @@ static fvar_status scale_step_impl(fvar_ctx *ctx, const void *tokens, bool token
         aa.wait_cycles = ctx->wait_cycles;
         attention_plan(E, H, r, L_prev + r, ctx->num_sms, &aa.tiles_per_cta, &aa.kv_splits);
         ctx->prof_begin(FVAR_KCLASS_ATTENTION, 4.0 * E * r * (L_prev + r) * C, 4.0 * E * (L_prev + r) * C + 4.0 * E * r * C);
-        FV_CUDA(ctx, launch_attention(ctx->q_map, ctx->kmap[blk], ctx->vmap[blk], aa, st), "attention");
+        FV_CUDA(ctx, launch_attention(ctx->q_map, ctx->kmap[blk], ctx->vmap[blk], aa, ctx->num_sms, st), "attention");
         ctx->launched();
       }
       {
@@ -1171,7 +1171,7 @@ static fvar_status scale_step_impl(fvar_ctx *ctx, const void *tokens, bool token
         aa.wait_cycles = ctx->wait_cycles;
         attention_plan(E, H, r, ctx->cfg.ctx_len, ctx->num_sms, &aa.tiles_per_cta, &aa.kv_splits);
         ctx->prof_begin(FVAR_KCLASS_ATTENTION, 4.0 * E * r * ctx->cfg.ctx_len * C, 4.0 * E * ctx->cfg.ctx_len * C + 4.0 * E * r * C);
-        FV_CUDA(ctx, launch_attention(ctx->q_map, ctx->ckmap[blk], ctx->cvmap[blk], aa, st), "cross attention");
+        FV_CUDA(ctx, launch_attention(ctx->q_map, ctx->ckmap[blk], ctx->cvmap[blk], aa, ctx->num_sms, st), "cross attention");
         ctx->launched();
         GemmArgs go = gemm_args(R, C, C);
         go.rows_per_batch = r; go.bmul = bmul; go.boff = boff;
@@ -1588,9 +1588,10 @@ fvar_status fvar_attention(const void *q, const void *Kc, const void *Vt, int B,
   int dev = 0, sms = 0;
   FK_CUDA(cudaGetDevice(&dev), "get device");
   FK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device attribute");
+  FK_CUDA(attention_prepare(), "attention set-up");
   attention_plan(B, H, r, L, sms, &a.tiles_per_cta, &a.kv_splits);
   if (!a.status) return kfail(FVAR_ECUDA, "attention: status word");
-  FK_CUDA(launch_attention(tq, tk, tv, a, static_cast<cudaStream_t>(stream)), "attention");
+  FK_CUDA(launch_attention(tq, tk, tv, a, sms, static_cast<cudaStream_t>(stream)), "attention");
   return FVAR_OK;
 }
 

@@ -143,7 +143,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       // ---------------------------------------------------------------- MMA issuer
       // The whole warp walks the loop (so that stage counters, addresses and descriptors are
       // warp-uniform values); one elected lane issues the MMAs and the commits.
-      const bool leader = elect_one();
+      const uint32_t leader = elect_one() ? 1u : 0u;
       const uint32_t idesc = umma_idesc_bf16(kBlockM, BN) | (p.w_mn_major ? (1u << 16) : 0u);   // bit 16: B is MN-major
       int stage = 0;
       uint32_t phase = 0;
@@ -173,20 +173,16 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           }
           const uint32_t kstep_b = p.w_mn_major ? (2048u >> 4) : 2u;      // descriptor advance per 16 of K
           const uint32_t acc_first = (kb > kb0) ? 1u : 0u;
-          if (leader) {
 #pragma unroll
           for (int ka = 0; ka < kKAtoms; ++ka) {
 #pragma unroll
             for (int k = 0; k < kBlockK / 16; ++k)
-              umma_bf16(d_tmem, da[ka] + 2 * k, db[ka] + kstep_b * k, idesc, (ka != 0 || k != 0) ? 1u : acc_first);
+              umma_bf16_if(leader, d_tmem, da[ka] + 2 * k, db[ka] + kstep_b * k, idesc, (ka != 0 || k != 0) ? 1u : acc_first);
           }
-          umma_commit(empty_bar(stage));
-          }
-          __syncwarp();
+          umma_commit_if(leader, empty_bar(stage));
           if (++stage == S) { stage = 0; phase ^= 1u; }
         }
-        if (ok && leader) umma_commit(tfull_bar(a));
-        __syncwarp();
+        if (ok) umma_commit_if(leader, tfull_bar(a));
       }
     }
   } else {

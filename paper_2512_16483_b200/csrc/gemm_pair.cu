@@ -124,7 +124,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   } else if (warp == 1) {
     if (rank == 0) {
       // ---------------------------------------------------------------- MMA issuer (rank 0 only)
-      const bool leader = elect_one();
+      const uint32_t leader = elect_one() ? 1u : 0u;
       constexpr uint32_t idesc = umma_idesc_bf16(2 * kBlockM, BN);
       int stage = 0;
       uint32_t phase = 0;
@@ -149,20 +149,16 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             db[ka] = smem_desc_sw128(sa + Cfg::kStageBytesA + ka * Cfg::kAtomBytesB);
           }
           const uint32_t acc_first = (kb > 0) ? 1u : 0u;
-          if (leader) {
 #pragma unroll
-            for (int ka = 0; ka < kKAtoms; ++ka) {
+          for (int ka = 0; ka < kKAtoms; ++ka) {
 #pragma unroll
-              for (int k = 0; k < kBlockK / 16; ++k)
-                umma_bf16_pair(d_tmem, da[ka] + 2 * k, db[ka] + 2 * k, idesc, (ka != 0 || k != 0) ? 1u : acc_first);
-            }
-            umma_commit_pair(empty_bar(stage));       // frees this stage in both CTAs
+            for (int k = 0; k < kBlockK / 16; ++k)
+              umma_bf16_pair_if(leader, d_tmem, da[ka] + 2 * k, db[ka] + 2 * k, idesc, (ka != 0 || k != 0) ? 1u : acc_first);
           }
-          __syncwarp();
+          umma_commit_pair_if(leader, empty_bar(stage));       // frees this stage in both CTAs
           if (++stage == S) { stage = 0; phase ^= 1u; }
         }
-        if (ok && leader) umma_commit_pair(tfull_bar(a));   // accumulator ready in both CTAs
-        __syncwarp();
+        if (ok) umma_commit_pair_if(leader, tfull_bar(a));   // accumulator ready in both CTAs
       }
     }
   } else {

@@ -227,7 +227,7 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     // ------------------------------------------------------------------ MMA issuer
     pdl_wait();
     pdl_launch_dependents();
-    const bool leader = elect_one();
+    const uint32_t leader = elect_one() ? 1u : 0u;
     const uint32_t idesc = umma_idesc_bf16(kBlockM, rp);
     for (int i = 0; i < nst; ++i) {
       const int stage = i % nstages;
@@ -236,31 +236,27 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
       tc_fence_after();
       const uint32_t sa = ring + stage * stage_bytes;
       const int kvalid = min(nk, nkb - i * nk);              // K blocks of this stage inside the CTA's range
-      if (leader) {
-        // descriptor words: the address field counts 16-byte units, so a K block further on adds its size >> 4
-        uint64_t dw = smem_desc_sw128(sa), da0 = smem_desc_sw128(sa + w_stage);
-        const uint64_t da1_off = static_cast<uint64_t>((nk * a_bytes) >> 4);
-        uint32_t acc = i > 0 ? 1u : 0u;
-        for (int kk = 0; kk < kvalid; ++kk) {
+      // descriptor words: the address field counts 16-byte units, so a K block further on adds its size >> 4
+      uint64_t dw = smem_desc_sw128(sa), da0 = smem_desc_sw128(sa + w_stage);
+      const uint64_t da1_off = static_cast<uint64_t>((nk * a_bytes) >> 4);
+      uint32_t acc = i > 0 ? 1u : 0u;
+      for (int kk = 0; kk < kvalid; ++kk) {
 #pragma unroll
-          for (int k = 0; k < kBlockK / 16; ++k) {
-            if (ROWS) {
-              umma_bf16(tmem_base, da0 + 2 * k, dw + 2 * k, idesc, acc);       // rows x features
-            } else {
-              umma_bf16(tmem_base, dw + 2 * k, da0 + 2 * k, idesc, acc);       // features x rows
-              if (nchunks > 1) umma_bf16(tmem_base + rp32, dw + 2 * k, da0 + da1_off + 2 * k, idesc, acc);
-            }
-            acc = 1u;
+        for (int k = 0; k < kBlockK / 16; ++k) {
+          if (ROWS) {
+            umma_bf16_if(leader, tmem_base, da0 + 2 * k, dw + 2 * k, idesc, acc);       // rows x features
+          } else {
+            umma_bf16_if(leader, tmem_base, dw + 2 * k, da0 + 2 * k, idesc, acc);       // features x rows
+            if (nchunks > 1) umma_bf16_if(leader, tmem_base + rp32, dw + 2 * k, da0 + da1_off + 2 * k, idesc, acc);
           }
-          dw += kSkinnyWAtom >> 4;
-          da0 += a_bytes >> 4;
+          acc = 1u;
         }
-        umma_commit(empty_bar(stage));
+        dw += kSkinnyWAtom >> 4;
+        da0 += a_bytes >> 4;
       }
-      __syncwarp();
+      umma_commit_if(leader, empty_bar(stage));
     }
-    if (ok && leader) umma_commit(tfull_bar);
-    __syncwarp();
+    if (ok) umma_commit_if(leader, tfull_bar);
   } else {
     pdl_wait();
     pdl_launch_dependents();

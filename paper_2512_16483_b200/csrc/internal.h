@@ -135,6 +135,10 @@ cudaError_t gemm_prepare();
 cudaError_t gemm_pair_prepare();
 cudaError_t attention_prepare();
 
+// Division by an invariant d: mul = ceil(2^32 / d), or 0 where that would not be exact.
+struct FastDiv {
+  unsigned d, mul;
+};
 struct AttnArgs {
   int B_eff, H, r, D, L, L_cap;
   int bmul, boff;          // caller batch element (cache slot) of computed element e
@@ -146,11 +150,13 @@ struct AttnArgs {
   int kv_splits;
   int tiles_per_cta;       // 1: one 128-row query tile per CTA; otherwise two
   long long wait_cycles;   // budget of every bounded wait (0: the default)
+  int units;               // without key ranges: query tile groups over all heads and elements, walked by the CTAs
+  FastDiv div_nqt, div_h;  // unit -> (query tile group, head, element); filled by launch_attention
 };
 // Query tiles per CTA (1 or 2) and key ranges per launch (1 = no split; at most 6).
 void attention_plan(int B_eff, int H, int r, int L, int num_sms, int *tiles_per_cta, int *kv_splits);
 cudaError_t launch_attention(const CUtensorMap &tmQ, const CUtensorMap &tmK, const CUtensorMap &tmV,
-                             const AttnArgs &a, cudaStream_t st);
+                             const AttnArgs &a, int num_sms, cudaStream_t st);
 
 // Launch with programmatic stream serialization (see pdl_wait in ptx.cuh).
 template <typename... KArgs, typename... Args>

@@ -1,0 +1,44 @@
+"""Kernels at the edges of their launch rules: the sizes where one form hands over to another, remainders of tiles, and
+several units of work in one thread block.  Each against a plain PyTorch fp32 reference of the same operation."""
+import pytest
+import torch
+
+from helpers import rel_err
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fv():
+    from paper_2512_16483_b200 import binding
+    binding.load_library()
+    return binding
+
+
+@pytest.mark.parametrize("B,H,D,r,L", [
+    (12, 16, 64, 169, 424),     # more units than SMs; the second tile of every unit is a remainder of 41 rows
+    (3, 16, 128, 1600, 300),    # units of two tiles and of one (1600 = 6 * 256 + 64) walked by the same blocks, 3 key blocks
+    (5, 16, 128, 700, 129),     # the same with an even number of key blocks, the last with a single key
+    (10, 30, 64, 100, 100),     # one key block: set-up, softmax and store of consecutive units only
+    (2, 16, 128, 1100, 1500),   # lone tiles walked: 9 tiles a head, the last of 76 rows
+    (1, 16, 128, 400, 2921),    # key ranges over a cluster, four tiles, the last of 16 rows
+    (1, 3, 128, 5, 6441),       # six ranges, fewer rows than a slice's share for every block
+    (1, 40, 64, 257, 1030),     # pairs whose second unit is one row
+    (1, 16, 128, 128, 128), (1, 1, 64, 1, 1),
+])
+def test_attention_launch_shapes(fv, B, H, D, r, L):
+    g = torch.Generator(device="cuda").manual_seed(B * 1000 + r)
+    L_cap = (L + 127) // 128 * 128
+    q = torch.randn((B, r, H * D), generator=g, device="cuda").bfloat16()
+    K = torch.randn((B, H, L_cap, D), generator=g, device="cuda").bfloat16()
+    Vt = torch.randn((B, H, D, L_cap), generator=g, device="cuda").bfloat16()
+    q[:, ::3] *= 6.0            # rows whose maximum moves: the accumulator is rescaled in some blocks only
+    for _ in range(3):          # blocks of work follow one another differently from launch to launch
+        out = fv.fvar_attention(q, K, Vt, L)
+    assert fv.kernel_poll_status() == fv.OK
+    s = torch.einsum("brhd,bhld->bhrl", q.float().view(B, r, H, D), K[:, :, :L].float()) * D ** -0.5
+    ref = torch.einsum("bhrl,bhdl->brhd", s.softmax(-1), Vt[..., :L].float()).reshape(B, r, H * D)
+    _, cos = rel_err(out.float().cpu().numpy(), ref.cpu().numpy())
+    # P and the result are rounded to bf16 (2^-8 of the value at most each); sharp rows are many times the RMS
+    bad = (out.float() - ref).abs() - (2.0 ** -6 * ref.abs() + 3e-2 * ref.square().mean().sqrt())
+    assert bad.max() <= 0 and cos >= 0.9999, (float(bad.max()), cos)

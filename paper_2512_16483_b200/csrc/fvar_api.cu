@@ -141,13 +141,15 @@ struct fvar_ctx {
   std::vector<CUtensorMap> csplit_map; // [scale]
   int lls_rank_cap;                    // min(kLlsMaxRank, Mmax)
   bool last_lls;                       // the last step restored by LLS (no index sets)
-  // transition between scale steps: codebook (caller's memory), half-norms, packed arg-max words, codes and
-  // the accumulated feature map F_k at the last scale's resolution
+  // transition between scale steps: codebook (caller's memory), half-norms, two buffers of packed arg-max words
+  // (transitions alternate: each leaves the other buffer zeroed for the next) and the accumulated feature map F_k
+  // at the last scale's resolution
   const bf16 *codebook;
   int codebook_V;
   float *tr_hn, *tr_F;
-  unsigned long long *tr_best;
-  int *tr_codes;
+  unsigned long long *tr_best[2];
+  int tr_buf;                          // buffer the next codeword search uses
+  long long tr_dirty[2];               // words of each buffer that a search may have set
   int tr_scale;                        // last scale accumulated into tr_F (-1: none)
   int tr_B;
   // pipelined host entry point: two staging slots each way, one stream per copy direction
@@ -246,7 +248,7 @@ namespace {
 struct Layout {
   size_t status, split_partial, split_counters, kc, vt, ckc, cvt, ada, silu_c, gcache, x0, xs, y, q, a, hbuf, xsplit[2], scores, idx, inv, qt_pool, total;
   size_t cup, csplit, lls_xhat, lls_chat, lls_G, lls_Ginv, lls_T, lls_P;
-  size_t tr_hn, tr_best, tr_codes, tr_F;
+  size_t tr_hn, tr_best[2], tr_F;
   size_t hin[2], hout[2];
   std::vector<size_t> qt_off;
 };
@@ -325,8 +327,8 @@ Layout make_layout(const fvar_cfg *c) {
   take(pool * 2);
   const size_t M_last = static_cast<size_t>(c->scale_hw[2 * (c->n_scales - 1)]) * c->scale_hw[2 * (c->n_scales - 1) + 1];
   L.tr_hn = take(static_cast<size_t>(kMaxCodebook) * 4);
-  L.tr_best = take(B * Mmax * 8);
-  L.tr_codes = take(B * Mmax * 4);
+  L.tr_best[0] = take(B * Mmax * 8);
+  L.tr_best[1] = take(B * Mmax * 8);
   L.tr_F = take(B * M_last * C * 4);
   for (int s2 = 0; s2 < 2; ++s2) {
     L.hin[s2] = take(B * Mmax * C * 2);
@@ -515,7 +517,11 @@ fvar_status fvar_init(const fvar_weights *weights, const fvar_cfg *cfg, void *wo
   c->idx = reinterpret_cast<int *>(at(L.idx)); c->inv = reinterpret_cast<int *>(at(L.inv));
   c->qt_pool = reinterpret_cast<bf16 *>(at(L.qt_pool));
   c->tr_hn = reinterpret_cast<float *>(at(L.tr_hn)); c->tr_F = reinterpret_cast<float *>(at(L.tr_F));
-  c->tr_best = reinterpret_cast<unsigned long long *>(at(L.tr_best)); c->tr_codes = reinterpret_cast<int *>(at(L.tr_codes));
+  c->tr_buf = 0;
+  for (int t = 0; t < 2; ++t) {
+    c->tr_best[t] = reinterpret_cast<unsigned long long *>(at(L.tr_best[t]));
+    c->tr_dirty[t] = 0;                // the workspace is zeroed below
+  }
   c->codebook = nullptr; c->codebook_V = 0; c->tr_scale = -1; c->tr_B = 0;
   for (int s2 = 0; s2 < 2; ++s2) {
     c->hin[s2] = reinterpret_cast<bf16 *>(at(L.hin[s2]));
@@ -880,30 +886,57 @@ static fvar_status transition_impl(fvar_ctx *ctx, const void *fo, int scale_idx,
   cudaStream_t st = ctx->st;
 
   // R_k = Q(F_k^o): scores F_k^o Z^T - |Z|^2 / 2 on the tensor cores, arg-max in the epilogue
-  const GemmPlan plan = gemm_plan(R, 1, V, C, ctx->num_sms, ctx->max_clusters, 1, 0);
-  CUtensorMap ta, tw;
-  if (!tmap_2d(&ta, fo, C, R, C, 128) || !tmap_2d(&tw, ctx->codebook, C, V, C, plan.pair ? plan.block_n / 2 : plan.block_n))
-    return fail(ctx, FVAR_EINVAL, "scale_transition: fo must be 16-byte aligned");
-  FV_CUDA(ctx, cudaMemsetAsync(ctx->tr_best, 0, static_cast<size_t>(R) * 8, st), "arg-max words clear");
+  const int buf = ctx->tr_buf;
+  if (ctx->tr_dirty[buf] > 0) {                  // only after a transition that failed half way
+    FV_CUDA(ctx, cudaMemsetAsync(ctx->tr_best[buf], 0, static_cast<size_t>(ctx->tr_dirty[buf]) * 8, st), "arg-max words clear");
+    ctx->tr_dirty[buf] = 0;
+  }
   GemmArgs g = gemm_args(R, V, C);
   g.col_sub = ctx->tr_hn;
-  g.best = ctx->tr_best;
+  g.best = ctx->tr_best[buf];
   g.status = ctx->status;
-  ctx->prof_begin(FVAR_KCLASS_GEMM, 2.0 * R * V * C, 2.0 * (static_cast<double>(V) * C + static_cast<double>(R) * C) + 8.0 * R);
-  if (plan.pair)
+  g.wait_cycles = ctx->wait_cycles;
+  CUtensorMap ta, tw;
+  bool maps_ok = false, split = false;
+  const double gflops = 2.0 * R * V * C, gbytes = 2.0 * (static_cast<double>(V) * C + static_cast<double>(R) * C) + 8.0 * R;
+  // few rows: the search streams the codebook once, so it takes the cluster-split forms by the rule of the step's GEMMs
+  // (R = 1 .. 16, V = 8192, C = 2048: 12.5 -> 8.8 us)
+  if (V % 8 == 0 && R <= ctx->skinny_max_rows) {
+    const bool rows = gemm_ksplit_wins(R, V, C);
+    if (rows || R <= gemm_skinny_row_limit(V, C)) {
+      g.sk_tiles_m = rows ? (R + 127) / 128 : 0;
+      g.splits = gemm_skinny_pick_splits(V, C, 0, g.sk_tiles_m, !rows && R <= 64);
+      gemm_skinny_shape(g);
+      split = g.splits > 0 && g.sk_stages >= 1;
+      if (split)
+        maps_ok = gemm_skinny_map(&ta, fo, R, C, C, rows ? 128 : g.sk_rp, g.sk_nk) && gemm_skinny_map(&tw, ctx->codebook, V, C, C, 128, g.sk_nk);
+      else
+        g.sk_tiles_m = g.splits = 0;
+    }
+  }
+  GemmPlan plan{false, 64, 1};
+  if (!split) {
+    plan = gemm_plan(R, 1, V, C, ctx->num_sms, ctx->max_clusters, 1, 0);
+    maps_ok = tmap_2d(&ta, fo, C, R, C, 128) && tmap_2d(&tw, ctx->codebook, C, V, C, plan.pair ? plan.block_n / 2 : plan.block_n);
+  }
+  if (!maps_ok) return fail(ctx, FVAR_EINVAL, "scale_transition: fo must be 16-byte aligned");
+  ctx->tr_dirty[buf] = R;
+  ctx->prof_begin(FVAR_KCLASS_GEMM, gflops, gbytes);
+  if (split)
+    FV_CUDA(ctx, launch_gemm_skinny(EPI_ARGMAX, ta, tw, g, st), "codeword search");
+  else if (plan.pair)
     FV_CUDA(ctx, launch_gemm_pair(EPI_ARGMAX, plan.block_n, ta, tw, g, st), "codeword search");
   else
     FV_CUDA(ctx, launch_gemm(EPI_ARGMAX, plan.block_n, ta, tw, g, ctx->num_sms, st), "codeword search");
   ctx->launched();
-  ctx->prof_begin(FVAR_KCLASS_CONVERT, 0.0, 12.0 * R);
-  FV_CUDA(ctx, launch_unpack_codes(ctx->tr_best, R, V, ctx->tr_codes, ctx->status, st), "unpack codes");
-  ctx->launched();
-  if (codes) FV_CUDA(ctx, cudaMemcpyAsync(codes, ctx->tr_codes, static_cast<size_t>(R) * 4, cudaMemcpyDeviceToDevice, st), "codes copy");
 
-  // F_k = F_{k-1} + Up(R_k, (h_K, w_K))
+  // F_k = F_{k-1} + Up(R_k, (h_K, w_K)); the same launch decodes the codes and clears the other buffer's words
   ctx->prof_begin(FVAR_KCLASS_RTR_FILL, 0.0, (scale_idx == 0 ? 4.0 : 8.0) * B * hK * wK * C + 2.0 * R * C);
-  FV_CUDA(ctx, launch_up_accumulate(ctx->codebook, ctx->tr_codes, B, hk, wk, hK, wK, C, scale_idx == 0, ctx->tr_F, st), "up_accumulate");
+  FV_CUDA(ctx, launch_up_accumulate(ctx->codebook, ctx->tr_best[buf], V, B, hk, wk, hK, wK, C, scale_idx == 0, ctx->tr_F, codes,
+                                    ctx->tr_best[buf ^ 1], ctx->tr_dirty[buf ^ 1], ctx->status, st), "up_accumulate");
   ctx->launched();
+  ctx->tr_dirty[buf ^ 1] = 0;
+  ctx->tr_buf = buf ^ 1;
   // next input = Down(F_k, (h_{k+1}, w_{k+1}))
   if (next_tokens) {
     const int hn = ctx->hw[2 * (scale_idx + 1)], wn = ctx->hw[2 * (scale_idx + 1) + 1];

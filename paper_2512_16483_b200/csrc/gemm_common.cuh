@@ -27,6 +27,15 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<uint32_t *>(&v);
 }
 
+// One candidate of the arg-max epilogue: ordered score bits << 32 | ~column, so that an unsigned max takes the largest
+// score and the lowest column on ties; a NaN score ranks as -inf.
+__device__ __forceinline__ unsigned long long argmax_word(float score, int col) {
+  if (score != score) score = -INFINITY;
+  const unsigned u = __float_as_uint(score);
+  const unsigned key = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+  return (static_cast<unsigned long long>(key) << 32) | (0xFFFFFFFFu - static_cast<unsigned>(col));
+}
+
 // Warp-wide row-major stores through a 4 KiB shared-memory staging tile.  After tcgen05.ld each lane
 // holds 32 consecutive columns of its own row; storing those directly makes every instruction touch
 // 32 different rows 16 bytes at a time.  Instead the lanes park their pieces in shared memory (16-byte
@@ -137,11 +146,7 @@ __device__ __forceinline__ void epilogue_chunk(const GemmArgs &p, const uint32_t
           }
         }
       }
-      if (best_c >= 0) {
-        const unsigned u = __float_as_uint(best_v);
-        const unsigned key = (u & 0x80000000u) ? ~u : (u | 0x80000000u);  // unsigned order = float order
-        atomicMax(p.best + grow, (static_cast<unsigned long long>(key) << 32) | (0xFFFFFFFFu - static_cast<unsigned>(best_c)));
-      }
+      if (best_c >= 0) atomicMax(p.best + grow, argmax_word(best_v, best_c));
     }
   } else if constexpr (EPI == EPI_QKV) {
     const int e = row / p.rows_per_batch, j = row - e * p.rows_per_batch;

@@ -46,10 +46,29 @@ __device__ __forceinline__ uint2 pack4_bf16(float a, float b, float c, float d) 
   return make_uint2(pack_bf16(a, b), pack_bf16(c, d));
 }
 
+// What the epilogue of (row, features n .. n + 3) reads besides the sums: fetched together with them, so that a row pays
+// one memory latency and not two.
+struct SkinnyFetch {
+  float4 resid;
+  int jo;                  // output row within the element (after the scatter)
+};
+template <int EPI>
+__device__ __forceinline__ SkinnyFetch skinny_fetch(const GemmArgs &p, int row, int n) {
+  SkinnyFetch f;
+  f.resid = make_float4(0.f, 0.f, 0.f, 0.f);
+  f.jo = 0;
+  if constexpr (EPI == EPI_RESID) {
+    const int e = row / p.rows_per_batch, j = row - e * p.rows_per_batch;
+    f.resid = *reinterpret_cast<const float4 *>(p.resid + (static_cast<long long>(e * p.rmap.bmul + p.rmap.boff) * p.rmap.rpb + j) * p.ld_out + n);
+    f.jo = p.scatter ? __ldg(p.scatter + static_cast<long long>(e) * p.rows_per_batch + j) : j;
+  }
+  return f;
+}
+
 // Epilogue of one thread for output row `row` (row of the flattened [R] rows), features n .. n + 3 (n % 4 == 0,
 // n + 3 < N): the four sums arrive in `acc`.
 template <int EPI>
-__device__ __forceinline__ void skinny_store(const GemmArgs &p, float4 acc, int row, int n) {
+__device__ __forceinline__ void skinny_store(const GemmArgs &p, float4 acc, const SkinnyFetch &f, int row, int n) {
   float v[4] = {acc.x, acc.y, acc.z, acc.w};
   if (p.bias != nullptr) {
     const uint2 u = __ldg(reinterpret_cast<const uint2 *>(p.bias + n));
@@ -82,11 +101,9 @@ __device__ __forceinline__ void skinny_store(const GemmArgs &p, float4 acc, int 
       for (int i = 0; i < 4; ++i) dst[static_cast<long long>(i) * p.L_cap] = __float2bfloat16_rn(v[i]);
     }
   } else if constexpr (EPI == EPI_RESID) {
-    const int e = row / p.rows_per_batch, j = row - e * p.rows_per_batch;
-    const int b = e * p.bmul + p.boff;
-    const float4 r4 = *reinterpret_cast<const float4 *>(
-        p.resid + (static_cast<long long>(e * p.rmap.bmul + p.rmap.boff) * p.rmap.rpb + j) * p.ld_out + n);
-    const int jo = p.scatter ? __ldg(p.scatter + static_cast<long long>(e) * p.rows_per_batch + j) : j;
+    const int e = row / p.rows_per_batch, b = e * p.bmul + p.boff;
+    const float4 r4 = f.resid;
+    const int jo = f.jo;
     const float4 g4 = p.gate ? __ldg(reinterpret_cast<const float4 *>(p.gate + static_cast<long long>(b) * p.gate_stride + n))
                              : make_float4(1.f, 1.f, 1.f, 1.f);
     v[0] = fmaf(g4.x, v[0], r4.x);
@@ -106,13 +123,29 @@ __device__ __forceinline__ void skinny_store(const GemmArgs &p, float4 acc, int 
   }
 }
 
+// Arg-max epilogue of one warp for output row `row`: lane l holds the sums of features n .. n + 3 of the 128-feature
+// tile.  One packed word per row and tile leaves the warp (see GemmArgs::best).
+__device__ __forceinline__ void skinny_argmax(const GemmArgs &p, float4 acc, int row, int n, int lane) {
+  unsigned long long word = 0ull;                            // nothing: every real score packs to more
+  if (n < p.N) {                                             // n % 4 == 0 and N % 8 == 0: all four or none
+    const float4 h4 = __ldg(reinterpret_cast<const float4 *>(p.col_sub + n));
+    word = argmax_word(acc.x - h4.x, n);
+    word = max(word, argmax_word(acc.y - h4.y, n + 1));
+    word = max(word, argmax_word(acc.z - h4.z, n + 2));
+    word = max(word, argmax_word(acc.w - h4.w, n + 3));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) word = max(word, __shfl_xor_sync(0xffffffffu, word, o));
+  if (lane == 0) atomicMax(p.best + row, word);
+}
+
 // tmA: the activation rows [R][K], box of sk_rp rows; tmW: the weight rows [N][K], box of 128 rows (gemm_skinny_map).
 // ROWS = false: the form described at the top (weights on the M side, all rows on the N side).  ROWS = true: the same
 // pipeline, K split and cluster reduction for 128 x 128 output tiles with the rows back on the M side -- for a few
 // hundred rows and a narrow output, where the row-tiled kernels have too few tiles to fill the SMs and each of their
 // CTAs walks all of K; cluster c then owns tile (row tile c % sk_tiles_m, feature tile c / sk_tiles_m).
 template <int EPI, bool ROWS>
-__global__ void __launch_bounds__(kSkinnyThreads, 1)
+__global__ void __launch_bounds__(kSkinnyThreads, ROWS ? 1 : 2)      // the small form shares an SM with the next GEMM
 gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
                    const __grid_constant__ GemmArgs p) {
   extern __shared__ uint8_t smem_raw[];
@@ -308,12 +341,15 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
       const int rpr = (rows_ch + S - 1) / S;
       const int lo = sp * rpr, hi = min(rows_ch, lo + rpr);
       const int n4 = (et & 31) * 4, n = tile * kBlockM + n4;
-      if (n < p.N) {
+      if (EPI == EPI_ARGMAX || n < p.N) {      // the arg-max shuffles need every lane
         uint32_t peer[8];
 #pragma unroll
         for (int t = 0; t < 8; ++t) peer[t] = mapa_shared(red, static_cast<uint32_t>(t < S ? t : 0));
+        // One row of a warp at a time: two or four rows' loads in flight together measured slower everywhere (a d16 block
+        // of 2 - 50 rows 33 -> 35 - 37 us), their unrolled code being fetched cold by every launch of the chain.
         for (int jj = lo + (et >> 5); jj < hi; jj += 8) {
           const uint32_t off = static_cast<uint32_t>(jj) * kPitch + static_cast<uint32_t>(n4) * 4u;
+          const SkinnyFetch fetch = skinny_fetch<EPI>(p, row0 + ch * rc + jj, n);
           float4 sum = ld_dsmem_f4(peer[0] + off);
 #pragma unroll
           for (int t = 1; t < 8; ++t)
@@ -321,7 +357,8 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
               const float4 v = ld_dsmem_f4(peer[t] + off);
               sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
             }
-          skinny_store<EPI>(p, sum, row0 + ch * rc + jj, n);
+          if constexpr (EPI == EPI_ARGMAX) skinny_argmax(p, sum, row0 + ch * rc + jj, n, lane);
+          else skinny_store<EPI>(p, sum, fetch, row0 + ch * rc + jj, n);
         }
       }
     }
@@ -384,16 +421,19 @@ cudaError_t gemm_skinny_prepare() {
   if (e == cudaSuccess) e = skinny_prepare_one<EPI_GELU_BF16, false>();
   if (e == cudaSuccess) e = skinny_prepare_one<EPI_QKV, false>();
   if (e == cudaSuccess) e = skinny_prepare_one<EPI_RESID, false>();
+  if (e == cudaSuccess) e = skinny_prepare_one<EPI_ARGMAX, false>();
   if (e == cudaSuccess) e = skinny_prepare_one<EPI_F32, true>();
   if (e == cudaSuccess) e = skinny_prepare_one<EPI_BF16, true>();
   if (e == cudaSuccess) e = skinny_prepare_one<EPI_GELU_BF16, true>();
   if (e == cudaSuccess) e = skinny_prepare_one<EPI_QKV, true>();
   if (e == cudaSuccess) e = skinny_prepare_one<EPI_RESID, true>();
+  if (e == cudaSuccess) e = skinny_prepare_one<EPI_ARGMAX, true>();
   return e;
 }
 
 bool gemm_skinny_supported(int epi, int R, int N, int K) {
-  return epi != EPI_ARGMAX && R >= 1 && R <= 512 && N % 8 == 0 && K % 8 == 0 && N >= 8;
+  (void)epi;
+  return R >= 1 && R <= 512 && N % 8 == 0 && K % 8 == 0 && N >= 8;
 }
 
 // Which of the two cluster-split modes, if any, beats the row-tiled kernels -- set from measurements in the step on B200
@@ -505,7 +545,7 @@ bool gemm_skinny_map(CUtensorMap *m, const void *base, uint64_t rows, uint64_t K
 // tmA / tmW: gemm_skinny_map over the activation rows (box of a.sk_rp rows) and the weight rows (box of 128 rows).
 // a.splits = cluster size, set before gemm_skinny_shape.
 cudaError_t launch_gemm_skinny(int epi, const CUtensorMap &tmA, const CUtensorMap &tmW, const GemmArgs &a, cudaStream_t st) {
-  if (a.nbatch != 1 || a.w_mn_major || a.sk_stages < 1 || epi == EPI_ARGMAX || a.N % 8 || a.K % 8 ||
+  if (a.nbatch != 1 || a.w_mn_major || a.sk_stages < 1 || a.N % 8 || a.K % 8 ||
       (a.sk_tiles_m <= 0 && !gemm_skinny_supported(epi, a.R, a.N, a.K)))
     return cudaErrorInvalidValue;
   if (a.sk_tiles_m > 0) {
@@ -515,6 +555,7 @@ cudaError_t launch_gemm_skinny(int epi, const CUtensorMap &tmA, const CUtensorMa
       case EPI_GELU_BF16: return skinny_launch_one<EPI_GELU_BF16, true>(tmA, tmW, a, st);
       case EPI_QKV: return skinny_launch_one<EPI_QKV, true>(tmA, tmW, a, st);
       case EPI_RESID: return skinny_launch_one<EPI_RESID, true>(tmA, tmW, a, st);
+      case EPI_ARGMAX: return skinny_launch_one<EPI_ARGMAX, true>(tmA, tmW, a, st);
     }
     return cudaErrorInvalidValue;
   }
@@ -524,6 +565,7 @@ cudaError_t launch_gemm_skinny(int epi, const CUtensorMap &tmA, const CUtensorMa
     case EPI_GELU_BF16: return skinny_launch_one<EPI_GELU_BF16, false>(tmA, tmW, a, st);
     case EPI_QKV: return skinny_launch_one<EPI_QKV, false>(tmA, tmW, a, st);
     case EPI_RESID: return skinny_launch_one<EPI_RESID, false>(tmA, tmW, a, st);
+    case EPI_ARGMAX: return skinny_launch_one<EPI_ARGMAX, false>(tmA, tmW, a, st);
   }
   return cudaErrorInvalidValue;
 }

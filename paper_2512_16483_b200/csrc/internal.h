@@ -197,12 +197,13 @@ cudaError_t launch_tokens_to_f32(const bf16 *tok, float *x, int E, int M, int C,
 cudaError_t launch_out_to_bf16(const float *x, RowMap xmap, int E, int M, int C, bf16 *out, cudaStream_t st);
 cudaError_t launch_generate_projection(bf16 *qt, int M, int Mk, int r, unsigned long long seed, int group, int scale,
                                        cudaStream_t st);
-// Between two scale steps: codeword half-norms, the packed argmax words, Up-accumulate and area Down.
+// Between two scale steps: codeword half-norms, Up-accumulate and area Down.
 cudaError_t launch_half_norms(const bf16 *Z, int V, int C, float *hn, cudaStream_t st);
-cudaError_t launch_unpack_codes(const unsigned long long *best, long long n, int V, int *codes, unsigned *status,
-                                cudaStream_t st);
-cudaError_t launch_up_accumulate(const bf16 *Z, const int *codes, int B, int h0, int w0, int h1, int w1, int C,
-                                 bool overwrite, float *F, cudaStream_t st);
+// best: the arg-max words of the codeword search, one per source cell; codes (optional): where the decoded ones go;
+// clear[0 .. n_clear): zeroed for a later search (not `best`).
+cudaError_t launch_up_accumulate(const bf16 *Z, const unsigned long long *best, int V, int B, int h0, int w0, int h1, int w1, int C,
+                                 bool overwrite, float *F, int *codes, unsigned long long *clear, long long n_clear, unsigned *status,
+                                 cudaStream_t st);
 cudaError_t launch_cfg_combine(const bf16 *pair, int pairs, long long per_elem, float s, bf16 *out, cudaStream_t st);
 // dup: every element is written twice, [2B][h1 * w1][C] (the two branches of a CFG pair).
 cudaError_t launch_down_area(const float *F, int B, int h0, int w0, int h1, int w1, int C, bf16 *tokens, bool dup, cudaStream_t st);

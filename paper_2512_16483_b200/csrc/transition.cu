@@ -1,7 +1,7 @@
 // Kernels of the transition between two scale steps (the paper's Algorithm 1, "Vanilla VAR" lines;
 // Eq. "var_upf", Eq. "var_downf"): R_k = Q(F_k^o), F_k = F_{k-1} + Up(R_k, (h_K, w_K)), next input =
 // Down(F_k, (h_{k+1}, w_{k+1})).  Q is the nearest codeword: its scores F_k^o Z^T - |Z_v|^2 / 2 come from the
-// tensor-core GEMM with the arg-max epilogue; the kernels here supply the half-norms, unpack the winning
+// tensor-core GEMM with the arg-max epilogue; the kernels here supply the half-norms, decode the winning
 // columns, gather + upsample + accumulate the codewords (HBM-bound, 16-byte accesses) and average the
 // accumulated map down to the next scale.
 #include "internal.h"
@@ -36,51 +36,57 @@ cudaError_t launch_half_norms(const bf16 *Z, int V, int C, float *hn, cudaStream
   return cudaGetLastError();
 }
 
-// The winning column of every row out of its packed word (low half = ~column).  A row no tile wrote
-// (word still zero) or a column out of range flags the status word and yields code 0.
-__global__ void __launch_bounds__(256) unpack_codes_kernel(const unsigned long long *__restrict__ best, long long n, int V,
-                                                           int *__restrict__ codes, unsigned *status) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const unsigned long long w = best[i];
-  const unsigned c = 0xFFFFFFFFu - static_cast<unsigned>(w & 0xFFFFFFFFull);
-  const bool bad = (w == 0ull) || c >= static_cast<unsigned>(V);
-  if (bad) atomicOr(status, kStatusBadIndex);
-  codes[i] = bad ? 0 : static_cast<int>(c);
-}
-
-cudaError_t launch_unpack_codes(const unsigned long long *best, long long n, int V, int *codes, unsigned *status,
-                                cudaStream_t st) {
-  if (n <= 0) return cudaSuccess;
-  return launch_pdl(unpack_codes_kernel, dim3(static_cast<unsigned>((n + 255) / 256)), dim3(256), 0, st, best, n, V, codes, status);
+// The winning column of a row out of its packed word (low half = ~column).  A row no tile wrote (word still zero)
+// or a column out of range yields code 0.
+__device__ __forceinline__ int code_of(unsigned long long word, int V, bool *bad) {
+  const unsigned c = 0xFFFFFFFFu - static_cast<unsigned>(word & 0xFFFFFFFFull);
+  *bad = (word == 0ull) || c >= static_cast<unsigned>(V);
+  return *bad ? 0 : static_cast<int>(c);
 }
 
 // F[b][p][:] (+)= sum over the four bilinear neighbours of pixel p on the (h0, w0) grid of weight x
-// Z[codes[b][neighbour]][:] (half-pixel centres, source coordinate clamped at 0, neighbours clamped at the
+// Z[code of neighbour][:] (half-pixel centres, source coordinate clamped at 0, neighbours clamped at the
 // edge: the library's Up).  One warp per target pixel; fp32 accumulator map.  C % 8 == 0.
-__global__ void __launch_bounds__(256) up_accumulate_kernel(const bf16 *__restrict__ Z, const int *__restrict__ codes, int B,
-                                                            int h0, int w0, int h1, int w1, int C, int overwrite,
-                                                            float *__restrict__ F) {
+// The codes are decoded from the arg-max words where they are used; the grid's threads also write them out for the
+// caller, flag the status word for a bad one, and zero the words the next codeword search will use (`clear`: a second
+// buffer, nobody's by now) -- in a chain of 3 us launches the memset, the unpacking kernel and the copy were half of
+// the transition's launches.  Bound by the map (8 C bytes a pixel, from L2 while it fits) and the gathered
+// codewords (as much again): B = 1, 64 x 64, C = 2048 14 us; with the three launches it replaces 24.
+__global__ void __launch_bounds__(256) up_accumulate_kernel(const bf16 *__restrict__ Z, const unsigned long long *__restrict__ best,
+                                                            int V, int B, int h0, int w0, int h1, int w1, int C, int overwrite,
+                                                            float *__restrict__ F, int *__restrict__ codes,
+                                                            unsigned long long *__restrict__ clear, long long n_clear, unsigned *status) {
   pdl_wait();
   pdl_launch_dependents();
   const int M1 = h1 * w1;
-  const long long gw = static_cast<long long>(blockIdx.x) * 8 + (threadIdx.x >> 5);
+  const long long n_codes = static_cast<long long>(B) * h0 * w0, nthreads = static_cast<long long>(gridDim.x) * blockDim.x;
+  const long long tid = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+  bool bad;
+  for (long long i = tid; i < n_codes; i += nthreads) {
+    const int c = code_of(best[i], V, &bad);
+    if (bad) atomicOr(status, kStatusBadIndex);
+    if (codes != nullptr) codes[i] = c;
+  }
+  for (long long i = tid; i < n_clear; i += nthreads) clear[i] = 0ull;
+  const long long gw = tid >> 5;
   if (gw >= static_cast<long long>(B) * M1) return;
   const int b = static_cast<int>(gw / M1), i = static_cast<int>(gw - static_cast<long long>(b) * M1);
   const int y = i / w1, xq = i - y * w1;
   const BilinearTap tap = bilinear_tap(y, xq, h0, w0, h1, w1);
   const int y0 = tap.y0, y1 = tap.y1, x0 = tap.x0, x1 = tap.x1;
-  const int *cb = codes + static_cast<long long>(b) * h0 * w0;
-  const uint4 *p00 = reinterpret_cast<const uint4 *>(Z + static_cast<long long>(__ldg(cb + y0 * w0 + x0)) * C);
-  const uint4 *p01 = reinterpret_cast<const uint4 *>(Z + static_cast<long long>(__ldg(cb + y0 * w0 + x1)) * C);
-  const uint4 *p10 = reinterpret_cast<const uint4 *>(Z + static_cast<long long>(__ldg(cb + y1 * w0 + x0)) * C);
-  const uint4 *p11 = reinterpret_cast<const uint4 *>(Z + static_cast<long long>(__ldg(cb + y1 * w0 + x1)) * C);
+  const unsigned long long *wb = best + static_cast<long long>(b) * h0 * w0;
+  auto row = [&](int yy, int xx) { return reinterpret_cast<const uint4 *>(Z + static_cast<long long>(code_of(__ldg(wb + yy * w0 + xx), V, &bad)) * C); };
+  const uint4 *p00 = row(y0, x0), *p01 = row(y0, x1), *p10 = row(y1, x0), *p11 = row(y1, x1);
   const float w00 = tap.w00, w01 = tap.w01, w10 = tap.w10, w11 = tap.w11;
   float4 *dst = reinterpret_cast<float4 *>(F + (static_cast<long long>(b) * M1 + i) * C);
+#pragma unroll 2
   for (int g = threadIdx.x & 31; g < C / 8; g += 32) {
     const uint4 a = __ldg(p00 + g), bq = __ldg(p01 + g), cq = __ldg(p10 + g), d = __ldg(p11 + g);
+    float4 plo = make_float4(0.f, 0.f, 0.f, 0.f), phi = plo;
+    if (!overwrite) {
+      plo = dst[2 * g];
+      phi = dst[2 * g + 1];
+    }
     const __nv_bfloat162 *ha = reinterpret_cast<const __nv_bfloat162 *>(&a), *hb = reinterpret_cast<const __nv_bfloat162 *>(&bq);
     const __nv_bfloat162 *hc = reinterpret_cast<const __nv_bfloat162 *>(&cq), *hd = reinterpret_cast<const __nv_bfloat162 *>(&d);
     float o[8];
@@ -91,85 +97,87 @@ __global__ void __launch_bounds__(256) up_accumulate_kernel(const bf16 *__restri
       o[2 * t] = w00 * fa.x + w01 * fb.x + w10 * fc.x + w11 * fd.x;
       o[2 * t + 1] = w00 * fa.y + w01 * fb.y + w10 * fc.y + w11 * fd.y;
     }
-    float4 lo = make_float4(o[0], o[1], o[2], o[3]), hi = make_float4(o[4], o[5], o[6], o[7]);
-    if (!overwrite) {
-      const float4 plo = dst[2 * g], phi = dst[2 * g + 1];
-      lo.x += plo.x; lo.y += plo.y; lo.z += plo.z; lo.w += plo.w;
-      hi.x += phi.x; hi.y += phi.y; hi.z += phi.z; hi.w += phi.w;
-    }
-    dst[2 * g] = lo;
-    dst[2 * g + 1] = hi;
+    dst[2 * g] = make_float4(o[0] + plo.x, o[1] + plo.y, o[2] + plo.z, o[3] + plo.w);
+    dst[2 * g + 1] = make_float4(o[4] + phi.x, o[5] + phi.y, o[6] + phi.z, o[7] + phi.w);
   }
 }
 
-cudaError_t launch_up_accumulate(const bf16 *Z, const int *codes, int B, int h0, int w0, int h1, int w1, int C,
-                                 bool overwrite, float *F, cudaStream_t st) {
+cudaError_t launch_up_accumulate(const bf16 *Z, const unsigned long long *best, int V, int B, int h0, int w0, int h1, int w1, int C,
+                                 bool overwrite, float *F, int *codes, unsigned long long *clear, long long n_clear, unsigned *status,
+                                 cudaStream_t st) {
   const long long warps = static_cast<long long>(B) * h1 * w1;
   if (warps <= 0) return cudaSuccess;
   if (C % 8 != 0) return cudaErrorInvalidValue;
-  return launch_pdl(up_accumulate_kernel, dim3(static_cast<unsigned>((warps + 7) / 8)), dim3(256), 0, st, Z, codes, B, h0, w0,
-                    h1, w1, C, overwrite ? 1 : 0, F);
+  return launch_pdl(up_accumulate_kernel, dim3(static_cast<unsigned>((warps + 7) / 8)), dim3(256), 0, st, Z, best, V, B, h0, w0,
+                    h1, w1, C, overwrite ? 1 : 0, F, codes, clear, n_clear, status);
 }
 
 // tokens[b][q][:] = mean of F over the source cells target cell q = (y, x) of the (h1, w1) grid covers:
-// rows [floor(y h0 / h1), ceil((y + 1) h0 / h1)), columns likewise ("area" resampling); bf16 out.
-// One warp per target cell: the lanes walk the channels four float4 groups at a time (so that several
-// loads per lane are in flight), the window cell by cell inside.  C % 4 == 0.
-__global__ void __launch_bounds__(256) down_area_kernel(const float *__restrict__ F, int B, int h0, int w0, int h1, int w1,
-                                                        int C, bf16 *__restrict__ tokens, int dup) {
+// rows [floor(y h0 / h1), ceil((y + 1) h0 / h1)), columns likewise ("area" resampling); bf16 out.  C % 4 == 0.
+// A thread owns four channels of one target cell; G groups of threads share the window's cells (group g takes cells g,
+// g + G, ...) and their partial sums are added in group order through shared memory.  Bound by latency while the target
+// has few cells -- the map is in L2 then -- so G grows until about two thousand threads an SM are at work.  One warp a
+// cell with all channels, the form before, took 95 us for a 2 x 2 target of a 64 x 64 map with C = 2048 and 15 - 17 us
+// from 16 x 16 to 40 x 40; now 9 - 10.
+template <int G>
+__global__ void __launch_bounds__(256) down_area_kernel(const float *__restrict__ F, int h0, int w0, int h1, int w1, int C, int slabs,
+                                                        bf16 *__restrict__ tokens, int dup) {
+  constexpr int kLanes = 256 / G;
+  __shared__ float4 part[G > 1 ? 256 : 1];
   pdl_wait();
   pdl_launch_dependents();
-  const int M1 = h1 * w1, lane = threadIdx.x & 31;
-  const long long cell = static_cast<long long>(blockIdx.x) * 8 + (threadIdx.x >> 5);
-  if (cell >= static_cast<long long>(B) * M1) return;
-  const int b = static_cast<int>(cell / M1), q = static_cast<int>(cell - static_cast<long long>(b) * M1);
+  const int M1 = h1 * w1, b = blockIdx.y, q = blockIdx.x / slabs, slab = blockIdx.x - q * slabs;
   const int y = q / w1, x = q - y * w1;
   const int ya = (y * h0) / h1, yb = ((y + 1) * h0 + h1 - 1) / h1;
   const int xa = (x * w0) / w1, xb = ((x + 1) * w0 + w1 - 1) / w1;
-  const float inv = 1.0f / static_cast<float>((yb - ya) * (xb - xa));
-  const float4 *src = reinterpret_cast<const float4 *>(F + static_cast<long long>(b) * h0 * w0 * C);
-  // dup: element b is written twice, as elements 2b and 2b + 1 (both branches of a CFG pair read the same tokens)
-  uint2 *dst = reinterpret_cast<uint2 *>(tokens + (static_cast<long long>(dup ? 2 * b : b) * M1 + q) * C);
-  const long long dup_off = static_cast<long long>(M1) * C / 4;      // one element further on, in uint2 units
-  const int ngroups = C / 4, row4 = C / 4;
-  for (int g0 = lane; g0 < ngroups; g0 += 128) {
-    float4 acc[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int yy = ya; yy < yb; ++yy)
-      for (int xx = xa; xx < xb; ++xx) {
-        const float4 *cellp = src + (static_cast<long long>(yy) * w0 + xx) * row4;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int g = g0 + 32 * u;
-          if (g < ngroups) {
-            const float4 v = __ldg(cellp + g);
-            acc[u].x += v.x; acc[u].y += v.y; acc[u].z += v.z; acc[u].w += v.w;
-          }
-        }
-      }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int g = g0 + 32 * u;
-      if (g < ngroups) {
-        const __nv_bfloat162 o0 = __floats2bfloat162_rn(acc[u].x * inv, acc[u].y * inv);
-        const __nv_bfloat162 o1 = __floats2bfloat162_rn(acc[u].z * inv, acc[u].w * inv);
-        uint2 pk;
-        pk.x = *reinterpret_cast<const uint32_t *>(&o0);
-        pk.y = *reinterpret_cast<const uint32_t *>(&o1);
-        dst[g] = pk;
-        if (dup) dst[g + dup_off] = pk;
-      }
+  const int nx = xb - xa, cells = (yb - ya) * nx;
+  const int grp = threadIdx.x / kLanes, c4 = slab * kLanes + threadIdx.x % kLanes;      // this thread's four channels
+  const bool in = c4 < C / 4;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (in) {
+    const float4 *src = reinterpret_cast<const float4 *>(F + static_cast<long long>(b) * h0 * w0 * C) + c4;
+#pragma unroll 4
+    for (int i = grp; i < cells; i += G) {
+      const int yy = ya + i / nx, xx = xa + i % nx;
+      const float4 v = __ldg(src + (static_cast<long long>(yy) * w0 + xx) * (C / 4));
+      acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
     }
+  }
+  if constexpr (G > 1) {
+    part[threadIdx.x] = acc;
+    __syncthreads();
+    if (grp > 0) return;
+#pragma unroll
+    for (int t = 1; t < G; ++t) {
+      const float4 v = part[t * kLanes + threadIdx.x];
+      acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+    }
+  }
+  if (in) {
+    const float inv = 1.0f / static_cast<float>(cells);
+    const __nv_bfloat162 o0 = __floats2bfloat162_rn(acc.x * inv, acc.y * inv), o1 = __floats2bfloat162_rn(acc.z * inv, acc.w * inv);
+    const uint2 pk = make_uint2(*reinterpret_cast<const uint32_t *>(&o0), *reinterpret_cast<const uint32_t *>(&o1));
+    // dup: element b is written twice, as elements 2b and 2b + 1 (both branches of a CFG pair read the same tokens)
+    uint2 *dst = reinterpret_cast<uint2 *>(tokens + (static_cast<long long>(dup ? 2 * b : b) * M1 + q) * C) + c4;
+    dst[0] = pk;
+    if (dup) dst[static_cast<long long>(M1) * C / 4] = pk;
   }
 }
 
+template <int G>
+static cudaError_t launch_down(const float *F, int B, int h0, int w0, int h1, int w1, int C, bf16 *tokens, bool dup, cudaStream_t st) {
+  const int slabs = (C / 4 + 256 / G - 1) / (256 / G);
+  return launch_pdl(down_area_kernel<G>, dim3(static_cast<unsigned>(h1 * w1 * slabs), B), dim3(256), 0, st, F, h0, w0, h1, w1, C, slabs, tokens, dup ? 1 : 0);
+}
+
 cudaError_t launch_down_area(const float *F, int B, int h0, int w0, int h1, int w1, int C, bf16 *tokens, bool dup, cudaStream_t st) {
-  if (C % 4 != 0) return cudaErrorInvalidValue;
-  const long long warps = static_cast<long long>(B) * h1 * w1;
-  if (warps <= 0) return cudaSuccess;
-  return launch_pdl(down_area_kernel, dim3(static_cast<unsigned>((warps + 7) / 8)), dim3(256), 0, st, F, B, h0, w0, h1, w1, C,
-                    tokens, dup ? 1 : 0);
+  if (C % 4 != 0 || B > 65535) return cudaErrorInvalidValue;
+  if (B <= 0 || h1 <= 0 || w1 <= 0) return cudaSuccess;
+  const double threads = static_cast<double>(B) * h1 * w1 * (C / 4), cells = static_cast<double>(h0) * w0 / (static_cast<double>(h1) * w1);
+  const double want = 300000.0 / threads < cells ? 300000.0 / threads : cells;      // groups for 148 x 2048 threads, at most one a cell
+  if (want > 8.0) return launch_down<16>(F, B, h0, w0, h1, w1, C, tokens, dup, st);
+  if (want > 2.0) return launch_down<4>(F, B, h0, w0, h1, w1, C, tokens, dup, st);
+  return launch_down<1>(F, B, h0, w0, h1, w1, C, tokens, dup, st);
 }
 
 // Classifier-free guidance on CFG pairs: out[p] = null + s (prompt - null) with (prompt, null) = elements

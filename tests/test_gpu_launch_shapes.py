@@ -3,7 +3,8 @@ several units of work in one thread block.  Each against a plain PyTorch fp32 re
 import pytest
 import torch
 
-from helpers import rel_err
+import synth_inputs as si
+from helpers import rel_err, to_bf16_cuda, weights_to_cuda
 
 pytestmark = pytest.mark.gpu
 
@@ -42,3 +43,28 @@ def test_attention_launch_shapes(fv, B, H, D, r, L):
     # P and the result are rounded to bf16 (2^-8 of the value at most each); sharp rows are many times the RMS
     bad = (out.float() - ref).abs() - (2.0 ** -6 * ref.abs() + 3e-2 * ref.square().mean().sqrt())
     assert bad.max() <= 0 and cos >= 0.9999, (float(bad.max()), cos)
+
+
+@pytest.mark.parametrize("V", [8, 1000, 2048, 4104])
+def test_transitions_repeat_on_one_context(fv, V):
+    """Codeword search in every form its rule takes (1 to 512 rows, few and many codewords); the chain run twice on one
+    context gives the same codes, map and tokens, and the codes are those of the fp32 scores."""
+    shp, B = si.shape_tiny(n_blocks=1, scales=(1, 2, 3, 8, 16)), 2
+    ctx = fv.Fvar(weights_to_cuda(si.make_weights(5, shp)), blocks_per_group=1, n_heads=shp.n_heads, head_dim=shp.head_dim,
+                  ffn_dim=shp.ffn_dim, scale_hw=shp.hw(), max_batch=B, ctx_len=0, ctx_width=0)
+    Ms, C = shp.tokens_per_scale(), shp.width
+    Z = to_bf16_cuda(si.make_codebook(6, V, C))
+    ctx.set_codebook(Z)
+    got = []
+    for _ in range(2):
+        run = []
+        for k in range(len(Ms)):
+            fo = to_bf16_cuda(si.make_step_outputs(7, k, B, Ms[k], si.make_codebook(6, V, C), 0.1))
+            codes, nxt = ctx.scale_transition(fo, k, Ms[k + 1] if k + 1 < len(Ms) else None, pairs=True)
+            score = fo.float() @ Z.float().T - 0.5 * Z.float().square().sum(-1)
+            assert torch.equal(codes.long(), score.argmax(-1)), k
+            run += [codes.clone()] + ([nxt.clone()] if nxt is not None else [])
+        got.append(run + [ctx.get_feature(B, Ms[-1], C)])
+    assert ctx.poll_status() == fv.OK
+    for a, b in zip(*got):
+        assert torch.equal(a, b)

@@ -203,24 +203,19 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       const uint32_t aphase = (it >> 1) & 1u;
       const int row_local = quad * 32 + lane;
       const int row = m_idx * kBlockM + row_local;
-      // The residual rows of the first two column chunks are fetched while the main loop still runs:
-      // with one tile per CTA nothing else hides that latency.
+      // The residual of the first two column chunks is fetched while the main loop still runs: with one tile per CTA
+      // nothing else hides that latency; later chunks are fetched two ahead.
       constexpr int kPre = (kChunks < 2) ? kChunks : 2;
       float4 pre[kPre][8];
-      bool have_pre = false;
+      ResidRow rr{-1, 0, 0, 0};
+      auto col_of = [&](int ci) { return n_idx * BN + (ci * kEpiColGroups + cg) * 32; };
+      auto in_tile = [&](int ci) { return (ci * kEpiColGroups + cg) * 32 < BN && col_of(ci) < p.N; };    // uniform across the warp
       if constexpr (EPI == EPI_RESID) {
-        if (splits == 1 && row < p.R) {
-          const int e2 = row / p.rows_per_batch, j2 = row - e2 * p.rows_per_batch;
-          const float *res = p.resid + (static_cast<long long>(e2 * p.rmap.bmul + p.rmap.boff) * p.rmap.rpb + j2) * p.ld_out + n_idx * BN;
+        rr = resid_row(p, row);
+        if (splits == 1) {
 #pragma unroll
-          for (int ci = 0; ci < kPre; ++ci) {
-            const int c = ci * kEpiColGroups + cg;
-            if (n_idx * BN + c * 32 < p.N) {
-#pragma unroll
-              for (int q = 0; q < 8; ++q) pre[ci][q] = reinterpret_cast<const float4 *>(res + c * 32)[q];
-            }
-          }
-          have_pre = true;
+        for (int ci = 0; ci < kPre; ++ci)
+          if (in_tile(ci)) resid_fetch(p, rr, col_of(ci), lane, pre[ci]);
         }
       }
       ok = __all_sync(0xffffffffu, mbar_wait(tfull_bar(a), aphase, p.status, &abort_flag, wb));
@@ -228,20 +223,23 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       tc_fence_after();
       const uint32_t taddr = tmem_base + a * BN + (static_cast<uint32_t>(quad * 32) << 16);
       if (splits == 1) {
-        auto do_chunk = [&](int ci, const float4 *prep) {
-          const int c = ci * kEpiColGroups + cg;
-          const int col0 = n_idx * BN + c * 32;
-          if (c * 32 < BN && col0 < p.N) {       // uniform across the warp
-            uint32_t acc[32];
-            tmem_ld32(taddr + c * 32, acc);
-            tmem_ld_wait();
-            epilogue_chunk<EPI>(p, acc, e, row, col0, row < p.R, ep_stage, lane, prep);
-          }
-        };
-#pragma unroll
-        for (int ci = 0; ci < kPre; ++ci) do_chunk(ci, have_pre ? pre[ci] : nullptr);
 #pragma unroll 1
-        for (int ci = kPre; ci < kChunks; ++ci) do_chunk(ci, nullptr);
+        for (int c0 = 0; c0 < kChunks; c0 += kPre) {
+#pragma unroll
+          for (int u = 0; u < kPre; ++u) {
+            const int ci = c0 + u;
+            if (!in_tile(ci)) continue;
+            uint32_t acc[32];
+            tmem_ld32(taddr + (ci * kEpiColGroups + cg) * 32, acc);
+            tmem_ld_wait();
+            if constexpr (EPI == EPI_RESID) {
+              resid_chunk(p, acc, rr, col_of(ci), ep_stage, lane, pre[u]);
+              if (ci + kPre < kChunks && in_tile(ci + kPre)) resid_fetch(p, rr, col_of(ci + kPre), lane, pre[u]);
+            } else {
+              epilogue_chunk<EPI>(p, acc, e, row, col_of(ci), row < p.R, ep_stage, lane);
+            }
+          }
+        }
         tc_fence_before();
         mbar_arrive(tempty_bar(a));
       } else {
@@ -290,7 +288,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             uint32_t acc[32];
 #pragma unroll
             for (int i = 0; i < 32; ++i) acc[i] = __float_as_uint(sum[i]);
-            epilogue_chunk<EPI>(p, acc, e, row, col0, row < p.R, ep_stage, lane);
+            if constexpr (EPI == EPI_RESID) {
+              resid_fetch(p, rr, col0, lane, pre[0]);
+              resid_chunk(p, acc, rr, col0, ep_stage, lane, pre[0]);
+            } else {
+              epilogue_chunk<EPI>(p, acc, e, row, col0, row < p.R, ep_stage, lane);
+            }
           }
           if (threadIdx.x == 64) p.counters[tile] = 0;      // ready for the next launch
         }

@@ -85,12 +85,11 @@ __device__ __forceinline__ void warp_store_bf16(uint32_t stage, int lane, const 
   __syncwarp();
 }
 
-// Epilogue of one warp for 32 rows x 32 consecutive columns starting at col0 (col0 % 32 == 0): each
+// Epilogue (all but EPI_RESID) of one warp for 32 rows x 32 consecutive columns starting at col0 (col0 % 32 == 0): each
 // lane owns one row (`valid` false: row past the end).  Every lane of the warp must call.
 template <int EPI>
 __device__ __forceinline__ void epilogue_chunk(const GemmArgs &p, const uint32_t (&acc)[32], int batch, int row,
-                                               int col0, bool valid, uint32_t stage, int lane,
-                                               const float4 *resid_pre = nullptr) {
+                                               int col0, bool valid, uint32_t stage, int lane) {
   float v[32];
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(acc[i]);
@@ -165,40 +164,79 @@ __device__ __forceinline__ void epilogue_chunk(const GemmArgs &p, const uint32_t
 #pragma unroll
       for (int i = 0; i < 32; ++i) base[static_cast<long long>(i) * p.L_cap] = __float2bfloat16_rn(v[i]);
     }
-  } else {  // EPI_RESID
-    float *dst = nullptr;
-    if (valid) {
-      const int e = row / p.rows_per_batch, j = row - e * p.rows_per_batch;
-      const int b = e * p.bmul + p.boff;
-      const float *res = p.resid + (static_cast<long long>(e * p.rmap.bmul + p.rmap.boff) * p.rmap.rpb + j) * p.ld_out + col0;
-      const int jo = p.scatter ? __ldg(p.scatter + static_cast<long long>(e) * p.rows_per_batch + j) : j;
-      dst = p.out_f32 + (static_cast<long long>(e * p.omap.bmul + p.omap.boff) * p.omap.rpb + jo) * p.ld_out + col0;
-      const float *g = p.gate ? p.gate + static_cast<long long>(b) * p.gate_stride + col0 : nullptr;
+  }
+}
+
+// Rows of the residual epilogue as a warp shares them: lane l holds where row l of its 32 rows goes and what it adds to.
+struct ResidRow {
+  int out, res, b, split;      // output row (-1: past the end), residual row, caller batch element, row of the hi half
+};
+__device__ __forceinline__ ResidRow resid_row(const GemmArgs &p, int row) {
+  ResidRow r{-1, 0, 0, 0};
+  if (row < p.R) {
+    const int e = row / p.rows_per_batch, j = row - e * p.rows_per_batch;
+    const int jo = p.scatter ? __ldg(p.scatter + static_cast<long long>(e) * p.rows_per_batch + j) : j;
+    r.b = e * p.bmul + p.boff;
+    r.res = (e * p.rmap.bmul + p.rmap.boff) * p.rmap.rpb + j;
+    r.out = (e * p.omap.bmul + p.omap.boff) * p.omap.rpb + jo;
+    r.split = e * 2 * p.xsplit_mk + jo;
+  }
+  return r;
+}
+// The residual values of one 32-column chunk in the order the epilogue wants them: lane l, step it holds 4 columns of
+// row 4 it + l / 8, so that eight lanes read 128 consecutive bytes.  (A row a lane, every access of a warp touched 32
+// lines and half of the sectors came from L2 twice.)
+__device__ __forceinline__ void resid_fetch(const GemmArgs &p, const ResidRow &rr, int col0, int lane, float4 (&pre)[8]) {
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        float4 r4 = resid_pre ? resid_pre[q] : reinterpret_cast<const float4 *>(res)[q];
-        float4 g4 = g ? __ldg(reinterpret_cast<const float4 *>(g) + q) : make_float4(1.f, 1.f, 1.f, 1.f);
-        v[q * 4] = fmaf(g4.x, v[q * 4], r4.x);
-        v[q * 4 + 1] = fmaf(g4.y, v[q * 4 + 1], r4.y);
-        v[q * 4 + 2] = fmaf(g4.z, v[q * 4 + 2], r4.z);
-        v[q * 4 + 3] = fmaf(g4.w, v[q * 4 + 3], r4.w);
-      }
-    }
-    warp_store_f32(stage, lane, v, dst);
-    if (p.xsplit != nullptr) {                   // uniform across the grid
-      bf16 *hi = nullptr;
-      if (valid) {
-        const int e = row / p.rows_per_batch, j = row - e * p.rows_per_batch;
-        const int jo = p.scatter ? __ldg(p.scatter + static_cast<long long>(e) * p.rows_per_batch + j) : j;
-        hi = p.xsplit + (static_cast<long long>(e) * 2 * p.xsplit_mk + jo) * p.ld_out + col0;
-      }
-      float lo[32];
+  for (int it = 0; it < 8; ++it) {
+    const int r = it * 4 + (lane >> 3);
+    const int out = __shfl_sync(0xffffffffu, rr.out, r), res = __shfl_sync(0xffffffffu, rr.res, r);
+    if (out >= 0) pre[it] = *reinterpret_cast<const float4 *>(p.resid + static_cast<long long>(res) * p.ld_out + col0 + (lane & 7) * 4);
+  }
+}
+// EPI_RESID of one warp for its 32 rows x 32 columns starting at col0 (col0 + 32 <= N).  Every lane must call.
+__device__ __forceinline__ void resid_chunk(const GemmArgs &p, const uint32_t (&acc)[32], const ResidRow &rr, int col0, uint32_t stage, int lane,
+                                            const float4 (&pre)[8]) {
 #pragma unroll
-      for (int i = 0; i < 32; ++i) lo[i] = v[i] - __bfloat162float(__float2bfloat16_rn(v[i]));
-      warp_store_bf16(stage, lane, v, hi);
-      warp_store_bf16(stage, lane, lo, hi ? hi + static_cast<long long>(p.xsplit_mk) * p.ld_out : nullptr);
+  for (int q = 0; q < 8; ++q)
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stage + lane * 128 + ((q ^ (lane & 7)) << 4)), "r"(acc[q * 4]), "r"(acc[q * 4 + 1]),
+                 "r"(acc[q * 4 + 2]), "r"(acc[q * 4 + 3]) : "memory");
+  const int c = lane & 7, col = col0 + c * 4;
+  float bias[4] = {0.f, 0.f, 0.f, 0.f};
+  if (p.bias != nullptr) {
+    const uint2 u = __ldg(reinterpret_cast<const uint2 *>(p.bias + col));
+    const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&u);
+    const float2 f0 = __bfloat1622float2(h[0]), f1 = __bfloat1622float2(h[1]);
+    bias[0] = f0.x; bias[1] = f0.y; bias[2] = f1.x; bias[3] = f1.y;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int it = 0; it < 8; ++it) {
+    const int r = it * 4 + (lane >> 3);
+    const int out = __shfl_sync(0xffffffffu, rr.out, r), b = __shfl_sync(0xffffffffu, rr.b, r), split = __shfl_sync(0xffffffffu, rr.split, r);
+    float4 o;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(o.x), "=f"(o.y), "=f"(o.z), "=f"(o.w)
+                 : "r"(stage + r * 128 + ((c ^ (r & 7)) << 4)));
+    if (out >= 0) {
+      const float4 g = p.gate ? __ldg(reinterpret_cast<const float4 *>(p.gate + static_cast<long long>(b) * p.gate_stride + col))
+                              : make_float4(1.f, 1.f, 1.f, 1.f);
+      o.x = fmaf(g.x, o.x + bias[0], pre[it].x);
+      o.y = fmaf(g.y, o.y + bias[1], pre[it].y);
+      o.z = fmaf(g.z, o.z + bias[2], pre[it].z);
+      o.w = fmaf(g.w, o.w + bias[3], pre[it].w);
+      *reinterpret_cast<float4 *>(p.out_f32 + static_cast<long long>(out) * p.ld_out + col) = o;
+      if (p.xsplit != nullptr) {
+        bf16 *hi = p.xsplit + static_cast<long long>(split) * p.ld_out + col;
+        const uint2 h2 = make_uint2(pack_bf16(o.x, o.y), pack_bf16(o.z, o.w));
+        const __nv_bfloat162 *hh = reinterpret_cast<const __nv_bfloat162 *>(&h2);
+        const float2 f0 = __bfloat1622float2(hh[0]), f1 = __bfloat1622float2(hh[1]);
+        *reinterpret_cast<uint2 *>(hi) = h2;
+        *reinterpret_cast<uint2 *>(hi + static_cast<long long>(p.xsplit_mk) * p.ld_out) =
+            make_uint2(pack_bf16(o.x - f0.x, o.y - f0.y), pack_bf16(o.z - f1.x, o.w - f1.y));
+      }
     }
   }
+  __syncwarp();
 }
 
 }  // namespace fvar

@@ -203,171 +203,100 @@ cudaError_t launch_copy_indices(const int *forced, int B, int M, int r, int ld_f
 }
 
 // ------------------------------------------------------------------------------------------------
-// y = LN(x) * (1 + scale) + shift  (or LN(x) * gamma): one CTA of 128 threads per row, the row
-// held in registers (two-pass mean / variance), bf16 output, 16-byte accesses.
+// y = LN(x) * (1 + scale) + shift  (or LN(x) * gamma): one CTA of 128 threads per row, the row held in registers as T
+// float4 a thread (two-pass mean / variance), bf16 output.
+// In the step a row count of 2 .. 8192 is a launch of 1 - 18 us between two GEMMs, so it is the chain of latencies that
+// counts: the vectors a row is modulated with are requested together with the row, or before the wait for the preceding
+// kernel where the caller says that no kernel in flight writes them (`early`: the step's AdaLN vectors and gamma are
+// written by fvar_set_cond only).  Rows x columns, in a chain of such launches, against the form before (warp a row from
+// 4096 rows, vectors after the statistics): 16 x 2048 4.8 -> 1.4 us, 400 x 2048 5.6 -> 2.5, 2704 x 1024 5.1 -> 4.7,
+// 8192 x 2048 30 -> 18 (5.6 TB/s of 6.5).  A warp or two a row, or two rows a CTA, are level at best.
 constexpr int kLnThreads = 128;
-constexpr int kLnMaxVec = 8;                    // 8 x (8 elements) x 128 threads = 8192 columns
+constexpr int kLnMaxVec = 16;                   // float4 a thread: 8192 columns
 
-// Normalises, modulates (or scales by gamma) and stores one group of 8 consecutive elements of a row: group g of
-// the row whose values are in v, statistics mean / rstd; shift and scale at float offset voff, y row at yr.
-__device__ __forceinline__ void ln_store_group(const float (&v)[8], float mean, float rstd, const bf16 *__restrict__ gamma,
-                                               const float *__restrict__ scale, const float *__restrict__ shift, long long voff,
-                                               int g, bf16 *__restrict__ yr) {
-  float o[8];
-  if (gamma != nullptr) {
-    const uint4 gu = __ldg(reinterpret_cast<const uint4 *>(gamma) + g);
-    const __nv_bfloat162 *gh = reinterpret_cast<const __nv_bfloat162 *>(&gu);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float2 gf = __bfloat1622float2(gh[i]);
-      o[2 * i] = (v[2 * i] - mean) * rstd * gf.x;
-      o[2 * i + 1] = (v[2 * i + 1] - mean) * rstd * gf.y;
-    }
-  } else {
-    const float4 *sc = reinterpret_cast<const float4 *>(scale + voff) + 2 * g;
-    const float4 *sh = reinterpret_cast<const float4 *>(shift + voff) + 2 * g;
-    const float4 s0 = __ldg(sc), s1 = __ldg(sc + 1), h0 = __ldg(sh), h1 = __ldg(sh + 1);
-    const float scv[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
-    const float shv[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
-#pragma unroll
-    for (int i = 0; i < 8; ++i) o[i] = fmaf((v[i] - mean) * rstd, 1.0f + scv[i], shv[i]);
-  }
-  uint32_t w[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    __nv_bfloat162 h2 = __floats2bfloat162_rn(o[2 * i], o[2 * i + 1]);
-    w[i] = *reinterpret_cast<uint32_t *>(&h2);
-  }
-  reinterpret_cast<uint4 *>(yr)[g] = make_uint4(w[0], w[1], w[2], w[3]);
-}
-
-__global__ void __launch_bounds__(kLnThreads) ln_modulate_kernel(const float *__restrict__ x, RowMap xmap, int rows,
-                                                                 int C, const float *__restrict__ shift,
-                                                                 const float *__restrict__ scale,
-                                                                 long long vec_stride, int bmul, int boff,
-                                                                 const bf16 *__restrict__ gamma, float eps,
-                                                                 bf16 *__restrict__ y) {
-  pdl_launch_dependents();      // nothing precedes the wait: the successor may start its own prologue right away
-  pdl_wait();
-  __shared__ float red[kLnThreads / 32];
+template <int T>
+__global__ void __launch_bounds__(kLnThreads) ln_modulate_kernel(const float *__restrict__ x, RowMap xmap, int rows, int C,
+                                                                 const float *__restrict__ shift, const float *__restrict__ scale,
+                                                                 long long vec_stride, int bmul, int boff, const bf16 *__restrict__ gamma,
+                                                                 float eps, int early, bf16 *__restrict__ y) {
+  pdl_launch_dependents();      // nothing precedes the wait but loads: the successor may start its own prologue right away
+  __shared__ float red[2][kLnThreads / 32];
+  constexpr bool kHold = T <= 4;                // the vectors fit in registers beside the row
   const int e = blockIdx.x / rows, j = blockIdx.x - e * rows;
-  const float *xr = x + (static_cast<long long>(e * xmap.bmul + xmap.boff) * xmap.rpb + j) * C;
-  bf16 *yr = y + static_cast<long long>(blockIdx.x) * C;
-  const int nvec = C / 8;                       // 8-element groups in the row
-  float v[kLnMaxVec][8];
+  const int n4 = C / 4, tid = threadIdx.x;
+  const long long voff = static_cast<long long>(e * bmul + boff) * vec_stride;
+  float4 mul[kHold ? T : 1], add[kHold ? T : 1];
+  auto vec_mul = [&](int g) {                   // what the normalised value is multiplied with ...
+    if (gamma == nullptr) {
+      const float4 s = __ldg(reinterpret_cast<const float4 *>(scale + voff) + g);
+      return make_float4(1.0f + s.x, 1.0f + s.y, 1.0f + s.z, 1.0f + s.w);
+    }
+    const uint2 u = __ldg(reinterpret_cast<const uint2 *>(gamma) + g);
+    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.x)), b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.y));
+    return make_float4(a.x, a.y, b.x, b.y);
+  };
+  auto vec_add = [&](int g) {                   // ... and what is added
+    return gamma == nullptr ? __ldg(reinterpret_cast<const float4 *>(shift + voff) + g) : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  auto fetch_vecs = [&]() {
+#pragma unroll
+    for (int t = 0; t < T; ++t)
+      if (tid + t * kLnThreads < n4) { mul[kHold ? t : 0] = vec_mul(tid + t * kLnThreads); add[kHold ? t : 0] = vec_add(tid + t * kLnThreads); }
+  };
+  if (kHold && early) fetch_vecs();
+  pdl_wait();
+  if (kHold && !early) fetch_vecs();
+  const float4 *xr = reinterpret_cast<const float4 *>(x + (static_cast<long long>(e * xmap.bmul + xmap.boff) * xmap.rpb + j) * C);
+  float4 v[T];
   float sum = 0.f;
 #pragma unroll
-  for (int t = 0; t < kLnMaxVec; ++t) {
-    const int g = threadIdx.x + t * kLnThreads;
-    if (g < nvec) {
-      const float4 a = reinterpret_cast<const float4 *>(xr)[2 * g], c = reinterpret_cast<const float4 *>(xr)[2 * g + 1];
-      v[t][0] = a.x; v[t][1] = a.y; v[t][2] = a.z; v[t][3] = a.w;
-      v[t][4] = c.x; v[t][5] = c.y; v[t][6] = c.z; v[t][7] = c.w;
+  for (int t = 0; t < T; ++t) v[t] = tid + t * kLnThreads < n4 ? xr[tid + t * kLnThreads] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) sum += v[t][i];
-    }
-  }
-  auto block_sum = [&](float val) {
+  for (int t = 0; t < T; ++t) sum += (v[t].x + v[t].y) + (v[t].z + v[t].w);
+  auto block_sum = [&](float val, int k) {
     val = warp_sum(val);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = val;
+    if ((tid & 31) == 0) red[k][tid >> 5] = val;
     __syncthreads();
     float tot = 0.f;
 #pragma unroll
-    for (int w = 0; w < kLnThreads / 32; ++w) tot += red[w];
+    for (int w = 0; w < kLnThreads / 32; ++w) tot += red[k][w];
     return tot;
   };
-  const float mean = block_sum(sum) / C;
-  float sq = 0.f;
-#pragma unroll
-  for (int t = 0; t < kLnMaxVec; ++t) {
-    const int g = threadIdx.x + t * kLnThreads;
-    if (g < nvec) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float d = v[t][i] - mean;
-        sq = fmaf(d, d, sq);
-      }
-    }
-  }
-  const float rstd = rsqrtf(block_sum(sq) / C + eps);
-  const long long voff = static_cast<long long>(e * bmul + boff) * vec_stride;
-#pragma unroll
-  for (int t = 0; t < kLnMaxVec; ++t) {
-    const int g = threadIdx.x + t * kLnThreads;
-    if (g < nvec) {
-      ln_store_group(v[t], mean, rstd, gamma, scale, shift, voff, g, yr);
-    }
-  }
-}
-
-// Warp-per-row variant for C <= 256 * T: the row lives in the registers of one warp (T groups of 8
-// elements per lane), statistics by shuffles only, no block-wide barrier; 8 rows per CTA.
-template <int T>
-__global__ void __launch_bounds__(256) ln_modulate_warp_kernel(const float *__restrict__ x, RowMap xmap, int rows, int total_rows,
-                                                               int C, const float *__restrict__ shift,
-                                                               const float *__restrict__ scale, long long vec_stride,
-                                                               int bmul, int boff, const bf16 *__restrict__ gamma, float eps,
-                                                               bf16 *__restrict__ y) {
-  pdl_launch_dependents();      // nothing precedes the wait: the successor may start its own prologue right away
-  pdl_wait();
-  const int grow = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (grow >= total_rows) return;
-  const int lane = threadIdx.x & 31;
-  const int e = grow / rows, j = grow - e * rows;
-  const float *xr = x + (static_cast<long long>(e * xmap.bmul + xmap.boff) * xmap.rpb + j) * C;
-  bf16 *yr = y + static_cast<long long>(grow) * C;
-  const int nvec = C / 8;
-  float v[T][8];
-  float sum = 0.f;
-#pragma unroll
-  for (int t = 0; t < T; ++t) {
-    const int g = lane + t * 32;
-    if (g < nvec) {
-      const float4 a = __ldg(reinterpret_cast<const float4 *>(xr) + 2 * g), c = __ldg(reinterpret_cast<const float4 *>(xr) + 2 * g + 1);
-      v[t][0] = a.x; v[t][1] = a.y; v[t][2] = a.z; v[t][3] = a.w;
-      v[t][4] = c.x; v[t][5] = c.y; v[t][6] = c.z; v[t][7] = c.w;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) sum += v[t][i];
-    }
-  }
-  const float mean = warp_sum(sum) / C;
+  const float mean = block_sum(sum, 0) / C;
   float sq = 0.f;
 #pragma unroll
   for (int t = 0; t < T; ++t)
-    if (lane + t * 32 < nvec) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float d = v[t][i] - mean;
-        sq = fmaf(d, d, sq);
-      }
+    if (tid + t * kLnThreads < n4) {
+      const float a = v[t].x - mean, b = v[t].y - mean, c = v[t].z - mean, d = v[t].w - mean;
+      sq = fmaf(a, a, sq); sq = fmaf(b, b, sq); sq = fmaf(c, c, sq); sq = fmaf(d, d, sq);
     }
-  const float rstd = rsqrtf(warp_sum(sq) / C + eps);
-  const long long voff = static_cast<long long>(e * bmul + boff) * vec_stride;
+  const float rstd = rsqrtf(block_sum(sq, 1) / C + eps);
+  uint2 *yr = reinterpret_cast<uint2 *>(y + static_cast<long long>(blockIdx.x) * C);
 #pragma unroll
   for (int t = 0; t < T; ++t) {
-    const int g = lane + t * 32;
-    if (g < nvec) {
-      ln_store_group(v[t], mean, rstd, gamma, scale, shift, voff, g, yr);
+    const int g = tid + t * kLnThreads;
+    if (g < n4) {
+      const float4 m = kHold ? mul[kHold ? t : 0] : vec_mul(g), h = kHold ? add[kHold ? t : 0] : vec_add(g);
+      const __nv_bfloat162 o0 = __floats2bfloat162_rn(fmaf((v[t].x - mean) * rstd, m.x, h.x), fmaf((v[t].y - mean) * rstd, m.y, h.y));
+      const __nv_bfloat162 o1 = __floats2bfloat162_rn(fmaf((v[t].z - mean) * rstd, m.z, h.z), fmaf((v[t].w - mean) * rstd, m.w, h.w));
+      yr[g] = make_uint2(*reinterpret_cast<const uint32_t *>(&o0), *reinterpret_cast<const uint32_t *>(&o1));
     }
   }
 }
 
 cudaError_t launch_ln_modulate(const float *x, RowMap xmap, int E, int rows, int C, const float *shift,
                                const float *scale, long long vec_stride, int bmul, int boff, const bf16 *gamma,
-                               float eps, bf16 *y, cudaStream_t st) {
+                               float eps, bool early, bf16 *y, cudaStream_t st) {
   if (E * rows <= 0) return cudaSuccess;
-  if (C % 8 != 0 || C > 8 * kLnThreads * kLnMaxVec) return cudaErrorInvalidValue;
-  const int total = E * rows;
-  // few rows: a CTA per row finishes sooner (more threads per row); many rows: a warp per row streams better
-  if (total >= 4096 && C <= 1024)
-    return launch_pdl(ln_modulate_warp_kernel<4>, dim3((total + 7) / 8), dim3(256), 0, st, x, xmap, rows, total, C, shift, scale,
-                      vec_stride, bmul, boff, gamma, eps, y);
-  if (total >= 4096 && C <= 2048)
-    return launch_pdl(ln_modulate_warp_kernel<8>, dim3((total + 7) / 8), dim3(256), 0, st, x, xmap, rows, total, C, shift, scale,
-                      vec_stride, bmul, boff, gamma, eps, y);
-  return launch_pdl(ln_modulate_kernel, dim3(E * rows), dim3(kLnThreads), 0, st, x, xmap, rows, C, shift, scale, vec_stride, bmul, boff, gamma,
-                                                      eps, y);
+  if (C % 8 != 0 || C > 4 * kLnThreads * kLnMaxVec) return cudaErrorInvalidValue;
+  auto go = [&](auto kern) {
+    return launch_pdl(kern, dim3(E * rows), dim3(kLnThreads), 0, st, x, xmap, rows, C, shift, scale, vec_stride, bmul, boff, gamma, eps, early ? 1 : 0, y);
+  };
+  if (C <= 512) return go(ln_modulate_kernel<1>);
+  if (C <= 1024) return go(ln_modulate_kernel<2>);
+  if (C <= 2048) return go(ln_modulate_kernel<4>);
+  if (C <= 4096) return go(ln_modulate_kernel<8>);
+  return go(ln_modulate_kernel<16>);
 }
 
 // ------------------------------------------------------------------------------------------------

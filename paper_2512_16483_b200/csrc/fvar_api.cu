@@ -1160,7 +1160,7 @@ static fvar_status scale_step_impl(fvar_ctx *ctx, const void *tokens, bool token
 
       ctx->prof_begin(FVAR_KCLASS_LN, 0.0, 6.0 * R * C);
       FV_CUDA(ctx, launch_ln_modulate(in_ptr, in_map, E, r, C, ada, ada + C, 6 * C, bmul, boff, nullptr,
-                                      ctx->cfg.ln_eps, ctx->y, st), "ln_modulate 1");
+                                      ctx->cfg.ln_eps, true, ctx->y, st), "ln_modulate 1");
       ctx->launched();
       {
         GemmArgs ga = gemm_args(R, 3 * C, C);
@@ -1194,7 +1194,7 @@ static fvar_status scale_step_impl(fvar_ctx *ctx, const void *tokens, bool token
       if (ctx->cfg.has_cross_attn) {
         ctx->prof_begin(FVAR_KCLASS_LN, 0.0, 6.0 * R * C);
         FV_CUDA(ctx, launch_ln_modulate(ctx->xs, smap, E, r, C, nullptr, nullptr, 0, bmul, boff, ctx->ln_c_gamma[blk],
-                                        ctx->cfg.ln_eps, ctx->y, st), "ln cross");
+                                        ctx->cfg.ln_eps, true, ctx->y, st), "ln cross");
         ctx->launched();
         GemmArgs gq = gemm_args(R, C, C);
         gq.out_bf16 = ctx->q; gq.ld_out = C;
@@ -1214,7 +1214,7 @@ static fvar_status scale_step_impl(fvar_ctx *ctx, const void *tokens, bool token
       }
       ctx->prof_begin(FVAR_KCLASS_LN, 0.0, 6.0 * R * C);
       FV_CUDA(ctx, launch_ln_modulate(ctx->xs, smap, E, r, C, ada + 3 * C, ada + 4 * C, 6 * C, bmul, boff, nullptr,
-                                      ctx->cfg.ln_eps, ctx->y, st), "ln_modulate 2");
+                                      ctx->cfg.ln_eps, true, ctx->y, st), "ln_modulate 2");
       ctx->launched();
       {
         GemmArgs ga = gemm_args(R, F, C);
@@ -1515,7 +1515,7 @@ fvar_status fvar_ln_modulate(const float *x, int R, int C, int rows_per_batch, c
   if (!x || !y || !shift || !scale || R <= 0 || C <= 0 || C % 8 || C > 8192 || rows_per_batch <= 0 || R % rows_per_batch)
     return kfail(FVAR_EINVAL, "ln_modulate: bad arguments");
   FK_CUDA(launch_ln_modulate(x, RowMap{1, 0, rows_per_batch}, R / rows_per_batch, rows_per_batch, C, shift, scale,
-                             vec_stride, 1, 0, nullptr, eps, static_cast<bf16 *>(y), static_cast<cudaStream_t>(stream)),
+                             vec_stride, 1, 0, nullptr, eps, false, static_cast<bf16 *>(y), static_cast<cudaStream_t>(stream)),
           "ln_modulate");
   return FVAR_OK;
 }

@@ -183,9 +183,11 @@ cudaError_t launch_row_scores(const float *x, RowMap xmap, int E, int M, int C, 
 cudaError_t launch_select_topr(const float *scores, int B, int M, int r, int *idx, int *inv, cudaStream_t st);
 cudaError_t launch_copy_indices(const int *forced, int B, int M, int r, int ld_forced, int *idx, int *inv,
                                 unsigned *status, cudaStream_t st);
+// early: shift, scale and gamma are not written by any kernel that may still be in flight (they may then be read before
+// the preceding kernel has finished).
 cudaError_t launch_ln_modulate(const float *x, RowMap xmap, int E, int rows, int C, const float *shift,
                                const float *scale, long long vec_stride, int bmul, int boff,
-                               const bf16 *gamma, float eps, bf16 *y, cudaStream_t st);
+                               const bf16 *gamma, float eps, bool early, bf16 *y, cudaStream_t st);
 // xsplit (optional): the filled rows also go out as their two-term bf16 split, [E][2][mk][C] (see GemmArgs::xsplit).
 cudaError_t launch_rtr_fill(const float *prev, float *out, int E, int bmul, int boff, int h0, int w0, int h1,
                             int w1, int C, const int *inv, bf16 *xsplit, int mk, cudaStream_t st);

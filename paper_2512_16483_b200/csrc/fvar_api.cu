@@ -353,11 +353,8 @@ fvar_status cuda_fail(fvar_ctx *ctx, cudaError_t e, const char *what) {
     if (e__ != cudaSuccess) return cuda_fail(ctx, e__, what);   \
   } while (0)
 
-// out = A W^T (+ epilogue) on the context's stream; picks the tile width from the problem size.
-fvar_status run_gemm_map(fvar_ctx *ctx, int epi, const CUtensorMap &tmA, int blk, int wid, GemmArgs &g, const char *what);
-
-// A operand from one of the library's activation buffers: a single row tile takes the shortest box
-// that covers its rows.
+// out = A W^T (+ epilogue) on the context's stream; form and tile width from the problem size.  A operand: one of the
+// library's activation buffers; a single row tile takes the shortest box that covers its rows.
 fvar_status run_gemm(fvar_ctx *ctx, int epi, const fvar_ctx::ActMaps &maps, int blk, int wid, GemmArgs &g, const char *what) {
   if (g.nbatch == 1 && g.R <= ctx->skinny_max_rows && g.R <= gemm_skinny_row_limit(g.N, g.K) && !gemm_ksplit_wins(g.R, g.N, g.K) &&
       gemm_skinny_supported(epi, g.R, g.N, g.K)) {
@@ -403,17 +400,8 @@ fvar_status run_gemm(fvar_ctx *ctx, int epi, const fvar_ctx::ActMaps &maps, int 
     g.sk_tiles_m = 0;
     g.splits = 1;
   }
-  int t = 3;
-  if (g.nbatch == 1 && g.R <= 64) t = g.R <= 16 ? 0 : (g.R <= 32 ? 1 : 2);
-  g.a_box_rows = 16 << t;
-  return run_gemm_map(ctx, epi, maps.m[t], blk, wid, g, what);
-}
-
-fvar_status run_gemm_map(fvar_ctx *ctx, int epi, const CUtensorMap &tmA, int blk, int wid, GemmArgs &g, const char *what) {
-  // CTA pairs need the full 128-row A box (tmA is then the activation buffer's 128-row map)
-  const GemmPlan plan = gemm_plan(g.R, g.nbatch, g.N, g.K, ctx->num_sms, (g.a_box_rows == 128 || g.a_box_rows == 0) ? ctx->max_clusters : 0,
-                                  ctx->max_splits, kSplitScratchBytes);
-  const int bn = plan.block_n;
+  const GemmPlan plan = gemm_plan(g.R, g.nbatch, g.N, g.K, ctx->num_sms, ctx->max_clusters, ctx->max_splits, kSplitScratchBytes,
+                                  gemm_flex_supported(epi, g.N, g.K));
   g.splits = plan.splits;
   g.partial = ctx->split_partial;
   g.counters = ctx->split_counters;
@@ -422,10 +410,21 @@ fvar_status run_gemm_map(fvar_ctx *ctx, int epi, const CUtensorMap &tmA, int blk
   ctx->prof_begin(FVAR_KCLASS_GEMM, 2.0 * g.R * g.N * g.K * g.nbatch,
                   2.0 * (static_cast<double>(g.N) * g.K + static_cast<double>(g.R) * g.K * g.nbatch) +
                       (epi == EPI_F32 || epi == EPI_RESID ? 4.0 : 2.0) * g.R * g.N * g.nbatch);
-  if (plan.pair)
-    FV_CUDA(ctx, launch_gemm_pair(epi, bn, tmA, ctx->wm(blk, wid, bn / 2), g, ctx->launch_st), what);
-  else
-    FV_CUDA(ctx, launch_gemm(epi, bn, tmA, ctx->wm(blk, wid, bn), g, ctx->num_sms, ctx->launch_st), what);
+  if (plan.form == kGemmFlex) {
+    g.fx_nb = plan.block_n;
+    gemm_flex_shape(g);
+    CUtensorMap tmA, tmW;
+    if (!gemm_skinny_map(&tmA, maps.base, maps.rows, maps.cols, maps.cols, g.fx_nb / 2, g.fx_nk) || !gemm_skinny_map(&tmW, ctx->w[wid][blk], g.N, g.K, g.K, 128, g.fx_nk))
+      return fail(ctx, FVAR_ECUDA, "tensor map encoding failed");
+    FV_CUDA(ctx, launch_gemm_flex(epi, tmA, tmW, g, ctx->max_clusters, ctx->launch_st), what);
+  } else if (plan.form == kGemmPair) {             // CTA pairs take the full 128-row A box
+    g.a_box_rows = 128;
+    FV_CUDA(ctx, launch_gemm_pair(epi, plan.block_n, maps.m[3], ctx->wm(blk, wid, plan.block_n / 2), g, ctx->launch_st), what);
+  } else {
+    const int t = (g.nbatch == 1 && g.R <= 64) ? (g.R <= 16 ? 0 : (g.R <= 32 ? 1 : 2)) : 3;
+    g.a_box_rows = 16 << t;
+    FV_CUDA(ctx, launch_gemm(epi, plan.block_n, maps.m[t], ctx->wm(blk, wid, plan.block_n), g, ctx->num_sms, ctx->launch_st), what);
+  }
   ctx->launched();
   return FVAR_OK;
 }
@@ -621,7 +620,7 @@ fvar_status fvar_init(const fvar_weights *weights, const fvar_cfg *cfg, void *wo
     c->host_pipe_ok = cudaEventCreateWithFlags(&c->ev_in[s2], cudaEventDisableTiming) == cudaSuccess &&
                       cudaEventCreateWithFlags(&c->ev_cmp[s2], cudaEventDisableTiming) == cudaSuccess &&
                       cudaEventCreateWithFlags(&c->ev_out[s2], cudaEventDisableTiming) == cudaSuccess;
-  if (lls_prepare() != cudaSuccess || gemm_prepare() != cudaSuccess || gemm_pair_prepare() != cudaSuccess || gemm_skinny_prepare() != cudaSuccess ||
+  if (lls_prepare() != cudaSuccess || gemm_prepare() != cudaSuccess || gemm_pair_prepare() != cudaSuccess || gemm_skinny_prepare() != cudaSuccess || gemm_flex_prepare() != cudaSuccess ||
       attention_prepare() != cudaSuccess)
     return destroy_fail(FVAR_ECUDA, "kernel attribute set-up failed");
   c->max_clusters = gemm_pair_max_clusters();
@@ -790,10 +789,14 @@ fvar_status fvar_set_cond(fvar_ctx *ctx, int B, const void *cond, const void *co
     if (s != FVAR_OK) return s;
   }
   if (ctx->cfg.has_cross_attn) {
-    CUtensorMap ctx_map;
+    fvar_ctx::ActMaps ctx_map;
     const int T = ctx->cfg.ctx_len, Wc = ctx->cfg.ctx_width;
-    if (!tmap_2d(&ctx_map, context, Wc, static_cast<uint64_t>(B) * T, Wc, 128))
-      return fail(ctx, FVAR_EINVAL, "set_cond: context must be 16-byte aligned");
+    ctx_map.base = static_cast<const bf16 *>(context);
+    ctx_map.cols = Wc;
+    ctx_map.rows = static_cast<uint64_t>(B) * T;
+    for (int t = 0; t < 4; ++t)
+      if (!tmap_2d(&ctx_map.m[t], context, Wc, static_cast<uint64_t>(B) * T, Wc, 16u << t))
+        return fail(ctx, FVAR_EINVAL, "set_cond: context must be 16-byte aligned");
     for (int blk = 0; blk < nb; ++blk) {
       GemmArgs g = gemm_args(B * T, 2 * C, Wc);
       g.rows_per_batch = T;
@@ -801,7 +804,7 @@ fvar_status fvar_set_cond(fvar_ctx *ctx, int B, const void *cond, const void *co
       g.vt = ctx->cvt + blk * ctx->ckv_block_elems();
       g.C = C; g.H = ctx->H; g.D = ctx->D; g.L_cap = ctx->ctx_cap; g.L_prev = 0; g.col_base = C;
       g.out_bf16 = ctx->q; g.ld_out = C;           // unused: no column maps to the q part
-      fvar_status s = run_gemm_map(ctx, EPI_QKV, ctx_map, blk, W_CKV, g, "context kv gemm");
+      fvar_status s = run_gemm(ctx, EPI_QKV, ctx_map, blk, W_CKV, g, "context kv gemm");
       if (s != FVAR_OK) return s;
     }
   }
@@ -914,17 +917,17 @@ static fvar_status transition_impl(fvar_ctx *ctx, const void *fo, int scale_idx,
         g.sk_tiles_m = g.splits = 0;
     }
   }
-  GemmPlan plan{false, 64, 1};
+  GemmPlan plan{kGemmSingle, 64, 1};
   if (!split) {
-    plan = gemm_plan(R, 1, V, C, ctx->num_sms, ctx->max_clusters, 1, 0);
-    maps_ok = tmap_2d(&ta, fo, C, R, C, 128) && tmap_2d(&tw, ctx->codebook, C, V, C, plan.pair ? plan.block_n / 2 : plan.block_n);
+    plan = gemm_plan(R, 1, V, C, ctx->num_sms, ctx->max_clusters, 1, 0, false);
+    maps_ok = tmap_2d(&ta, fo, C, R, C, 128) && tmap_2d(&tw, ctx->codebook, C, V, C, plan.form == kGemmPair ? plan.block_n / 2 : plan.block_n);
   }
   if (!maps_ok) return fail(ctx, FVAR_EINVAL, "scale_transition: fo must be 16-byte aligned");
   ctx->tr_dirty[buf] = R;
   ctx->prof_begin(FVAR_KCLASS_GEMM, gflops, gbytes);
   if (split)
     FV_CUDA(ctx, launch_gemm_skinny(EPI_ARGMAX, ta, tw, g, st), "codeword search");
-  else if (plan.pair)
+  else if (plan.form == kGemmPair)
     FV_CUDA(ctx, launch_gemm_pair(EPI_ARGMAX, plan.block_n, ta, tw, g, st), "codeword search");
   else
     FV_CUDA(ctx, launch_gemm(EPI_ARGMAX, plan.block_n, ta, tw, g, ctx->num_sms, st), "codeword search");
@@ -1523,7 +1526,8 @@ fvar_status fvar_ln_modulate(const float *x, int R, int C, int rows_per_batch, c
 fvar_status fvar_gemm_bf16_form(const void *A, const void *W, const void *bias, int R, int N, int K, int form,
                                 int block_n, float *out, void *stream) {
   if (!A || !W || !out || R <= 0 || N <= 0 || K <= 0 || K % 8) return kfail(FVAR_EINVAL, "gemm: bad arguments");
-  if (form != FVAR_GEMM_AUTO && form != FVAR_GEMM_SINGLE && form != FVAR_GEMM_PAIR && form != FVAR_GEMM_SKINNY && form != FVAR_GEMM_KSPLIT)
+  if (form != FVAR_GEMM_AUTO && form != FVAR_GEMM_SINGLE && form != FVAR_GEMM_PAIR && form != FVAR_GEMM_SKINNY && form != FVAR_GEMM_KSPLIT &&
+      form != FVAR_GEMM_FLEX)
     return kfail(FVAR_EINVAL, "gemm: bad form");
   if (form == FVAR_GEMM_SKINNY || form == FVAR_GEMM_KSPLIT) {
     const int tiles_m = form == FVAR_GEMM_KSPLIT ? (R + 127) / 128 : 0;
@@ -1553,11 +1557,17 @@ fvar_status fvar_gemm_bf16_form(const void *A, const void *W, const void *bias, 
   FK_CUDA(cudaGetDevice(&dev), "get device");
   FK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device attribute");
   const int max_clusters = form == FVAR_GEMM_SINGLE ? 0 : gemm_pair_max_clusters();
-  GemmPlan plan = gemm_plan(R, 1, N, K, sms, max_clusters, 1, 0);
+  const bool flex_ok = gemm_flex_supported(EPI_F32, N, K);
+  GemmPlan plan = gemm_plan(R, 1, N, K, sms, max_clusters, 1, 0, flex_ok && (form == FVAR_GEMM_AUTO || form == FVAR_GEMM_FLEX));
   if (form == FVAR_GEMM_PAIR) {
     if (R <= 128 || max_clusters <= 0) return kfail(FVAR_EINVAL, "gemm: the pair form needs R > 128 and a device that runs CTA pairs");
     if (block_n != 0 && block_n != 128 && block_n != 256) return kfail(FVAR_EINVAL, "gemm: pair block_n must be 128 or 256");
-    if (!plan.pair) plan = GemmPlan{true, (N > 128) ? 256 : 128, 1};
+    if (plan.form != kGemmPair) plan = GemmPlan{kGemmPair, (N > 128) ? 256 : 128, 1};
+    if (block_n) plan.block_n = block_n;
+  } else if (form == FVAR_GEMM_FLEX) {
+    if (!flex_ok || max_clusters <= 0) return kfail(FVAR_EINVAL, "gemm: the free-width pair form needs N % 64 == 0 and a device that runs CTA pairs");
+    if (block_n != 0 && (block_n < 32 || block_n > 256 || block_n % 32)) return kfail(FVAR_EINVAL, "gemm: free-width block_n must be a multiple of 32 up to 256");
+    if (plan.form != kGemmFlex) plan = GemmPlan{kGemmFlex, R < 256 ? (R + 31) / 32 * 32 : 256, 1};
     if (block_n) plan.block_n = block_n;
   } else if (block_n != 0) {
     if (form == FVAR_GEMM_AUTO) return kfail(FVAR_EINVAL, "gemm: block_n needs an explicit form");
@@ -1565,16 +1575,25 @@ fvar_status fvar_gemm_bf16_form(const void *A, const void *W, const void *bias, 
     plan.block_n = block_n;
   }
   const int bn = plan.block_n;
-  CUtensorMap ta, tw;
-  if (!tmap_2d(&ta, A, K, R, K, 128) || !tmap_2d(&tw, W, K, N, K, plan.pair ? bn / 2 : bn))
-    return kfail(FVAR_EINVAL, "gemm: operands must be 16-byte aligned");
   GemmArgs g = gemm_args(R, N, K);
   g.bias = static_cast<const bf16 *>(bias);
   g.out_f32 = out;
   g.ld_out = N;
   g.status = kernel_status_ptr();
   if (!g.status) return kfail(FVAR_ECUDA, "gemm: status word");
-  if (plan.pair)
+  CUtensorMap ta, tw;
+  bool maps_ok;
+  if (plan.form == kGemmFlex) {
+    g.fx_nb = bn;
+    gemm_flex_shape(g);
+    maps_ok = gemm_skinny_map(&ta, A, R, K, K, bn / 2, g.fx_nk) && gemm_skinny_map(&tw, W, N, K, K, 128, g.fx_nk);
+  } else {
+    maps_ok = tmap_2d(&ta, A, K, R, K, 128) && tmap_2d(&tw, W, K, N, K, plan.form == kGemmPair ? bn / 2 : bn);
+  }
+  if (!maps_ok) return kfail(FVAR_EINVAL, "gemm: operands must be 16-byte aligned");
+  if (plan.form == kGemmFlex)
+    FK_CUDA(launch_gemm_flex(EPI_F32, ta, tw, g, max_clusters, static_cast<cudaStream_t>(stream)), "gemm");
+  else if (plan.form == kGemmPair)
     FK_CUDA(launch_gemm_pair(EPI_F32, bn, ta, tw, g, static_cast<cudaStream_t>(stream)), "gemm");
   else
     FK_CUDA(launch_gemm(EPI_F32, bn, ta, tw, g, sms, static_cast<cudaStream_t>(stream)), "gemm");

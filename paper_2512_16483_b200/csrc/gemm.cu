@@ -309,12 +309,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   }
 }
 
-// Cost model fitted to measurements on B200: an SM takes in about 100 GB/s from L2, so one K step
-// of a 128 x BN tile (16 KiB of A + BN * 128 B of W) costs t_k microseconds; a wave of work items
-// costs its K steps plus an epilogue that is only hidden behind the next item of the same CTA.
-// Splitting K trades a reduction through the scratch area for more CTAs streaming the operands.
-// microseconds per K block and per epilogue of a single-CTA tile of 64 / 128 / 256 columns
-static const float kTileTk[3] = {0.24f, 0.30f, 0.47f}, kTileTepi[3] = {1.0f, 1.5f, 2.5f};
+// Cost model of a launch on B200, fitted to measured ones (R = 100 .. 4096, N = 1024 .. 8192, K = 1024 .. 8192): fixed part
+// (set-up, first operands, the last tile's epilogue) + waves of tiles x K blocks x time a K block, in microseconds; the
+// epilogue of every tile but the last hides behind the main loop of the next.  Splitting K trades a reduction through
+// the scratch area for more CTAs streaming the operands.
+// Single CTAs, 128 rows x 64 / 128 / 256 features, and pairs, 256 rows x 128 / 256 features:
+static const float kTileTk[3] = {0.161f, 0.226f, 0.37f}, kTileFixed[3] = {3.2f, 4.2f, 6.0f};
+static const float kPairTk[2] = {0.197f, 0.295f}, kPairFixed[2] = {4.4f, 6.9f};
 
 void gemm_pick_tile(int tiles_m_total, int N, int K, int num_sms, int max_splits, size_t scratch_bytes, int *block_n,
                     int *splits) {
@@ -332,7 +333,7 @@ void gemm_pick_tile(int tiles_m_total, int N, int K, int num_sms, int max_splits
         break;
       const long long waves = (tiles * sp + num_sms - 1) / num_sms;
       const int kb = (num_kb + sp - 1) / sp;
-      float cost = waves * (kb * kTileTk[i] + kTileTepi[i]);
+      float cost = kTileFixed[i] + waves * kb * kTileTk[i];
       if (sp > 1) cost += 1.5f + 0.6f * sp * cand[i] / 128.0f;      // park + fixed-order reduction by one CTA
       if (cost < best_cost) {
         best_cost = cost;
@@ -344,28 +345,40 @@ void gemm_pick_tile(int tiles_m_total, int N, int K, int num_sms, int max_splits
 }
 
 
-GemmPlan gemm_plan(int R, int nbatch, int N, int K, int num_sms, int max_clusters, int max_splits, size_t scratch_bytes) {
-  GemmPlan plan{false, 64, 1};
+GemmPlan gemm_plan(int R, int nbatch, int N, int K, int num_sms, int max_clusters, int max_splits, size_t scratch_bytes, bool flex) {
+  GemmPlan plan{kGemmSingle, 64, 1};
   const int tiles_m = (R + kBlockM - 1) / kBlockM * nbatch;
   gemm_pick_tile(tiles_m, N, K, num_sms, max_splits, scratch_bytes, &plan.block_n, &plan.splits);
-  if (nbatch != 1 || R <= kBlockM || max_clusters <= 0) return plan;
+  if (nbatch != 1 || max_clusters <= 0) return plan;
   // Cost of the single-CTA choice.
   const int num_kb = (K + kBlockK - 1) / kBlockK;
   const int i1 = plan.block_n == 64 ? 0 : (plan.block_n == 128 ? 1 : 2);
   const long long tiles1 = static_cast<long long>(tiles_m) * ((N + plan.block_n - 1) / plan.block_n) * plan.splits;
-  float cost1 = ((tiles1 + num_sms - 1) / num_sms) * (((num_kb + plan.splits - 1) / plan.splits) * kTileTk[i1] + kTileTepi[i1]);
-  if (plan.splits > 1) cost1 += 1.5f + 0.6f * plan.splits * plan.block_n / 128.0f;
-  // A pair CTA moves, per K step, what a single CTA of half the tile width moves, for twice the output.
-  const int cand2[2] = {128, 256};
-  const int tiles_m2 = (R + 2 * kBlockM - 1) / (2 * kBlockM);
-  float best2 = 1e30f;
-  int bn2 = 0;
-  for (int i = 0; i < 2; ++i) {
-    const long long t2 = static_cast<long long>(tiles_m2) * ((N + cand2[i] - 1) / cand2[i]);
-    const float c = ((t2 + max_clusters - 1) / max_clusters) * (num_kb * kTileTk[i] + kTileTepi[i + 1]);
-    if (c < best2) { best2 = c; bn2 = cand2[i]; }
+  const long long waves1 = (tiles1 + num_sms - 1) / num_sms;
+  float best = kTileFixed[i1] + waves1 * ((num_kb + plan.splits - 1) / plan.splits) * kTileTk[i1] * (waves1 > 2 ? 1.15f : 1.0f);
+  if (plan.splits > 1) best += 1.5f + 0.6f * plan.splits * plan.block_n / 128.0f;
+  // From the third wave on the operands' way from L2 and the power cap slow every form: 2048 x 7680 x 1920 takes 0.36 us a
+  // K block on pairs of 256 columns, 0.30 with 192 rows a tile.
+  auto work = [&](long long tiles, float t, float crowded) {
+    const long long w = (tiles + max_clusters - 1) / max_clusters;
+    return static_cast<float>(w) * num_kb * t * (w > 2 ? crowded : 1.0f);
+  };
+  if (R > kBlockM) {
+    // A pair CTA moves, per K step, what a single CTA of half the tile width moves, for twice the output.
+    for (int i = 0; i < 2; ++i) {
+      const int bn = 128 << i;
+      const float c = kPairFixed[i] + work(static_cast<long long>((R + 2 * kBlockM - 1) / (2 * kBlockM)) * ((N + bn - 1) / bn), kPairTk[i], i == 0 ? 1.2f : 1.15f);
+      if (c < best) { best = c; plan = GemmPlan{kGemmPair, bn, 1}; }
+    }
   }
-  if (bn2 && best2 < cost1) plan = GemmPlan{true, bn2, 1};
+  // The free-width form has to be clearly ahead, as full tiles are level; up to 32 rows its narrowest tile is half padding.
+  if (flex && R > 32) {
+    for (int nb = 64; nb <= 256; nb += 32) {
+      const float t = 0.098f + 0.00077f * nb < 0.155f ? 0.155f : 0.098f + 0.00077f * nb;
+      const float c = 2.0f + 0.019f * nb + work(static_cast<long long>((N + 2 * kBlockM - 1) / (2 * kBlockM)) * ((R + nb - 1) / nb), t, 1.28f);
+      if (c < 0.97f * best) { best = c / 0.97f; plan = GemmPlan{kGemmFlex, nb, 1}; }
+    }
+  }
   return plan;
 }
 

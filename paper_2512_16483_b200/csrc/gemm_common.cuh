@@ -194,6 +194,28 @@ __device__ __forceinline__ void resid_fetch(const GemmArgs &p, const ResidRow &r
     if (out >= 0) pre[it] = *reinterpret_cast<const float4 *>(p.resid + static_cast<long long>(res) * p.ld_out + col0 + (lane & 7) * 4);
   }
 }
+// Gate + residual (and the hi / lo split) of four columns `col` .. col + 3 of row r of the warp's 32 rows: o = sums with
+// bias.  Every lane of the warp must call.
+__device__ __forceinline__ void resid_store(const GemmArgs &p, const ResidRow &rr, float4 o, const float4 &res, int r, int col) {
+  const int out = __shfl_sync(0xffffffffu, rr.out, r), b = __shfl_sync(0xffffffffu, rr.b, r), split = __shfl_sync(0xffffffffu, rr.split, r);
+  if (out < 0) return;
+  const float4 g = p.gate ? __ldg(reinterpret_cast<const float4 *>(p.gate + static_cast<long long>(b) * p.gate_stride + col))
+                          : make_float4(1.f, 1.f, 1.f, 1.f);
+  o.x = fmaf(g.x, o.x, res.x);
+  o.y = fmaf(g.y, o.y, res.y);
+  o.z = fmaf(g.z, o.z, res.z);
+  o.w = fmaf(g.w, o.w, res.w);
+  *reinterpret_cast<float4 *>(p.out_f32 + static_cast<long long>(out) * p.ld_out + col) = o;
+  if (p.xsplit != nullptr) {
+    bf16 *hi = p.xsplit + static_cast<long long>(split) * p.ld_out + col;
+    const uint2 h2 = make_uint2(pack_bf16(o.x, o.y), pack_bf16(o.z, o.w));
+    const __nv_bfloat162 *hh = reinterpret_cast<const __nv_bfloat162 *>(&h2);
+    const float2 f0 = __bfloat1622float2(hh[0]), f1 = __bfloat1622float2(hh[1]);
+    *reinterpret_cast<uint2 *>(hi) = h2;
+    *reinterpret_cast<uint2 *>(hi + static_cast<long long>(p.xsplit_mk) * p.ld_out) =
+        make_uint2(pack_bf16(o.x - f0.x, o.y - f0.y), pack_bf16(o.z - f1.x, o.w - f1.y));
+  }
+}
 // EPI_RESID of one warp for its 32 rows x 32 columns starting at col0 (col0 + 32 <= N).  Every lane must call.
 __device__ __forceinline__ void resid_chunk(const GemmArgs &p, const uint32_t (&acc)[32], const ResidRow &rr, int col0, uint32_t stage, int lane,
                                             const float4 (&pre)[8]) {
@@ -202,39 +224,20 @@ __device__ __forceinline__ void resid_chunk(const GemmArgs &p, const uint32_t (&
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stage + lane * 128 + ((q ^ (lane & 7)) << 4)), "r"(acc[q * 4]), "r"(acc[q * 4 + 1]),
                  "r"(acc[q * 4 + 2]), "r"(acc[q * 4 + 3]) : "memory");
   const int c = lane & 7, col = col0 + c * 4;
-  float bias[4] = {0.f, 0.f, 0.f, 0.f};
+  float2 f0 = make_float2(0.f, 0.f), f1 = f0;
   if (p.bias != nullptr) {
     const uint2 u = __ldg(reinterpret_cast<const uint2 *>(p.bias + col));
     const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&u);
-    const float2 f0 = __bfloat1622float2(h[0]), f1 = __bfloat1622float2(h[1]);
-    bias[0] = f0.x; bias[1] = f0.y; bias[2] = f1.x; bias[3] = f1.y;
+    f0 = __bfloat1622float2(h[0]);
+    f1 = __bfloat1622float2(h[1]);
   }
   __syncwarp();
 #pragma unroll
   for (int it = 0; it < 8; ++it) {
     const int r = it * 4 + (lane >> 3);
-    const int out = __shfl_sync(0xffffffffu, rr.out, r), b = __shfl_sync(0xffffffffu, rr.b, r), split = __shfl_sync(0xffffffffu, rr.split, r);
-    float4 o;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(o.x), "=f"(o.y), "=f"(o.z), "=f"(o.w)
-                 : "r"(stage + r * 128 + ((c ^ (r & 7)) << 4)));
-    if (out >= 0) {
-      const float4 g = p.gate ? __ldg(reinterpret_cast<const float4 *>(p.gate + static_cast<long long>(b) * p.gate_stride + col))
-                              : make_float4(1.f, 1.f, 1.f, 1.f);
-      o.x = fmaf(g.x, o.x + bias[0], pre[it].x);
-      o.y = fmaf(g.y, o.y + bias[1], pre[it].y);
-      o.z = fmaf(g.z, o.z + bias[2], pre[it].z);
-      o.w = fmaf(g.w, o.w + bias[3], pre[it].w);
-      *reinterpret_cast<float4 *>(p.out_f32 + static_cast<long long>(out) * p.ld_out + col) = o;
-      if (p.xsplit != nullptr) {
-        bf16 *hi = p.xsplit + static_cast<long long>(split) * p.ld_out + col;
-        const uint2 h2 = make_uint2(pack_bf16(o.x, o.y), pack_bf16(o.z, o.w));
-        const __nv_bfloat162 *hh = reinterpret_cast<const __nv_bfloat162 *>(&h2);
-        const float2 f0 = __bfloat1622float2(hh[0]), f1 = __bfloat1622float2(hh[1]);
-        *reinterpret_cast<uint2 *>(hi) = h2;
-        *reinterpret_cast<uint2 *>(hi + static_cast<long long>(p.xsplit_mk) * p.ld_out) =
-            make_uint2(pack_bf16(o.x - f0.x, o.y - f0.y), pack_bf16(o.z - f1.x, o.w - f1.y));
-      }
-    }
+    float4 o = ld_shared_f4(stage + r * 128 + ((c ^ (r & 7)) << 4));
+    o.x += f0.x; o.y += f0.y; o.z += f1.x; o.w += f1.y;
+    resid_store(p, rr, o, pre[it], r, col);
   }
   __syncwarp();
 }

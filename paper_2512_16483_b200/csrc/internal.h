@@ -78,6 +78,9 @@ struct GemmArgs {
   // MMA width of a chunk, chunks (1 or 2) and pipeline stages -- filled by gemm_skinny_shape
   int sk_rows_chunk, sk_rp, sk_nchunks, sk_stages, sk_small, sk_nk;
   int sk_tiles_m;          // > 0: the 128 x 128-tile mode of that kernel with this many row tiles (rows on the M side)
+  // CTA-pair form with a free row width (gemm_flex.cu): rows of a tile (a multiple of 32 up to 256), K blocks per
+  // pipeline stage, stages
+  int fx_nb, fx_nk, fx_stages;
   // optional: weights the next GEMM of the chain will stream; every CTA asks L2 to prefetch its share
   const void *pf_ptr;
   unsigned long long pf_bytes;
@@ -108,15 +111,15 @@ cudaError_t launch_gemm_pair(int epi, int block_n, const CUtensorMap &tmA, const
                              cudaStream_t st);
 // Largest number of CTA pairs of the pair kernel that can be resident at once (0: pairs unavailable).
 int gemm_pair_max_clusters();
-// How a GEMM is launched: by single CTAs (block_n in {64, 128, 256}, optional split-K) or by CTA pairs
-// (block_n in {128, 256}).
+// How a GEMM is launched: by single CTAs (block_n in {64, 128, 256} features, optional split-K), by CTA pairs of 256 rows
+// x block_n in {128, 256} features, or by CTA pairs of 256 features x block_n rows (gemm_flex.cu).
+enum GemmForm { kGemmSingle = 0, kGemmPair = 1, kGemmFlex = 2 };
 struct GemmPlan {
-  bool pair;
-  int block_n, splits;
+  int form, block_n, splits;
 };
-// Picks the launch form and tile width from the measured cost model.  tiles_m_total: 128-row tiles over
-// all batches; pairs are considered only for a single problem with more than one row tile.
-GemmPlan gemm_plan(int R, int nbatch, int N, int K, int num_sms, int max_clusters, int max_splits, size_t scratch_bytes);
+// Picks the launch form and tile width from the measured cost model.  flex: the free-width form may be taken (it needs
+// N % 64 == 0 and an epilogue it has); pairs of either kind are considered only for a single problem.
+GemmPlan gemm_plan(int R, int nbatch, int N, int K, int num_sms, int max_clusters, int max_splits, size_t scratch_bytes, bool flex);
 
 // Weight-streaming form for R <= 512 rows (gemm_skinny.cu): the weights are the M side of the MMA, the K range of
 // a 128-feature tile is split over a cluster of `splits` CTAs that reduce through distributed shared memory.
@@ -129,6 +132,13 @@ void gemm_skinny_shape(GemmArgs &a);      // needs a.R, a.K and a.splits
 bool gemm_skinny_map(CUtensorMap *m, const void *base, uint64_t rows, uint64_t K, uint64_t ld, uint32_t box_rows, int nk);
 cudaError_t launch_gemm_skinny(int epi, const CUtensorMap &tmA, const CUtensorMap &tmW, const GemmArgs &a, cudaStream_t st);
 cudaError_t gemm_skinny_prepare();
+
+// CTA-pair form with a free row width (gemm_flex.cu).  gemm_flex_shape fills the pipeline fields for a.fx_nb;
+// tmA / tmW: gemm_skinny_map with boxes of fx_nb / 2 and 128 rows.
+bool gemm_flex_supported(int epi, int N, int K);
+void gemm_flex_shape(GemmArgs &a);
+cudaError_t launch_gemm_flex(int epi, const CUtensorMap &tmA, const CUtensorMap &tmW, const GemmArgs &a, int max_clusters, cudaStream_t st);
+cudaError_t gemm_flex_prepare();
 
 // Set the dynamic shared-memory attribute of every instantiation (once, outside any stream capture).
 cudaError_t gemm_prepare();

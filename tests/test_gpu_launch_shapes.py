@@ -68,3 +68,47 @@ def test_transitions_repeat_on_one_context(fv, V):
     assert ctx.poll_status() == fv.OK
     for a, b in zip(*got):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("R,N,K,width", [
+    (33, 64, 64, 32), (400, 192, 2048, 160), (400, 6144, 200, 224),     # half a feature tile, a remainder of one, K not whole blocks
+    (255, 1920, 1920, 64), (257, 1920, 128, 256), (1, 256, 4096, 0),    # an odd number of 128-feature halves, one row past a tile
+    (5000, 320, 136, 96), (2704, 1024, 1024, 0), (97, 8192, 2048, 0),   # several tiles a pair, the picked widths
+])
+def test_gemm_free_width_pairs(fv, R, N, K, width):
+    g = torch.Generator(device="cuda").manual_seed(R + N + K)
+    A = torch.randn((R, K), generator=g, device="cuda").bfloat16()
+    W = torch.randn((N, K), generator=g, device="cuda").bfloat16()
+    bias = torch.randn((N,), generator=g, device="cuda").bfloat16()
+    out = fv.fvar_gemm_bf16_form(A, W, bias, fv.GEMM_FLEX, width)
+    assert fv.kernel_poll_status() == fv.OK
+    ref = A.double() @ W.double().T + bias.double()
+    bound = 1e-5 * (A.double().abs() @ W.double().abs().T).max()
+    assert (out.double() - ref).abs().max() <= bound
+
+
+@pytest.mark.parametrize("shape,B,k,bar", [("d16", 16, 8, 2e-2), ("infinity", 1, 7, 3e-2)])
+def test_step_epilogues_of_the_free_width_pairs(fv, shape, B, k, bar):
+    """One dense block at sizes where QKV, out-proj and both FFN GEMMs take that form between them (2704 rows of 1024
+    columns; 400 rows of 2048): every epilogue of it, KV cache included, against the CPU oracle."""
+    import numpy as np
+    from oracle import fvar_oracle as orc
+    from helpers import assert_close
+    shp = si.shape_var_d16(n_blocks=1) if shape == "d16" else si.shape_infinity_2b(n_blocks=1, blocks_per_group=1)
+    w = si.make_weights(11, shp)
+    ctx = fv.Fvar(weights_to_cuda(w), blocks_per_group=1, n_heads=shp.n_heads, head_dim=shp.head_dim, ffn_dim=shp.ffn_dim, scale_hw=shp.hw(),
+                  max_batch=B, ctx_len=shp.ctx_len, ctx_width=shp.ctx_width)
+    o = orc.Oracle(w, shp.n_heads, 1, shp.hw(), shp.ln_eps)
+    cond = si.make_cond(12, B, shp.width)
+    text = si.make_context(13, B, shp.ctx_len, shp.ctx_width) if shp.has_cross_attn else None
+    ctx.set_cond(to_bf16_cuda(cond), to_bf16_cuda(text) if text is not None else None)
+    o.set_cond(cond, text)
+    M = shp.tokens_per_scale()[k]
+    for scale in (k, k):                # the second time over the keys and values the first one left in the cache
+        toks = si.make_tokens(14, B, M, shp.width)
+        ctx.scale_step(to_bf16_cuda(toks), scale)
+        o.scale_step(toks, scale, orc.Policy("dense", "pair"))
+        assert_close(ctx.get_group_output(0, M).cpu().numpy(), np.stack([o.group_cache[0][b] for b in range(B)]), max_rel=bar, what=shape)
+        ctx.kv_append(scale)
+        o.kv_append(scale)
+    assert ctx.poll_status() == fv.OK

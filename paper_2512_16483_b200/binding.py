@@ -136,8 +136,16 @@ EXPORTED = ("fvar_workspace_bytes", "fvar_init", "fvar_set_cond", "fvar_set_proj
             "fvar_infinity_schedule")
 
 
+# A kernel-level call is a launch of a few microseconds, and the public way to the current stream's handle builds two
+# Python objects (3.3 us measured, as much as the launch itself); this is the lookup underneath (0.1 us).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    if _raw_stream is None or _raw_device is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_raw_device())
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
@@ -160,7 +168,7 @@ def fvar_row_scores(x: torch.Tensor) -> torch.Tensor:
     """x fp32 [B][M][C] -> scores fp32 [B][M]."""
     _dev(x, torch.float32)
     B, M, C = x.shape
-    s = torch.empty((B, M), dtype=torch.float32, device=x.device)
+    s = x.new_empty((B, M))
     _check_kernel(load_library().fvar_row_scores(x.data_ptr(), B, M, C, s.data_ptr(), _stream()))
     return s
 
@@ -169,7 +177,7 @@ def fvar_row_keys(x: torch.Tensor, noise: torch.Tensor) -> torch.Tensor:
     """x fp32 [B][M][C], noise fp32 [B][M] (Exp(1) variates) -> sampling keys fp32 [B][M] = score / noise."""
     _dev(x, torch.float32), _dev(noise, torch.float32)
     B, M, C = x.shape
-    k = torch.empty((B, M), dtype=torch.float32, device=x.device)
+    k = x.new_empty((B, M))
     _check_kernel(load_library().fvar_row_keys(x.data_ptr(), noise.data_ptr(), B, M, C, k.data_ptr(), _stream()))
     return k
 
@@ -178,8 +186,8 @@ def fvar_select_topr(scores: torch.Tensor, r: int):
     """scores fp32 [B][M] -> (idx int32 [B][r] ascending, inv int32 [B][M])."""
     _dev(scores, torch.float32)
     B, M = scores.shape
-    idx = torch.empty((B, r), dtype=torch.int32, device=scores.device)
-    inv = torch.empty((B, M), dtype=torch.int32, device=scores.device)
+    idx = scores.new_empty((B, r), dtype=torch.int32)
+    inv = scores.new_empty((B, M), dtype=torch.int32)
     _check_kernel(load_library().fvar_select_topr(scores.data_ptr(), B, M, r, idx.data_ptr(), inv.data_ptr(), _stream()))
     return idx, inv
 
@@ -188,7 +196,7 @@ def fvar_ln_modulate(x: torch.Tensor, shift: torch.Tensor, scale: torch.Tensor, 
     """x fp32 [B][n][C], shift/scale fp32 [B][C] -> bf16 [B][n][C]."""
     _dev(x, torch.float32), _dev(shift, torch.float32), _dev(scale, torch.float32)
     B, n, C = x.shape
-    y = torch.empty((B, n, C), dtype=torch.bfloat16, device=x.device)
+    y = x.new_empty((B, n, C), dtype=torch.bfloat16)
     _check_kernel(load_library().fvar_ln_modulate(x.data_ptr(), B * n, C, n, shift.data_ptr(), scale.data_ptr(), C,
                                                   eps, y.data_ptr(), _stream()))
     return y
@@ -204,7 +212,7 @@ def fvar_gemm_bf16_form(A: torch.Tensor, W: torch.Tensor, bias: Optional[torch.T
     _dev(A, torch.bfloat16), _dev(W, torch.bfloat16)
     R, K = A.shape
     N = W.shape[0]
-    out = torch.empty((R, N), dtype=torch.float32, device=A.device)
+    out = A.new_empty((R, N), dtype=torch.float32)
     _check_kernel(load_library().fvar_gemm_bf16_form(A.data_ptr(), W.data_ptr(), _ptr(bias), R, N, K, form, block_n,
                                                      out.data_ptr(), _stream()))
     return out
@@ -215,7 +223,7 @@ def fvar_gemm_bf16_wt(A: torch.Tensor, Wt: torch.Tensor, bias: Optional[torch.Te
     _dev(A, torch.bfloat16), _dev(Wt, torch.bfloat16)
     R, K = A.shape
     N = Wt.shape[1]
-    out = torch.empty((R, N), dtype=torch.float32, device=A.device)
+    out = A.new_empty((R, N), dtype=torch.float32)
     _check_kernel(load_library().fvar_gemm_bf16_wt(A.data_ptr(), Wt.data_ptr(), _ptr(bias), R, N, K, block_n, out.data_ptr(), _stream()))
     return out
 
@@ -225,7 +233,7 @@ def fvar_cfg_combine(pair: torch.Tensor, guidance: float) -> torch.Tensor:
     _dev(pair, torch.bfloat16)
     B = pair.shape[0]
     per = pair[0].numel()
-    out = torch.empty((B // 2,) + tuple(pair.shape[1:]), dtype=torch.bfloat16, device=pair.device)
+    out = pair.new_empty((B // 2,) + tuple(pair.shape[1:]), dtype=torch.bfloat16)
     _check_kernel(load_library().fvar_cfg_combine(pair.data_ptr(), B, per, float(guidance), out.data_ptr(), _stream()))
     return out
 

@@ -88,7 +88,7 @@ __device__ __forceinline__ int fast_div(int u, const FastDiv &f) {
 // How the units of work are spread over the grid: each CTA walks several, has one, or shares one with its cluster.
 enum { kWalk = 0, kOne = 1, kRanges = 2 };
 
-template <int D, int MODE>
+template <int D, int MODE, bool DUAL>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                  const __grid_constant__ CUtensorMap tmV, const __grid_constant__ AttnArgs p) {
@@ -200,11 +200,16 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             tma_load_2d(q_smem + t * Cfg::kTileBytes + a * kAtomBytes, &tmQ, q_full, x.h * D + a * 64, x.e * p.r + x.q0 + t * kQRows);
         ++q_units;
         for (int i = 0; i < 2 * nkv; ++i) {            // even i: K of block i/2, odd i: V^T of block i/2
-          const int j = i >> 1;
+          int j = i >> 1, v = i & 1;
+          if (DUAL) {                                  // K 0, K 1, V 0, K 2, V 1, K 3, ... V nkv-2, V nkv-1
+            const int k = i - 2, alt = 2 * (nkv - 2);
+            v = k >= alt || (k >= 0 && (k & 1) == 0);
+            j = k < 0 ? i : k < alt ? (k >> 1) + (v ? 0 : 2) : k - alt + nkv - 2;
+          }
           if (!mbar_wait(ring_empty(slot), phase ^ 1u, p.status, &abort_flag, wb)) { ok = false; break; }
           mbar_expect_tx(ring_full(slot), Cfg::kTileBytes);
           const uint32_t dst = ring_smem + slot * Cfg::kTileBytes;
-          if ((i & 1) == 0) {
+          if (v == 0) {
 #pragma unroll
             for (int a = 0; a < D / 64; ++a) tma_load_3d(dst + a * kAtomBytes, &tmK, ring_full(slot), a * 64, (jb0 + j) * kKeys, bh);
           } else {
@@ -269,7 +274,37 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         for (int t = 0; t < ntiles; ++t) issue_s(t, t, base % NR);
         umma_commit_if(leader, ring_empty(base % NR));
         if (nkv == 1) umma_commit_if(leader, q_empty);
-        if (ntiles == 1) {
+        if (DUAL) {
+          // one tile, two streams of key blocks: stream t owns S buffer t, accumulator t and the blocks t, t + 2, ...
+          unsigned pos = base + 1;
+          if (!full(pos)) { ok = false; break; }
+          tc_fence_after();
+          issue_s(0, 1, pos % NR);
+          umma_commit_if(leader, ring_empty(pos % NR));
+          if (nkv == 2) umma_commit_if(leader, q_empty);
+          ++pos;
+          for (int j = 0; j < nkv; ++j) {
+            const int t = j & 1;
+            const uint32_t par = ((pbits >> t) ^ (j >> 1)) & 1u;
+            if (!wait(p_half(t), par) || !full(pos)) { ok = false; break; }
+            tc_fence_after();
+            issue_pv(t, t, pos % NR, 0, j > 1);
+            if (!wait(p_full(t), par)) { ok = false; break; }
+            tc_fence_after();
+            issue_pv(t, t, pos % NR, 1, true, j + 2 >= nkv);
+            umma_commit_if(leader, ring_empty(pos % NR));
+            ++pos;
+            if (j + 2 < nkv) {
+              if (!full(pos)) { ok = false; break; }
+              tc_fence_after();
+              issue_s(0, t, pos % NR);
+              umma_commit_if(leader, ring_empty(pos % NR));
+              if (j + 3 == nkv) umma_commit_if(leader, q_empty);
+              ++pos;
+            }
+          }
+          pbits ^= (((nkv + 1) >> 1) & 1u) | (((nkv >> 1) & 1u) << 1);
+        } else if (ntiles == 1) {
           // A single query tile has no partner to alternate with: the idle tile's S columns serve as
           // a second S buffer, so that Q K^T of block j+1 runs while the softmax works on block j.  The idle tile's P
           // barriers alternate with its own too: the softmax may be done with block j+1 while this thread still waits
@@ -337,16 +372,17 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     bool ok = true;
     for (int u = unit0; ok && u < nunits; u += unit_step) {
       const int ntiles = unit_at(u).ntiles;
-      const bool single = (ntiles == 1);               // then S alternates between the two S buffers
+      const bool single = (ntiles == 1) && !DUAL;               // then S alternates between the two S buffers
       m_ref = -INFINITY;
       l_run = 0.f;
-      for (int j = 0; t < ntiles && j < nkv; ++j) {
+      const int nblk = DUAL ? (nkv + 1 - t) >> 1 : nkv;   // blocks of this warp-group: all, or those of its stream
+      for (int j = 0; (DUAL || t < ntiles) && j < nblk; ++j) {
         const int sbuf = single ? (j & 1) : t;
         const uint32_t s_addr = s_base + sbuf * kKeys;
         ok = __all_sync(0xffffffffu, mbar_wait(s_full(sbuf), ((sbits >> sbuf) ^ (single ? (j >> 1) : j)) & 1u, p.status, &abort_flag, wb));
         if (!ok) break;
         tc_fence_after();
-        const int valid = p.L - (jb0 + j) * kKeys;       // keys of this block below L (>= 128: all)
+        const int valid = p.L - (jb0 + (DUAL ? 2 * j + t : j)) * kKeys;       // keys of this block below L (>= 128: all)
         // the whole S row (128 fp32) in registers: four TMEM loads in flight, one wait
         uint32_t v[4][32];
 #pragma unroll
@@ -421,30 +457,58 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         unpack_f2(add_f2(ls[0], ls[1]), l0, l1);
         l_run += l0 + l1;
       }
-      if (t < ntiles) {
+      if (DUAL || t < ntiles) {
         // a barrier of its own: the blocks' o_full phases have not been waited for one by one, so their parity is no
         // safe guide here
         ok = ok && __all_sync(0xffffffffu, mbar_wait(o_last(t), last_bit, p.status, &abort_flag, wb));
         final_ok = ok;
+        const uint32_t swap = q_smem + Cfg::kTileBytes + row_local * 8;
+        if constexpr (DUAL) {
+          // The two streams meet: a row's maximum and sum change sides through shared memory (the second query tile's room,
+          // which no lone unit has), and each warp-group finishes half of the columns from both accumulators.  The barrier
+          // carries the outcome of the waits: either all eight warps go on or none.
+          asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(swap + t * (kQRows * 8)), "f"(m_ref), "f"(l_run) : "memory");
+          ok = ok && __all_sync(0xffffffffu, mbar_wait(o_last(t ^ 1), last_bit, p.status, &abort_flag, wb));
+          ok = bar_and(1, 256, ok);
+        }
         if (MODE != kRanges && ok) {
           tc_fence_after();
           int u2 = u;                                    // decoded again: kept in registers through the loop, the unit spills
           asm volatile("" : "+r"(u2));
           const Unit x = unit_at(u2);
-          const int rib = x.q0 + t * kQRows + row_local;
+          const int rib = x.q0 + (DUAL ? 0 : t * kQRows) + row_local;
           bf16 *dst = p.out + (static_cast<long long>(x.e) * p.r + rib) * (p.H * D) + x.h * D;
-          const float inv_l = 1.0f / l_run;
+          float inv_l, other = 0.f;
+          if constexpr (DUAL) {
+            const float2 ml = ld_shared_f2(swap + (t ^ 1) * (kQRows * 8));
+            const float m_all = fmaxf(m_ref, ml.x), w0 = exp2f((m_ref - m_all) * c), w1 = exp2f((ml.x - m_all) * c);
+            const float l_all = t == 0 ? fmaf(l_run, w0, ml.y * w1) : fmaf(ml.y, w1, l_run * w0);   // the same sum on both sides
+            inv_l = w0 / l_all;
+            other = w1 / l_all;
+          } else {
+            inv_l = 1.0f / l_run;
+          }
+          constexpr int kCols = DUAL ? D / 64 : D / 32;
+          const int cc0 = DUAL ? t * kCols : 0;
           const bool wide = (reinterpret_cast<uintptr_t>(p.out) & 31) == 0;
 #pragma unroll 1
-          for (int cc = 0; cc < D / 32; ++cc) {
+          for (int cc = cc0; cc < cc0 + kCols; ++cc) {
             uint32_t v[32];
             tmem_ld32(o_addr + cc * 32, v);
             tmem_ld_wait();
+            if constexpr (DUAL) {
+              uint32_t v1[32];
+              tmem_ld32(o_addr + (t == 0 ? D : -D) + cc * 32, v1);
+              tmem_ld_wait();
+#pragma unroll
+              for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(fmaf(__uint_as_float(v1[i]), other, __uint_as_float(v[i]) * inv_l));
+            }
             if (rib < p.r) {
+              const float norm = DUAL ? 1.f : inv_l;
               uint32_t w[16];
 #pragma unroll
               for (int i = 0; i < 16; ++i) {
-                __nv_bfloat162 v2 = __floats2bfloat162_rn(__uint_as_float(v[i * 2]) * inv_l, __uint_as_float(v[i * 2 + 1]) * inv_l);
+                __nv_bfloat162 v2 = __floats2bfloat162_rn(__uint_as_float(v[i * 2]) * norm, __uint_as_float(v[i * 2 + 1]) * norm);
                 w[i] = *reinterpret_cast<uint32_t *>(&v2);
               }
               // every lane has a row of its own: the wider the store, the fewer passes over 32 lines each
@@ -458,14 +522,18 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             }
           }
         }
-        o_bit ^= (nkv - 1) & 1u;
+        // nobody hands over a P of the next unit, and so lets an accumulator be overwritten, before both halves are out
+        if constexpr (MODE == kWalk && DUAL) {
+          if (ok) asm volatile("bar.sync 1, 256;" ::: "memory");
+        }
+        o_bit ^= (nblk - 1) & 1u;
         last_bit ^= 1u;
       } else {
         // a unit with one tile uses both S buffers: its end is awaited, or the parity of the next wait would be ambiguous
         ok = __all_sync(0xffffffffu, mbar_wait(o_last(0), unit_bit, p.status, &abort_flag, wb));
       }
       unit_bit ^= 1u;
-      sbits ^= single ? ((((nkv + 1) >> 1) & 1u) | (((nkv >> 1) & 1u) << 1)) : ((nkv & 1) ? 3u : 0u);
+      sbits ^= single || DUAL ? ((((nkv + 1) >> 1) & 1u) | (((nkv >> 1) & 1u) << 1)) : ((nkv & 1) ? 3u : 0u);
     }
   }
 
@@ -543,29 +611,35 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   }
 }
 
-template <int D, int MODE>
+template <int D, int MODE, bool DUAL>
 static cudaError_t set_attr() {
   static bool attr_set = false;
   if (attr_set) return cudaSuccess;
   // The register split draws on what the block was launched with: refuse a build whose kernel got fewer.
   cudaFuncAttributes fa;
-  cudaError_t err = cudaFuncGetAttributes(&fa, attention_kernel<D, MODE>);
+  cudaError_t err = cudaFuncGetAttributes(&fa, attention_kernel<D, MODE, DUAL>);
   if (err != cudaSuccess) return err;
   if (kAttnThreads * fa.numRegs < 32 * kSoftmaxWarp * kRegsIssue + (kAttnThreads - 32 * kSoftmaxWarp) * kRegsSoftmax) return cudaErrorInvalidConfiguration;
-  err = cudaFuncSetAttribute(attention_kernel<D, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<D>::kSmemBytes);
+  err = cudaFuncSetAttribute(attention_kernel<D, MODE, DUAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<D>::kSmemBytes);
   if (err == cudaSuccess) attr_set = true;
   return err;
 }
 
 static int g_max_clusters[9];       // resident clusters of s CTAs (0: not asked or not launchable); the same for both widths: one CTA an SM
 
+template <int D>
+static cudaError_t set_attrs() {
+  cudaError_t e = set_attr<D, kWalk, false>();
+  if (e == cudaSuccess) e = set_attr<D, kWalk, true>();
+  if (e == cudaSuccess) e = set_attr<D, kOne, false>();
+  if (e == cudaSuccess) e = set_attr<D, kOne, true>();
+  if (e == cudaSuccess) e = set_attr<D, kRanges, false>();
+  return e;
+}
+
 cudaError_t attention_prepare() {
-  cudaError_t e = set_attr<64, kWalk>();
-  if (e == cudaSuccess) e = set_attr<64, kOne>();
-  if (e == cudaSuccess) e = set_attr<64, kRanges>();
-  if (e == cudaSuccess) e = set_attr<128, kWalk>();
-  if (e == cudaSuccess) e = set_attr<128, kOne>();
-  if (e == cudaSuccess) e = set_attr<128, kRanges>();
+  cudaError_t e = set_attrs<64>();
+  if (e == cudaSuccess) e = set_attrs<128>();
   if (e != cudaSuccess || g_max_clusters[1] > 0) return e;
   for (int s = 8; s >= 1; --s) {
     cudaLaunchConfig_t cfg = {};
@@ -580,7 +654,7 @@ cudaError_t attention_prepare() {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, attention_kernel<128, kRanges>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, attention_kernel<128, kRanges, false>, &cfg) != cudaSuccess) {
       cudaGetLastError();
       n = 0;
     }
@@ -594,7 +668,7 @@ static FastDiv make_fast_div(unsigned d, unsigned long long max_u) {
   return FastDiv{d, (d > 1 && max_u * d < (1ull << 32)) ? static_cast<unsigned>(((1ull << 32) + d - 1) / d) : 0u};
 }
 
-template <int D>
+template <int D, bool DUAL>
 static cudaError_t launch_d(const CUtensorMap &tmQ, const CUtensorMap &tmK, const CUtensorMap &tmV, AttnArgs a, int num_sms,
                             cudaStream_t st) {
   using Cfg = AttnCfg<D>;
@@ -603,22 +677,22 @@ static cudaError_t launch_d(const CUtensorMap &tmQ, const CUtensorMap &tmK, cons
   if (units > INT_MAX) return cudaErrorInvalidValue;
   if (a.kv_splits <= 1 && units <= num_sms) {
     // the walk's bookkeeping is 0.5 us of a 4 us launch
-    cudaError_t err = set_attr<D, kOne>();
+    cudaError_t err = set_attr<D, kOne, DUAL>();
     if (err != cudaSuccess) return err;
-    return launch_pdl(attention_kernel<D, kOne>, dim3(nqt, a.H, a.B_eff), dim3(kAttnThreads), Cfg::kSmemBytes, st, tmQ, tmK, tmV, a);
+    return launch_pdl(attention_kernel<D, kOne, DUAL>, dim3(nqt, a.H, a.B_eff), dim3(kAttnThreads), Cfg::kSmemBytes, st, tmQ, tmK, tmV, a);
   }
   if (a.kv_splits <= 1) {
     // one CTA an SM, each walking its share of the units: the set-up and first operands of a unit hide behind the last
     // blocks of the one before (D = 128: B = 2, r = 4096 over 256 context keys 42.3 -> 29.2 us; D = 64: B = 32, H = 30,
     // r = 128 over 552 keys 70.6 -> 48.7)
-    cudaError_t err = set_attr<D, kWalk>();
+    cudaError_t err = set_attr<D, kWalk, DUAL>();
     if (err != cudaSuccess) return err;
     a.units = static_cast<int>(units);
     a.div_nqt = make_fast_div(nqt, units);
     a.div_h = make_fast_div(a.H, units);
-    return launch_pdl(attention_kernel<D, kWalk>, dim3(num_sms), dim3(kAttnThreads), Cfg::kSmemBytes, st, tmQ, tmK, tmV, a);
+    return launch_pdl(attention_kernel<D, kWalk, DUAL>, dim3(num_sms), dim3(kAttnThreads), Cfg::kSmemBytes, st, tmQ, tmK, tmV, a);
   }
-  cudaError_t err = set_attr<D, kRanges>();
+  cudaError_t err = set_attr<D, kRanges, false>();
   if (err != cudaSuccess) return err;
   if (a.kv_splits > 8) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
@@ -635,18 +709,27 @@ static cudaError_t launch_d(const CUtensorMap &tmQ, const CUtensorMap &tmK, cons
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, attention_kernel<D, kRanges>, tmQ, tmK, tmV, a);
+  return cudaLaunchKernelEx(&cfg, attention_kernel<D, kRanges, false>, tmQ, tmK, tmV, a);
 }
 
 // Launch shape of an attention call: query tiles per CTA (two: each K / V block feeds two tiles, the softmax of one
 // overlapping the MMAs of the other; one: twice the units when there are few) and key ranges per unit (a cluster of up
 // to 6 CTAs).  The pair with the least estimated time wins.  The estimate (microseconds) is fitted to forced launches of
 // 21 shapes on B200, r = 16 .. 4096 over 55 .. 10521 keys, which it ranks as measured: a block of 128 keys takes a
-// tile pair 1.6 and a lone tile 1.0; a unit 4 or 3 more for its own first operands and store; a launch 3.5; ranges pay
+// tile pair 1.6 and a lone tile 1.0 (0.85 as two streams); a unit 4 or 3 more for its own first operands and store; a launch 3.5; ranges pay
 // for their set-up, the barriers and the rows that cross the cluster, and 4 more for each wave after the first (a new
 // cluster starts only when all of its SMs are free).  Resident clusters come from the occupancy query, which a probe
 // confirmed to the cluster (74 / 45 / 33 / 26 / 22 of 2 .. 6 CTAs, but 15 of 7 or 8, hence the limit).
 constexpr int kMaxRanges = 6;
+
+// A launch of lone query tiles without ranges has both warp-groups on each tile, one on every other key block: two streams
+// keep the tensor core and the special-function units busy where one is a chain (B = 1, r = 16 over 6441 keys in one
+// range 55.9 -> 45.4 us; B = 16, H = 16, D = 64, r = 100 over 680 keys 18.5 -> 17.1).  Both need a block; at two and three
+// blocks they gain little but lose nothing.  In ranges the streams' meeting costs what they gain (r = 400 over 2921
+// keys in two ranges 20.7 -> 21.1), so those stay one stream.
+static bool dual_streams(int tiles_per_cta, int r, int L, int splits) {
+  return (tiles_per_cta == 1 || r <= kQRows) && splits <= 1 && L > kKeys;
+}
 
 void attention_plan(int B_eff, int H, int r, int L, int num_sms, int *tiles_per_cta, int *kv_splits) {
   const int nkv = (L + kKeys - 1) / kKeys;
@@ -663,7 +746,7 @@ void attention_plan(int B_eff, int H, int r, int L, int num_sms, int *tiles_per_
       const int per = (nkv + s - 1) / s;
       double cost;
       if (s == 1) {
-        cost = 3.5 + static_cast<double>((units + num_sms - 1) / num_sms) * (per * t_block + (pair ? 4.0 : 3.0));
+        cost = 3.5 + static_cast<double>((units + num_sms - 1) / num_sms) * (per * (pair ? 1.6 : 0.85) + (pair ? 4.0 : 3.0));
       } else {
         if (per < 4 || (nkv + per - 1) / per != s || g_max_clusters[s] <= 0) continue;   // at least four key blocks a range
         const double waves = static_cast<double>((units + g_max_clusters[s] - 1) / g_max_clusters[s]);
@@ -677,8 +760,9 @@ void attention_plan(int B_eff, int H, int r, int L, int num_sms, int *tiles_per_
 cudaError_t launch_attention(const CUtensorMap &tmQ, const CUtensorMap &tmK, const CUtensorMap &tmV,
                              const AttnArgs &a, int num_sms, cudaStream_t st) {
   if (a.r <= 0 || a.L <= 0) return cudaErrorInvalidValue;
-  if (a.D == 64) return launch_d<64>(tmQ, tmK, tmV, a, num_sms, st);
-  if (a.D == 128) return launch_d<128>(tmQ, tmK, tmV, a, num_sms, st);
+  const bool dual = dual_streams(a.tiles_per_cta, a.r, a.L, a.kv_splits);
+  if (a.D == 64) return dual ? launch_d<64, true>(tmQ, tmK, tmV, a, num_sms, st) : launch_d<64, false>(tmQ, tmK, tmV, a, num_sms, st);
+  if (a.D == 128) return dual ? launch_d<128, true>(tmQ, tmK, tmV, a, num_sms, st) : launch_d<128, false>(tmQ, tmK, tmV, a, num_sms, st);
   return cudaErrorInvalidValue;
 }
 

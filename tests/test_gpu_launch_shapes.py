@@ -24,6 +24,8 @@ def fv():
     (2, 16, 128, 1100, 1500),   # lone tiles walked: 9 tiles a head, the last of 76 rows
     (1, 16, 128, 400, 2921),    # key ranges over a cluster, four tiles, the last of 16 rows
     (1, 3, 128, 5, 6441),       # six ranges, fewer rows than a slice's share for every block
+    (16, 16, 64, 100, 600),     # lone tiles walked as two streams of 3 and 2 blocks
+    (9, 16, 64, 128, 513),      # the same, a unit a block, the last block with a single key
     (1, 40, 64, 257, 1030),     # pairs whose second unit is one row
     (1, 16, 128, 128, 128), (1, 1, 64, 1, 1),
 ])

@@ -206,7 +206,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       // The residual of the first two column chunks is fetched while the main loop still runs: with one tile per CTA
       // nothing else hides that latency; later chunks are fetched two ahead.
       constexpr int kPre = (kChunks < 2) ? kChunks : 2;
-      float4 pre[kPre][8];
+      ResidPre pre[kPre];
       ResidRow rr{-1, 0, 0, 0};
       auto col_of = [&](int ci) { return n_idx * BN + (ci * kEpiColGroups + cg) * 32; };
       auto in_tile = [&](int ci) { return (ci * kEpiColGroups + cg) * 32 < BN && col_of(ci) < p.N; };    // uniform across the warp

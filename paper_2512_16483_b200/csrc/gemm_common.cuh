@@ -183,24 +183,36 @@ __device__ __forceinline__ ResidRow resid_row(const GemmArgs &p, int row) {
   }
   return r;
 }
-// The residual values of one 32-column chunk in the order the epilogue wants them: lane l, step it holds 4 columns of
-// row 4 it + l / 8, so that eight lanes read 128 consecutive bytes.  (A row a lane, every access of a warp touched 32
-// lines and half of the sectors came from L2 twice.)
-__device__ __forceinline__ void resid_fetch(const GemmArgs &p, const ResidRow &rr, int col0, int lane, float4 (&pre)[8]) {
+// What the epilogue of one 32-column chunk reads besides the sums, in the order it wants it: lane l, step it holds 4 columns
+// of the residual of row 4 it + l / 8, so that eight lanes read 128 consecutive bytes (a row a lane, every access of a warp
+// touched 32 lines and half of the sectors came from L2 twice), and the gate of the batch element of its first row, which
+// nearly always is that of all 32 (a load a row in the chain of each store: three dense d16 scales 5332 us, without 5270).
+struct ResidPre {
+  float4 v[8], gate;
+  int b;
+};
+__device__ __forceinline__ float4 resid_gate(const GemmArgs &p, int b, int col) {
+  return p.gate ? __ldg(reinterpret_cast<const float4 *>(p.gate + static_cast<long long>(b) * p.gate_stride + col)) : make_float4(1.f, 1.f, 1.f, 1.f);
+}
+__device__ __forceinline__ void resid_fetch(const GemmArgs &p, const ResidRow &rr, int col0, int lane, ResidPre &pre) {
+  const int col = col0 + (lane & 7) * 4;
 #pragma unroll
   for (int it = 0; it < 8; ++it) {
     const int r = it * 4 + (lane >> 3);
     const int out = __shfl_sync(0xffffffffu, rr.out, r), res = __shfl_sync(0xffffffffu, rr.res, r);
-    if (out >= 0) pre[it] = *reinterpret_cast<const float4 *>(p.resid + static_cast<long long>(res) * p.ld_out + col0 + (lane & 7) * 4);
+    if (out >= 0) pre.v[it] = *reinterpret_cast<const float4 *>(p.resid + static_cast<long long>(res) * p.ld_out + col);
   }
+  pre.b = __shfl_sync(0xffffffffu, rr.b, 0);
+  pre.gate = resid_gate(p, pre.b, col);
 }
-// Gate + residual (and the hi / lo split) of four columns `col` .. col + 3 of row r of the warp's 32 rows: o = sums with
-// bias.  Every lane of the warp must call.
-__device__ __forceinline__ void resid_store(const GemmArgs &p, const ResidRow &rr, float4 o, const float4 &res, int r, int col) {
+// Gate + residual (and the hi / lo split) of four columns `col` .. col + 3 of row r = 4 it + lane / 8 of the warp's 32 rows:
+// o = sums with bias.  Every lane of the warp must call.
+__device__ __forceinline__ void resid_store(const GemmArgs &p, const ResidRow &rr, float4 o, const ResidPre &pre, int it, int r, int col) {
   const int out = __shfl_sync(0xffffffffu, rr.out, r), b = __shfl_sync(0xffffffffu, rr.b, r), split = __shfl_sync(0xffffffffu, rr.split, r);
   if (out < 0) return;
-  const float4 g = p.gate ? __ldg(reinterpret_cast<const float4 *>(p.gate + static_cast<long long>(b) * p.gate_stride + col))
-                          : make_float4(1.f, 1.f, 1.f, 1.f);
+  float4 g = pre.gate;
+  if (b != pre.b) g = resid_gate(p, b, col);
+  const float4 res = pre.v[it];
   o.x = fmaf(g.x, o.x, res.x);
   o.y = fmaf(g.y, o.y, res.y);
   o.z = fmaf(g.z, o.z, res.z);
@@ -218,7 +230,7 @@ __device__ __forceinline__ void resid_store(const GemmArgs &p, const ResidRow &r
 }
 // EPI_RESID of one warp for its 32 rows x 32 columns starting at col0 (col0 + 32 <= N).  Every lane must call.
 __device__ __forceinline__ void resid_chunk(const GemmArgs &p, const uint32_t (&acc)[32], const ResidRow &rr, int col0, uint32_t stage, int lane,
-                                            const float4 (&pre)[8]) {
+                                            const ResidPre &pre) {
 #pragma unroll
   for (int q = 0; q < 8; ++q)
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stage + lane * 128 + ((q ^ (lane & 7)) << 4)), "r"(acc[q * 4]), "r"(acc[q * 4 + 1]),
@@ -232,12 +244,16 @@ __device__ __forceinline__ void resid_chunk(const GemmArgs &p, const uint32_t (&
     f1 = __bfloat1622float2(h[1]);
   }
   __syncwarp();
+  float4 o[8];
 #pragma unroll
   for (int it = 0; it < 8; ++it) {
     const int r = it * 4 + (lane >> 3);
-    float4 o = ld_shared_f4(stage + r * 128 + ((c ^ (r & 7)) << 4));
-    o.x += f0.x; o.y += f0.y; o.z += f1.x; o.w += f1.y;
-    resid_store(p, rr, o, pre[it], r, col);
+    o[it] = ld_shared_f4(stage + r * 128 + ((c ^ (r & 7)) << 4));
+  }
+#pragma unroll
+  for (int it = 0; it < 8; ++it) {
+    o[it].x += f0.x; o[it].y += f0.y; o[it].z += f1.x; o[it].w += f1.y;
+    resid_store(p, rr, o[it], pre, it, it * 4 + (lane >> 3), col);
   }
   __syncwarp();
 }

@@ -30,7 +30,8 @@ constexpr int kFlexSmemBytes = 1024 /*alignment*/ + kFlexRing + 256 /*barriers*/
 constexpr int kFlexWAtom = kBlockM * kBlockK * 2;         // 128 weight rows x 64 K
 static_assert(kFlexSmemBytes <= 227 * 1024 && kFlexSmemBytes > 116 * 1024, "one CTA per SM");
 
-template <int EPI>
+// PRE: chunks of a warp whose residual is held in registers ahead of their sums (EPI_RESID; see launch_gemm_flex).
+template <int EPI, int PRE>
 __global__ void __launch_bounds__(kFlexThreads, 1)
 gemm_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, const __grid_constant__ GemmArgs p) {
   extern __shared__ uint8_t smem_raw[];
@@ -163,18 +164,29 @@ gemm_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       const int a = it & 1, n0 = (2 * ft + static_cast<int>(half)) * kBlockM + quad * 32;
       const int row0 = ch * nb, rows = min(nb, p.R - row0);
       RowsEpilogue<EPI> ep(p, n0, ep_stage, lane);
-      if (n0 < p.N && cg * 32 < rows) ep.prefetch(row0 + cg * 32);           // hides behind the main loop
+      // EPI_RESID: what the first PRE chunks read besides their sums is requested while the main loop runs (with one tile
+      // a CTA nothing else hides it), the later ones' PRE ahead
+      typename RowsEpilogue<EPI>::Fetch fetch[PRE];
+#pragma unroll
+      for (int u = 0; u < PRE; ++u)
+        if (n0 < p.N && (cg + u * kEpiColGroups) * 32 < rows) ep.prefetch(row0 + (cg + u * kEpiColGroups) * 32, fetch[u]);
       ok = __all_sync(0xffffffffu, mbar_wait(tfull_bar(a), (it >> 1) & 1u, p.status, &abort_flag, wb));
       if (!ok) break;
       tc_fence_after();
       const uint32_t taddr = tmem_base + a * 256 + (static_cast<uint32_t>(quad * 32) << 16);
       if (n0 < p.N) {                                                          // N % 64 == 0: whole 32-feature groups
 #pragma unroll 1
-        for (int c = cg; c * 32 < rows; c += kEpiColGroups) {
-          uint32_t acc[32];
-          tmem_ld32(taddr + c * 32, acc);
-          tmem_ld_wait();
-          ep.chunk(acc, row0 + c * 32, (c + kEpiColGroups) * 32 < rows ? row0 + (c + kEpiColGroups) * 32 : -1);
+        for (int c0 = cg; c0 * 32 < rows; c0 += PRE * kEpiColGroups) {
+#pragma unroll
+          for (int u = 0; u < PRE; ++u) {
+            const int c = c0 + u * kEpiColGroups, ahead = c + PRE * kEpiColGroups;
+            if (c * 32 >= rows) continue;
+            uint32_t acc[32];
+            tmem_ld32(taddr + c * 32, acc);
+            tmem_ld_wait();
+            ep.chunk(acc, row0 + c * 32, fetch[u]);
+            if (ahead * 32 < rows) ep.prefetch(row0 + ahead * 32, fetch[u]);
+          }
         }
       }
       tc_fence_before();
@@ -194,21 +206,22 @@ gemm_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 }
 
 // ------------------------------------------------------------------------------------------------ host
-template <int EPI>
+template <int EPI, int PRE>
 static cudaError_t flex_prepare_one() {
   static bool ready = false;
   if (ready) return cudaSuccess;
-  const cudaError_t err = cudaFuncSetAttribute(gemm_flex_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFlexSmemBytes);
+  const cudaError_t err = cudaFuncSetAttribute(gemm_flex_kernel<EPI, PRE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFlexSmemBytes);
   if (err == cudaSuccess) ready = true;
   return err;
 }
 
 cudaError_t gemm_flex_prepare() {
-  cudaError_t e = flex_prepare_one<EPI_F32>();
-  if (e == cudaSuccess) e = flex_prepare_one<EPI_BF16>();
-  if (e == cudaSuccess) e = flex_prepare_one<EPI_GELU_BF16>();
-  if (e == cudaSuccess) e = flex_prepare_one<EPI_QKV>();
-  if (e == cudaSuccess) e = flex_prepare_one<EPI_RESID>();
+  cudaError_t e = flex_prepare_one<EPI_F32, 1>();
+  if (e == cudaSuccess) e = flex_prepare_one<EPI_BF16, 1>();
+  if (e == cudaSuccess) e = flex_prepare_one<EPI_GELU_BF16, 1>();
+  if (e == cudaSuccess) e = flex_prepare_one<EPI_QKV, 1>();
+  if (e == cudaSuccess) e = flex_prepare_one<EPI_RESID, 1>();
+  if (e == cudaSuccess) e = flex_prepare_one<EPI_RESID, 2>();
   return e;
 }
 
@@ -223,9 +236,9 @@ void gemm_flex_shape(GemmArgs &a) {
   a.fx_stages = stages > kFlexMaxStages ? kFlexMaxStages : stages;
 }
 
-template <int EPI>
+template <int EPI, int PRE>
 static cudaError_t flex_launch_one(const CUtensorMap &tmA, const CUtensorMap &tmW, const GemmArgs &a, int max_clusters, cudaStream_t st) {
-  const cudaError_t err = flex_prepare_one<EPI>();
+  const cudaError_t err = flex_prepare_one<EPI, PRE>();
   if (err != cudaSuccess) return err;
   const long long tiles = static_cast<long long>((a.N + 2 * kBlockM - 1) / (2 * kBlockM)) * ((a.R + a.fx_nb - 1) / a.fx_nb);
   cudaLaunchConfig_t cfg = {};
@@ -242,7 +255,7 @@ static cudaError_t flex_launch_one(const CUtensorMap &tmA, const CUtensorMap &tm
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, gemm_flex_kernel<EPI>, tmA, tmW, a);
+  return cudaLaunchKernelEx(&cfg, gemm_flex_kernel<EPI, PRE>, tmA, tmW, a);
 }
 
 // tmA: gemm_skinny_map over the activation rows (box of a.fx_nb / 2 rows), tmW: over the weight rows (box of 128), both
@@ -252,11 +265,14 @@ cudaError_t launch_gemm_flex(int epi, const CUtensorMap &tmA, const CUtensorMap 
       a.fx_nb % 32 || a.fx_stages < 2 || max_clusters <= 0)
     return cudaErrorInvalidValue;
   switch (epi) {
-    case EPI_F32: return flex_launch_one<EPI_F32>(tmA, tmW, a, max_clusters, st);
-    case EPI_BF16: return flex_launch_one<EPI_BF16>(tmA, tmW, a, max_clusters, st);
-    case EPI_GELU_BF16: return flex_launch_one<EPI_GELU_BF16>(tmA, tmW, a, max_clusters, st);
-    case EPI_QKV: return flex_launch_one<EPI_QKV>(tmA, tmW, a, max_clusters, st);
-    case EPI_RESID: return flex_launch_one<EPI_RESID>(tmA, tmW, a, max_clusters, st);
+    case EPI_F32: return flex_launch_one<EPI_F32, 1>(tmA, tmW, a, max_clusters, st);
+    case EPI_BF16: return flex_launch_one<EPI_BF16, 1>(tmA, tmW, a, max_clusters, st);
+    case EPI_GELU_BF16: return flex_launch_one<EPI_GELU_BF16, 1>(tmA, tmW, a, max_clusters, st);
+    case EPI_QKV: return flex_launch_one<EPI_QKV, 1>(tmA, tmW, a, max_clusters, st);
+    // Up to 64 rows a tile each warp has one chunk, and the code for two only makes a cold launch longer (a step of 1 - 100
+    // rows 2391 against 2404 us); beyond, two ahead is better than one (2704 rows, three scales: 5232 against 5272).
+    case EPI_RESID:
+      return a.fx_nb <= 64 ? flex_launch_one<EPI_RESID, 1>(tmA, tmW, a, max_clusters, st) : flex_launch_one<EPI_RESID, 2>(tmA, tmW, a, max_clusters, st);
   }
   return cudaErrorInvalidValue;
 }

@@ -12,17 +12,18 @@ __device__ __forceinline__ uint2 pack4_bf16(float a, float b, float c, float d) 
 // What the epilogue of (row, features n .. n + 3) reads besides the sums: fetched together with them, so that a row pays
 // one memory latency and not two.
 struct SkinnyFetch {
-  float4 resid;
+  float4 resid, gate;
   int jo;                  // output row within the element (after the scatter)
 };
 template <int EPI>
 __device__ __forceinline__ SkinnyFetch skinny_fetch(const GemmArgs &p, int row, int n) {
   SkinnyFetch f;
-  f.resid = make_float4(0.f, 0.f, 0.f, 0.f);
+  f.resid = f.gate = make_float4(0.f, 0.f, 0.f, 0.f);
   f.jo = 0;
   if constexpr (EPI == EPI_RESID) {
     const int e = row / p.rows_per_batch, j = row - e * p.rows_per_batch;
     f.resid = *reinterpret_cast<const float4 *>(p.resid + (static_cast<long long>(e * p.rmap.bmul + p.rmap.boff) * p.rmap.rpb + j) * p.ld_out + n);
+    f.gate = resid_gate(p, e * p.bmul + p.boff, n);
     f.jo = p.scatter ? __ldg(p.scatter + static_cast<long long>(e) * p.rows_per_batch + j) : j;
   }
   return f;
@@ -64,11 +65,8 @@ __device__ __forceinline__ void skinny_store(const GemmArgs &p, float4 acc, cons
       for (int i = 0; i < 4; ++i) dst[static_cast<long long>(i) * p.L_cap] = __float2bfloat16_rn(v[i]);
     }
   } else if constexpr (EPI == EPI_RESID) {
-    const int e = row / p.rows_per_batch, b = e * p.bmul + p.boff;
-    const float4 r4 = f.resid;
-    const int jo = f.jo;
-    const float4 g4 = p.gate ? __ldg(reinterpret_cast<const float4 *>(p.gate + static_cast<long long>(b) * p.gate_stride + n))
-                             : make_float4(1.f, 1.f, 1.f, 1.f);
+    const int e = row / p.rows_per_batch, jo = f.jo;
+    const float4 r4 = f.resid, g4 = f.gate;
     v[0] = fmaf(g4.x, v[0], r4.x);
     v[1] = fmaf(g4.y, v[1], r4.y);
     v[2] = fmaf(g4.z, v[2], r4.z);
@@ -111,22 +109,23 @@ struct RowsEpilogue {
   const int n0, lane;
   const uint32_t stage;                // 32 x 132 bytes of shared memory of this warp
   float bias;                          // of this lane's feature
-  float4 pre[8];                       // EPI_RESID: residual of the next chunk
-  ResidRow rr;
-
   __device__ __forceinline__ RowsEpilogue(const GemmArgs &args, int first_feature, uint32_t stage_addr, int l)
-      : p(args), n0(first_feature), lane(l), stage(stage_addr), rr{-1, 0, 0, 0} {
+      : p(args), n0(first_feature), lane(l), stage(stage_addr) {
     bias = (p.bias != nullptr && n0 < p.N) ? __bfloat162float(p.bias[n0 + lane]) : 0.f;
   }
-  // Requests what the chunk of rows `row0` .. row0 + 31 reads besides its sums.
-  __device__ __forceinline__ void prefetch(int row0) {
+  // What the chunk of rows `row0` .. row0 + 31 reads besides its sums (EPI_RESID).
+  struct Fetch {
+    ResidRow rr;
+    ResidPre pre;
+  };
+  __device__ __forceinline__ void prefetch(int row0, Fetch &f) const {
     if constexpr (EPI == EPI_RESID) {
-      rr = resid_row(p, row0 + lane);
-      resid_fetch(p, rr, n0, lane, pre);
+      f.rr = resid_row(p, row0 + lane);
+      resid_fetch(p, f.rr, n0, lane, f.pre);
     }
   }
-  // acc[i] = sum of row row0 + i; next_row0 >= 0: the warp's next chunk, to be prefetched.
-  __device__ __forceinline__ void chunk(const uint32_t (&acc)[32], int row0, int next_row0) {
+  // acc[i] = sum of row row0 + i.
+  __device__ __forceinline__ void chunk(const uint32_t (&acc)[32], int row0, const Fetch &f) const {
     const int vc0 = n0 + p.col_base;
     if (EPI == EPI_QKV && vc0 >= 2 * p.C) {              // uniform across the warp: C % 64 == 0
 #pragma unroll
@@ -163,12 +162,15 @@ struct RowsEpilogue {
     __syncwarp();
     const int c4 = lane & 7, n = n0 + c4 * 4, vc = vc0 + c4 * 4;
     const int ck = vc - p.C, hk = (EPI == EPI_QKV) ? ck / p.D : 0, dk = ck - hk * p.D;
+    float4 v[8];                         // all of them, then the stores: neither waits for the other row by row
+#pragma unroll
+    for (int it = 0; it < 8; ++it) v[it] = ld_shared_f4(stage + (it * 4 + (lane >> 3)) * 128 + c4 * 16);
 #pragma unroll
     for (int it = 0; it < 8; ++it) {
       const int r = it * 4 + (lane >> 3), row = row0 + r;
-      const float4 o = ld_shared_f4(stage + r * 128 + c4 * 16);
+      const float4 o = v[it];
       if constexpr (EPI == EPI_RESID) {
-        resid_store(p, rr, o, pre[it], r, n);
+        resid_store(p, f.rr, o, f.pre, it, r, n);
       } else if constexpr (EPI == EPI_F32) {
         if (row < p.R) *reinterpret_cast<float4 *>(p.out_f32 + static_cast<long long>(row) * p.ld_out + n) = o;
       } else if constexpr (EPI == EPI_QKV) {
@@ -183,7 +185,6 @@ struct RowsEpilogue {
       }
     }
     __syncwarp();
-    if (next_row0 >= 0) prefetch(next_row0);
   }
 };
 

@@ -89,10 +89,10 @@ def test_gemm_free_width_pairs(fv, R, N, K, width):
     assert (out.double() - ref).abs().max() <= bound
 
 
-@pytest.mark.parametrize("shape,B,k,bar", [("d16", 16, 8, 2e-2), ("infinity", 1, 7, 3e-2)])
+@pytest.mark.parametrize("shape,B,k,bar", [("d16", 16, 8, 2e-2), ("d16", 2, 7, 2e-2), ("infinity", 1, 7, 3e-2)])
 def test_step_epilogues_of_the_free_width_pairs(fv, shape, B, k, bar):
     """One dense block at sizes where QKV, out-proj and both FFN GEMMs take that form between them (2704 rows of 1024
-    columns; 400 rows of 2048): every epilogue of it, KV cache included, against the CPU oracle."""
+    columns; 200; 400 rows of 2048): every epilogue of it, KV cache included, against the CPU oracle."""
     import numpy as np
     from oracle import fvar_oracle as orc
     from helpers import assert_close

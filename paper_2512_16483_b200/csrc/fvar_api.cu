@@ -412,6 +412,7 @@ fvar_status run_gemm(fvar_ctx *ctx, int epi, const fvar_ctx::ActMaps &maps, int 
                       (epi == EPI_F32 || epi == EPI_RESID ? 4.0 : 2.0) * g.R * g.N * g.nbatch);
   if (plan.form == kGemmFlex) {
     g.fx_nb = plan.block_n;
+    g.fx_early = 1;                                // the caller's weights: no kernel of the library writes them
     gemm_flex_shape(g);
     CUtensorMap tmA, tmW;
     if (!gemm_skinny_map(&tmA, maps.base, maps.rows, maps.cols, maps.cols, g.fx_nb / 2, g.fx_nk) || !gemm_skinny_map(&tmW, ctx->w[wid][blk], g.N, g.K, g.K, 128, g.fx_nk))

@@ -80,6 +80,19 @@ gemm_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   cluster_sync_all();                 // the peer's barriers are initialised before anything signals them
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_holder;
+  const uint32_t full0 = mapa_shared(full_bar(0), 0);
+  const int pre = p.fx_early ? min(nstages, nst) : 0;
+  if (threadIdx.x == 0) {
+    // While the predecessor drains: the weights of the first stages, which wait for nothing but the barriers just
+    // initialised.  A loop of its own -- a test per stage inside the producer's made it miss its pace (400 x 6144 x 2048
+    // 13.0 -> 14.9 us) and hid that this gains (Infinity 40 with table 3698 -> 3665 us).
+    const int row_w = (2 * (tile0 / chunks) + static_cast<int>(half)) * kBlockM;
+    for (int i = 0; i < pre; ++i) {
+      if (half == 0) mbar_expect_tx(full_bar(i), 2u * stage_bytes);
+      if (nk > 1) tma_load_3d_pair(ring + i * stage_bytes, &tmW, full0 + 8u * i, 0, row_w, i * nk);
+      else tma_load_2d_pair(ring + i * stage_bytes, &tmW, full0 + 8u * i, i * kBlockK, row_w);
+    }
+  }
   pdl_wait();
   pdl_launch_dependents();
   bool ok = true;
@@ -87,14 +100,19 @@ gemm_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   if (warp == 0) {
     if (lane == 0) {
       // ---------------------------------------------------------------- TMA producer (both CTAs)
-      const uint32_t full0 = mapa_shared(full_bar(0), 0);
-      int stage = 0;
-      uint32_t phase = 0;
-      bool issued = false;
+      const int row_a0 = (tile0 % chunks) * nb + static_cast<int>(half) * (nb / 2);
+      for (int i = 0; i < pre; ++i) {
+        const uint32_t sa = ring + i * stage_bytes + nk * kFlexWAtom;
+        if (nk > 1) tma_load_3d_pair(sa, &tmA, full0 + 8u * i, 0, row_a0, i * nk);
+        else tma_load_2d_pair(sa, &tmA, full0 + 8u * i, i * kBlockK, row_a0);
+      }
+      int stage = pre == nstages ? 0 : pre, first = pre;
+      uint32_t phase = pre == nstages ? 1u : 0u;
+      bool issued = pre > 0;
       for (int tile = tile0; ok && tile < total; tile += tile_step) {
         const int ft = tile / chunks, ch = tile - ft * chunks;
         const int row_w = (2 * ft + static_cast<int>(half)) * kBlockM, row_a = ch * nb + static_cast<int>(half) * (nb / 2);
-        for (int i = 0; i < nst; ++i) {
+        for (int i = first; i < nst; ++i) {
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, p.status, &abort_flag, wb)) { ok = false; break; }
           if (half == 0) mbar_expect_tx(full_bar(stage), 2u * stage_bytes);
           const uint32_t sa = ring + stage * stage_bytes, fb = full0 + 8u * stage;
@@ -108,6 +126,7 @@ gemm_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           issued = true;
           if (++stage == nstages) { stage = 0; phase ^= 1u; }
         }
+        first = 0;
       }
       if (!ok && issued) {
         // The byte counts of this CTA's copies go to the even CTA's barriers, which cannot be polled from here in

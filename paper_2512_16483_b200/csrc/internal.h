@@ -81,6 +81,7 @@ struct GemmArgs {
   // CTA-pair form with a free row width (gemm_flex.cu): rows of a tile (a multiple of 32 up to 256), K blocks per
   // pipeline stage, stages
   int fx_nb, fx_nk, fx_stages;
+  int fx_early;            // nothing in flight writes the weights: the first stages of them are requested before the wait
   // optional: weights the next GEMM of the chain will stream; every CTA asks L2 to prefetch its share
   const void *pf_ptr;
   unsigned long long pf_bytes;

@@ -214,11 +214,13 @@ cudaError_t launch_copy_indices(const int *forced, int B, int M, int r, int ld_f
 constexpr int kLnThreads = 128;
 constexpr int kLnMaxVec = 16;                   // float4 a thread: 8192 columns
 
-template <int T>
-__global__ void __launch_bounds__(kLnThreads) ln_modulate_kernel(const float *__restrict__ x, RowMap xmap, int rows, int C,
+// PARTS: the row is completed first, x += gate * (sum of the K ranges of the GEMM before it, in range order, + bias),
+// and written back; the reads of the ranges hide in the latency that the row's own have.
+template <int T, bool PARTS>
+__global__ void __launch_bounds__(kLnThreads) ln_modulate_kernel(const float *x, RowMap xmap, int rows, int C,
                                                                  const float *__restrict__ shift, const float *__restrict__ scale,
                                                                  long long vec_stride, int bmul, int boff, const bf16 *__restrict__ gamma,
-                                                                 float eps, int early, bf16 *__restrict__ y) {
+                                                                 float eps, int early, bf16 *__restrict__ y, LnParts parts) {
   pdl_launch_dependents();      // nothing precedes the wait but loads: the successor may start its own prologue right away
   __shared__ float red[2][kLnThreads / 32];
   constexpr bool kHold = T <= 4;                // the vectors fit in registers beside the row
@@ -244,6 +246,18 @@ __global__ void __launch_bounds__(kLnThreads) ln_modulate_kernel(const float *__
       if (tid + t * kLnThreads < n4) { mul[kHold ? t : 0] = vec_mul(tid + t * kLnThreads); add[kHold ? t : 0] = vec_add(tid + t * kLnThreads); }
   };
   if (kHold && early) fetch_vecs();
+  float4 gate[PARTS ? T : 1], bias[PARTS ? T : 1];
+  if constexpr (PARTS) {
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+      const int g = tid + t * kLnThreads;
+      if (g >= n4) continue;
+      gate[t] = __ldg(reinterpret_cast<const float4 *>(parts.gate + voff) + g);
+      const uint2 u = __ldg(reinterpret_cast<const uint2 *>(parts.bias) + g);
+      const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.x)), b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.y));
+      bias[t] = make_float4(a.x, a.y, b.x, b.y);
+    }
+  }
   pdl_wait();
   if (kHold && !early) fetch_vecs();
   const float4 *xr = reinterpret_cast<const float4 *>(x + (static_cast<long long>(e * xmap.bmul + xmap.boff) * xmap.rpb + j) * C);
@@ -251,6 +265,27 @@ __global__ void __launch_bounds__(kLnThreads) ln_modulate_kernel(const float *__
   float sum = 0.f;
 #pragma unroll
   for (int t = 0; t < T; ++t) v[t] = tid + t * kLnThreads < n4 ? xr[tid + t * kLnThreads] : make_float4(0.f, 0.f, 0.f, 0.f);
+  if constexpr (PARTS) {
+    const float4 *pr = reinterpret_cast<const float4 *>(parts.part + static_cast<long long>(blockIdx.x) * C);
+    float4 *xw = const_cast<float4 *>(xr);
+    float4 q[kMaxParts][T];
+#pragma unroll
+    for (int s = 0; s < kMaxParts; ++s)
+#pragma unroll
+      for (int t = 0; t < T; ++t)
+        q[s][t] = (s < parts.splits && tid + t * kLnThreads < n4) ? pr[s * (parts.stride >> 2) + tid + t * kLnThreads] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+      if (tid + t * kLnThreads >= n4) continue;
+      float4 a = q[0][t];
+#pragma unroll
+      for (int s = 1; s < kMaxParts; ++s) { a.x += q[s][t].x; a.y += q[s][t].y; a.z += q[s][t].z; a.w += q[s][t].w; }
+      a.x += bias[t].x; a.y += bias[t].y; a.z += bias[t].z; a.w += bias[t].w;
+      v[t].x = fmaf(gate[t].x, a.x, v[t].x); v[t].y = fmaf(gate[t].y, a.y, v[t].y);
+      v[t].z = fmaf(gate[t].z, a.z, v[t].z); v[t].w = fmaf(gate[t].w, a.w, v[t].w);
+      xw[tid + t * kLnThreads] = v[t];
+    }
+  }
 #pragma unroll
   for (int t = 0; t < T; ++t) sum += (v[t].x + v[t].y) + (v[t].z + v[t].w);
   auto block_sum = [&](float val, int k) {
@@ -290,13 +325,27 @@ cudaError_t launch_ln_modulate(const float *x, RowMap xmap, int E, int rows, int
   if (E * rows <= 0) return cudaSuccess;
   if (C % 8 != 0 || C > 4 * kLnThreads * kLnMaxVec) return cudaErrorInvalidValue;
   auto go = [&](auto kern) {
-    return launch_pdl(kern, dim3(E * rows), dim3(kLnThreads), 0, st, x, xmap, rows, C, shift, scale, vec_stride, bmul, boff, gamma, eps, early ? 1 : 0, y);
+    return launch_pdl(kern, dim3(E * rows), dim3(kLnThreads), 0, st, x, xmap, rows, C, shift, scale, vec_stride, bmul, boff, gamma, eps, early ? 1 : 0, y, LnParts{});
   };
-  if (C <= 512) return go(ln_modulate_kernel<1>);
-  if (C <= 1024) return go(ln_modulate_kernel<2>);
-  if (C <= 2048) return go(ln_modulate_kernel<4>);
-  if (C <= 4096) return go(ln_modulate_kernel<8>);
-  return go(ln_modulate_kernel<16>);
+  if (C <= 512) return go(ln_modulate_kernel<1, false>);
+  if (C <= 1024) return go(ln_modulate_kernel<2, false>);
+  if (C <= 2048) return go(ln_modulate_kernel<4, false>);
+  if (C <= 4096) return go(ln_modulate_kernel<8, false>);
+  return go(ln_modulate_kernel<16, false>);
+}
+
+// C <= 2048: gemm_partial_plan takes no wider output.
+cudaError_t launch_ln_parts(float *x, RowMap xmap, int E, int rows, int C, const LnParts &parts, const float *shift, const float *scale,
+                            long long vec_stride, int bmul, int boff, float eps, bf16 *y, cudaStream_t st) {
+  if (E * rows <= 0) return cudaSuccess;
+  if (C % 8 != 0 || C > 2048 || parts.splits < 1 || parts.splits > kMaxParts || parts.stride % 4 != 0) return cudaErrorInvalidValue;
+  auto go = [&](auto kern) {
+    return launch_pdl(kern, dim3(E * rows), dim3(kLnThreads), 0, st, static_cast<const float *>(x), xmap, rows, C, shift, scale, vec_stride, bmul, boff,
+                      static_cast<const bf16 *>(nullptr), eps, 1, y, parts);
+  };
+  if (C <= 512) return go(ln_modulate_kernel<1, true>);
+  if (C <= 1024) return go(ln_modulate_kernel<2, true>);
+  return go(ln_modulate_kernel<4, true>);
 }
 
 // ------------------------------------------------------------------------------------------------

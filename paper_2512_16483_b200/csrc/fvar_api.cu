@@ -353,6 +353,28 @@ fvar_status cuda_fail(fvar_ctx *ctx, cudaError_t e, const char *what) {
     if (e__ != cudaSuccess) return cuda_fail(ctx, e__, what);   \
   } while (0)
 
+GemmArgs gemm_args(int R, int N, int K);
+
+// The sums of `ranges` K ranges of A W^T, each [R][N], to the scratch area (gemm_partial_plan).
+fvar_status run_gemm_parts(fvar_ctx *ctx, const fvar_ctx::ActMaps &maps, int blk, int wid, int R, int N, int K, int ranges, int rows_tile) {
+  GemmArgs g = gemm_args(R, N, K);
+  g.out_f32 = ctx->split_partial;
+  g.ld_out = N;
+  g.splits = ranges;
+  g.fx_nb = rows_tile;
+  g.fx_early = 1;
+  g.status = ctx->status;
+  g.wait_cycles = ctx->wait_cycles;
+  gemm_flex_shape(g);
+  CUtensorMap tmA, tmW;
+  if (!gemm_skinny_map(&tmA, maps.base, maps.rows, maps.cols, maps.cols, g.fx_nb / 2, g.fx_nk) || !gemm_skinny_map(&tmW, ctx->w[wid][blk], N, K, K, 128, g.fx_nk))
+    return fail(ctx, FVAR_ECUDA, "tensor map encoding failed");
+  ctx->prof_begin(FVAR_KCLASS_GEMM, 2.0 * R * N * K, 2.0 * (static_cast<double>(N) * K + static_cast<double>(R) * K) + 4.0 * ranges * R * N);
+  FV_CUDA(ctx, launch_gemm_flex(EPI_PARTIAL, tmA, tmW, g, ctx->max_clusters, ctx->launch_st), "gemm in K ranges");
+  ctx->launched();
+  return FVAR_OK;
+}
+
 // out = A W^T (+ epilogue) on the context's stream; form and tile width from the problem size.  A operand: one of the
 // library's activation buffers; a single row tile takes the shortest box that covers its rows.
 fvar_status run_gemm(fvar_ctx *ctx, int epi, const fvar_ctx::ActMaps &maps, int blk, int wid, GemmArgs &g, const char *what) {
@@ -1149,6 +1171,7 @@ static fvar_status scale_step_impl(fvar_ctx *ctx, const void *tokens, bool token
       ctx->launched();
     }
 
+    LnParts parts{};                      // fc2 of the block before, left in K ranges for this block's first LayerNorm
     for (int t = 0; t < bpg; ++t) {
       const int blk = g * bpg + t;
       const bool first_dense = (t == 0) && !late, last = (t == bpg - 1);
@@ -1163,8 +1186,12 @@ static fvar_status scale_step_impl(fvar_ctx *ctx, const void *tokens, bool token
       };
 
       ctx->prof_begin(FVAR_KCLASS_LN, 0.0, 6.0 * R * C);
-      FV_CUDA(ctx, launch_ln_modulate(in_ptr, in_map, E, r, C, ada, ada + C, 6 * C, bmul, boff, nullptr,
-                                      ctx->cfg.ln_eps, true, ctx->y, st), "ln_modulate 1");
+      if (parts.splits > 0)
+        FV_CUDA(ctx, launch_ln_parts(ctx->xs, smap, E, r, C, parts, ada, ada + C, 6 * C, bmul, boff, ctx->cfg.ln_eps, ctx->y, st), "ln_modulate 1");
+      else
+        FV_CUDA(ctx, launch_ln_modulate(in_ptr, in_map, E, r, C, ada, ada + C, 6 * C, bmul, boff, nullptr,
+                                        ctx->cfg.ln_eps, true, ctx->y, st), "ln_modulate 1");
+      parts.splits = 0;
       ctx->launched();
       {
         GemmArgs ga = gemm_args(R, 3 * C, C);
@@ -1242,7 +1269,15 @@ static fvar_status scale_step_impl(fvar_ctx *ctx, const void *tokens, bool token
           ga.out_f32 = ctx->xs; ga.omap = smap;
         }
         prefetch_next(ga, blk + 1, W_QKV);
-        if ((s = run_gemm(ctx, EPI_RESID, ctx->h_map, blk, W_FC2, ga, "fc2 gemm")) != FVAR_OK) return s;
+        int rows_tile = 0;
+        const int ranges = (last || ctx->skinny_max_rows <= 0 || ctx->b_fc2[blk] == nullptr) ? 0 : gemm_partial_plan(R, C, F, ctx->max_clusters, &rows_tile);
+        if (ranges > 0 && static_cast<size_t>(ranges) * R * C * 4 <= kSplitScratchBytes) {
+          // the next block's first LayerNorm adds the K ranges up; the residual stream stays where it is until then
+          parts = LnParts{ctx->split_partial, ranges, static_cast<long long>(R) * C, ctx->b_fc2[blk], ga.gate};
+          if ((s = run_gemm_parts(ctx, ctx->h_map, blk, W_FC2, R, C, F, ranges, rows_tile)) != FVAR_OK) return s;
+        } else {
+          if ((s = run_gemm(ctx, EPI_RESID, ctx->h_map, blk, W_FC2, ga, "fc2 gemm")) != FVAR_OK) return s;
+        }
       }
       ctx->staged[blk] = r;
     }

@@ -51,11 +51,14 @@ gemm_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const int nb = p.fx_nb, nk = p.fx_nk, nstages = p.fx_stages;
   const int tiles_f = (p.N + 2 * kBlockM - 1) / (2 * kBlockM), chunks = (p.R + nb - 1) / nb;
   const int total = tiles_f * chunks;
-  const int tile0 = static_cast<int>(cluster_id_x()), tile_step = static_cast<int>(cluster_nctaid_x());
+  constexpr bool kPart = EPI == EPI_PARTIAL;
+  const int range = kPart ? static_cast<int>(cluster_id_x()) / total : 0;            // kPart: one tile and K range a pair
+  const int tile0 = static_cast<int>(cluster_id_x()) - range * total, tile_step = kPart ? total : static_cast<int>(cluster_nctaid_x());
   const uint32_t b_bytes = static_cast<uint32_t>(nb / 2) * (kBlockK * 2);            // this CTA's rows of one K block
   const uint32_t stage_bytes = nk * (kFlexWAtom + b_bytes);
   const int num_kb = (p.K + kBlockK - 1) / kBlockK;
-  const int nst = (num_kb + nk - 1) / nk;                                            // stages of a tile
+  const int nst = (num_kb + nk - 1) / nk / (kPart ? p.splits : 1);                   // stages of a tile
+  const int k0 = kPart ? range * nst * nk : 0;                                       // first K block
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -89,8 +92,8 @@ gemm_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const int row_w = (2 * (tile0 / chunks) + static_cast<int>(half)) * kBlockM;
     for (int i = 0; i < pre; ++i) {
       if (half == 0) mbar_expect_tx(full_bar(i), 2u * stage_bytes);
-      if (nk > 1) tma_load_3d_pair(ring + i * stage_bytes, &tmW, full0 + 8u * i, 0, row_w, i * nk);
-      else tma_load_2d_pair(ring + i * stage_bytes, &tmW, full0 + 8u * i, i * kBlockK, row_w);
+      if (nk > 1) tma_load_3d_pair(ring + i * stage_bytes, &tmW, full0 + 8u * i, 0, row_w, k0 + i * nk);
+      else tma_load_2d_pair(ring + i * stage_bytes, &tmW, full0 + 8u * i, (k0 + i) * kBlockK, row_w);
     }
   }
   pdl_wait();
@@ -103,8 +106,8 @@ gemm_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       const int row_a0 = (tile0 % chunks) * nb + static_cast<int>(half) * (nb / 2);
       for (int i = 0; i < pre; ++i) {
         const uint32_t sa = ring + i * stage_bytes + nk * kFlexWAtom;
-        if (nk > 1) tma_load_3d_pair(sa, &tmA, full0 + 8u * i, 0, row_a0, i * nk);
-        else tma_load_2d_pair(sa, &tmA, full0 + 8u * i, i * kBlockK, row_a0);
+        if (nk > 1) tma_load_3d_pair(sa, &tmA, full0 + 8u * i, 0, row_a0, k0 + i * nk);
+        else tma_load_2d_pair(sa, &tmA, full0 + 8u * i, (k0 + i) * kBlockK, row_a0);
       }
       int stage = pre == nstages ? 0 : pre, first = pre;
       uint32_t phase = pre == nstages ? 1u : 0u;
@@ -117,11 +120,11 @@ gemm_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           if (half == 0) mbar_expect_tx(full_bar(stage), 2u * stage_bytes);
           const uint32_t sa = ring + stage * stage_bytes, fb = full0 + 8u * stage;
           if (nk > 1) {              // K blocks past the end of K are zero-filled and not multiplied
-            tma_load_3d_pair(sa, &tmW, fb, 0, row_w, i * nk);
-            tma_load_3d_pair(sa + nk * kFlexWAtom, &tmA, fb, 0, row_a, i * nk);
+            tma_load_3d_pair(sa, &tmW, fb, 0, row_w, k0 + i * nk);
+            tma_load_3d_pair(sa + nk * kFlexWAtom, &tmA, fb, 0, row_a, k0 + i * nk);
           } else {
-            tma_load_2d_pair(sa, &tmW, fb, i * kBlockK, row_w);
-            tma_load_2d_pair(sa + kFlexWAtom, &tmA, fb, i * kBlockK, row_a);
+            tma_load_2d_pair(sa, &tmW, fb, (k0 + i) * kBlockK, row_w);
+            tma_load_2d_pair(sa + kFlexWAtom, &tmA, fb, (k0 + i) * kBlockK, row_a);
           }
           issued = true;
           if (++stage == nstages) { stage = 0; phase ^= 1u; }
@@ -156,7 +159,7 @@ gemm_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           tc_fence_after();
           const uint32_t sa = ring + stage * stage_bytes;
           uint64_t dw = smem_desc_sw128(sa), da = smem_desc_sw128(sa + nk * kFlexWAtom);
-          const int kvalid = min(nk, num_kb - i * nk);
+          const int kvalid = min(nk, num_kb - k0 - i * nk);
           for (int kk = 0; kk < kvalid; ++kk) {
 #pragma unroll
             for (int k = 0; k < kBlockK / 16; ++k) {
@@ -182,7 +185,7 @@ gemm_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       const int ft = tile / chunks, ch = tile - ft * chunks;
       const int a = it & 1, n0 = (2 * ft + static_cast<int>(half)) * kBlockM + quad * 32;
       const int row0 = ch * nb, rows = min(nb, p.R - row0);
-      RowsEpilogue<EPI> ep(p, n0, ep_stage, lane);
+      RowsEpilogue<EPI> ep(p, n0, ep_stage, lane, range);
       // EPI_RESID: what the first PRE chunks read besides their sums is requested while the main loop runs (with one tile
       // a CTA nothing else hides it), the later ones' PRE ahead
       typename RowsEpilogue<EPI>::Fetch fetch[PRE];
@@ -239,6 +242,7 @@ cudaError_t gemm_flex_prepare() {
   if (e == cudaSuccess) e = flex_prepare_one<EPI_BF16, 1>();
   if (e == cudaSuccess) e = flex_prepare_one<EPI_GELU_BF16, 1>();
   if (e == cudaSuccess) e = flex_prepare_one<EPI_QKV, 1>();
+  if (e == cudaSuccess) e = flex_prepare_one<EPI_PARTIAL, 1>();
   if (e == cudaSuccess) e = flex_prepare_one<EPI_RESID, 1>();
   if (e == cudaSuccess) e = flex_prepare_one<EPI_RESID, 2>();
   return e;
@@ -255,11 +259,26 @@ void gemm_flex_shape(GemmArgs &a) {
   a.fx_stages = stages > kFlexMaxStages ? kFlexMaxStages : stages;
 }
 
+// The reduction of a K split over CTAs costs a cluster barrier and a round of remote reads after the last MMA, and the
+// 128 x 128 tiles of that form (gemm_skinny.cu) move twice the operands of 256 x 224.  Where a LayerNorm follows, it
+// can add up the ranges while it reads its rows: 400 x 2048 x 8192 with its gate and residual 25.9 us in the chain, now 17 and 1 in the
+// LayerNorm (Infinity 40 with table 3693 -> 3578 us, three late scales 11014 -> 10650).  Taken where that form is the
+// alternative (gemm_ksplit_wins) and the rows are more than one chunk; at least three ranges, or too few pairs work.
+int gemm_partial_plan(int R, int N, int K, int max_clusters, int *rows_tile) {
+  if (R <= 256 || !gemm_ksplit_wins(R, N, K) || !gemm_flex_supported(EPI_PARTIAL, N, K) || K % kBlockK != 0) return 0;
+  const int tiles_f = (N + 2 * kBlockM - 1) / (2 * kBlockM), chunks = (R + 255) / 256, num_kb = K / kBlockK;
+  *rows_tile = ((R + chunks - 1) / chunks + 31) / 32 * 32;
+  for (int s = kMaxParts; s >= 3; --s)
+    if (num_kb % (2 * s) == 0 && tiles_f * chunks * s <= max_clusters) return s;
+  return 0;
+}
+
 template <int EPI, int PRE>
 static cudaError_t flex_launch_one(const CUtensorMap &tmA, const CUtensorMap &tmW, const GemmArgs &a, int max_clusters, cudaStream_t st) {
   const cudaError_t err = flex_prepare_one<EPI, PRE>();
   if (err != cudaSuccess) return err;
-  const long long tiles = static_cast<long long>((a.N + 2 * kBlockM - 1) / (2 * kBlockM)) * ((a.R + a.fx_nb - 1) / a.fx_nb);
+  const long long tiles = static_cast<long long>((a.N + 2 * kBlockM - 1) / (2 * kBlockM)) * ((a.R + a.fx_nb - 1) / a.fx_nb) * (EPI == EPI_PARTIAL ? a.splits : 1);
+  if (EPI == EPI_PARTIAL && (tiles > max_clusters || a.K % (kBlockK * a.fx_nk * a.splits) != 0)) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * static_cast<unsigned>(tiles < max_clusters ? tiles : max_clusters));
   cfg.blockDim = dim3(kFlexThreads);
@@ -280,13 +299,14 @@ static cudaError_t flex_launch_one(const CUtensorMap &tmA, const CUtensorMap &tm
 // tmA: gemm_skinny_map over the activation rows (box of a.fx_nb / 2 rows), tmW: over the weight rows (box of 128), both
 // with a.fx_nk K blocks.  max_clusters: resident CTA pairs (gemm_pair_max_clusters).
 cudaError_t launch_gemm_flex(int epi, const CUtensorMap &tmA, const CUtensorMap &tmW, const GemmArgs &a, int max_clusters, cudaStream_t st) {
-  if (a.nbatch != 1 || a.w_mn_major || a.splits > 1 || a.R <= 0 || !gemm_flex_supported(epi, a.N, a.K) || a.fx_nb < 32 || a.fx_nb > 256 ||
+  if (a.nbatch != 1 || a.w_mn_major || (a.splits > 1 && epi != EPI_PARTIAL) || a.splits < 0 || a.R <= 0 || !gemm_flex_supported(epi, a.N, a.K) || a.fx_nb < 32 || a.fx_nb > 256 ||
       a.fx_nb % 32 || a.fx_stages < 2 || max_clusters <= 0)
     return cudaErrorInvalidValue;
   switch (epi) {
     case EPI_F32: return flex_launch_one<EPI_F32, 1>(tmA, tmW, a, max_clusters, st);
     case EPI_BF16: return flex_launch_one<EPI_BF16, 1>(tmA, tmW, a, max_clusters, st);
     case EPI_GELU_BF16: return flex_launch_one<EPI_GELU_BF16, 1>(tmA, tmW, a, max_clusters, st);
+    case EPI_PARTIAL: return a.splits > 0 ? flex_launch_one<EPI_PARTIAL, 1>(tmA, tmW, a, max_clusters, st) : cudaErrorInvalidValue;
     case EPI_QKV: return flex_launch_one<EPI_QKV, 1>(tmA, tmW, a, max_clusters, st);
     // Up to 64 rows a tile each warp has one chunk, and the code for two only makes a cold launch longer (a step of 1 - 100
     // rows 2391 against 2404 us); beyond, two ahead is better than one (2704 rows, three scales: 5232 against 5272).

@@ -108,9 +108,10 @@ struct RowsEpilogue {
   const GemmArgs &p;
   const int n0, lane;
   const uint32_t stage;                // 32 x 132 bytes of shared memory of this warp
+  const int range;                     // EPI_PARTIAL: K range
   float bias;                          // of this lane's feature
-  __device__ __forceinline__ RowsEpilogue(const GemmArgs &args, int first_feature, uint32_t stage_addr, int l)
-      : p(args), n0(first_feature), lane(l), stage(stage_addr) {
+  __device__ __forceinline__ RowsEpilogue(const GemmArgs &args, int first_feature, uint32_t stage_addr, int l, int k_range)
+      : p(args), n0(first_feature), lane(l), stage(stage_addr), range(k_range) {
     bias = (p.bias != nullptr && n0 < p.N) ? __bfloat162float(p.bias[n0 + lane]) : 0.f;
   }
   // What the chunk of rows `row0` .. row0 + 31 reads besides its sums (EPI_RESID).
@@ -171,8 +172,9 @@ struct RowsEpilogue {
       const float4 o = v[it];
       if constexpr (EPI == EPI_RESID) {
         resid_store(p, f.rr, o, f.pre, it, r, n);
-      } else if constexpr (EPI == EPI_F32) {
-        if (row < p.R) *reinterpret_cast<float4 *>(p.out_f32 + static_cast<long long>(row) * p.ld_out + n) = o;
+      } else if constexpr (EPI == EPI_F32 || EPI == EPI_PARTIAL) {
+        const int at = EPI == EPI_PARTIAL ? range * p.R + row : row;
+        if (row < p.R) *reinterpret_cast<float4 *>(p.out_f32 + static_cast<long long>(at) * p.ld_out + n) = o;
       } else if constexpr (EPI == EPI_QKV) {
         const int ko = __shfl_sync(0xffffffffu, k_off, r);
         if (row < p.R) {

@@ -33,7 +33,7 @@ __host__ __device__ inline BilinearTap bilinear_tap(int y, int x, int h0, int w0
   return t;
 }
 
-enum EpiMode { EPI_F32 = 0, EPI_BF16 = 1, EPI_GELU_BF16 = 2, EPI_QKV = 3, EPI_RESID = 4, EPI_ARGMAX = 5 };
+enum EpiMode { EPI_F32 = 0, EPI_BF16 = 1, EPI_GELU_BF16 = 2, EPI_QKV = 3, EPI_RESID = 4, EPI_ARGMAX = 5, EPI_PARTIAL = 6 };
 
 struct GemmArgs {
   int R, N, K;            // out[R][N] = A[R][K] * W[N][K]^T, per batch
@@ -81,6 +81,8 @@ struct GemmArgs {
   // CTA-pair form with a free row width (gemm_flex.cu): rows of a tile (a multiple of 32 up to 256), K blocks per
   // pipeline stage, stages
   int fx_nb, fx_nk, fx_stages;
+  // EPI_PARTIAL (that form only): `splits` K ranges of whole stages, each one's sums [R][ld_out] fp32 (no bias) at
+  // out_f32 + range * R * ld_out; one tile a pair
   int fx_early;            // nothing in flight writes the weights: the first stages of them are requested before the wait
   // optional: weights the next GEMM of the chain will stream; every CTA asks L2 to prefetch its share
   const void *pf_ptr;
@@ -138,6 +140,8 @@ cudaError_t gemm_skinny_prepare();
 // tmA / tmW: gemm_skinny_map with boxes of fx_nb / 2 and 128 rows.
 bool gemm_flex_supported(int epi, int N, int K);
 void gemm_flex_shape(GemmArgs &a);
+// K ranges (and rows a tile) for an R x N x K product whose sums the following LayerNorm adds up; 0: other forms are better.
+int gemm_partial_plan(int R, int N, int K, int max_clusters, int *rows_tile);
 cudaError_t launch_gemm_flex(int epi, const CUtensorMap &tmA, const CUtensorMap &tmW, const GemmArgs &a, int max_clusters, cudaStream_t st);
 cudaError_t gemm_flex_prepare();
 
@@ -194,6 +198,17 @@ cudaError_t launch_row_scores(const float *x, RowMap xmap, int E, int M, int C, 
 cudaError_t launch_select_topr(const float *scores, int B, int M, int r, int *idx, int *inv, cudaStream_t st);
 cudaError_t launch_copy_indices(const int *forced, int B, int M, int r, int ld_forced, int *idx, int *inv,
                                 unsigned *status, cudaStream_t st);
+// K ranges of the GEMM before a LayerNorm that the latter adds up first: x += gate * (sum of the parts + bias), in place.
+struct LnParts {
+  const float *part;               // [splits][E * rows][C]
+  int splits;                      // up to kMaxParts
+  long long stride;                // floats between two parts
+  const bf16 *bias;                // [C]
+  const float *gate;               // [caller element][vec_stride]
+};
+constexpr int kMaxParts = 4;
+cudaError_t launch_ln_parts(float *x, RowMap xmap, int E, int rows, int C, const LnParts &parts, const float *shift, const float *scale,
+                            long long vec_stride, int bmul, int boff, float eps, bf16 *y, cudaStream_t st);
 // early: shift, scale and gamma are not written by any kernel that may still be in flight (they may then be read before
 // the preceding kernel has finished).
 cudaError_t launch_ln_modulate(const float *x, RowMap xmap, int E, int rows, int C, const float *shift,

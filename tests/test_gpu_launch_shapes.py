@@ -89,18 +89,20 @@ def test_gemm_free_width_pairs(fv, R, N, K, width):
     assert (out.double() - ref).abs().max() <= bound
 
 
-@pytest.mark.parametrize("shape,B,k,bar", [("d16", 16, 8, 2e-2), ("d16", 2, 7, 2e-2), ("infinity", 1, 7, 3e-2)])
-def test_step_epilogues_of_the_free_width_pairs(fv, shape, B, k, bar):
-    """One dense block at sizes where QKV, out-proj and both FFN GEMMs take that form between them (2704 rows of 1024
-    columns; 200; 400 rows of 2048): every epilogue of it, KV cache included, against the CPU oracle."""
+@pytest.mark.parametrize("shape,B,k,blocks,bar", [("d16", 16, 8, 1, 2e-2), ("d16", 2, 7, 1, 2e-2), ("infinity", 1, 7, 1, 3e-2),
+                                                  ("infinity", 1, 7, 2, 3e-2), ("d16", 2, 8, 2, 2e-2)])
+def test_step_epilogues_of_the_free_width_pairs(fv, shape, B, k, blocks, bar):
+    """A dense block at sizes where QKV, out-proj and both FFN GEMMs take that form between them (2704 rows of 1024
+    columns; 200; 400 rows of 2048): every epilogue of it, KV cache included, against the CPU oracle.
+    With two blocks a group (400 and 338 rows), the first one's last GEMM in K ranges that the second's LayerNorm adds up."""
     import numpy as np
     from oracle import fvar_oracle as orc
     from helpers import assert_close
-    shp = si.shape_var_d16(n_blocks=1) if shape == "d16" else si.shape_infinity_2b(n_blocks=1, blocks_per_group=1)
+    shp = si.shape_var_d16(n_blocks=blocks) if shape == "d16" else si.shape_infinity_2b(n_blocks=blocks, blocks_per_group=blocks)
     w = si.make_weights(11, shp)
-    ctx = fv.Fvar(weights_to_cuda(w), blocks_per_group=1, n_heads=shp.n_heads, head_dim=shp.head_dim, ffn_dim=shp.ffn_dim, scale_hw=shp.hw(),
+    ctx = fv.Fvar(weights_to_cuda(w), blocks_per_group=blocks, n_heads=shp.n_heads, head_dim=shp.head_dim, ffn_dim=shp.ffn_dim, scale_hw=shp.hw(),
                   max_batch=B, ctx_len=shp.ctx_len, ctx_width=shp.ctx_width)
-    o = orc.Oracle(w, shp.n_heads, 1, shp.hw(), shp.ln_eps)
+    o = orc.Oracle(w, shp.n_heads, blocks, shp.hw(), shp.ln_eps)
     cond = si.make_cond(12, B, shp.width)
     text = si.make_context(13, B, shp.ctx_len, shp.ctx_width) if shp.has_cross_attn else None
     ctx.set_cond(to_bf16_cuda(cond), to_bf16_cuda(text) if text is not None else None)

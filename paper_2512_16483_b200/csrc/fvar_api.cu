@@ -362,7 +362,7 @@ fvar_status run_gemm_parts(fvar_ctx *ctx, const fvar_ctx::ActMaps &maps, int blk
   g.ld_out = N;
   g.splits = ranges;
   g.fx_nb = rows_tile;
-  g.fx_early = 1;
+  g.w_early = 1;
   g.status = ctx->status;
   g.wait_cycles = ctx->wait_cycles;
   gemm_flex_shape(g);
@@ -389,6 +389,7 @@ fvar_status run_gemm(fvar_ctx *ctx, int epi, const fvar_ctx::ActMaps &maps, int 
     if (S > 0 && g.sk_stages >= 1 && gemm_skinny_map(&tmA, maps.base, maps.rows, maps.cols, maps.cols, g.sk_rp, g.sk_nk) &&
         gemm_skinny_map(&tmW, ctx->w[wid][blk], g.N, g.K, g.K, 128, g.sk_nk)) {
       g.splits = S;
+      g.w_early = 1;                               // the caller's weights: what wrote them precedes silu or tokens_to_f32, which wait
       g.status = ctx->status;
       g.wait_cycles = ctx->wait_cycles;
       ctx->prof_begin(FVAR_KCLASS_GEMM, 2.0 * g.R * g.N * g.K,
@@ -410,6 +411,7 @@ fvar_status run_gemm(fvar_ctx *ctx, int epi, const fvar_ctx::ActMaps &maps, int 
     CUtensorMap tmA, tmW;
     if (S > 0 && g.sk_stages >= 1 && gemm_skinny_map(&tmA, maps.base, maps.rows, maps.cols, maps.cols, 128, g.sk_nk) &&
         gemm_skinny_map(&tmW, ctx->w[wid][blk], g.N, g.K, g.K, 128, g.sk_nk)) {
+      g.w_early = 1;
       g.status = ctx->status;
       g.wait_cycles = ctx->wait_cycles;
       ctx->prof_begin(FVAR_KCLASS_GEMM, 2.0 * g.R * g.N * g.K,
@@ -434,7 +436,7 @@ fvar_status run_gemm(fvar_ctx *ctx, int epi, const fvar_ctx::ActMaps &maps, int 
                       (epi == EPI_F32 || epi == EPI_RESID ? 4.0 : 2.0) * g.R * g.N * g.nbatch);
   if (plan.form == kGemmFlex) {
     g.fx_nb = plan.block_n;
-    g.fx_early = 1;                                // the caller's weights: no kernel of the library writes them
+    g.w_early = 1;
     gemm_flex_shape(g);
     CUtensorMap tmA, tmW;
     if (!gemm_skinny_map(&tmA, maps.base, maps.rows, maps.cols, maps.cols, g.fx_nb / 2, g.fx_nk) || !gemm_skinny_map(&tmW, ctx->w[wid][blk], g.N, g.K, g.K, 128, g.fx_nk))
@@ -920,6 +922,7 @@ static fvar_status transition_impl(fvar_ctx *ctx, const void *fo, int scale_idx,
   GemmArgs g = gemm_args(R, V, C);
   g.col_sub = ctx->tr_hn;
   g.best = ctx->tr_best[buf];
+  g.w_early = 1;                                 // the codebook: what wrote it precedes half_norms, which starts after its end
   g.status = ctx->status;
   g.wait_cycles = ctx->wait_cycles;
   CUtensorMap ta, tw;

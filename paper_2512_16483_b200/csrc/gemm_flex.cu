@@ -84,7 +84,7 @@ gemm_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_holder;
   const uint32_t full0 = mapa_shared(full_bar(0), 0);
-  const int pre = p.fx_early ? min(nstages, nst) : 0;
+  const int pre = p.w_early ? min(nstages, nst) : 0;
   if (threadIdx.x == 0) {
     // While the predecessor drains: the weights of the first stages, which wait for nothing but the barriers just
     // initialised.  A loop of its own -- a test per stage inside the producer's made it miss its pace (400 x 6144 x 2048

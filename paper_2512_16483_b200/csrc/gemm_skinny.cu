@@ -15,7 +15,7 @@
 // set the throughput of a single SM's copy unit).
 //
 // Roles: warp 0 feeds the stage ring with TMA (the weight halves of the first stages are requested before
-// griddepcontrol.wait: weights never depend on the preceding kernel), warp 1 issues the MMAs into TMEM,
+// griddepcontrol.wait, so the launch overlaps its predecessor only where that does not write them: w_early), warp 1 issues the MMAs into TMEM,
 // warps 2-9 dump, reduce and store.  After its last load the producer asks L2 to prefetch this CTA's share
 // of the weights the next GEMM of the chain will stream.  Every mbarrier wait is bounded; a CTA that gives
 // up flags the status word and still joins every cluster barrier, so its peers never wait for it.
@@ -107,7 +107,7 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     mbar_init(tfull_bar, 1);
     mbar_fence_init();
     // The weights of the first stages are requested at once, by the thread that will go on producing: they depend
-    // on no other kernel, and on nothing of this CTA but the barriers just initialised.
+    // on no kernel in flight (w_early), and on nothing of this CTA but the barriers just initialised.
     for (int i = 0; i < pre; ++i) {
       mbar_expect_tx(full_bar(i), stage_bytes);
       load_w(i);
@@ -403,7 +403,7 @@ static cudaError_t skinny_launch_one(const CUtensorMap &tmA, const CUtensorMap &
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = a.w_early ? 2 : 1;      // the kernel requests weights before its wait: else it starts when its predecessor has ended
   return cudaLaunchKernelEx(&cfg, gemm_skinny_kernel<EPI, ROWS>, tmA, tmW, a);
 }
 

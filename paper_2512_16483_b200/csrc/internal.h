@@ -74,6 +74,9 @@ struct GemmArgs {
   float *partial;
   int *counters;
   unsigned *status;
+  // The forms with the weights' first stages requested before the wait for the preceding kernel (gemm_skinny.cu,
+  // gemm_flex.cu): no kernel that may still be in flight writes the weights.  0: they are requested after it.
+  int w_early;
   // Weight-streaming form (gemm_skinny.cu; `splits` is then the cluster size): rows per column chunk, the padded
   // MMA width of a chunk, chunks (1 or 2) and pipeline stages -- filled by gemm_skinny_shape
   int sk_rows_chunk, sk_rp, sk_nchunks, sk_stages, sk_small, sk_nk;
@@ -83,7 +86,6 @@ struct GemmArgs {
   int fx_nb, fx_nk, fx_stages;
   // EPI_PARTIAL (that form only): `splits` K ranges of whole stages, each one's sums [R][ld_out] fp32 (no bias) at
   // out_f32 + range * R * ld_out; one tile a pair
-  int fx_early;            // nothing in flight writes the weights: the first stages of them are requested before the wait
   // optional: weights the next GEMM of the chain will stream; every CTA asks L2 to prefetch its share
   const void *pf_ptr;
   unsigned long long pf_bytes;

@@ -116,3 +116,21 @@ def test_step_epilogues_of_the_free_width_pairs(fv, shape, B, k, blocks, bar):
         ctx.kv_append(scale)
         o.kv_append(scale)
     assert ctx.poll_status() == fv.OK
+
+
+@pytest.mark.parametrize("form,R,N,K", [("GEMM_SKINNY", 16, 8192, 2048), ("GEMM_KSPLIT", 100, 2048, 8192), ("GEMM_FLEX", 400, 8192, 2048),
+                                        ("GEMM_SINGLE", 100, 8192, 2048), ("GEMM_PAIR", 400, 8192, 2048)])
+def test_gemm_waits_for_a_weight_that_the_call_before_writes(fv, form, R, N, K):
+    """The second operand comes from the library call just before, which lets its successor start early: every form
+    has to read it after that call has ended."""
+    g = torch.Generator(device="cuda").manual_seed(R + N)
+    A = torch.randn((R, K), generator=g, device="cuda").bfloat16()
+    pair = torch.randn((2, N, K), generator=g, device="cuda").bfloat16()
+    for s in (1.0, 0.0, -1.0, 2.0, 1.0, 0.0):          # the buffer of the weight is reused: it holds an earlier one
+        W = fv.fvar_cfg_combine(pair, s)
+        out = fv.fvar_gemm_bf16_form(A, W[0], None, getattr(fv, form), 0)
+        ref = A.double() @ W[0].double().T
+        bound = 1e-5 * (A.double().abs() @ W[0].double().abs().T).max()       # fp32 sums of at most 8192 products
+        del W
+        assert (out.double() - ref).abs().max() <= bound, s
+    assert fv.kernel_poll_status() == fv.OK

@@ -11,6 +11,9 @@
  * Conventions
  *   - "dev" pointers are device memory of the current CUDA device, "host" pointers are host memory.
  *   - bf16 arrays are raw 16-bit patterns.  All matrices are row-major.
+ *   - Device arrays that hold rows or vectors of features start on a 16-byte boundary, as allocations do; 8 bytes suffice
+ *     for ln_c_gamma, next_tokens and the output of fvar_ln_modulate.  FVAR_EINVAL otherwise (fvar_init answers FVAR_ECUDA
+ *     for a weight matrix).  Scores, keys, index lists, cond and arrays that are only copied need no more than their type.
  *   - Weight matrices are stored [out_features][in_features] (y = x W^T + b).
  *   - The library never allocates or frees device memory and never synchronises unless a function
  *     says so; all work is enqueued on the stream given to fvar_init.  The caller owns weights,

@@ -578,6 +578,7 @@ fvar_status fvar_init(const fvar_weights *weights, const fvar_cfg *cfg, void *wo
     if (!bsrc[i]) return destroy_fail(FVAR_EINVAL, "a bias array is NULL");
     for (int b = 0; b < nb; ++b) {
       if (!bsrc[i][b]) return destroy_fail(FVAR_EINVAL, "a bias pointer is NULL");
+      if (off_grid(bsrc[i][b], i == 5 ? 8 : 16)) return destroy_fail(FVAR_EINVAL, "biases must be 16-byte, ln_c_gamma 8-byte aligned");
       bdst[i]->push_back(static_cast<const bf16 *>(bsrc[i][b]));
     }
   }
@@ -889,7 +890,7 @@ fvar_status fvar_set_codebook(fvar_ctx *ctx, const void *Z, int V) {
   if (!ctx) return FVAR_EINVAL;
   if (!Z || V <= 0) return fail(ctx, FVAR_EINVAL, "set_codebook: NULL codebook or V <= 0");
   if (V > kMaxCodebook) return fail(ctx, FVAR_EUNSUPPORTED, "set_codebook: more than 65536 codewords");
-  if (reinterpret_cast<uintptr_t>(Z) & 15) return fail(ctx, FVAR_EINVAL, "set_codebook: codebook must be 16-byte aligned");
+  if (off_grid(Z, 16)) return fail(ctx, FVAR_EINVAL, "set_codebook: codebook must be 16-byte aligned");
   FV_CUDA(ctx, launch_half_norms(static_cast<const bf16 *>(Z), V, ctx->C, ctx->tr_hn, ctx->st), "half_norms");
   ctx->launched();
   ctx->codebook = static_cast<const bf16 *>(Z);
@@ -906,6 +907,7 @@ static fvar_status transition_impl(fvar_ctx *ctx, const void *fo, int scale_idx,
     return fail(ctx, FVAR_EINVAL, "scale_transition: bad arguments");
   if (scale_idx == nS - 1 && next_tokens != nullptr)
     return fail(ctx, FVAR_EINVAL, "scale_transition: there is no next input after the last scale (next_tokens must be NULL)");
+  if (off_grid(next_tokens, 8)) return fail(ctx, FVAR_EINVAL, "scale_transition: next_tokens must be 8-byte aligned");
   if (scale_idx > 0 && (ctx->tr_scale != scale_idx - 1 || ctx->tr_B != B))
     return fail(ctx, FVAR_ESTATE, "scale_transition: scales must be accumulated in order, 0 first, with one batch size");
   const int C = ctx->C, V = ctx->codebook_V, M = ctx->Mk[scale_idx], R = B * M;
@@ -1038,6 +1040,7 @@ static fvar_status scale_step_impl(fvar_ctx *ctx, const void *tokens, bool token
   if (pol->mode != FVAR_DENSE && pol->mode != FVAR_LOWRANK_RTR) return fail(ctx, FVAR_EINVAL, "scale_step: bad mode");
   if (pol->cfg_mode != FVAR_CFG_PAIR && pol->cfg_mode != FVAR_CFG_NULL_ONLY) return fail(ctx, FVAR_EINVAL, "scale_step: bad cfg_mode");
   if (!tokens || !out) return fail(ctx, FVAR_EINVAL, "scale_step: NULL tokens / out");
+  if (off_grid(tokens, 16) || off_grid(out, 16)) return fail(ctx, FVAR_EINVAL, "scale_step: tokens and out must be 16-byte aligned");
   if (ctx->B <= 0) return fail(ctx, FVAR_ESTATE, "scale_step before set_cond");
   if (scale_idx < 0 || scale_idx >= ctx->cfg.n_scales) return fail(ctx, FVAR_EINVAL, "scale_step: bad scale_idx");
   if (scale_idx < ctx->last_scale) return fail(ctx, FVAR_ESTATE, "scale_step: scale_idx decreased");
@@ -1536,12 +1539,14 @@ static fvar_status kfail(fvar_status s, const char *m) { g_init_error = m; retur
 
 fvar_status fvar_row_scores(const float *x, int B, int M, int C, float *scores, void *stream) {
   if (!x || !scores || B <= 0 || M <= 0 || C <= 0 || C % 4) return kfail(FVAR_EINVAL, "row_scores: bad arguments");
+  if (off_grid(x, 16)) return kfail(FVAR_EINVAL, "row_scores: x must be 16-byte aligned");
   FK_CUDA(launch_row_scores(x, RowMap{1, 0, M}, B, M, C, nullptr, scores, static_cast<cudaStream_t>(stream)), "row_scores");
   return FVAR_OK;
 }
 
 fvar_status fvar_row_keys(const float *x, const float *noise, int B, int M, int C, float *keys, void *stream) {
   if (!x || !noise || !keys || B <= 0 || M <= 0 || C <= 0 || C % 4) return kfail(FVAR_EINVAL, "row_keys: bad arguments");
+  if (off_grid(x, 16)) return kfail(FVAR_EINVAL, "row_keys: x must be 16-byte aligned");
   FK_CUDA(launch_row_scores(x, RowMap{1, 0, M}, B, M, C, noise, keys, static_cast<cudaStream_t>(stream)), "row_keys");
   return FVAR_OK;
 }
@@ -1556,15 +1561,23 @@ fvar_status fvar_ln_modulate(const float *x, int R, int C, int rows_per_batch, c
                              long long vec_stride, float eps, void *y, void *stream) {
   if (!x || !y || !shift || !scale || R <= 0 || C <= 0 || C % 8 || C > 8192 || rows_per_batch <= 0 || R % rows_per_batch)
     return kfail(FVAR_EINVAL, "ln_modulate: bad arguments");
+  if (off_grid(x, 16) || off_grid(shift, 16) || off_grid(scale, 16) || vec_stride % 4 || off_grid(y, 8))
+    return kfail(FVAR_EINVAL, "ln_modulate: x, shift, scale and every vector of theirs must be 16-byte, y 8-byte aligned");
   FK_CUDA(launch_ln_modulate(x, RowMap{1, 0, rows_per_batch}, R / rows_per_batch, rows_per_batch, C, shift, scale,
                              vec_stride, 1, 0, nullptr, eps, false, static_cast<bf16 *>(y), static_cast<cudaStream_t>(stream)),
           "ln_modulate");
   return FVAR_OK;
 }
 
+// Rows of 4 k columns leave as 16-byte stores; 32 whole columns, or 8 k in the cluster-split forms, take their bias so.
+static bool gemm_off_grid(const void *bias, const float *out, int N) {
+  return (N % 4 == 0 && off_grid(out, 16)) || ((N >= 32 || N % 8 == 0) && off_grid(bias, 16));
+}
+
 fvar_status fvar_gemm_bf16_form(const void *A, const void *W, const void *bias, int R, int N, int K, int form,
                                 int block_n, float *out, void *stream) {
   if (!A || !W || !out || R <= 0 || N <= 0 || K <= 0 || K % 8) return kfail(FVAR_EINVAL, "gemm: bad arguments");
+  if (gemm_off_grid(bias, out, N)) return kfail(FVAR_EINVAL, "gemm: bias and out must be 16-byte aligned");
   if (form != FVAR_GEMM_AUTO && form != FVAR_GEMM_SINGLE && form != FVAR_GEMM_PAIR && form != FVAR_GEMM_SKINNY && form != FVAR_GEMM_KSPLIT &&
       form != FVAR_GEMM_FLEX)
     return kfail(FVAR_EINVAL, "gemm: bad form");
@@ -1642,6 +1655,7 @@ fvar_status fvar_gemm_bf16_form(const void *A, const void *W, const void *bias, 
 fvar_status fvar_gemm_bf16_wt(const void *A, const void *Wt, const void *bias, int R, int N, int K, int block_n, float *out,
                               void *stream) {
   if (!A || !Wt || !out || R <= 0 || N <= 0 || K <= 0 || K % 8 || N % 8) return kfail(FVAR_EINVAL, "gemm_wt: bad arguments");
+  if (gemm_off_grid(bias, out, N)) return kfail(FVAR_EINVAL, "gemm_wt: bias and out must be 16-byte aligned");
   int dev = 0, sms = 0;
   FK_CUDA(cudaGetDevice(&dev), "get device");
   FK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device attribute");
@@ -1668,6 +1682,7 @@ fvar_status fvar_attention(const void *q, const void *Kc, const void *Vt, int B,
                            void *out, void *stream) {
   if (!q || !Kc || !Vt || !out || B <= 0 || H <= 0 || r <= 0 || (D != 64 && D != 128) || L <= 0 || L > L_cap || L_cap % 8)
     return kfail(FVAR_EINVAL, "attention: bad arguments");
+  if (off_grid(out, 16)) return kfail(FVAR_EINVAL, "attention: out must be 16-byte aligned");
   CUtensorMap tq, tk, tv;
   const uint64_t BH = static_cast<uint64_t>(B) * H;
   if (!tmap_2d(&tq, q, static_cast<uint64_t>(H) * D, static_cast<uint64_t>(B) * r, static_cast<uint64_t>(H) * D, 128) ||
@@ -1687,8 +1702,7 @@ fvar_status fvar_attention(const void *q, const void *Kc, const void *Vt, int B,
 }
 
 fvar_status fvar_cfg_combine(const void *pair, int B, long long per_elem, float guidance, void *out, void *stream) {
-  if (!pair || !out || B <= 0 || (B & 1) || per_elem <= 0 || per_elem % 8 || (reinterpret_cast<uintptr_t>(pair) & 15) ||
-      (reinterpret_cast<uintptr_t>(out) & 15))
+  if (!pair || !out || B <= 0 || (B & 1) || per_elem <= 0 || per_elem % 8 || off_grid(pair, 16) || off_grid(out, 16))
     return kfail(FVAR_EINVAL, "cfg_combine: bad arguments");
   FK_CUDA(launch_cfg_combine(static_cast<const bf16 *>(pair), B / 2, per_elem, guidance, static_cast<bf16 *>(out),
                              static_cast<cudaStream_t>(stream)), "cfg_combine");
@@ -1707,7 +1721,7 @@ fvar_status fvar_selftest_wait_timeout(fvar_ctx *ctx, long long cycles, void *st
 }
 
 fvar_status fvar_l2_prefetch(const void *ptr, size_t bytes, void *stream) {
-  if (!ptr || (reinterpret_cast<uintptr_t>(ptr) & 15)) return kfail(FVAR_EINVAL, "l2_prefetch: NULL or unaligned pointer");
+  if (!ptr || off_grid(ptr, 16)) return kfail(FVAR_EINVAL, "l2_prefetch: NULL or unaligned pointer");
   FK_CUDA(launch_l2_prefetch(ptr, bytes, static_cast<cudaStream_t>(stream)), "l2_prefetch");
   return FVAR_OK;
 }
@@ -1716,6 +1730,7 @@ fvar_status fvar_rtr_fill(const float *prev, int B, int h0, int w0, int h1, int 
                           void *stream) {
   if (!prev || !out || B <= 0 || h0 <= 0 || w0 <= 0 || h1 <= 0 || w1 <= 0 || C <= 0 || C % 4)
     return kfail(FVAR_EINVAL, "rtr_fill: bad arguments");
+  if (off_grid(prev, 16) || off_grid(out, 16)) return kfail(FVAR_EINVAL, "rtr_fill: prev and out must be 16-byte aligned");
   FK_CUDA(launch_rtr_fill(prev, out, B, 1, 0, h0, w0, h1, w1, C, inv, nullptr, 0, static_cast<cudaStream_t>(stream)), "rtr_fill");
   return FVAR_OK;
 }

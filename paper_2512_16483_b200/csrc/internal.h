@@ -191,6 +191,10 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
+// The kernels read and write a caller's buffers 8 or 16 bytes at a time: an address off that grid is refused at the entry
+// points (a launch would fault).
+inline bool off_grid(const void *p, unsigned bytes) { return (reinterpret_cast<uintptr_t>(p) & (bytes - 1)) != 0; }
+
 // Records the message fvar_last_error(NULL) returns.
 void set_global_error(const char *msg);
 

@@ -50,6 +50,10 @@ extern "C" fvar_status fvar_select_rows_static(const float *x, int B, int M, int
     set_global_error("select_rows_static: bad arguments");
     return FVAR_EINVAL;
   }
+  if (off_grid(x, 16)) {
+    set_global_error("select_rows_static: x must be 16-byte aligned");
+    return FVAR_EINVAL;
+  }
   if (static_cast<long long>(B) * M > kStaticScoreCapacity) {
     set_global_error(("select_rows_static: B * M = " + std::to_string(static_cast<long long>(B) * M) +
                       " exceeds the built-in scratch of " + std::to_string(kStaticScoreCapacity) +

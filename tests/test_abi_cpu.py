@@ -4,6 +4,7 @@ import os
 import re
 
 import numpy as np
+import pytest
 
 import synth_inputs as si
 from paper_2512_16483_b200 import build as fbuild
@@ -47,6 +48,34 @@ def test_workspace_bytes_and_bad_shapes_without_gpu():
     assert st == binding.EINVAL and not ctx.value
     assert b"shape" in lib.fvar_last_error(None)
     assert lib.fvar_kv_append(None, 0) == binding.EINVAL
+
+
+@pytest.mark.parametrize("call,args,vary", [
+    ("fvar_row_scores", (64, 1, 4, 8, 64, None), {0: 16}),
+    ("fvar_row_keys", (64, 64, 1, 4, 8, 64, None), {0: 16}),
+    ("fvar_ln_modulate", (64, 4, 8, 4, 64, 64, 8, 1e-6, 64, None), {0: 16, 4: 16, 5: 16, 8: 8}),
+    ("fvar_gemm_bf16", (64, 64, 64, 4, 64, 8, 64, None), {2: 16, 6: 16}),
+    ("fvar_gemm_bf16_form", (64, 64, 64, 4, 8, 8, 3, 0, 64, None), {2: 16, 8: 16}),
+    ("fvar_gemm_bf16_wt", (64, 64, 64, 4, 64, 8, 0, 64, None), {2: 16, 7: 16}),
+    ("fvar_attention", (64, 64, 64, 1, 1, 4, 64, 4, 8, 64, None), {9: 16}),
+    ("fvar_cfg_combine", (64, 2, 8, 1.0, 64, None), {0: 16, 4: 16}),
+    ("fvar_rtr_fill", (64, 1, 2, 2, 4, 4, 8, 64, 64, None), {0: 16, 8: 16}),
+    ("fvar_select_rows_static", (64, 1, 4, 8, 2, 64, 64, None), {0: 16}),
+])
+def test_kernel_calls_refuse_addresses_off_their_vector_grid(call, args, vary):
+    """The kernels move 8 or 16 bytes at a time; a buffer off that grid has to come back as FVAR_EINVAL, before anything
+    is launched.  (The addresses here are numbers, not memory: only refused calls are made.)"""
+    from paper_2512_16483_b200 import binding
+    fn = getattr(binding.load_library(), call)
+    for pos, grid in vary.items():
+        for off in (2, 4, 8):
+            if off % grid:
+                bad = list(args)
+                bad[pos] += off
+                assert fn(*bad) == binding.EINVAL, (call, pos, off)
+                assert b"aligned" in binding.load_library().fvar_last_error(None) or call == "fvar_cfg_combine"
+    if call == "fvar_ln_modulate":                       # rows of shift and scale off the grid
+        assert fn(*args[:6], 6, *args[7:]) == binding.EINVAL
 
 
 def test_schedule_matches_printed_table():

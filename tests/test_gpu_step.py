@@ -278,6 +278,37 @@ def test_state_and_argument_errors(fv):
     assert p2.gpu.poll_status() == fv.OK                                       # cleared by the read
 
 
+def test_buffers_off_the_vector_grid_are_refused(fv):
+    """A contiguous view that starts one element into an allocation: an error, not a launch that faults."""
+    shp = si.shape_tiny(n_blocks=1, width=128, n_heads=2, head_dim=64, ffn_dim=256, scales=(2, 3), cross=True)
+    p = Pair(fv, shp, seed=107, B=2)
+    g, M, C = p.gpu, 4, 128
+
+    def shifted(*shape):
+        n = int(np.prod(shape))
+        return torch.zeros(n + 1, dtype=torch.bfloat16, device="cuda")[1:].view(shape)
+
+    good = to_bf16_cuda(si.make_tokens(107, 2, M, C))
+    for call in (lambda: g.scale_step(shifted(2, M, C), 0), lambda: g.scale_step(good, 0, out=shifted(2, M, C))):
+        with pytest.raises(fv.FvarError) as e:
+            call()
+        assert e.value.status == fv.EINVAL
+    got, ref = _step_both(p, si.make_tokens(107, 2, M, C), 0, mode=fv.DENSE)          # the context is as it was
+    assert_out_close(got, ref, what="step after refused ones")
+    g.set_codebook(to_bf16_cuda(si.make_codebook(107, 16, C)))
+    codes = torch.empty((2, M), dtype=torch.int32, device="cuda")
+    for fo, nxt in ((shifted(2, M, C), good), (good, shifted(2, 9, C))):
+        assert g.lib.fvar_scale_transition(g.ctx, fo.data_ptr(), 0, 2, codes.data_ptr(), nxt.data_ptr()) == fv.EINVAL
+    for name in ("b_qkv", "b_fc2", "ln_c_gamma"):
+        w = weights_to_cuda(si.make_weights(107, shp))
+        w[0][name] = shifted(w[0][name].numel())
+        with pytest.raises(fv.FvarError) as e:
+            fv.Fvar(w, blocks_per_group=1, n_heads=2, head_dim=64, ffn_dim=256, scale_hw=shp.hw(), max_batch=2, ctx_len=shp.ctx_len,
+                    ctx_width=shp.ctx_width)
+        assert e.value.status == fv.EINVAL
+    assert g.poll_status() == fv.OK
+
+
 def test_graph_replay_matches_direct_launch(fv):
     """The step body is captured into a CUDA graph on first use and replayed afterwards; capture,
     replay and direct launches must give the same bits, and the cache bookkeeping must not differ."""

@@ -1445,13 +1445,14 @@ fvar_status fvar_scale_step_host(fvar_ctx *ctx, const void *tokens_host, int sca
   if (pol->mode == FVAR_SKIP) return FVAR_OK;
   if (!tokens_host || !out_host) return fail(ctx, FVAR_EINVAL, "scale_step_host: NULL tokens / out");
   if (scale_idx < 0 || scale_idx >= ctx->cfg.n_scales || ctx->B <= 0) return fail(ctx, FVAR_EINVAL, "scale_step_host: bad scale_idx or no cond");
-  // Staging: the bf16 tokens land in the hidden-activation buffer (free until the first fc1) and
-  // the bf16 output in the attention-output buffer (free after the last out-proj).
+  // Staging: the bf16 tokens land in the query buffer (free until the first QKV GEMM, which the
+  // input conversion precedes) and the bf16 output in the attention-output buffer (free after the last out-proj); both
+  // hold max_batch x tokens x width whatever the FFN width is.
   const size_t M = ctx->Mk[scale_idx];
   const bool null_only = pol->cfg_mode == FVAR_CFG_NULL_ONLY && ctx->B % 2 == 0;
   const int E = null_only ? ctx->B / 2 : ctx->B;
-  FV_CUDA(ctx, upload_tokens(ctx, ctx->hbuf, tokens_host, M * ctx->C * 2, null_only, ctx->st), "tokens H2D");
-  fvar_status s = scale_step_impl(ctx, ctx->hbuf, null_only, scale_idx, pol, ctx->a);
+  FV_CUDA(ctx, upload_tokens(ctx, ctx->q, tokens_host, M * ctx->C * 2, null_only, ctx->st), "tokens H2D");
+  fvar_status s = scale_step_impl(ctx, ctx->q, null_only, scale_idx, pol, ctx->a);
   if (s != FVAR_OK) return s;
   FV_CUDA(ctx, cudaMemcpyAsync(out_host, ctx->a, static_cast<size_t>(E) * M * ctx->C * 2, cudaMemcpyDeviceToHost, ctx->st), "out D2H");
   FV_CUDA(ctx, cudaStreamSynchronize(ctx->st), "stream synchronize");

@@ -234,6 +234,24 @@ def test_host_entry_point_matches_device_entry_point(fv):
     assert torch.equal(outs[0], outs[1])
 
 
+def test_host_entry_point_with_an_ffn_narrower_than_the_rows(fv):
+    """ffn_dim < width, both branches of a late step: the uploaded tokens need more room than the hidden activations do."""
+    shp = si.shape_tiny(n_blocks=2, width=256, n_heads=4, head_dim=64, ffn_dim=64, scales=(8, 16))
+    toks = si.make_tokens(108, 4, 256, 256)
+    outs = []
+    for host in (False, True):
+        p = Pair(fv, shp, seed=108, B=4)
+        p.prefill(1)
+        p.set_projections(1, [128, 128])
+        if host:
+            oh = torch.empty((4, 256, 256), dtype=torch.bfloat16).pin_memory()
+            outs.append(p.gpu.scale_step_host(to_bf16_cuda(toks).cpu().pin_memory(), 1, oh, mode=fv.LOWRANK_RTR, keep_ratio=0.5).clone())
+        else:
+            outs.append(p.gpu.scale_step(to_bf16_cuda(toks), 1, mode=fv.LOWRANK_RTR, keep_ratio=0.5).cpu())
+        p.check_ok()
+    assert torch.equal(outs[0], outs[1])
+
+
 def test_state_and_argument_errors(fv):
     shp = si.shape_tiny(n_blocks=2, width=128, n_heads=2, head_dim=64, ffn_dim=256, scales=(2, 3, 4))
     p = Pair(fv, shp, seed=106, B=2)

@@ -251,7 +251,8 @@ fvar_status fvar_restore_loaded(fvar_ctx *ctx);
  * thread-block cluster that reduces through distributed shared memory; it is bound by reading the weights
  * once.  0 never uses it.
  * FVAR_OPT_WAIT_KCYCLES (default 0 = about half a second): budget, in thousands of clock cycles, of every
- * bounded wait inside the step's kernels; a wait that runs out sets FVAR_ETIMEOUT (fvar_poll_status). */
+ * bounded wait inside the step's kernels; a wait that runs out sets FVAR_ETIMEOUT (fvar_poll_status).  Values of 1 to
+ * 9999 count as 10000 (about 5 ms): a shorter budget could end a kernel while its copies are still on the way. */
 enum { FVAR_OPT_CUDA_GRAPHS = 0, FVAR_OPT_GEMM_MAX_SPLITS = 1, FVAR_OPT_SKINNY_MAX_ROWS = 2, FVAR_OPT_WAIT_KCYCLES = 3 };
 fvar_status fvar_set_option(fvar_ctx *ctx, int option, int value);
 

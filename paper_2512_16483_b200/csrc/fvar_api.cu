@@ -698,7 +698,9 @@ fvar_status fvar_set_option(fvar_ctx *ctx, int option, int value) {
     if (value < 0) return fail(ctx, FVAR_EINVAL, "set_option: the wait budget must not be negative");
     FV_CUDA(ctx, cudaStreamSynchronize(ctx->st), "stream synchronize");
     ctx->drop_graphs();
-    ctx->wait_cycles = static_cast<long long>(value) * 1000;
+    // Never below kMinWaitCycles: a CTA whose consumers give up after its producer has issued its last copy leaves without
+    // draining, which is sound only if a budget is far longer than a copy takes.
+    ctx->wait_cycles = value == 0 ? 0 : std::max(static_cast<long long>(value) * 1000, kMinWaitCycles);
     return FVAR_OK;
   }
   if (option == FVAR_OPT_SKINNY_MAX_ROWS) {

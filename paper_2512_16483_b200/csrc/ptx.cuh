@@ -15,6 +15,7 @@ enum : unsigned { kStatusTimeout = 1u, kStatusBadIndex = 2u };
 // Default budget of a bounded wait in clock cycles (about half a second at boost clock); kernels take the
 // budget as an argument (0 = this default), so that a test can make a wait run out in a millisecond.
 constexpr long long kWaitCycles = 1000000000ll;
+constexpr long long kMinWaitCycles = 10000000ll;      // least budget of a kernel with copies in flight: 5 ms, a copy takes microseconds
 __host__ __device__ constexpr long long wait_budget(long long cycles) { return cycles > 0 ? cycles : kWaitCycles; }
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {

@@ -35,6 +35,22 @@ def test_wait_runs_out_on_a_context_and_the_context_survives(fv):
         p.oracle.kv_append(k)
 
 
+def test_the_smallest_budget_never_ends_a_healthy_step(fv):
+    """A budget below what an operand copy takes would end kernels with copies in flight; the library raises it."""
+    shp = si.shape_tiny(n_blocks=2, blocks_per_group=1, width=128, n_heads=2, head_dim=64, ffn_dim=256, scales=(1, 2, 3, 16))
+    p = Pair(fv, shp, seed=72, B=2, std=0.05)
+    p.gpu.set_option(fv.OPT_WAIT_KCYCLES, 1)
+    for k in range(4):
+        toks = si.make_tokens(72, 2, shp.tokens_per_scale()[k], 128)
+        got, ref = _step_both(p, toks, k, mode=fv.DENSE)
+        assert_out_close(got, ref, what="dense step %d" % k)
+        assert p.gpu.poll_status() == fv.OK
+        p.gpu.kv_append(k)
+        p.oracle.kv_append(k)
+    with pytest.raises(fv.FvarError):
+        p.gpu.set_option(fv.OPT_WAIT_KCYCLES, -1)
+
+
 def test_wait_runs_out_at_kernel_level_then_a_gemm_passes(fv):
     lib = fv.load_library()
     assert fv.kernel_poll_status() == fv.OK

@@ -487,11 +487,13 @@ fvar_status fvar_init(const fvar_weights *weights, const fvar_cfg *cfg, void *wo
   const Layout L = make_layout(cfg);
   if (bytes < L.total) return fail(nullptr, FVAR_ENOMEM, "workspace too small");
 
-  int dev = 0;
-  cudaDeviceProp prop;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess)
+  // Two attributes, not cudaGetDeviceProperties: that asks the driver for everything (2.5 ms of a 3 ms fvar_init, up to
+  // 80 ms when the host is busy).
+  int dev = 0, major = 0, num_sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return fail(nullptr, FVAR_ECUDA, "no CUDA device");
-  if (prop.major != 10) return fail(nullptr, FVAR_ECUDA, "libfvar needs an sm_100 device (B200)");
+  if (major != 10) return fail(nullptr, FVAR_ECUDA, "libfvar needs an sm_100 device (B200)");
   if (!tmap_init_driver()) return fail(nullptr, FVAR_ECUDA, "cuTensorMapEncodeTiled is not available");
 
   fvar_ctx *c = new fvar_ctx();
@@ -510,7 +512,7 @@ fvar_status fvar_init(const fvar_weights *weights, const fvar_cfg *cfg, void *wo
   }
   c->L_cap = static_cast<int>(align_up(Ltot, 128));
   c->ctx_cap = cfg->has_cross_attn ? static_cast<int>(align_up(cfg->ctx_len, 128)) : 0;
-  c->num_sms = prop.multiProcessorCount;
+  c->num_sms = num_sms;
   c->st = static_cast<cudaStream_t>(cuda_stream);
   c->launch_st = c->st;
   c->cap_st = nullptr;

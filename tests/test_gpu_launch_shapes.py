@@ -90,15 +90,17 @@ def test_gemm_free_width_pairs(fv, R, N, K, width):
 
 
 @pytest.mark.parametrize("shape,B,k,blocks,bar", [("d16", 16, 8, 1, 2e-2), ("d16", 2, 7, 1, 2e-2), ("infinity", 1, 7, 1, 3e-2),
-                                                  ("infinity", 1, 7, 2, 3e-2), ("d16", 2, 8, 2, 2e-2)])
+                                                  ("infinity", 1, 7, 2, 3e-2), ("d16", 2, 8, 2, 2e-2), ("narrow", 1, 3, 3, 2e-2)])
 def test_step_epilogues_of_the_free_width_pairs(fv, shape, B, k, blocks, bar):
-    """A dense block at sizes where QKV, out-proj and both FFN GEMMs take that form between them (2704 rows of 1024
-    columns; 200; 400 rows of 2048): every epilogue of it, KV cache included, against the CPU oracle.
-    With two blocks a group (400 and 338 rows), the first one's last GEMM in K ranges that the second's LayerNorm adds up."""
+    """Dense blocks at sizes where that form is taken for out-proj and fc2 (2704 rows of 1024 columns) and for QKV and fc1
+    (400 rows of 2048), every epilogue of it and the KV cache against the CPU oracle; at 200 rows of 1024 columns no GEMM
+    takes it.  With several blocks a group (400, 338 and 324 rows), fc2 of all but the last in K ranges that the next
+    block's LayerNorm adds up: four of them, or three where K / 64 = 66 is a multiple of 6 and not of 8."""
     import numpy as np
     from oracle import fvar_oracle as orc
     from helpers import assert_close
-    shp = si.shape_var_d16(n_blocks=blocks) if shape == "d16" else si.shape_infinity_2b(n_blocks=blocks, blocks_per_group=blocks)
+    shp = (si.shape_var_d16(n_blocks=blocks) if shape == "d16" else si.shape_infinity_2b(n_blocks=blocks, blocks_per_group=blocks) if shape == "infinity"
+           else si.shape_tiny(n_blocks=blocks, blocks_per_group=blocks, width=512, n_heads=8, head_dim=64, ffn_dim=4224, scales=(1, 2, 3, 18, 19)))
     w = si.make_weights(11, shp)
     ctx = fv.Fvar(weights_to_cuda(w), blocks_per_group=blocks, n_heads=shp.n_heads, head_dim=shp.head_dim, ffn_dim=shp.ffn_dim, scale_hw=shp.hw(),
                   max_batch=B, ctx_len=shp.ctx_len, ctx_width=shp.ctx_width)

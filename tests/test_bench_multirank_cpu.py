@@ -1,6 +1,8 @@
 """The multi-GPU leg of bench.py is "replicas only": ranks share nothing but a barrier and the maximum of
 their times.  This runs that aggregation on two gloo ranks on the CPU."""
+import json
 import os
+import subprocess
 import sys
 
 import torch
@@ -37,3 +39,11 @@ def test_single_rank_needs_no_process_group():
     import bench
     assert bench.max_over_ranks(7.5, None, "cpu") == 7.5
     assert bench.whole_job_value(100, 10, 1, 2000.0) == 500.0
+
+
+def test_reference_arm_says_that_there_is_no_reference_implementation():
+    p = subprocess.run([sys.executable, os.path.join(ROOT, "bench.py"), "--impl", "reference", "--gpus", "1", "--steps", "2", "--warmup", "1"],
+                       capture_output=True, text=True, timeout=300)
+    assert p.returncode == 0, p.stderr
+    line = json.loads(p.stdout)
+    assert line["impl"] == "reference" and line["unavailable"] and "value" not in line

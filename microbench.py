@@ -1,10 +1,11 @@
 """Stand-alone timings of the library's kernels through the C ABI (CUDA events, one GPU).
 
-    python microbench.py gemm [single|pair <64|128|256>]   # the library's choice, or a given launch form and tile width
+    python microbench.py gemm [single|pair <64|128|256> | flex <rows>]   # the library's choice, or a given launch form and tile width
     python microbench.py skinny      # the weight-streaming form on the Infinity-2B-shaped late GEMMs
     python microbench.py skinny_one R N K [S]  # eight launches of that form on one shape (for ncu)
+    python microbench.py flex_one R N K [rows]   # eight launches of the pairs with a free row width on one shape (for ncu)
     python microbench.py attention_one B H D r L   # four attention launches on one shape (for ncu)
-    python microbench.py gemmk [single|pair <width>]       # the same over K at fixed R x N: fixed cost and cost per K step
+    python microbench.py gemmk [single|pair|flex <width>]       # the same over K at fixed R x N: fixed cost and cost per K step
     python microbench.py attention
     python microbench.py memory      # score, LayerNorm + modulate, restoration fill, selection
     python microbench.py transition  # between two scale steps: codeword search, Up-accumulate, Down
@@ -35,9 +36,10 @@ def _time(fn, n=20, warm=3):
 
 
 def _form_args():
-    """Optional launch form after the sub-command: `single|pair <tile width>`; default: the library's cost model."""
-    if len(sys.argv) > 3 and sys.argv[2] in ("single", "pair"):
-        return (fv.GEMM_SINGLE if sys.argv[2] == "single" else fv.GEMM_PAIR), int(sys.argv[3]), "%s %s" % (sys.argv[2], sys.argv[3])
+    """Optional launch form after the sub-command: `single|pair|flex <tile width>`; default: the library's cost model."""
+    forms = {"single": fv.GEMM_SINGLE, "pair": fv.GEMM_PAIR, "flex": fv.GEMM_FLEX}
+    if len(sys.argv) > 3 and sys.argv[2] in forms:
+        return forms[sys.argv[2]], int(sys.argv[3]), "%s %s" % (sys.argv[2], sys.argv[3])
     return fv.GEMM_AUTO, 0, "picked"
 
 
@@ -86,8 +88,8 @@ def skinny():
                 R, N, K, auto, sk, N * K * 2 / sk / 1e3, 2 * R * N * K / sk / 1e6), flush=True)
 
 
-def skinny_one():
-    """A few launches of the weight-streaming form over rotating weight copies (for a profiler): R N K [ranges]."""
+def _form_one(form, what):
+    """A few launches of one form over rotating weight copies (for a profiler): R N K [ranges or rows a tile]."""
     lib = fv.load_library()
     R, N, K = (int(x) for x in sys.argv[2:5])
     S = int(sys.argv[5]) if len(sys.argv) > 5 else 0
@@ -95,10 +97,18 @@ def skinny_one():
     Ws = [torch.randn(N, K, device="cuda").bfloat16() * 0.02 for _ in range(8)]
     out = torch.empty(R, N, device="cuda", dtype=torch.float32)
     for W in Ws:
-        assert lib.fvar_gemm_bf16_form(A.data_ptr(), W.data_ptr(), None, R, N, K, fv.GEMM_SKINNY, S, out.data_ptr(),
+        assert lib.fvar_gemm_bf16_form(A.data_ptr(), W.data_ptr(), None, R, N, K, form, S, out.data_ptr(),
                                        torch.cuda.current_stream().cuda_stream) == 0
     torch.cuda.synchronize()
-    print("launched 8 weight-streaming GEMMs R=%d N=%d K=%d" % (R, N, K))
+    print("launched 8 %s GEMMs R=%d N=%d K=%d" % (what, R, N, K))
+
+
+def skinny_one():
+    _form_one(fv.GEMM_SKINNY, "weight-streaming")
+
+
+def flex_one():
+    _form_one(fv.GEMM_FLEX, "free-width pair")
 
 
 def attention_one():
@@ -200,8 +210,9 @@ def transition():
         chain()
     gemm_t = ctx.profile_dump(fv.KCLASSES.index("gemm"))          # per pass: search of scale 0, of scale 1
     up_t = ctx.profile_dump(fv.KCLASSES.index("rtr_fill"))        # per pass: Up of scale 0 (write), of scale 1 (accumulate)
-    cv_t = ctx.profile_dump(fv.KCLASSES.index("convert"))         # per pass: unpack, Down 64->48, unpack, Down 64->64
-    t_g, t_u, t_d = 1e3 * min(gemm_t[1::2]), 1e3 * min(up_t[1::2]), 1e3 * min(cv_t[1::4])
+    cv_t = ctx.profile_dump(fv.KCLASSES.index("convert"))         # per pass: Down 64->48, Down 64->64
+    t_g, t_u, t_d = 1e3 * min(gemm_t[1::2]), 1e3 * min(up_t[1::2]), 1e3 * min(cv_t[0::2])
+    assert len(gemm_t) == len(up_t) == len(cv_t) == 10
     print("codeword search  R=%d V=%d K=%d: %.1f us  %.0f TFLOP/s" % (B * Ms[1], V, C, t_g, 2.0 * B * Ms[1] * V * C / t_g / 1e6))
     print("up_accumulate    B=%d 48x48 -> 64x64 C=%d: %.1f us  %.0f GB/s (fp32 map read and written once)" % (
         B, C, t_u, 8.0 * B * Ms[2] * C / t_u / 1e3))
@@ -213,4 +224,4 @@ def transition():
 if __name__ == "__main__":
     which = sys.argv[1] if len(sys.argv) > 1 else "gemm"
     {"gemm": gemm, "gemmk": gemmk, "attention": attention, "memory": memory, "transition": transition, "skinny": skinny,
-     "ksplit": ksplit, "skinny_one": skinny_one, "attention_one": attention_one}[which]()
+     "ksplit": ksplit, "skinny_one": skinny_one, "flex_one": flex_one, "attention_one": attention_one}[which]()

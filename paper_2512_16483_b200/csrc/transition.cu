@@ -114,11 +114,11 @@ cudaError_t launch_up_accumulate(const bf16 *Z, const unsigned long long *best, 
 
 // tokens[b][q][:] = mean of F over the source cells target cell q = (y, x) of the (h1, w1) grid covers:
 // rows [floor(y h0 / h1), ceil((y + 1) h0 / h1)), columns likewise ("area" resampling); bf16 out.  C % 4 == 0.
-// A thread owns four channels of one target cell; G groups of threads share the window's cells (group g takes cells g,
-// g + G, ...) and their partial sums are added in group order through shared memory.  Bound by latency while the target
-// has few cells -- the map is in L2 then -- so G grows until about two thousand threads an SM are at work.  One warp a
-// cell with all channels, the form before, took 95 us for a 2 x 2 target of a 64 x 64 map with C = 2048 and 15 - 17 us
-// from 16 x 16 to 40 x 40; now 9 - 10.
+// Two forms, chosen in launch_down_area.
+//
+// Few target cells, long windows: a thread owns four channels of one target cell; G groups of threads share the window's
+// cells (group g takes cells g, g + G, ...) and their partial sums are added in group order through shared memory.  Bound
+// by latency -- the map is in L2 then -- so G grows until about two thousand threads an SM are at work.
 template <int G>
 __global__ void __launch_bounds__(256) down_area_kernel(const float *__restrict__ F, int h0, int w0, int h1, int w1, int C, int slabs,
                                                         bf16 *__restrict__ tokens, int dup) {
@@ -164,6 +164,49 @@ __global__ void __launch_bounds__(256) down_area_kernel(const float *__restrict_
   }
 }
 
+// Many target cells, short windows: a warp a cell with all channels, four groups of four channels a lane at a time, so
+// that a block is eight whole cells and not a slice of one, whose start and end then cost more than its reads of 4 KB:
+// eight elements of a 64 x 64 map to 64 x 64 tokens for both branches, 537 MB, 161 us in the other form, 88 in this one.
+__global__ void __launch_bounds__(256) down_area_cells_kernel(const float *__restrict__ F, int B, int h0, int w0, int h1, int w1, int C,
+                                                              bf16 *__restrict__ tokens, int dup) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const int M1 = h1 * w1, lane = threadIdx.x & 31;
+  const long long cell = static_cast<long long>(blockIdx.x) * 8 + (threadIdx.x >> 5);
+  if (cell >= static_cast<long long>(B) * M1) return;
+  const int b = static_cast<int>(cell / M1), q = static_cast<int>(cell - static_cast<long long>(b) * M1);
+  const int y = q / w1, x = q - y * w1;
+  const int ya = (y * h0) / h1, yb = ((y + 1) * h0 + h1 - 1) / h1;
+  const int xa = (x * w0) / w1, xb = ((x + 1) * w0 + w1 - 1) / w1;
+  const float inv = 1.0f / static_cast<float>((yb - ya) * (xb - xa));
+  const int n4 = C / 4;
+  const float4 *src = reinterpret_cast<const float4 *>(F + static_cast<long long>(b) * h0 * w0 * C);
+  uint2 *dst = reinterpret_cast<uint2 *>(tokens + (static_cast<long long>(dup ? 2 * b : b) * M1 + q) * C);
+  for (int g0 = lane; g0 < n4; g0 += 128) {
+    float4 acc[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int yy = ya; yy < yb; ++yy)
+      for (int xx = xa; xx < xb; ++xx) {
+        const float4 *cellp = src + (static_cast<long long>(yy) * w0 + xx) * n4;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (g0 + 32 * u < n4) {
+            const float4 v = __ldg(cellp + g0 + 32 * u);
+            acc[u].x += v.x; acc[u].y += v.y; acc[u].z += v.z; acc[u].w += v.w;
+          }
+      }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (g0 + 32 * u < n4) {
+        const __nv_bfloat162 o0 = __floats2bfloat162_rn(acc[u].x * inv, acc[u].y * inv), o1 = __floats2bfloat162_rn(acc[u].z * inv, acc[u].w * inv);
+        const uint2 pk = make_uint2(*reinterpret_cast<const uint32_t *>(&o0), *reinterpret_cast<const uint32_t *>(&o1));
+        dst[g0 + 32 * u] = pk;
+        if (dup) dst[static_cast<long long>(M1) * n4 + g0 + 32 * u] = pk;
+      }
+  }
+}
+
 template <int G>
 static cudaError_t launch_down(const float *F, int B, int h0, int w0, int h1, int w1, int C, bf16 *tokens, bool dup, cudaStream_t st) {
   const int slabs = (C / 4 + 256 / G - 1) / (256 / G);
@@ -171,8 +214,17 @@ static cudaError_t launch_down(const float *F, int B, int h0, int w0, int h1, in
 }
 
 cudaError_t launch_down_area(const float *F, int B, int h0, int w0, int h1, int w1, int C, bf16 *tokens, bool dup, cudaStream_t st) {
-  if (C % 4 != 0 || B > 65535) return cudaErrorInvalidValue;
+  if (C % 4 != 0) return cudaErrorInvalidValue;
   if (B <= 0 || h1 <= 0 || w1 <= 0) return cudaSuccess;
+  // A warp a cell walks a chain of (cells of a window) x (C / 512) rounds of loads, which it hides behind the other warps
+  // only if there are many: it is the faster form from about 40 warps a round on.  64 x 64 map, C = 2048, both forms (us
+  // in the per-kernel timing, a warp a cell first), targets 16 20 24 32 40 48 64: one element 25 25 21 13 15 12 12 against
+  // 13 15 14 13 21 21 25; two 27 25 21 15 19 19 23 against 15 19 21 21 33 37 45; four 48 48 37 29 43 42 48 against 31 39
+  // 41 39 58 66 82; eight 62 64 64 64 72 76 88 against 60 68 70 66 107 123 161; a 2 x 2 target 1047 - 1972 against 21 - 69.
+  const double warps = static_cast<double>(B) * h1 * w1, rounds = static_cast<double>(h0) * w0 / (static_cast<double>(h1) * w1) * C / 512.0;
+  if (warps >= 40.0 * rounds || B > 65535)         // 65535: rows of the other form's grid
+    return launch_pdl(down_area_cells_kernel, dim3(static_cast<unsigned>((static_cast<long long>(B) * h1 * w1 + 7) / 8)), dim3(256), 0, st, F, B, h0, w0, h1, w1, C,
+                      tokens, dup ? 1 : 0);
   const double threads = static_cast<double>(B) * h1 * w1 * (C / 4), cells = static_cast<double>(h0) * w0 / (static_cast<double>(h1) * w1);
   const double want = 300000.0 / threads < cells ? 300000.0 / threads : cells;      // groups for 148 x 2048 threads, at most one a cell
   if (want > 8.0) return launch_down<16>(F, B, h0, w0, h1, w1, C, tokens, dup, st);

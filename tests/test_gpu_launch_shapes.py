@@ -72,6 +72,29 @@ def test_transitions_repeat_on_one_context(fv, V):
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("C,hw,B", [
+    (640, ((3, 5), (7, 11), (16, 18)), 3),        # long windows, then short ones: both forms; 160 groups of four channels
+    (192, ((1, 1), (2, 9), (13, 7), (13, 13)), 2),    # one window for all, a taller and a wider window, equal sizes a side
+    (64, ((1, 2), (20, 33), (40, 40)), 1),        # fewer channels than a warp's round
+])
+def test_down_in_both_forms(fv, C, hw, B):
+    """The next tokens are the window means of the accumulated map, whichever form the number of windows picks."""
+    shp = si.shape_tiny(n_blocks=1, width=C, n_heads=C // 64, head_dim=64, ffn_dim=64, scale_hw=hw)
+    ctx = fv.Fvar(weights_to_cuda(si.make_weights(8, shp)), blocks_per_group=1, n_heads=shp.n_heads, head_dim=64, ffn_dim=64, scale_hw=shp.hw(),
+                  max_batch=B, ctx_len=0, ctx_width=0)
+    Ms, Z = shp.tokens_per_scale(), si.make_codebook(9, 64, C)
+    ctx.set_codebook(to_bf16_cuda(Z))
+    for k in range(len(Ms) - 1):
+        fo = to_bf16_cuda(si.make_step_outputs(10, k, B, Ms[k], Z, 0.1))
+        _, nxt = ctx.scale_transition(fo, k, Ms[k + 1], pairs=True)
+        F = ctx.get_feature(B, Ms[-1], C).double().view(B, *hw[-1], C).permute(0, 3, 1, 2)
+        pool = torch.nn.functional.adaptive_avg_pool2d
+        ref, mag = (pool(x, hw[k + 1]).permute(0, 2, 3, 1).reshape(B, Ms[k + 1], C) for x in (F, F.abs()))
+        for half in (0, 1):                       # both branches; bf16 rounding and an fp32 sum over the window
+            assert ((nxt[half::2].double() - ref).abs() <= 2.0 ** -8 * ref.abs() + 1e-5 * mag).all(), (k, half)
+    assert ctx.poll_status() == fv.OK
+
+
 @pytest.mark.parametrize("R,N,K,width", [
     (33, 64, 64, 32), (400, 192, 2048, 160), (400, 6144, 200, 224),     # half a feature tile, a remainder of one, K not whole blocks
     (255, 1920, 1920, 64), (257, 1920, 128, 256), (1, 256, 4096, 0),    # an odd number of 128-feature halves, one row past a tile

@@ -210,7 +210,10 @@ cudaError_t launch_copy_indices(const int *forced, int B, int M, int r, int ld_f
 // kernel where the caller says that no kernel in flight writes them (`early`: the step's AdaLN vectors and gamma are
 // written by fvar_set_cond only).  Rows x columns, in a chain of such launches, against the form before (warp a row from
 // 4096 rows, vectors after the statistics): 16 x 2048 4.8 -> 1.4 us, 400 x 2048 5.6 -> 2.5, 2704 x 1024 5.1 -> 4.7,
-// 8192 x 2048 30 -> 18 (5.6 TB/s of 6.5).  A warp or two a row, or two rows a CTA, are level at best.
+// 8192 x 2048 30 -> 18 (5.6 TB/s of 6.5).  Timed one by one inside a step, where no launch overlaps the next, little of
+// that is left: 16 x 2048 7.8 before and after, a launch of three dense d16 scales 11.4 -> 10.6, of three dense Infinity
+// scales 22.2 -> 20.9; one that adds K ranges up takes longer (three late Infinity scales 8.1 -> 8.5).  A warp or two a
+// row, or two rows a CTA, are level at best.
 constexpr int kLnThreads = 128;
 constexpr int kLnMaxVec = 16;                   // float4 a thread: 8192 columns
 

@@ -312,7 +312,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 // Cost model of a launch on B200, fitted to measured ones (R = 100 .. 4096, N = 1024 .. 8192, K = 1024 .. 8192): fixed part
 // (set-up, first operands, the last tile's epilogue) + waves of tiles x K blocks x time a K block, in microseconds; the
 // epilogue of every tile but the last hides behind the main loop of the next.  Splitting K trades a reduction through
-// the scratch area for more CTAs streaming the operands.
+// the scratch area for more CTAs streaming the operands.  The constants rank forms, they are no times: a K block of a
+// 256 x 256 pair takes 0.28 us with 16 of 74 pairs at work, 0.33 with 48 and 0.36 a wave in four waves, single CTAs of 64
+// features 0.155 with 128 of 148 at work and 0.16 a wave beyond, all launched on their own at 1965 MHz; under the power
+// cap of a dense step each is longer.
 // Single CTAs, 128 rows x 64 / 128 / 256 features, and pairs, 256 rows x 128 / 256 features:
 static const float kTileTk[3] = {0.161f, 0.226f, 0.37f}, kTileFixed[3] = {3.2f, 4.2f, 6.0f};
 static const float kPairTk[2] = {0.197f, 0.295f}, kPairFixed[2] = {4.4f, 6.9f};
@@ -350,7 +353,8 @@ GemmPlan gemm_plan(int R, int nbatch, int N, int K, int num_sms, int max_cluster
   const int tiles_m = (R + kBlockM - 1) / kBlockM * nbatch;
   gemm_pick_tile(tiles_m, N, K, num_sms, max_splits, scratch_bytes, &plan.block_n, &plan.splits);
   if (nbatch != 1 || max_clusters <= 0) return plan;
-  // Cost of the single-CTA choice.
+  // Cost of the single-CTA choice.  Its width was picked without the slowdown from the third wave on that is priced in
+  // here; with it no plan changes (1024, 1920 and 2048 columns, 33 to 8192 rows, every GEMM of a block).
   const int num_kb = (K + kBlockK - 1) / kBlockK;
   const int i1 = plan.block_n == 64 ? 0 : (plan.block_n == 128 ? 1 : 2);
   const long long tiles1 = static_cast<long long>(tiles_m) * ((N + plan.block_n - 1) / plan.block_n) * plan.splits;

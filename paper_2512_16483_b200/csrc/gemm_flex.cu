@@ -262,8 +262,11 @@ void gemm_flex_shape(GemmArgs &a) {
 // The reduction of a K split over CTAs costs a cluster barrier and a round of remote reads after the last MMA, and the
 // 128 x 128 tiles of that form (gemm_skinny.cu) move twice the operands of 256 x 224.  Where a LayerNorm follows, it
 // can add up the ranges while it reads its rows: 400 x 2048 x 8192 with its gate and residual 25.9 us in the chain, now 17 and 1 in the
-// LayerNorm (Infinity 40 with table 3693 -> 3578 us, three late scales 11014 -> 10650).  Taken where that form is the
-// alternative (gemm_ksplit_wins) and the rows are more than one chunk; at least three ranges, or too few pairs work.
+// LayerNorm (Infinity 40 with table 3693 -> 3578 us, three late scales 11014 -> 10650).  The line is drawn by rows, not by
+// an estimate: taken where that form is the alternative (gemm_ksplit_wins: N <= 2048, K >= 4096, up to 512 rows) and the
+// rows are more than one chunk.  It is the better one at both ends (a step of the 48 x 48 scale with ranges and without,
+// us: 258 rows 3762 and 3966, 320 rows 3845 and 4039, 400 rows 4160 and 4289, 512 rows 4450 and 4520); up to 256 rows
+// ranges gained nothing.  Four ranges, or three where K / 64 is a multiple of 6 and not of 8; with two, too few pairs work.
 int gemm_partial_plan(int R, int N, int K, int max_clusters, int *rows_tile) {
   if (R <= 256 || !gemm_ksplit_wins(R, N, K) || !gemm_flex_supported(EPI_PARTIAL, N, K) || K % kBlockK != 0) return 0;
   const int tiles_f = (N + 2 * kBlockM - 1) / (2 * kBlockM), chunks = (R + 255) / 256, num_kb = K / kBlockK;
@@ -308,8 +311,9 @@ cudaError_t launch_gemm_flex(int epi, const CUtensorMap &tmA, const CUtensorMap 
     case EPI_GELU_BF16: return flex_launch_one<EPI_GELU_BF16, 1>(tmA, tmW, a, max_clusters, st);
     case EPI_PARTIAL: return a.splits > 0 ? flex_launch_one<EPI_PARTIAL, 1>(tmA, tmW, a, max_clusters, st) : cudaErrorInvalidValue;
     case EPI_QKV: return flex_launch_one<EPI_QKV, 1>(tmA, tmW, a, max_clusters, st);
-    // Up to 64 rows a tile each warp has one chunk, and the code for two only makes a cold launch longer (a step of 1 - 100
-    // rows 2391 against 2404 us); beyond, two ahead is better than one (2704 rows, three scales: 5232 against 5272).
+    // Up to 64 rows a tile each warp has one chunk, and the code for two only makes a cold launch longer: a step of 544 rows
+    // of 2048 columns, where out-proj and cross out-proj take 64 rows a tile, 5001 against 5024 us (2364 rows of 1024
+    // columns: level).  Beyond, two ahead is better than one (2704 rows, three scales: 5232 against 5272).
     case EPI_RESID:
       return a.fx_nb <= 64 ? flex_launch_one<EPI_RESID, 1>(tmA, tmW, a, max_clusters, st) : flex_launch_one<EPI_RESID, 2>(tmA, tmW, a, max_clusters, st);
   }

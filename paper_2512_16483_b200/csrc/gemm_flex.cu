@@ -7,9 +7,9 @@
 //
 // What bounds it: the operands' way from L2 (12 - 15 TB/s over the chip) and the tensor pipe, 0.10 + 0.00077 * width us per
 // 64 of K and wave; a launch adds 2 us of set-up and first operands and 0.019 * width us of the last tile's epilogue.
-// Against pairs of 256 rows (us, rows x features x K): 400 x 6144 x 2048 16.4 -> 12.8 with 160 rows a tile, 72 tiles;
-// 283 x 8192 x 2048 16.4 -> 13.1; 680 x 4096 x 1024 11.1 -> 9.3; 2704 x 1024 x 1024 11.6 -> 8.9; 2704 x 1024 x 4096
-// 25.6 -> 19.5; full tiles are level.  Spreading the K range of a tile over a cluster of pairs was built and left out:
+// Against the best of the pairs of 256 rows (us, rows x features x K, launched through the kernel-level entry, which
+// requests no weights early): 400 x 6144 x 2048 16.6 -> 13.9 with 160 rows a tile, 72 tiles; 283 x 8192 x 2048 16.9 -> 13.9;
+// 680 x 4096 x 1024 10.8 -> 10.3; 2704 x 1024 x 1024 10.6 -> 9.5; 2704 x 1024 x 4096 25.6 -> 20.8; full tiles are level.  Spreading the K range of a tile over a cluster of pairs was built and left out:
 // its reduction costs 4 - 6 us, 400 x 2048 x 8192 took 22.5 us against 21.7 of 128 x 128 tiles split the same way.
 //
 // Roles per CTA: warp 0 feeds the stage ring with TMA (cta_group::2: the bytes of both CTAs are counted on the barrier of

@@ -218,12 +218,15 @@ cudaError_t launch_down_area(const float *F, int B, int h0, int w0, int h1, int 
   if (C % 4 != 0) return cudaErrorInvalidValue;
   if (B <= 0 || h1 <= 0 || w1 <= 0) return cudaSuccess;
   // A warp a cell walks a chain of (cells of a window) x (C / 512) rounds of loads, which it hides behind the other warps
-  // only if there are many: it is the faster form from about 40 warps a round on.  64 x 64 map, C = 2048, both forms (us
-  // in the per-kernel timing, a warp a cell first), targets 16 20 24 32 40 48 64: one element 25 25 21 13 15 12 12 against
-  // 13 15 14 13 21 21 25; two 27 25 21 15 19 19 23 against 15 19 21 21 33 37 45; four 48 48 37 29 43 42 48 against 31 39
-  // 41 39 58 66 82; eight 62 64 64 64 72 76 88 against 60 68 70 66 107 123 161; a 2 x 2 target 1047 - 1972 against 21 - 69.
+  // only if there are many: it is taken from 160 warps a round on.  Whole chains of transitions (guidance, search, Up,
+  // Down; 64 x 64 map, C = 2048, us), the line at 160 against the shared form alone: up to 40 x 40 cells, which that line
+  // leaves to the shared form for one element, level (one 523 and 522, two 826 and 829, four 1513 and 1518, eight 2900 and
+  // 2894); up to 64 x 64 one 734 and 748, two 1247 and 1275, four 2424 and 2523, eight 4902 and 5039.  Timed launch by
+  // launch a warp a cell wins from 40 warps a round on (64 x 64 cells of one element 12 against 25 us, of eight 88 against
+  // 161), but a line there costs in the chain: one element 536 and 747, two 843 and 1264.  For 2 x 2 cells it takes 1047 -
+  // 1972 us, the other form 21 - 69.
   const double warps = static_cast<double>(B) * h1 * w1, rounds = static_cast<double>(h0) * w0 / (static_cast<double>(h1) * w1) * C / 512.0;
-  if (warps >= 40.0 * rounds || B > 65535)         // 65535: rows of the other form's grid
+  if (warps >= 160.0 * rounds || B > 65535)        // 65535: rows of the other form's grid
     return launch_pdl(down_area_cells_kernel, dim3(static_cast<unsigned>((static_cast<long long>(B) * h1 * w1 + 7) / 8)), dim3(256), 0, st, F, B, h0, w0, h1, w1, C,
                       tokens, dup ? 1 : 0);
   const double threads = static_cast<double>(B) * h1 * w1 * (C / 4), cells = static_cast<double>(h0) * w0 / (static_cast<double>(h1) * w1);

@@ -73,7 +73,7 @@ def test_transitions_repeat_on_one_context(fv, V):
 
 
 @pytest.mark.parametrize("C,hw,B", [
-    (640, ((3, 5), (7, 11), (16, 18)), 3),        # long windows, then short ones: both forms; 160 groups of four channels
+    (640, ((3, 5), (5, 7), (14, 16), (16, 18)), 3),    # long windows, then short ones: both forms; 160 groups of four channels
     (192, ((1, 1), (2, 9), (13, 7), (13, 13)), 2),    # one window for all, a taller and a wider window, equal sizes a side
     (64, ((1, 2), (20, 33), (40, 40)), 1),        # fewer channels than a warp's round
 ])

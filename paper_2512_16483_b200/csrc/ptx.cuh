@@ -31,12 +31,13 @@ __device__ __forceinline__ bool elect_one() {
 }
 
 // ------------------------------------------------------------------------------------ dependent launch
-// Every kernel of the library is launched with programmatic stream serialization: its CTAs may be
+// The kernels of the step and of the transition are launched with programmatic stream serialization: their CTAs may be
 // scheduled while the previous kernel on the stream is still draining, so that launch latency and
 // the prologue (barrier init, TMEM allocation, descriptor prefetch) overlap the predecessor's tail.
 // pdl_wait() blocks until the predecessor grid has completed and its writes are visible; nothing
-// that reads or overwrites memory another kernel writes may precede it (weights, which no kernel
-// writes, may be requested earlier).  pdl_launch_dependents() lets the successor be scheduled and run
+// that reads or overwrites memory another kernel writes may precede it (weights may be requested
+// earlier where a kernel that waits stands between whatever wrote them and this one).
+// pdl_launch_dependents() lets the successor be scheduled and run
 // up to its own wait.  The tensor-core GEMMs release their successor only after their own wait; the
 // LayerNorm and attention kernels, whose successors do nothing but set up and request weights before
 // waiting, release it at once.  Completion order stays transitive along the stream (every kernel waits

@@ -103,6 +103,12 @@ __device__ __forceinline__ void st_global_32(void *p, const uint32_t *r) {
                "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
 }
 
+// 32 bytes in one load (coherent: not through the read-only path); p 32-byte aligned.
+__device__ __forceinline__ void ld_global_32(const void *p, float (&r)[8]) {
+  asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]) : "l"(p) : "memory");
+}
+
 // ------------------------------------------------------------------------------------ TMA
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap *m) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");

@@ -51,8 +51,10 @@ __device__ __forceinline__ int code_of(unsigned long long word, int V, bool *bad
 // caller, flag the status word for a bad one, and zero the words the next codeword search will use (`clear`: a second
 // buffer, nobody's by now) -- in a chain of 3 us launches the memset, the unpacking kernel and the copy were half of
 // the transition's launches.  Bound by the map (8 C bytes a pixel, from L2 while it fits) and the gathered
-// codewords (as much again).  Timed launch by launch, C = 2048, a 64 x 64 map: one element 19 us, eight 97; before, 17 and
-// 92, and 6 more for unpacking, besides the memset and the copy.
+// codewords (as much again).  The map moves 32 bytes a lane: as two accesses of 16 each of them touched half of every sector
+// it named, and the stores went to L2 as twice the masked halves (eleven transitions of one 64 x 64 map, C = 2048, 8192
+// codewords 522 -> 478 us, 1024 codewords 406 -> 354; thirteen of four maps 2470 -> 2395; one round of loads in flight
+// instead of four 517 and 380).  C % 8 == 0 and a map on a 32-byte grid (it is the workspace's).
 __global__ void __launch_bounds__(256) up_accumulate_kernel(const bf16 *__restrict__ Z, const unsigned long long *__restrict__ best,
                                                             int V, int B, int h0, int w0, int h1, int w1, int C, int overwrite,
                                                             float *__restrict__ F, int *__restrict__ codes,
@@ -79,27 +81,23 @@ __global__ void __launch_bounds__(256) up_accumulate_kernel(const bf16 *__restri
   auto row = [&](int yy, int xx) { return reinterpret_cast<const uint4 *>(Z + static_cast<long long>(code_of(__ldg(wb + yy * w0 + xx), V, &bad)) * C); };
   const uint4 *p00 = row(y0, x0), *p01 = row(y0, x1), *p10 = row(y1, x0), *p11 = row(y1, x1);
   const float w00 = tap.w00, w01 = tap.w01, w10 = tap.w10, w11 = tap.w11;
-  float4 *dst = reinterpret_cast<float4 *>(F + (static_cast<long long>(b) * M1 + i) * C);
-#pragma unroll 2
+  float *dst = F + (static_cast<long long>(b) * M1 + i) * C;
+#pragma unroll 4
   for (int g = threadIdx.x & 31; g < C / 8; g += 32) {
     const uint4 a = __ldg(p00 + g), bq = __ldg(p01 + g), cq = __ldg(p10 + g), d = __ldg(p11 + g);
-    float4 plo = make_float4(0.f, 0.f, 0.f, 0.f), phi = plo;
-    if (!overwrite) {
-      plo = dst[2 * g];
-      phi = dst[2 * g + 1];
-    }
+    float prev[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (!overwrite) ld_global_32(dst + 8 * g, prev);
     const __nv_bfloat162 *ha = reinterpret_cast<const __nv_bfloat162 *>(&a), *hb = reinterpret_cast<const __nv_bfloat162 *>(&bq);
     const __nv_bfloat162 *hc = reinterpret_cast<const __nv_bfloat162 *>(&cq), *hd = reinterpret_cast<const __nv_bfloat162 *>(&d);
-    float o[8];
+    uint32_t o[8];
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       const float2 fa = __bfloat1622float2(ha[t]), fb = __bfloat1622float2(hb[t]);
       const float2 fc = __bfloat1622float2(hc[t]), fd = __bfloat1622float2(hd[t]);
-      o[2 * t] = w00 * fa.x + w01 * fb.x + w10 * fc.x + w11 * fd.x;
-      o[2 * t + 1] = w00 * fa.y + w01 * fb.y + w10 * fc.y + w11 * fd.y;
+      o[2 * t] = __float_as_uint(w00 * fa.x + w01 * fb.x + w10 * fc.x + w11 * fd.x + prev[2 * t]);
+      o[2 * t + 1] = __float_as_uint(w00 * fa.y + w01 * fb.y + w10 * fc.y + w11 * fd.y + prev[2 * t + 1]);
     }
-    dst[2 * g] = make_float4(o[0] + plo.x, o[1] + plo.y, o[2] + plo.z, o[3] + plo.w);
-    dst[2 * g + 1] = make_float4(o[4] + phi.x, o[5] + phi.y, o[6] + phi.z, o[7] + phi.w);
+    st_global_32(dst + 8 * g, o);
   }
 }
 

@@ -223,7 +223,7 @@ template <int T, bool PARTS>
 __global__ void __launch_bounds__(kLnThreads) ln_modulate_kernel(const float *x, RowMap xmap, int rows, int C,
                                                                  const float *__restrict__ shift, const float *__restrict__ scale,
                                                                  long long vec_stride, int bmul, int boff, const bf16 *__restrict__ gamma,
-                                                                 float eps, int early, bf16 *__restrict__ y, LnParts parts) {
+                                                                 float eps, int early, bf16 *__restrict__ y, GemmParts parts) {
   pdl_launch_dependents();      // nothing precedes the wait but loads: the successor may start its own prologue right away
   __shared__ float red[2][kLnThreads / 32];
   constexpr bool kHold = T <= 4;                // the vectors fit in registers beside the row
@@ -256,21 +256,22 @@ __global__ void __launch_bounds__(kLnThreads) ln_modulate_kernel(const float *x,
       const int g = tid + t * kLnThreads;
       if (g >= n4) continue;
       gate[t] = __ldg(reinterpret_cast<const float4 *>(parts.gate + voff) + g);
-      const uint2 u = __ldg(reinterpret_cast<const uint2 *>(parts.bias) + g);
+      const uint2 u = parts.bias ? __ldg(reinterpret_cast<const uint2 *>(parts.bias) + g) : make_uint2(0u, 0u);
       const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.x)), b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.y));
       bias[t] = make_float4(a.x, a.y, b.x, b.y);
     }
   }
   pdl_wait();
   if (kHold && !early) fetch_vecs();
-  const float4 *xr = reinterpret_cast<const float4 *>(x + (static_cast<long long>(e * xmap.bmul + xmap.boff) * xmap.rpb + j) * C);
+  const RowMap rmap = PARTS ? parts.inmap : xmap;
+  const float4 *xr = reinterpret_cast<const float4 *>((PARTS ? parts.xin : x) + (static_cast<long long>(e * rmap.bmul + rmap.boff) * rmap.rpb + j) * C);
   float4 v[T];
   float sum = 0.f;
 #pragma unroll
   for (int t = 0; t < T; ++t) v[t] = tid + t * kLnThreads < n4 ? xr[tid + t * kLnThreads] : make_float4(0.f, 0.f, 0.f, 0.f);
   if constexpr (PARTS) {
     const float4 *pr = reinterpret_cast<const float4 *>(parts.part + static_cast<long long>(blockIdx.x) * C);
-    float4 *xw = const_cast<float4 *>(xr);
+    float4 *xw = reinterpret_cast<float4 *>(const_cast<float *>(x) + (static_cast<long long>(e * xmap.bmul + xmap.boff) * xmap.rpb + j) * C);
     float4 q[kMaxParts][T];
 #pragma unroll
     for (int s = 0; s < kMaxParts; ++s)
@@ -328,7 +329,7 @@ cudaError_t launch_ln_modulate(const float *x, RowMap xmap, int E, int rows, int
   if (E * rows <= 0) return cudaSuccess;
   if (C % 8 != 0 || C > 4 * kLnThreads * kLnMaxVec) return cudaErrorInvalidValue;
   auto go = [&](auto kern) {
-    return launch_pdl(kern, dim3(E * rows), dim3(kLnThreads), 0, st, x, xmap, rows, C, shift, scale, vec_stride, bmul, boff, gamma, eps, early ? 1 : 0, y, LnParts{});
+    return launch_pdl(kern, dim3(E * rows), dim3(kLnThreads), 0, st, x, xmap, rows, C, shift, scale, vec_stride, bmul, boff, gamma, eps, early ? 1 : 0, y, GemmParts{});
   };
   if (C <= 512) return go(ln_modulate_kernel<1, false>);
   if (C <= 1024) return go(ln_modulate_kernel<2, false>);
@@ -338,7 +339,7 @@ cudaError_t launch_ln_modulate(const float *x, RowMap xmap, int E, int rows, int
 }
 
 // C <= 2048: gemm_partial_plan takes no wider output.
-cudaError_t launch_ln_parts(float *x, RowMap xmap, int E, int rows, int C, const LnParts &parts, const float *shift, const float *scale,
+cudaError_t launch_ln_parts(float *x, RowMap xmap, int E, int rows, int C, const GemmParts &parts, const float *shift, const float *scale,
                             long long vec_stride, int bmul, int boff, float eps, bf16 *y, cudaStream_t st) {
   if (E * rows <= 0) return cudaSuccess;
   if (C % 8 != 0 || C > 2048 || parts.splits < 1 || parts.splits > kMaxParts || parts.stride % 4 != 0) return cudaErrorInvalidValue;
@@ -349,6 +350,73 @@ cudaError_t launch_ln_parts(float *x, RowMap xmap, int E, int rows, int C, const
   if (C <= 512) return go(ln_modulate_kernel<1, true>);
   if (C <= 1024) return go(ln_modulate_kernel<2, true>);
   return go(ln_modulate_kernel<4, true>);
+}
+
+// The K ranges of a group's last fc2 (see launch_finish_parts): one CTA of 128 threads a row, T float4 a thread, everything a
+// row reads in flight together.  Bound by latency and by the 4 C (ranges + 2) bytes a row, or 4 C more with the split, that
+// come from and stay in L2: in the chain about 3 us for 400 rows of 2048 columns in four ranges.  gemm_partial_plan has what the
+// GEMM and this launch take together against a GEMM that reduces by itself.
+template <int T>
+__global__ void __launch_bounds__(kLnThreads) finish_parts_kernel(GemmParts parts, int rows, int C, long long vec_stride, int bmul, int boff,
+                                                                  float *__restrict__ out, RowMap omap, const int *__restrict__ scatter,
+                                                                  bf16 *__restrict__ xsplit, int xsplit_mk) {
+  pdl_launch_dependents();
+  const int e = blockIdx.x / rows, j = blockIdx.x - e * rows, n4 = C / 4, tid = threadIdx.x;
+  float4 gate[T];
+  uint2 bias[T];
+#pragma unroll
+  for (int t = 0; t < T; ++t) {
+    const int g = tid + t * kLnThreads;
+    if (g >= n4) continue;
+    gate[t] = __ldg(reinterpret_cast<const float4 *>(parts.gate + static_cast<long long>(e * bmul + boff) * vec_stride) + g);
+    bias[t] = parts.bias ? __ldg(reinterpret_cast<const uint2 *>(parts.bias) + g) : make_uint2(0u, 0u);
+  }
+  pdl_wait();
+  const int jo = scatter ? scatter[static_cast<long long>(e) * rows + j] : j;
+  const float4 *xr = reinterpret_cast<const float4 *>(parts.xin + (static_cast<long long>(e * parts.inmap.bmul + parts.inmap.boff) * parts.inmap.rpb + j) * C);
+  const float4 *pr = reinterpret_cast<const float4 *>(parts.part + static_cast<long long>(blockIdx.x) * C);
+  float4 v[T], q[kMaxParts][T];
+#pragma unroll
+  for (int t = 0; t < T; ++t)
+    if (tid + t * kLnThreads < n4) v[t] = xr[tid + t * kLnThreads];
+#pragma unroll
+  for (int s = 0; s < kMaxParts; ++s)
+#pragma unroll
+    for (int t = 0; t < T; ++t)
+      q[s][t] = (s < parts.splits && tid + t * kLnThreads < n4) ? pr[s * (parts.stride >> 2) + tid + t * kLnThreads] : make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 *dst = reinterpret_cast<float4 *>(out + (static_cast<long long>(e * omap.bmul + omap.boff) * omap.rpb + jo) * C);
+  uint2 *hi = xsplit ? reinterpret_cast<uint2 *>(xsplit + (static_cast<long long>(e) * 2 * xsplit_mk + jo) * C) : nullptr;
+#pragma unroll
+  for (int t = 0; t < T; ++t) {
+    const int g = tid + t * kLnThreads;
+    if (g >= n4) continue;
+    float4 a = q[0][t];
+#pragma unroll
+    for (int s = 1; s < kMaxParts; ++s) { a.x += q[s][t].x; a.y += q[s][t].y; a.z += q[s][t].z; a.w += q[s][t].w; }
+    const float2 b0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&bias[t].x)), b1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&bias[t].y));
+    a.x = fmaf(gate[t].x, a.x + b0.x, v[t].x); a.y = fmaf(gate[t].y, a.y + b0.y, v[t].y);
+    a.z = fmaf(gate[t].z, a.z + b1.x, v[t].z); a.w = fmaf(gate[t].w, a.w + b1.y, v[t].w);
+    dst[g] = a;
+    if (hi != nullptr) {
+      const __nv_bfloat162 h0 = __floats2bfloat162_rn(a.x, a.y), h1 = __floats2bfloat162_rn(a.z, a.w);
+      const float2 f0 = __bfloat1622float2(h0), f1 = __bfloat1622float2(h1);
+      const __nv_bfloat162 l0 = __floats2bfloat162_rn(a.x - f0.x, a.y - f0.y), l1 = __floats2bfloat162_rn(a.z - f1.x, a.w - f1.y);
+      hi[g] = make_uint2(*reinterpret_cast<const uint32_t *>(&h0), *reinterpret_cast<const uint32_t *>(&h1));
+      hi[static_cast<long long>(xsplit_mk) * n4 + g] = make_uint2(*reinterpret_cast<const uint32_t *>(&l0), *reinterpret_cast<const uint32_t *>(&l1));
+    }
+  }
+}
+
+cudaError_t launch_finish_parts(const GemmParts &parts, int E, int rows, int C, long long vec_stride, int bmul, int boff, float *out, RowMap omap,
+                                const int *scatter, bf16 *xsplit, int xsplit_mk, cudaStream_t st) {
+  if (E * rows <= 0) return cudaSuccess;
+  if (C % 8 != 0 || C > 2048 || parts.splits < 1 || parts.splits > kMaxParts || parts.stride % 4 != 0) return cudaErrorInvalidValue;
+  auto go = [&](auto kern) {
+    return launch_pdl(kern, dim3(E * rows), dim3(kLnThreads), 0, st, parts, rows, C, vec_stride, bmul, boff, out, omap, scatter, xsplit, xsplit_mk);
+  };
+  if (C <= 512) return go(finish_parts_kernel<1>);
+  if (C <= 1024) return go(finish_parts_kernel<2>);
+  return go(finish_parts_kernel<4>);
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -1108,6 +1108,7 @@ static fvar_status scale_step_impl(fvar_ctx *ctx, const void *tokens, bool token
   // given (scale, ranks, cache lengths, slots) it is the same chain of launches every time: it is
   // captured into a CUDA graph on first use and replayed afterwards.
   auto body = [&]() -> fvar_status {
+  GemmParts parts{};                      // fc2 of the block before, left in K ranges for this block's first LayerNorm
   for (int g = 0; g < G; ++g) {
     const int r = rank[g];
     const bool late = r < M;
@@ -1181,7 +1182,6 @@ static fvar_status scale_step_impl(fvar_ctx *ctx, const void *tokens, bool token
       ctx->launched();
     }
 
-    LnParts parts{};                      // fc2 of the block before, left in K ranges for this block's first LayerNorm
     for (int t = 0; t < bpg; ++t) {
       const int blk = g * bpg + t;
       const bool first_dense = (t == 0) && !late, last = (t == bpg - 1);
@@ -1197,7 +1197,7 @@ static fvar_status scale_step_impl(fvar_ctx *ctx, const void *tokens, bool token
 
       ctx->prof_begin(FVAR_KCLASS_LN, 0.0, 6.0 * R * C);
       if (parts.splits > 0)
-        FV_CUDA(ctx, launch_ln_parts(ctx->xs, smap, E, r, C, parts, ada, ada + C, 6 * C, bmul, boff, ctx->cfg.ln_eps, ctx->y, st), "ln_modulate 1");
+        FV_CUDA(ctx, launch_ln_parts(const_cast<float *>(in_ptr), in_map, E, r, C, parts, ada, ada + C, 6 * C, bmul, boff, ctx->cfg.ln_eps, ctx->y, st), "ln_modulate 1");
       else
         FV_CUDA(ctx, launch_ln_modulate(in_ptr, in_map, E, r, C, ada, ada + C, 6 * C, bmul, boff, nullptr,
                                         ctx->cfg.ln_eps, true, ctx->y, st), "ln_modulate 1");
@@ -1270,22 +1270,32 @@ static fvar_status scale_step_impl(fvar_ctx *ctx, const void *tokens, bool token
         ga.rows_per_batch = r; ga.bmul = bmul; ga.boff = boff;
         ga.resid = ctx->xs; ga.rmap = smap; ga.ld_out = C;
         ga.gate = ada + 5 * C; ga.gate_stride = 6 * C;
-        if (last && !(lls && late)) {
-          if (forked) FV_CUDA(ctx, cudaStreamWaitEvent(st, ctx->ev_join, 0), "join wait");
+        const bool to_group = last && !(lls && late);      // the result is the group's output
+        if (to_group) {
           ga.out_f32 = gout; ga.omap = bmap;
           ga.scatter = late ? idx_g : nullptr;
           ga.xsplit = next_split; ga.xsplit_mk = Mk;
         } else {
           ga.out_f32 = ctx->xs; ga.omap = smap;
         }
+        auto join = [&]() { return to_group && forked ? cudaStreamWaitEvent(st, ctx->ev_join, 0) : cudaSuccess; };
         prefetch_next(ga, blk + 1, W_QKV);
         int rows_tile = 0;
-        const int ranges = (last || ctx->skinny_max_rows <= 0 || ctx->b_fc2[blk] == nullptr) ? 0 : gemm_partial_plan(R, C, F, ctx->max_clusters, &rows_tile);
+        const int ranges = ctx->skinny_max_rows > 0 ? gemm_partial_plan(R, C, F, ctx->max_clusters, &rows_tile) : 0;
         if (ranges > 0 && static_cast<size_t>(ranges) * R * C * 4 <= kSplitScratchBytes) {
-          // the next block's first LayerNorm adds the K ranges up; the residual stream stays where it is until then
-          parts = LnParts{ctx->split_partial, ranges, static_cast<long long>(R) * C, ctx->b_fc2[blk], ga.gate};
+          // the residual stream stays where it is until the sums are added up: by the next block's first LayerNorm, which
+          // writes this group's output where it is the next group's, or by a kernel of its own
+          parts = GemmParts{ctx->split_partial, ranges, static_cast<long long>(R) * C, ctx->b_fc2[blk], ga.gate, ctx->xs, smap};
           if ((s = run_gemm_parts(ctx, ctx->h_map, blk, W_FC2, R, C, F, ranges, rows_tile)) != FVAR_OK) return s;
+          if (last && (late || g + 1 == G || rank[g + 1] < M)) {
+            FV_CUDA(ctx, join(), "join wait");
+            ctx->prof_begin(FVAR_KCLASS_CONVERT, 0.0, 4.0 * R * C * (ranges + 2) + (ga.xsplit ? 4.0 * R * C : 0.0));
+            FV_CUDA(ctx, launch_finish_parts(parts, E, r, C, 6 * C, bmul, boff, ga.out_f32, ga.omap, ga.scatter, ga.xsplit, ga.xsplit_mk, st), "fc2 sums");
+            ctx->launched();
+            parts.splits = 0;
+          }
         } else {
+          FV_CUDA(ctx, join(), "join wait");
           if ((s = run_gemm(ctx, EPI_RESID, ctx->h_map, blk, W_FC2, ga, "fc2 gemm")) != FVAR_OK) return s;
         }
       }

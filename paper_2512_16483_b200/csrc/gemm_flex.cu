@@ -260,19 +260,25 @@ void gemm_flex_shape(GemmArgs &a) {
 }
 
 // The reduction of a K split over CTAs costs a cluster barrier and a round of remote reads after the last MMA, and the
-// 128 x 128 tiles of that form (gemm_skinny.cu) move twice the operands of 256 x 224.  Where a LayerNorm follows, it
-// can add up the ranges while it reads its rows: 400 x 2048 x 8192 with its gate and residual 25.9 us in the chain, now 17 and 1 in the
-// LayerNorm (Infinity 40 with table 3693 -> 3578 us, three late scales 11014 -> 10650).  The line is drawn by rows, not by
-// an estimate: taken where that form is the alternative (gemm_ksplit_wins: N <= 2048, K >= 4096, up to 512 rows) and the
-// rows are more than one chunk.  It is the better one at both ends (a step of the 48 x 48 scale with ranges and without,
-// us: 258 rows 3762 and 3966, 320 rows 3845 and 4039, 400 rows 4160 and 4289, 512 rows 4450 and 4520); up to 256 rows
-// ranges gained nothing.  Four ranges, or three where K / 64 is a multiple of 6 and not of 8; with two, too few pairs work.
+// 128 x 128 tiles of that form (gemm_skinny.cu) move twice the operands of 256 x 224.  The kernel that reads the rows next
+// can add up the ranges instead: the LayerNorm of the next block (400 x 2048 x 8192 with its gate and residual 25.9 us in the
+// chain of a step, now 17 and 1 in the LayerNorm), or after a group's last block, whose rows are scattered and split for a
+// projection, a pass of its own (26 us, now 17 and 3).
+// Taken where the ranges fill most of the pairs and are long division enough: three or four of them, 0.6 of the pairs at
+// work, two to four chunks of rows.  A step with ranges in every block and without (us):
+//   2048 columns, K = 8192, four ranges, 64 pairs: 257 rows 3659 and 3934, 400 rows 4061 and 4253, 512 rows 4344 and 4424;
+//   600 and 768 rows, where two ranges are all that fit: 5085 and 5039, 5554 and 5533 -- not taken;
+//   1920 columns, K = 7680: 340 rows (64 pairs) 2361 and 2548, 510 rows 3012 and 3153, 680 rows (three ranges, 72 pairs) 3350 and 3515;
+//   1024 columns, K = 4096: 576 rows (48 pairs) 787 and 858, 640 rows 833 and 885, 680 rows 1021 and 1041, 850 rows (64 pairs) 1205
+//   and 1215; 400 and 510 rows (32 pairs) 786 and 770, 950 and 925, 1020 rows (64 full chunks) 1244 and 1231 -- not taken.
+// One chunk (up to 256 rows) gains nowhere: 200 rows of 2048 columns 3365 and 3278.
 int gemm_partial_plan(int R, int N, int K, int max_clusters, int *rows_tile) {
-  if (R <= 256 || !gemm_ksplit_wins(R, N, K) || !gemm_flex_supported(EPI_PARTIAL, N, K) || K % kBlockK != 0) return 0;
-  const int tiles_f = (N + 2 * kBlockM - 1) / (2 * kBlockM), chunks = (R + 255) / 256, num_kb = K / kBlockK;
+  const int chunks = (R + 255) / 256, num_kb = K / kBlockK, tiles = (N + 2 * kBlockM - 1) / (2 * kBlockM) * chunks;
+  if (chunks < 2 || chunks > 4 || N > 2048 || K < 4096 || K % kBlockK != 0 || !gemm_flex_supported(EPI_PARTIAL, N, K)) return 0;
   *rows_tile = ((R + chunks - 1) / chunks + 31) / 32 * 32;
+  if (chunks == 4 && *rows_tile > 224) return 0;
   for (int s = kMaxParts; s >= 3; --s)
-    if (num_kb % (2 * s) == 0 && tiles_f * chunks * s <= max_clusters) return s;
+    if (num_kb % (2 * s) == 0 && tiles * s <= max_clusters) return 5 * tiles * s >= 3 * max_clusters ? s : 0;
   return 0;
 }
 

@@ -142,7 +142,7 @@ cudaError_t gemm_skinny_prepare();
 // tmA / tmW: gemm_skinny_map with boxes of fx_nb / 2 and 128 rows.
 bool gemm_flex_supported(int epi, int N, int K);
 void gemm_flex_shape(GemmArgs &a);
-// K ranges (and rows a tile) for an R x N x K product whose sums the following LayerNorm adds up; 0: other forms are better.
+// K ranges (and rows a tile) for an R x N x K product whose sums the following kernel adds up; 0: other forms are better.
 int gemm_partial_plan(int R, int N, int K, int max_clusters, int *rows_tile);
 cudaError_t launch_gemm_flex(int epi, const CUtensorMap &tmA, const CUtensorMap &tmW, const GemmArgs &a, int max_clusters, cudaStream_t st);
 cudaError_t gemm_flex_prepare();
@@ -204,17 +204,24 @@ cudaError_t launch_row_scores(const float *x, RowMap xmap, int E, int M, int C, 
 cudaError_t launch_select_topr(const float *scores, int B, int M, int r, int *idx, int *inv, cudaStream_t st);
 cudaError_t launch_copy_indices(const int *forced, int B, int M, int r, int ld_forced, int *idx, int *inv,
                                 unsigned *status, cudaStream_t st);
-// K ranges of the GEMM before a LayerNorm that the latter adds up first: x += gate * (sum of the parts + bias), in place.
-struct LnParts {
+// K ranges of a GEMM that the kernel after it adds up: x = xin + gate * (sum of the parts + bias).
+struct GemmParts {
   const float *part;               // [splits][E * rows][C]
   int splits;                      // up to kMaxParts
   long long stride;                // floats between two parts
-  const bf16 *bias;                // [C]
+  const bf16 *bias;                // [C] or nullptr
   const float *gate;               // [caller element][vec_stride]
+  const float *xin;                // what the sum is added to, rows by inmap
+  RowMap inmap;
 };
 constexpr int kMaxParts = 4;
-cudaError_t launch_ln_parts(float *x, RowMap xmap, int E, int rows, int C, const LnParts &parts, const float *shift, const float *scale,
+// The LayerNorm does: x (rows by xmap; it may be xin) is written, then normalised.
+cudaError_t launch_ln_parts(float *x, RowMap xmap, int E, int rows, int C, const GemmParts &parts, const float *shift, const float *scale,
                             long long vec_stride, int bmul, int boff, float eps, bf16 *y, cudaStream_t st);
+// No LayerNorm follows: row j of element e goes to row scatter[e][j] (j without scatter) of out, rows by omap, and as its
+// two-term bf16 split to xsplit (optional; see GemmArgs::xsplit).
+cudaError_t launch_finish_parts(const GemmParts &parts, int E, int rows, int C, long long vec_stride, int bmul, int boff, float *out, RowMap omap,
+                                const int *scatter, bf16 *xsplit, int xsplit_mk, cudaStream_t st);
 // early: shift, scale and gamma are not written by any kernel that may still be in flight (they may then be read before
 // the preceding kernel has finished).
 cudaError_t launch_ln_modulate(const float *x, RowMap xmap, int E, int rows, int C, const float *shift,

@@ -607,3 +607,21 @@ def test_lls_restoration_two_groups_and_limits(fv):
     with pytest.raises(fv.FvarError) as ei:
         p.gpu.scale_step(to_bf16_cuda(toks), 3, mode=fv.LOWRANK_RTR, rank_per_group=[200, 24], restore=fv.RESTORE_LLS)
     assert ei.value.status == fv.EUNSUPPORTED
+
+
+@pytest.mark.parametrize("B,k,blocks,ranks,kind,forced", [
+    (6, 7, 2, None, "normal", True),             # 600 rows dense: fc2 in K ranges that the next group's LayerNorm, or the last kernel, adds up
+    (7, 6, 1, None, "normal", True),             # 448 rows of 1024 columns: too few pairs, a GEMM that reduces by itself
+    (16, 8, 3, [85, 85, 85], "normal", True),    # 680 rows: scattered, with and without the split for the next group's projection
+    (16, 8, 2, [85, 169], "normal", True),       # a late group before a dense one
+    (16, 8, 1, [85], "spread", False),           # free selection, so through the graph whose second branch joins before the sums
+])
+def test_last_product_of_a_group_in_k_ranges(fv, B, k, blocks, ranks, kind, forced):
+    p = Pair(fv, si.shape_var_d16(n_blocks=blocks), seed=140 + B, B=B)
+    p.prefill(k)
+    M = p.shp.tokens_per_scale()[k]
+    toks = si.make_tokens(141, B, M, 1024, kind)
+    if ranks:
+        p.set_projections(k, ranks)
+    got, ref = _step_both(p, toks, k, mode=fv.LOWRANK_RTR if ranks else fv.DENSE, cfg="null_only" if ranks else "pair", ranks=ranks, forced=forced)
+    assert_out_close(got, ref, what="%d rows" % (B * M if not ranks else B // 2 * ranks[0]), max_rel=2e-2 * np.sqrt(blocks) if ranks else 2e-2)

@@ -170,8 +170,64 @@ __global__ void __launch_bounds__(kSelThreads) select_topr_kernel(const float *_
   }
 }
 
+// The same result for up to 256 rows by counting: row i is taken if fewer than r rows come before it, those with a larger
+// key and those with the same key and a lower index.  The M x M comparisons are spread over the block, part p of the rows
+// against all of them in warps of their own, so that every read of a key is a broadcast; with k_j >= 1, "k_j >= k_i" for
+// j < i and "k_j > k_i" for j > i are one comparison against k_i - 1 and k_i.  No histograms, so three barriers instead of
+// two dozen.  Bound by latency; in a chain of itself 169 rows 4.4 -> 3.3 us, 256 rows 4.3 -> 3.7, but 506 rows 4.4 -> 7.2, where the
+// comparisons are most of it, hence the line.  In a late step it runs beside the chain, whose QKV product cannot start on
+// the SMs that its 1024 threads fill: 13 x 13 scale of the 1024-column stack, eight elements, 1017 -> 1002 us.
+constexpr int kSelCountMax = 256;
+__global__ void __launch_bounds__(kSelThreads) select_count_kernel(const float *__restrict__ scores, int M, int r,
+                                                                   int *__restrict__ idx, int *__restrict__ inv) {
+  pdl_wait();
+  pdl_launch_dependents();
+  __shared__ __align__(16) unsigned keys[kSelCountMax];
+  __shared__ int before[kSelThreads];
+  __shared__ int warp_taken[kSelCountMax / 32];
+  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+  const int width = (M + 31) & ~31, parts = kSelThreads / width, part = tid / width, i = tid - part * width;
+  if (tid < kSelCountMax) keys[tid] = tid < M ? score_key(scores[static_cast<long long>(b) * M + tid]) : 0u;    // 0: before nobody
+  __syncthreads();
+  if (part < parts) {
+    const unsigned ki = keys[i];
+    const int chunks = (M + 3) / 4, per = (chunks + parts - 1) / parts;
+    const int c0 = part * per, c1 = min(chunks, c0 + per), own = i / 4;
+    int n = 0;
+    auto count = [&](int lo, int hi, unsigned t) {
+#pragma unroll 4
+      for (int c = lo; c < hi; ++c) {
+        const uint4 k = reinterpret_cast<const uint4 *>(keys)[c];
+        n += (k.x > t) + (k.y > t) + (k.z > t) + (k.w > t);
+      }
+    };
+    count(c0, min(c1, own), ki - 1u);
+    count(max(c0, own + 1), c1, ki);
+    if (own >= c0 && own < c1)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) n += keys[4 * own + e] > (4 * own + e < i ? ki - 1u : ki);
+    before[part * width + i] = n;
+  }
+  __syncthreads();
+  bool take = false;
+  if (tid < M) {
+    int n = 0;
+    for (int p = 0; p < parts; ++p) n += before[p * width + tid];
+    take = n < r;
+  }
+  const unsigned taken = __ballot_sync(0xffffffffu, take);
+  if (lane == 0 && tid < kSelCountMax) warp_taken[tid >> 5] = __popc(taken);
+  __syncthreads();
+  if (tid >= M) return;
+  int pos = __popc(taken & ((1u << lane) - 1u));
+  for (int w = 0; w < tid >> 5; ++w) pos += warp_taken[w];
+  if (take) idx[static_cast<long long>(b) * r + pos] = tid;
+  inv[static_cast<long long>(b) * M + tid] = take ? pos : -1;
+}
+
 cudaError_t launch_select_topr(const float *scores, int B, int M, int r, int *idx, int *inv, cudaStream_t st) {
   if (B <= 0) return cudaSuccess;
+  if (M <= kSelCountMax) return launch_pdl(select_count_kernel, dim3(B), dim3(kSelThreads), 0, st, scores, M, r, idx, inv);
   return launch_pdl(select_topr_kernel, dim3(B), dim3(kSelThreads), 0, st, scores, M, r, idx, inv);
 }
 

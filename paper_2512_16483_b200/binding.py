@@ -55,6 +55,7 @@ class _Policy(ct.Structure):
 
 
 _lib = None
+_calls = None                    # the short calls in native code (csrc/pycalls.cpp)
 
 
 def load_library() -> ct.CDLL:
@@ -121,8 +122,19 @@ def load_library() -> ct.CDLL:
     for name, (res, args) in sigs.items():
         fn = getattr(lib, name)
         fn.restype, fn.argtypes = res, args
-    _lib = lib
+    global _calls
+    try:
+        from . import _calls as calls
+    except ImportError as e:
+        raise FileNotFoundError("the library's call layer is not built: run `python -m paper_2512_16483_b200.build`") from e
+    _lib, _calls = lib, calls
     return lib
+
+
+def _native():
+    if _calls is None:
+        load_library()
+    return _calls
 
 
 EXPORTED = ("fvar_workspace_bytes", "fvar_init", "fvar_set_cond", "fvar_set_projection", "fvar_generate_projection",
@@ -157,6 +169,14 @@ def _check_kernel(status: int):
         raise FvarError(status, (load_library().fvar_last_error(None) or b"").decode())
 
 
+# The calls below that are a few microseconds long go through csrc/pycalls.cpp, which answers with the result, with the status
+# of a call that the library refused, or with None for anything but plain CUDA tensors; then the general way is taken.
+def _result(out):
+    if type(out) is int:
+        _check_kernel(out)
+    return out
+
+
 def _dev(t: torch.Tensor, dtype) -> torch.Tensor:
     assert t.is_cuda and t.dtype == dtype and t.is_contiguous(), (t.device, t.dtype, t.is_contiguous())
     return t
@@ -166,6 +186,9 @@ def _dev(t: torch.Tensor, dtype) -> torch.Tensor:
 
 def fvar_row_scores(x: torch.Tensor) -> torch.Tensor:
     """x fp32 [B][M][C] -> scores fp32 [B][M]."""
+    out = _native().row_scores(x)
+    if out is not None:
+        return _result(out)
     _dev(x, torch.float32)
     B, M, C = x.shape
     s = x.new_empty((B, M))
@@ -184,6 +207,9 @@ def fvar_row_keys(x: torch.Tensor, noise: torch.Tensor) -> torch.Tensor:
 
 def fvar_select_topr(scores: torch.Tensor, r: int):
     """scores fp32 [B][M] -> (idx int32 [B][r] ascending, inv int32 [B][M])."""
+    out = _native().select_topr(scores, r)
+    if out is not None:
+        return _result(out)
     _dev(scores, torch.float32)
     B, M = scores.shape
     idx = scores.new_empty((B, r), dtype=torch.int32)
@@ -194,6 +220,9 @@ def fvar_select_topr(scores: torch.Tensor, r: int):
 
 def fvar_ln_modulate(x: torch.Tensor, shift: torch.Tensor, scale: torch.Tensor, eps: float) -> torch.Tensor:
     """x fp32 [B][n][C], shift/scale fp32 [B][C] -> bf16 [B][n][C]."""
+    out = _native().ln_modulate(x, shift, scale, eps)
+    if out is not None:
+        return _result(out)
     _dev(x, torch.float32), _dev(shift, torch.float32), _dev(scale, torch.float32)
     B, n, C = x.shape
     y = x.new_empty((B, n, C), dtype=torch.bfloat16)
@@ -230,6 +259,9 @@ def fvar_gemm_bf16_wt(A: torch.Tensor, Wt: torch.Tensor, bias: Optional[torch.Te
 
 def fvar_cfg_combine(pair: torch.Tensor, guidance: float) -> torch.Tensor:
     """pair bf16 [B][...] with elements (2p, 2p + 1) = (prompt, null) -> bf16 [B / 2][...] = null + guidance (prompt - null)."""
+    res = _native().cfg_combine(pair, guidance)
+    if res is not None:
+        return _result(res)
     _dev(pair, torch.bfloat16)
     B = pair.shape[0]
     per = pair[0].numel()
@@ -251,6 +283,9 @@ def fvar_attention(q: torch.Tensor, Kc: torch.Tensor, Vt: torch.Tensor, L: int) 
 
 def fvar_rtr_fill(prev: torch.Tensor, hw_in, hw_out, inv: Optional[torch.Tensor], out: torch.Tensor) -> torch.Tensor:
     """Fills rows of out fp32 [B][h1*w1][C] whose inv < 0 with the upsampled rows of prev fp32 [B][h0*w0][C]."""
+    res = _native().rtr_fill(prev, hw_in, hw_out, inv, out)
+    if res is not None:
+        return _result(res)
     _dev(prev, torch.float32), _dev(out, torch.float32)
     B, _, C = prev.shape
     _check_kernel(load_library().fvar_rtr_fill(prev.data_ptr(), B, hw_in[0], hw_in[1], hw_out[0], hw_out[1], C,
@@ -359,6 +394,11 @@ class Fvar:
     def scale_transition(self, fo: torch.Tensor, scale_idx: int, next_M: Optional[int], pairs: bool = False):
         """fo bf16 [B][M_k][C] -> (codes int32 [B][M_k], next tokens bf16 [B][next_M][C] or None at the last scale).
         pairs: the next tokens come out as [2 B][next_M][C], every image's rows twice (both branches of its CFG pair)."""
+        res = _native().scale_transition(self.ctx.value, fo, scale_idx, next_M or 0, pairs)
+        if res is not None:
+            if type(res) is int:
+                self._check(res)
+            return res
         _dev(fo, torch.bfloat16)
         B, M, C = fo.shape
         codes = torch.empty((B, M), dtype=torch.int32, device=fo.device)

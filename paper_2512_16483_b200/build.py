@@ -1,14 +1,17 @@
-"""Builds libfvar.so (the C-ABI library) in-tree with nvcc for sm_100a."""
+"""Builds libfvar.so (the C-ABI library) in-tree with nvcc for sm_100a, and _calls.so (the binding's short calls) beside it."""
 from __future__ import annotations
 
 import concurrent.futures
+import importlib.util
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libfvar.so")
+CALLS = os.path.join(HERE, "_calls.so")
 OBJDIR = os.path.join(HERE, "_build")
 SOURCES = ("gemm.cu", "gemm_pair.cu", "gemm_skinny.cu", "gemm_flex.cu", "attention.cu", "elementwise.cu", "transition.cu", "lls.cu", "fvar_api.cu", "no_alloc.cu", "schedule.cu")
 NVCC_FLAGS = os.environ.get("FVAR_NVCC_EXTRA", "").split() + ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -25,9 +28,9 @@ def _sources():
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(CALLS):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(CALLS))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(HERE, "..", "include", "fvar.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -43,6 +46,20 @@ def _compile(src: str) -> str:
     return obj
 
 
+def _compile_calls() -> str:
+    """csrc/pycalls.cpp: host code against torch's headers, linked to the library beside it."""
+    torch_dir = importlib.util.find_spec("torch").submodule_search_locations[0]
+    inc, libs = os.path.join(torch_dir, "include"), os.path.join(torch_dir, "lib")
+    cuda = os.path.dirname(os.path.dirname(_nvcc())) or "/usr/local/cuda"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-I" + inc, "-I" + os.path.join(inc, "torch", "csrc", "api", "include"),
+           "-I" + os.path.join(cuda, "include"), "-I" + sysconfig.get_paths()["include"], os.path.join(CSRC, "pycalls.cpp"), "-o", CALLS,
+           "-L" + HERE, "-l:libfvar.so", "-L" + libs, "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python", "-Wl,-rpath,$ORIGIN"]
+    p = subprocess.run(cmd, capture_output=True, text=True)
+    if p.returncode != 0:
+        raise RuntimeError("g++ failed for pycalls.cpp:\n" + p.stderr[-4000:])
+    return CALLS
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     if not force and not _stale():
         return LIB
@@ -53,6 +70,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     p = subprocess.run(cmd, capture_output=True, text=True)
     if p.returncode != 0:
         raise RuntimeError("link failed:\n" + p.stderr[-4000:])
+    _compile_calls()
     if verbose:
         for o in objs:
             sys.stdout.write(open(o + ".log").read())

@@ -46,7 +46,7 @@ def _check_select(fv, scores: np.ndarray, r: int):
         assert np.array_equal(inv[b], exp_inv)
 
 
-@pytest.mark.parametrize("M", [1, 2, 33, 100, 169, 256, 1024, 1600, 4096, 5000])
+@pytest.mark.parametrize("M", [1, 2, 33, 100, 169, 255, 256, 257, 1024, 1600, 4096, 5000])
 def test_select_random_scores(fv, M):
     rng = np.random.default_rng(M)
     s = (rng.standard_normal((3, M)) ** 2).astype(np.float32) * 1000
@@ -320,3 +320,75 @@ def test_cluster_reductions_are_bit_stable(fv):
     for _ in range(3):
         assert torch.equal(first, fv.fvar_attention(q, Kc, Vt, L))
     _poll(fv)
+
+
+# ----------------------------------------------------------------------------- the two ways of a short call
+
+@pytest.mark.parametrize("B,h0,w0,h1,w1,C,r", [(1, 1, 1, 1, 1, 8, 1), (3, 2, 5, 7, 9, 1000, 63), (2, 13, 13, 16, 16, 1024, 128), (1, 20, 21, 23, 29, 72, 13)])
+def test_short_calls_native_and_general_way_agree(fv, monkeypatch, B, h0, w0, h1, w1, C, r):
+    """Kernel-level calls through native code and through ctypes are the same calls: equal results, bit for bit."""
+    g = torch.Generator(device="cuda").manual_seed(B * C + r)
+    rand = lambda *shape, dtype=torch.float32: torch.randn(shape, generator=g, device="cuda").to(dtype)
+    M = h1 * w1
+    x, kept, prev, sh, sc = rand(B, M, C), rand(B, r, C), rand(B, h0 * w0, C), rand(B, C), rand(B, C)
+    pair, dst = rand(2 * B, M, C, dtype=torch.bfloat16), rand(B, M, C)
+
+    def run():
+        s = fv.fvar_row_scores(x)
+        idx, inv = fv.fvar_select_topr(s, r)
+        out = dst.clone()
+        filled = fv.fvar_rtr_fill(prev, (h0, w0), (h1, w1), inv, out)
+        assert filled is out
+        whole = fv.fvar_rtr_fill(prev, (h0, w0), (h1, w1), None, dst.clone())
+        return [s, idx, inv, out, whole, fv.fvar_ln_modulate(kept, sh, sc, 1e-6), fv.fvar_cfg_combine(pair, 3.0)]
+
+    native = run()
+    monkeypatch.setattr(fv, "_native", lambda: type("Refuse", (), {"__getattr__": lambda self, name: lambda *a: None})())
+    for a, b in zip(native, run()):
+        assert a.dtype == b.dtype and a.shape == b.shape and torch.equal(a, b)
+
+
+def test_short_calls_refuse_what_they_refused(fv):
+    x = torch.randn((2, 6, 16), device="cuda")
+    for bad in (x.cpu(), x.double(), x.transpose(1, 2)):                    # another device, type, a strided view
+        with pytest.raises(AssertionError):
+            fv.fvar_row_scores(bad)
+    with pytest.raises(AssertionError):
+        torch.func.vmap(fv.fvar_row_scores, in_dims=3)(torch.randn((2, 6, 16, 3), device="cuda"))
+    with pytest.raises(ValueError):
+        fv.fvar_row_scores(x[0])                                            # two dimensions
+    s = fv.fvar_row_scores(x)
+    for r in (0, 7):
+        with pytest.raises(fv.FvarError) as e:
+            fv.fvar_select_topr(s, r)
+        assert e.value.status == fv.EINVAL
+    with pytest.raises(fv.FvarError):
+        fv.fvar_row_scores(x.view(-1)[1:].narrow(0, 0, 160).view(2, 5, 16))   # off the 16-byte grid
+    from torch.overrides import TorchFunctionMode
+    from torch.utils._python_dispatch import TorchDispatchMode
+    seen = []
+
+    class Functions(TorchFunctionMode):
+        def __torch_function__(self, func, types, args=(), kwargs=None):
+            seen.append("function")
+            return func(*args, **(kwargs or {}))
+
+    class Operators(TorchDispatchMode):
+        def __torch_dispatch__(self, func, types, args=(), kwargs=None):
+            seen.append("operator")
+            return func(*args, **(kwargs or {}))
+
+    for mode in (Functions, Operators):                                     # a mode sees the calls that it saw
+        with mode():
+            y = fv.fvar_row_scores(x)
+        assert torch.equal(y, s)
+    assert "function" in seen and "operator" in seen
+    inv = fv.fvar_select_topr(s, 2)[1]
+    out = fv.fvar_rtr_fill(x, [2, 3], [2, 3], inv, x.clone())               # lists and numpy numbers as before
+    assert torch.equal(out, fv.fvar_rtr_fill(x, (2, 3), (2, 3), inv, x.clone()))
+    assert torch.equal(fv.fvar_select_topr(s, np.int64(2))[1], inv)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):                                           # the current stream, and its allocations
+        a = fv.fvar_row_scores(x)
+    side.synchronize()
+    assert torch.equal(a, s)

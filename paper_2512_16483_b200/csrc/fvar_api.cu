@@ -434,9 +434,9 @@ fvar_status run_gemm(fvar_ctx *ctx, int epi, const fvar_ctx::ActMaps &maps, int 
   ctx->prof_begin(FVAR_KCLASS_GEMM, 2.0 * g.R * g.N * g.K * g.nbatch,
                   2.0 * (static_cast<double>(g.N) * g.K + static_cast<double>(g.R) * g.K * g.nbatch) +
                       (epi == EPI_F32 || epi == EPI_RESID ? 4.0 : 2.0) * g.R * g.N * g.nbatch);
+  g.w_early = 1;
   if (plan.form == kGemmFlex) {
     g.fx_nb = plan.block_n;
-    g.w_early = 1;
     gemm_flex_shape(g);
     CUtensorMap tmA, tmW;
     if (!gemm_skinny_map(&tmA, maps.base, maps.rows, maps.cols, maps.cols, g.fx_nb / 2, g.fx_nk) || !gemm_skinny_map(&tmW, ctx->w[wid][blk], g.N, g.K, g.K, 128, g.fx_nk))

@@ -89,15 +89,36 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_holder;
+  // While the predecessor drains: the weights of the first tile's first stages, in a loop of their own (as in gemm_flex.cu; a
+  // single problem whole along K, so that the tile is the block's index).  Here and in the pairs: one approximated step of
+  // 26 - 410 rows of 2048 columns 3544 -> 3507 us, of 680 rows of 1024 columns 1007 -> 996, of 200 rows of 1920 columns 2131 ->
+  // 2106.  With a test per stage inside the producer's loop the same requests cost 1 - 3 % instead.
+  const int pre = (p.w_early && splits == 1 && p.nbatch == 1) ? min(S, num_kb) : 0;
+  if (threadIdx.x == 0 && pre > 0) {
+    const int row_w = static_cast<int>(blockIdx.x) / tiles_m * BN;
+    for (int i = 0; i < pre; ++i) {
+      mbar_expect_tx(full_bar(i), a_tx_bytes + Cfg::kStageBytesB);
+#pragma unroll
+      for (int ka = 0; ka < kKAtoms; ++ka)
+        tma_load_2d(smem_base + i * Cfg::kStageBytes + Cfg::kStageBytesA + ka * Cfg::kAtomBytesB, &tmW, full_bar(i), (i * kKAtoms + ka) * kBlockK, row_w);
+    }
+  }
   pdl_wait();
   pdl_launch_dependents();
 
   if (warp == 0) {
     if (lane == 0) {
       // ---------------------------------------------------------------- TMA producer
-      int stage = 0;
-      uint32_t phase = 0;
-      uint32_t armed = 0;                      // bit s set: stage s has been armed at least once
+      if (pre > 0) {
+        const int row_a = static_cast<int>(blockIdx.x) % tiles_m * kBlockM;
+        for (int i = 0; i < pre; ++i)
+#pragma unroll
+          for (int ka = 0; ka < kKAtoms; ++ka)
+            tma_load_2d(smem_base + i * Cfg::kStageBytes + ka * Cfg::kAtomBytesA, &tmA, full_bar(i), (i * kKAtoms + ka) * kBlockK, row_a);
+      }
+      int stage = pre == S ? 0 : pre, first = pre;
+      uint32_t phase = pre == S ? 1u : 0u;
+      uint32_t armed = (1u << pre) - 1u;       // bit s set: stage s has been armed at least once
       uint32_t last_parity = 0;                // bit s: parity of the phase last armed on stage s
       bool ok = true;
       for (int work = blockIdx.x; ok && work < total_tiles; work += gridDim.x) {
@@ -107,7 +128,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         const int row_a = e * p.a_batch_rows + m_idx * kBlockM;
         const int row_w = p.w_mn_major ? e * p.b_batch_rows : e * p.b_batch_rows + n_idx * BN;
         const int kb0 = sp * kb_per_split, kb1 = min(num_kb, kb0 + kb_per_split);
-        for (int kb = kb0; kb < kb1; ++kb) {
+        for (int kb = kb0 + first; kb < kb1; ++kb) {
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, p.status, &abort_flag, wb)) { ok = false; break; }
           mbar_expect_tx(full_bar(stage), a_tx_bytes + Cfg::kStageBytesB);
           const uint32_t sa = smem_base + stage * Cfg::kStageBytes;
@@ -128,6 +149,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
           if (++stage == S) { stage = 0; phase ^= 1u; }
         }
+        first = 0;
       }
       if (!ok) {
         // Let every copy that was issued land before the CTA's shared memory is released.

@@ -85,21 +85,39 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   cluster_sync_all();                 // the peer's barriers are initialised before anything signals them
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_holder;
+  // While the predecessor drains: the weights of the first tile's first stages, in a loop of their own (see gemm.cu)
+  const uint32_t full0 = mapa_shared(full_bar(0), 0);        // the stage barriers of rank 0
+  const int pre = p.w_early ? min(S, num_kb) : 0;
+  if (threadIdx.x == 0) {
+    const int row_w = pair / tiles_m2 * BN + static_cast<int>(rank) * Cfg::kHalfN;
+    for (int i = 0; i < pre; ++i) {
+      if (rank == 0) mbar_expect_tx(full_bar(i), 2u * Cfg::kStageBytes);
+#pragma unroll
+      for (int ka = 0; ka < kKAtoms; ++ka)
+        tma_load_2d_pair(smem_base + i * Cfg::kStageBytes + Cfg::kStageBytesA + ka * Cfg::kAtomBytesB, &tmW, full0 + 8u * i, (i * kKAtoms + ka) * kBlockK, row_w);
+    }
+  }
   pdl_wait();
   pdl_launch_dependents();
 
   if (warp == 0) {
     if (lane == 0) {
       // ---------------------------------------------------------------- TMA producer (both CTAs)
-      const uint32_t full0 = mapa_shared(full_bar(0), 0);      // the stage barriers of rank 0
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true, issued = false;
+      {
+        const int row_a = (2 * (pair % tiles_m2) + static_cast<int>(rank)) * kBlockM;
+        for (int i = 0; i < pre; ++i)
+#pragma unroll
+          for (int ka = 0; ka < kKAtoms; ++ka)
+            tma_load_2d_pair(smem_base + i * Cfg::kStageBytes + ka * Cfg::kAtomBytesA, &tmA, full0 + 8u * i, (i * kKAtoms + ka) * kBlockK, row_a);
+      }
+      int stage = pre == S ? 0 : pre, first = pre;
+      uint32_t phase = pre == S ? 1u : 0u;
+      bool ok = true, issued = pre > 0;
       for (int work = pair; ok && work < total_tiles; work += npairs) {
         const int n_idx = work / tiles_m2, m2 = work - n_idx * tiles_m2;
         const int row_a = (2 * m2 + static_cast<int>(rank)) * kBlockM;
         const int row_w = n_idx * BN + static_cast<int>(rank) * Cfg::kHalfN;
-        for (int kb = 0; kb < num_kb; ++kb) {
+        for (int kb = first; kb < num_kb; ++kb) {
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, p.status, &abort_flag, wb)) { ok = false; break; }
           if (rank == 0) mbar_expect_tx(full_bar(stage), 2u * Cfg::kStageBytes);
           const uint32_t sa = smem_base + stage * Cfg::kStageBytes;
@@ -113,6 +131,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           issued = true;
           if (++stage == S) { stage = 0; phase ^= 1u; }
         }
+        first = 0;
       }
       if (!ok && issued) {
         // The byte counts of this CTA's copies go to rank 0's barriers, which cannot be polled from

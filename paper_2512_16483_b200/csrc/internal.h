@@ -74,8 +74,7 @@ struct GemmArgs {
   float *partial;
   int *counters;
   unsigned *status;
-  // The forms with the weights' first stages requested before the wait for the preceding kernel (gemm_skinny.cu,
-  // gemm_flex.cu): no kernel that may still be in flight writes the weights.  0: they are requested after it.
+  // The weights' first stages are requested before the wait for the preceding kernel: no kernel that may still be in flight writes the weights.  0: they are requested after it.
   int w_early;
   // Weight-streaming form (gemm_skinny.cu; `splits` is then the cluster size): rows per column chunk, the padded
   // MMA width of a chunk, chunks (1 or 2) and pipeline stages -- filled by gemm_skinny_shape

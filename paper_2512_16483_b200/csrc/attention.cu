@@ -176,6 +176,38 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_holder;
   pdl_launch_dependents();      // the successor (a GEMM) only requests weights before its own wait
+  // Tile i of a unit's stream of keys and values: K (v = 0) or V^T of which key block, and its request.
+  auto stream_item = [&](int i, int &j, int &v) {
+    j = i >> 1, v = i & 1;                         // even i: K of block i/2, odd i: V^T of block i/2
+    if (DUAL) {                                    // K 0, K 1, V 0, K 2, V 1, K 3, ... V nkv-2, V nkv-1
+      const int k = i - 2, alt = 2 * (nkv - 2);
+      v = k >= alt || (k >= 0 && (k & 1) == 0);
+      j = k < 0 ? i : k < alt ? (k >> 1) + (v ? 0 : 2) : k - alt + nkv - 2;
+    }
+  };
+  auto request = [&](int slot, int j, int v, int bh) {
+    mbar_expect_tx(ring_full(slot), Cfg::kTileBytes);
+    const uint32_t dst = ring_smem + slot * Cfg::kTileBytes;
+    if (v == 0) {
+#pragma unroll
+      for (int a = 0; a < D / 64; ++a) tma_load_3d(dst + a * kAtomBytes, &tmK, ring_full(slot), a * 64, (jb0 + j) * kKeys, bh);
+    } else {
+#pragma unroll
+      for (int a = 0; a < 2; ++a) tma_load_3d(dst + a * (D * 128), &tmV, ring_full(slot), (jb0 + j) * kKeys + a * 64, 0, bh);
+    }
+  };
+  // Tiles of the first unit that no kernel in flight writes are requested while the predecessor drains (see AttnArgs); as for the
+  // weights of the GEMMs in a loop of their own, ahead of the producer's.
+  int pre = 0;
+  if (threadIdx.x == 0 && p.early_rows > 0) {
+    const Unit x = unit_at(unit0);
+    for (; pre < min(p.early_tiles, min(NR, 2 * nkv)); ++pre) {
+      int j, v;
+      stream_item(pre, j, v);
+      if ((jb0 + j + 1) * kKeys > p.early_rows) break;
+      request(pre, j, v, (x.e * p.bmul + p.boff) * p.H + x.h);
+    }
+  }
   pdl_wait();
   float m_ref = -INFINITY, l_run = 0.f;      // softmax threads: running maximum and sum of this thread's query row
   bool final_ok = false;                      // softmax threads: the last P V of the row's tile has completed
@@ -185,10 +217,10 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   if (warp == 0) {
     if (lane == 0) {
       // ---------------------------------------------------------------- TMA producer
-      uint32_t armed = 0, last_parity = 0, q_units = 0;
+      uint32_t armed = (1u << pre) - 1u, last_parity = 0, q_units = 0;
       bool ok = true;
-      int slot = 0;
-      uint32_t phase = 0;
+      int slot = pre == NR ? 0 : pre, first = pre;
+      uint32_t phase = pre == NR ? 1u : 0u;
       for (int u = unit0; ok && u < nunits; u += unit_step) {
         const Unit x = unit_at(u);
         const int bh = (x.e * p.bmul + p.boff) * p.H + x.h;
@@ -199,27 +231,16 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           for (int a = 0; a < D / 64; ++a)
             tma_load_2d(q_smem + t * Cfg::kTileBytes + a * kAtomBytes, &tmQ, q_full, x.h * D + a * 64, x.e * p.r + x.q0 + t * kQRows);
         ++q_units;
-        for (int i = 0; i < 2 * nkv; ++i) {            // even i: K of block i/2, odd i: V^T of block i/2
-          int j = i >> 1, v = i & 1;
-          if (DUAL) {                                  // K 0, K 1, V 0, K 2, V 1, K 3, ... V nkv-2, V nkv-1
-            const int k = i - 2, alt = 2 * (nkv - 2);
-            v = k >= alt || (k >= 0 && (k & 1) == 0);
-            j = k < 0 ? i : k < alt ? (k >> 1) + (v ? 0 : 2) : k - alt + nkv - 2;
-          }
+        for (int i = first; i < 2 * nkv; ++i) {
+          int j, v;
+          stream_item(i, j, v);
           if (!mbar_wait(ring_empty(slot), phase ^ 1u, p.status, &abort_flag, wb)) { ok = false; break; }
-          mbar_expect_tx(ring_full(slot), Cfg::kTileBytes);
-          const uint32_t dst = ring_smem + slot * Cfg::kTileBytes;
-          if (v == 0) {
-#pragma unroll
-            for (int a = 0; a < D / 64; ++a) tma_load_3d(dst + a * kAtomBytes, &tmK, ring_full(slot), a * 64, (jb0 + j) * kKeys, bh);
-          } else {
-#pragma unroll
-            for (int a = 0; a < 2; ++a) tma_load_3d(dst + a * (D * 128), &tmV, ring_full(slot), (jb0 + j) * kKeys + a * 64, 0, bh);
-          }
+          request(slot, j, v, bh);
           armed |= 1u << slot;
           last_parity = (last_parity & ~(1u << slot)) | (phase << slot);
           if (++slot == NR) { slot = 0; phase ^= 1u; }
         }
+        first = 0;
       }
       if (!ok) {   // let every copy that was issued land before the shared memory is released
         const long long t0 = clock64();

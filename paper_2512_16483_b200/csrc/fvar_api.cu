@@ -1217,6 +1217,8 @@ static fvar_status scale_step_impl(fvar_ctx *ctx, const void *tokens, bool token
       {
         AttnArgs aa{E, H, r, D, L_prev + r, ctx->L_cap, bmul, boff, ctx->a, scale_log2, ctx->status, 1};
         aa.wait_cycles = ctx->wait_cycles;
+        aa.early_rows = L_prev;                      // the committed rows: written by earlier steps
+        aa.early_tiles = kEarlyTilesCache;
         attention_plan(E, H, r, L_prev + r, ctx->num_sms, &aa.tiles_per_cta, &aa.kv_splits);
         ctx->prof_begin(FVAR_KCLASS_ATTENTION, 4.0 * E * r * (L_prev + r) * C, 4.0 * E * (L_prev + r) * C + 4.0 * E * r * C);
         FV_CUDA(ctx, launch_attention(ctx->q_map, ctx->kmap[blk], ctx->vmap[blk], aa, ctx->num_sms, st), "attention");
@@ -1243,6 +1245,8 @@ static fvar_status scale_step_impl(fvar_ctx *ctx, const void *tokens, bool token
         if ((s = run_gemm(ctx, EPI_BF16, ctx->y_map, blk, W_CQ, gq, "cross q gemm")) != FVAR_OK) return s;
         AttnArgs aa{E, H, r, D, ctx->cfg.ctx_len, ctx->ctx_cap, bmul, boff, ctx->a, scale_log2, ctx->status, 1};
         aa.wait_cycles = ctx->wait_cycles;
+        aa.early_rows = ctx->ctx_cap;                // the context's: written by fvar_set_cond
+        aa.early_tiles = kEarlyTilesContext;
         attention_plan(E, H, r, ctx->cfg.ctx_len, ctx->num_sms, &aa.tiles_per_cta, &aa.kv_splits);
         ctx->prof_begin(FVAR_KCLASS_ATTENTION, 4.0 * E * r * ctx->cfg.ctx_len * C, 4.0 * E * ctx->cfg.ctx_len * C + 4.0 * E * r * C);
         FV_CUDA(ctx, launch_attention(ctx->q_map, ctx->ckmap[blk], ctx->cvmap[blk], aa, ctx->num_sms, st), "cross attention");

@@ -74,7 +74,8 @@ struct GemmArgs {
   float *partial;
   int *counters;
   unsigned *status;
-  // The weights' first stages are requested before the wait for the preceding kernel: no kernel that may still be in flight writes the weights.  0: they are requested after it.
+  // The weights' first stages are requested before the wait for the preceding kernel: no kernel that may still be in flight
+  // writes the weights.  0: they are requested after it.
   int w_early;
   // Weight-streaming form (gemm_skinny.cu; `splits` is then the cluster size): rows per column chunk, the padded
   // MMA width of a chunk, chunks (1 or 2) and pipeline stages -- filled by gemm_skinny_shape
@@ -166,9 +167,17 @@ struct AttnArgs {
   int kv_splits;
   int tiles_per_cta;       // 1: one 128-row query tile per CTA; otherwise two
   long long wait_cycles;   // budget of every bounded wait (0: the default)
+  // Tiles of 128 keys or values requested before the wait for the preceding kernel, of blocks that lie within the leading
+  // early_rows rows, which no kernel still in flight writes (0: none)
+  int early_rows, early_tiles;
   int units;               // without key ranges: query tile groups over all heads and elements, walked by the CTAs
   FastDiv div_nqt, div_h;  // unit -> (query tile group, head, element); filled by launch_attention
 };
+// How many such tiles pay.  The context's are few and wanted by few blocks: all that the ring takes (first scales of 800 and 1152
+// rows 5190 -> 5142 us, 16 rows 2577 -> 2558).  The cache's compete with the tail of the product before for the way from
+// memory: two (26 - 410 rows of 2048 columns 3491 -> 3469 us a step, one 3471, four 3481, ten 3486; 680 rows of 1024 columns 994 -> 973,
+// one 981, ten 981; 16 rows 2558 -> 2548, one 2554, ten 2560).
+constexpr int kEarlyTilesCache = 2, kEarlyTilesContext = 16;
 // Query tiles per CTA (1 or 2) and key ranges per launch (1 = no split; at most 6).
 void attention_plan(int B_eff, int H, int r, int L, int num_sms, int *tiles_per_cta, int *kv_splits);
 cudaError_t launch_attention(const CUtensorMap &tmQ, const CUtensorMap &tmK, const CUtensorMap &tmV,

@@ -416,7 +416,6 @@ template <int T>
 __global__ void __launch_bounds__(kLnThreads) finish_parts_kernel(GemmParts parts, int rows, int C, long long vec_stride, int bmul, int boff,
                                                                   float *__restrict__ out, RowMap omap, const int *__restrict__ scatter,
                                                                   bf16 *__restrict__ xsplit, int xsplit_mk) {
-  pdl_launch_dependents();
   const int e = blockIdx.x / rows, j = blockIdx.x - e * rows, n4 = C / 4, tid = threadIdx.x;
   float4 gate[T];
   uint2 bias[T];
@@ -428,6 +427,7 @@ __global__ void __launch_bounds__(kLnThreads) finish_parts_kernel(GemmParts part
     bias[t] = parts.bias ? __ldg(reinterpret_cast<const uint2 *>(parts.bias) + g) : make_uint2(0u, 0u);
   }
   pdl_wait();
+  pdl_launch_dependents();
   const int jo = scatter ? scatter[static_cast<long long>(e) * rows + j] : j;
   const float4 *xr = reinterpret_cast<const float4 *>(parts.xin + (static_cast<long long>(e * parts.inmap.bmul + parts.inmap.boff) * parts.inmap.rpb + j) * C);
   const float4 *pr = reinterpret_cast<const float4 *>(parts.part + static_cast<long long>(blockIdx.x) * C);
@@ -464,10 +464,14 @@ __global__ void __launch_bounds__(kLnThreads) finish_parts_kernel(GemmParts part
 }
 
 cudaError_t launch_finish_parts(const GemmParts &parts, int E, int rows, int C, long long vec_stride, int bmul, int boff, float *out, RowMap omap,
-                                const int *scatter, bf16 *xsplit, int xsplit_mk, cudaStream_t st) {
+                                const int *scatter, bf16 *xsplit, int xsplit_mk, bool at_join, cudaStream_t st) {
   if (E * rows <= 0) return cudaSuccess;
   if (C % 8 != 0 || C > 2048 || parts.splits < 1 || parts.splits > kMaxParts || parts.stride % 4 != 0) return cudaErrorInvalidValue;
   auto go = [&](auto kern) {
+    if (at_join) {
+      kern<<<dim3(E * rows), dim3(kLnThreads), 0, st>>>(parts, rows, C, vec_stride, bmul, boff, out, omap, scatter, xsplit, xsplit_mk);
+      return cudaGetLastError();
+    }
     return launch_pdl(kern, dim3(E * rows), dim3(kLnThreads), 0, st, parts, rows, C, vec_stride, bmul, boff, out, omap, scatter, xsplit, xsplit_mk);
   };
   if (C <= 512) return go(finish_parts_kernel<1>);

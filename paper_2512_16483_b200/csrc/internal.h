@@ -227,9 +227,11 @@ constexpr int kMaxParts = 4;
 cudaError_t launch_ln_parts(float *x, RowMap xmap, int E, int rows, int C, const GemmParts &parts, const float *shift, const float *scale,
                             long long vec_stride, int bmul, int boff, float eps, bf16 *y, cudaStream_t st);
 // No LayerNorm follows: row j of element e goes to row scatter[e][j] (j without scatter) of out, rows by omap, and as its
-// two-term bf16 split to xsplit (optional; see GemmArgs::xsplit).
+// two-term bf16 split to xsplit (optional; see GemmArgs::xsplit).  at_join: two branches of a graph meet at this launch.  It then
+// starts only when both have ended: its blocks, started early, would hold the SMs that the other branch may still need, and
+// blocks that let their own successor go before their wait would have that one queued in front of it.
 cudaError_t launch_finish_parts(const GemmParts &parts, int E, int rows, int C, long long vec_stride, int bmul, int boff, float *out, RowMap omap,
-                                const int *scatter, bf16 *xsplit, int xsplit_mk, cudaStream_t st);
+                                const int *scatter, bf16 *xsplit, int xsplit_mk, bool at_join, cudaStream_t st);
 // early: shift, scale and gamma are not written by any kernel that may still be in flight (they may then be read before
 // the preceding kernel has finished).
 cudaError_t launch_ln_modulate(const float *x, RowMap xmap, int E, int rows, int C, const float *shift,

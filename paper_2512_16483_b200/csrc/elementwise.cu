@@ -482,14 +482,19 @@ cudaError_t launch_finish_parts(const GemmParts &parts, int E, int rows, int C, 
 // ------------------------------------------------------------------------------------------------
 // Restoration fill: rows outside the index set take the bilinearly upsampled cached row
 // (half-pixel centres, source coordinate clamped at 0, neighbours clamped at the edge).
-// One warp per output row; rows inside the index set are skipped.
-__global__ void __launch_bounds__(256) rtr_fill_kernel(const float *__restrict__ prev, float *__restrict__ out, int E,
+// One warp per output row; rows inside the index set are skipped.  Bound by latency and by the map's way to
+// memory.  In a late step it runs beside the QKV product, whose blocks leave 11 K registers of an SM: four rows a block of at most 64
+// registers a thread fit beside it, eight of 56 waited for it to end and then held the SMs that the attention needs whole (a step
+// of 408 rows of 1920 columns 2112 -> 1994 us, of 2048 rows 7560 -> 7433, of 1632 rows of 1024 columns 1566 -> 1544; 40 registers spill:
+// 2106, 7670, 1625).  By itself 5.2 -> 4.8 us for 16 x 128 rows of 1024 columns.
+constexpr int kFillThreads = 128;
+__global__ void __launch_bounds__(kFillThreads, 8) rtr_fill_kernel(const float *__restrict__ prev, float *__restrict__ out, int E,
                                                        int bmul, int boff, int h0, int w0, int h1, int w1, int C,
                                                        const int *__restrict__ inv, bf16 *__restrict__ xsplit, int mk) {
   pdl_wait();
   pdl_launch_dependents();
   const int M1 = h1 * w1;
-  const long long gw = static_cast<long long>(blockIdx.x) * 8 + (threadIdx.x >> 5);
+  const long long gw = static_cast<long long>(blockIdx.x) * (kFillThreads / 32) + (threadIdx.x >> 5);
   if (gw >= static_cast<long long>(E) * M1) return;
   const int e = static_cast<int>(gw / M1), i = static_cast<int>(gw - static_cast<long long>(e) * M1);
   if (inv != nullptr && inv[static_cast<long long>(e) * M1 + i] >= 0) return;
@@ -529,7 +534,7 @@ cudaError_t launch_rtr_fill(const float *prev, float *out, int E, int bmul, int 
                             int C, const int *inv, bf16 *xsplit, int mk, cudaStream_t st) {
   const long long warps = static_cast<long long>(E) * h1 * w1;
   if (warps <= 0) return cudaSuccess;
-  return launch_pdl(rtr_fill_kernel, dim3(static_cast<unsigned>((warps + 7) / 8)), dim3(256), 0, st, prev, out, E, bmul, boff, h0, w0, h1, w1, C,
+  return launch_pdl(rtr_fill_kernel, dim3(static_cast<unsigned>((warps + kFillThreads / 32 - 1) / (kFillThreads / 32))), dim3(kFillThreads), 0, st, prev, out, E, bmul, boff, h0, w0, h1, w1, C,
                                                                          inv, xsplit, mk);
 }
 

@@ -552,6 +552,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       } else {
         // a unit with one tile uses both S buffers: its end is awaited, or the parity of the next wait would be ambiguous
         ok = __all_sync(0xffffffffu, mbar_wait(o_last(0), unit_bit, p.status, &abort_flag, wb));
+        final_ok = ok;
       }
       unit_bit ^= 1u;
       sbits ^= single || DUAL ? ((((nkv + 1) >> 1) & 1u) | (((nkv >> 1) & 1u) << 1)) : ((nkv & 1) ? 3u : 0u);
@@ -574,14 +575,17 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     cluster_sync_all();                                            // nobody's ring is in use any more
     if (warp >= kSoftmaxWarp && final_ok) {
       tc_fence_after();
-      const int t = (warp - kSoftmaxWarp) >> 2, row = (warp & 3) * 32 + lane, rpr = t == 0 ? rpr0 : rpr1;
+      // a lone tile is shared by both warp-groups, half of the columns each (with the merge below: a step of 26 - 410 rows
+      // of 2048 columns 3470 -> 3449 us, of 16 rows 2550 -> 2529)
+      const int wg = (warp - kSoftmaxWarp) >> 2, t = x.ntiles > 1 ? wg : 0, row = (warp & 3) * 32 + lane, rpr = t == 0 ? rpr0 : rpr1;
+      const int half = x.ntiles > 1 ? D / 32 : D / 64, cc0 = x.ntiles > 1 ? 0 : wg * half;
       const uint32_t o_addr = tmem_base + 256 + t * D + (static_cast<uint32_t>((warp & 3) * 32) << 16);
       const bool mine = x.q0 + t * kQRows + row < p.r;
       const int owner = mine ? row / rpr : 0, slot = (t == 0 ? 0 : splits * rpr0) + sp * rpr + row - owner * rpr;
       const uint32_t dst = mapa_shared(part_o + static_cast<uint32_t>(slot) * kPitch, static_cast<uint32_t>(owner));
       const uint32_t dst_m = mapa_shared(part_m + static_cast<uint32_t>(slot) * 8u, static_cast<uint32_t>(owner));
 #pragma unroll 1
-      for (int cc = 0; cc < D / 32; ++cc) {
+      for (int cc = cc0; cc < cc0 + half; ++cc) {
         uint32_t v[32];
         tmem_ld32(o_addr + cc * 32, v);
         tmem_ld_wait();
@@ -592,7 +596,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                          "r"(v[q * 4 + 2]), "r"(v[q * 4 + 3]) : "memory");
         }
       }
-      if (mine) asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(dst_m), "f"(m_ref), "f"(l_run) : "memory");
+      if (mine && t == wg) asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(dst_m), "f"(m_ref), "f"(l_run) : "memory");
     }
     tc_fence_before();
     cluster_sync_all();                                            // all rows have arrived; nobody touches a peer after this
@@ -600,24 +604,35 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       constexpr int G = D / 4;                                     // threads per row, one float4 each
       const int st = static_cast<int>(threadIdx.x) - 32 * kSoftmaxWarp, d4 = (st % G) * 4;
       const float c = p.scale_log2;
-      for (int k = st / G; k < rpr0 + rpr1; k += 256 / G) {
+#pragma unroll 1
+      for (int k0 = 0; k0 < rpr0 + rpr1; k0 += 256 / G) {            // every lane of a warp goes round as often
+        const bool there = k0 + st / G < rpr0 + rpr1;
+        const int k = there ? k0 + st / G : 0;
         const int tt = k < rpr0 ? 0 : 1, lrow = tt == 0 ? k : k - rpr0, rpr = tt == 0 ? rpr0 : rpr1;
         const int rib = x.q0 + tt * kQRows + sp * rpr + lrow;
-        if (rib >= p.r || sp * rpr + lrow >= kQRows) continue;
+        const bool live = there && rib < p.r && sp * rpr + lrow < kQRows;
         const uint32_t slot0 = static_cast<uint32_t>((tt == 0 ? 0 : splits * rpr0) + lrow);
-        float m_all = -INFINITY;
-        for (int t2 = 0; t2 < splits; ++t2) m_all = fmaxf(m_all, ld_shared_f2(part_m + (slot0 + t2 * rpr) * 8u).x);
-        float l_all = 0.f;
+        // A lane of the row's threads takes one range's maximum and sum; the weights are formed side by side and handed round
+        // (eight ranges at most), and the sum is the same whatever the timing.  One range after another in every thread, in two
+        // passes, was a chain of 640 clocks a row.  Code that runs once a launch has to be short: two rows a round cost
+        // 1.2 us of a 21 us launch instead of gaining.
+        const int l8 = st & 7;
+        const float2 ml = l8 < splits ? ld_shared_f2(part_m + (slot0 + l8 * rpr) * 8u) : make_float2(-INFINITY, 0.f);
+        float m_all = ml.x;
+#pragma unroll
+        for (int o2 = 4; o2 > 0; o2 >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xffffffffu, m_all, o2));
+        float w8 = exp2f((ml.x - m_all) * c), l_all = ml.y * w8;
+#pragma unroll
+        for (int o2 = 4; o2 > 0; o2 >>= 1) l_all += __shfl_xor_sync(0xffffffffu, l_all, o2);
+        w8 *= 1.0f / l_all;
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int t2 = 0; t2 < splits; ++t2) {                      // range order: the sum does not depend on timing
-          const float2 ml = ld_shared_f2(part_m + (slot0 + t2 * rpr) * 8u);
+        for (int t2 = 0; t2 < splits; ++t2) {
+          const float w = __shfl_sync(0xffffffffu, w8, t2, 8);
           const float4 v = ld_shared_f4(part_o + (slot0 + t2 * rpr) * kPitch + d4 * 4);
-          const float w = exp2f((ml.x - m_all) * c);
-          l_all = fmaf(ml.y, w, l_all);
           o.x = fmaf(w, v.x, o.x); o.y = fmaf(w, v.y, o.y); o.z = fmaf(w, v.z, o.z); o.w = fmaf(w, v.w, o.w);
         }
-        const float inv_l = 1.0f / l_all;
-        __nv_bfloat162 h0 = __floats2bfloat162_rn(o.x * inv_l, o.y * inv_l), h1 = __floats2bfloat162_rn(o.z * inv_l, o.w * inv_l);
+        if (!live) continue;
+        __nv_bfloat162 h0 = __floats2bfloat162_rn(o.x, o.y), h1 = __floats2bfloat162_rn(o.z, o.w);
         *reinterpret_cast<uint2 *>(p.out + (static_cast<long long>(x.e) * p.r + rib) * (p.H * D) + x.h * D + d4) =
             make_uint2(*reinterpret_cast<uint32_t *>(&h0), *reinterpret_cast<uint32_t *>(&h1));
       }

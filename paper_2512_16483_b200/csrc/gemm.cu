@@ -233,7 +233,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       auto col_of = [&](int ci) { return n_idx * BN + (ci * kEpiColGroups + cg) * 32; };
       auto in_tile = [&](int ci) { return (ci * kEpiColGroups + cg) * 32 < BN && col_of(ci) < p.N; };    // uniform across the warp
       if constexpr (EPI == EPI_RESID) {
-        rr = resid_row(p, row);
+        rr = resid_row(p, row, p.R);
         if (splits == 1) {
 #pragma unroll
         for (int ci = 0; ci < kPre; ++ci)
@@ -399,7 +399,7 @@ GemmPlan gemm_plan(int R, int nbatch, int N, int K, int num_sms, int max_cluster
   }
   // The free-width form has to be clearly ahead, as full tiles are level; up to 32 rows its narrowest tile is half padding.
   if (flex && R > 32) {
-    for (int nb = 64; nb <= 256; nb += 32) {
+    for (int nb = 64; nb <= 256; nb += 16) {
       const float t = 0.098f + 0.00077f * nb < 0.155f ? 0.155f : 0.098f + 0.00077f * nb;
       const float c = 2.0f + 0.019f * nb + work(static_cast<long long>((N + 2 * kBlockM - 1) / (2 * kBlockM)) * ((R + nb - 1) / nb), t, 1.28f);
       if (c < 0.97f * best) { best = c / 0.97f; plan = GemmPlan{kGemmFlex, nb, 1}; }

@@ -171,9 +171,9 @@ __device__ __forceinline__ void epilogue_chunk(const GemmArgs &p, const uint32_t
 struct ResidRow {
   int out, res, b, split;      // output row (-1: past the end), residual row, caller batch element, row of the hi half
 };
-__device__ __forceinline__ ResidRow resid_row(const GemmArgs &p, int row) {
+__device__ __forceinline__ ResidRow resid_row(const GemmArgs &p, int row, int row_end) {
   ResidRow r{-1, 0, 0, 0};
-  if (row < p.R) {
+  if (row < row_end) {
     const int e = row / p.rows_per_batch, j = row - e * p.rows_per_batch;
     const int jo = p.scatter ? __ldg(p.scatter + static_cast<long long>(e) * p.rows_per_batch + j) : j;
     r.b = e * p.bmul + p.boff;

@@ -1,7 +1,7 @@
 // GEMM on CTA pairs with a free tile width along the rows, sm_100a: out[R][N] = A[R][K] * W[N][K]^T.
 //
 // The weights are the M side of the MMA -- a pair of CTAs owns 256 output features, 128 each -- and a chunk of the rows,
-// any multiple of 32 up to 256, is the N side.  With the roles that way round the row count of a step, which is whatever
+// any multiple of 16 up to 256, is the N side.  With the roles that way round the row count of a step, which is whatever
 // rank or batch asks for, costs no padding to 256, and the chunk width is free to make the number of tiles match the 74
 // pairs of the chip.
 //
@@ -9,8 +9,11 @@
 // 64 of K and wave; a launch adds 2 us of set-up and first operands and 0.019 * width us of the last tile's epilogue.
 // Against the best of the pairs of 256 rows (us, rows x features x K, launched through the kernel-level entry, which
 // requests no weights early): 400 x 6144 x 2048 16.6 -> 13.9 with 160 rows a tile, 72 tiles; 283 x 8192 x 2048 16.9 -> 13.9;
-// 680 x 4096 x 1024 10.8 -> 10.3; 2704 x 1024 x 1024 10.6 -> 9.5; 2704 x 1024 x 4096 25.6 -> 20.8; full tiles are level.  Spreading the K range of a tile over a cluster of pairs was built and left out:
+// 680 x 4096 x 1024 10.8 -> 10.3; 2704 x 1024 x 1024 10.6 -> 9.5; 2704 x 1024 x 4096 25.6 -> 20.8; full tiles are level.  Multiples of 16 and not of 32 only (410 rows as two of 208 instead of 224,
+// or three of 144 instead of 160) are worth 1.2 % of such a step: 3455 -> 3414 us, 408 rows 4015 -> 3951.  Spreading the K range of a tile over a cluster of pairs was built and left out:
 // its reduction costs 4 - 6 us, 400 x 2048 x 8192 took 22.5 us against 21.7 of 128 x 128 tiles split the same way.
+//
+// The epilogue takes 32 rows at a time; what lies past the tile's end in its last chunk is the next tile's and not stored.
 //
 // Roles per CTA: warp 0 feeds the stage ring with TMA (cta_group::2: the bytes of both CTAs are counted on the barrier of
 // the pair's even CTA), warp 1 of the even CTA issues the MMAs into one of two TMEM accumulators, warps 2-9 drain the
@@ -185,7 +188,7 @@ gemm_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       const int ft = tile / chunks, ch = tile - ft * chunks;
       const int a = it & 1, n0 = (2 * ft + static_cast<int>(half)) * kBlockM + quad * 32;
       const int row0 = ch * nb, rows = min(nb, p.R - row0);
-      RowsEpilogue<EPI> ep(p, n0, ep_stage, lane, range);
+      RowsEpilogue<EPI> ep(p, n0, ep_stage, lane, range, row0 + rows);
       // EPI_RESID: what the first PRE chunks read besides their sums is requested while the main loop runs (with one tile
       // a CTA nothing else hides it), the later ones' PRE ahead
       typename RowsEpilogue<EPI>::Fetch fetch[PRE];
@@ -275,7 +278,7 @@ void gemm_flex_shape(GemmArgs &a) {
 int gemm_partial_plan(int R, int N, int K, int max_clusters, int *rows_tile) {
   const int chunks = (R + 255) / 256, num_kb = K / kBlockK, tiles = (N + 2 * kBlockM - 1) / (2 * kBlockM) * chunks;
   if (chunks < 2 || chunks > 4 || N > 2048 || K < 4096 || K % kBlockK != 0 || !gemm_flex_supported(EPI_PARTIAL, N, K)) return 0;
-  *rows_tile = ((R + chunks - 1) / chunks + 31) / 32 * 32;
+  *rows_tile = ((R + chunks - 1) / chunks + 15) / 16 * 16;
   if (chunks == 4 && *rows_tile > 224) return 0;
   for (int s = kMaxParts; s >= 3; --s)
     if (num_kb % (2 * s) == 0 && tiles * s <= max_clusters) return 5 * tiles * s >= 3 * max_clusters ? s : 0;
@@ -309,7 +312,7 @@ static cudaError_t flex_launch_one(const CUtensorMap &tmA, const CUtensorMap &tm
 // with a.fx_nk K blocks.  max_clusters: resident CTA pairs (gemm_pair_max_clusters).
 cudaError_t launch_gemm_flex(int epi, const CUtensorMap &tmA, const CUtensorMap &tmW, const GemmArgs &a, int max_clusters, cudaStream_t st) {
   if (a.nbatch != 1 || a.w_mn_major || (a.splits > 1 && epi != EPI_PARTIAL) || a.splits < 0 || a.R <= 0 || !gemm_flex_supported(epi, a.N, a.K) || a.fx_nb < 32 || a.fx_nb > 256 ||
-      a.fx_nb % 32 || a.fx_stages < 2 || max_clusters <= 0)
+      a.fx_nb % 16 || a.fx_stages < 2 || max_clusters <= 0)
     return cudaErrorInvalidValue;
   switch (epi) {
     case EPI_F32: return flex_launch_one<EPI_F32, 1>(tmA, tmW, a, max_clusters, st);

@@ -203,7 +203,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       auto col_of = [&](int ci) { return n_idx * BN + (ci * kEpiColGroups + cg) * 32; };
       auto in_tile = [&](int ci) { return (ci * kEpiColGroups + cg) * 32 < BN && col_of(ci) < p.N; };    // uniform across the warp
       if constexpr (EPI == EPI_RESID) {
-        rr = resid_row(p, row);
+        rr = resid_row(p, row, p.R);
 #pragma unroll
         for (int ci = 0; ci < kPre; ++ci)
           if (in_tile(ci)) resid_fetch(p, rr, col_of(ci), lane, pre[ci]);

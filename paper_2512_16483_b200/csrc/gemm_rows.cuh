@@ -109,9 +109,10 @@ struct RowsEpilogue {
   const int n0, lane;
   const uint32_t stage;                // 32 x 132 bytes of shared memory of this warp
   const int range;                     // EPI_PARTIAL: K range
+  const int row_end;                   // first row that is not this tile's
   float bias;                          // of this lane's feature
-  __device__ __forceinline__ RowsEpilogue(const GemmArgs &args, int first_feature, uint32_t stage_addr, int l, int k_range)
-      : p(args), n0(first_feature), lane(l), stage(stage_addr), range(k_range) {
+  __device__ __forceinline__ RowsEpilogue(const GemmArgs &args, int first_feature, uint32_t stage_addr, int l, int k_range, int end_row)
+      : p(args), n0(first_feature), lane(l), stage(stage_addr), range(k_range), row_end(end_row) {
     bias = (p.bias != nullptr && n0 < p.N) ? __bfloat162float(p.bias[n0 + lane]) : 0.f;
   }
   // What the chunk of rows `row0` .. row0 + 31 reads besides its sums (EPI_RESID).
@@ -121,7 +122,7 @@ struct RowsEpilogue {
   };
   __device__ __forceinline__ void prefetch(int row0, Fetch &f) const {
     if constexpr (EPI == EPI_RESID) {
-      f.rr = resid_row(p, row0 + lane);
+      f.rr = resid_row(p, row0 + lane, row_end);
       resid_fetch(p, f.rr, n0, lane, f.pre);
     }
   }
@@ -134,7 +135,7 @@ struct RowsEpilogue {
         asm volatile("st.shared.f32 [%0], %1;" ::"r"(stage + i * 132 + lane * 4), "f"(__uint_as_float(acc[i]) + bias) : "memory");
       __syncwarp();
       const int row = row0 + lane;
-      if (row < p.R) {
+      if (row < row_end) {
         const int e = row / p.rows_per_batch, j = row - e * p.rows_per_batch, b = e * p.bmul + p.boff;
         const int c = vc0 - 2 * p.C, h = c / p.D, d0 = c - h * p.D;
         bf16 *dst = p.vt + ((static_cast<long long>(b) * p.H + h) * p.D + d0) * p.L_cap + p.L_prev + j;
@@ -174,16 +175,16 @@ struct RowsEpilogue {
         resid_store(p, f.rr, o, f.pre, it, r, n);
       } else if constexpr (EPI == EPI_F32 || EPI == EPI_PARTIAL) {
         const int at = EPI == EPI_PARTIAL ? range * p.R + row : row;
-        if (row < p.R) *reinterpret_cast<float4 *>(p.out_f32 + static_cast<long long>(at) * p.ld_out + n) = o;
+        if (row < row_end) *reinterpret_cast<float4 *>(p.out_f32 + static_cast<long long>(at) * p.ld_out + n) = o;
       } else if constexpr (EPI == EPI_QKV) {
         const int ko = __shfl_sync(0xffffffffu, k_off, r);
-        if (row < p.R) {
+        if (row < row_end) {
           bf16 *dst = vc0 < p.C ? p.out_bf16 + static_cast<long long>(row) * p.ld_out + vc
                                 : p.kc + (static_cast<long long>(ko) + static_cast<long long>(hk) * p.L_cap) * p.D + dk;
           *reinterpret_cast<uint2 *>(dst) = pack4_bf16(o.x, o.y, o.z, o.w);
         }
       } else {
-        if (row < p.R) *reinterpret_cast<uint2 *>(p.out_bf16 + static_cast<long long>(row) * p.ld_out + n) = pack4_bf16(o.x, o.y, o.z, o.w);
+        if (row < row_end) *reinterpret_cast<uint2 *>(p.out_bf16 + static_cast<long long>(row) * p.ld_out + n) = pack4_bf16(o.x, o.y, o.z, o.w);
       }
     }
     __syncwarp();

@@ -81,7 +81,7 @@ struct GemmArgs {
   // MMA width of a chunk, chunks (1 or 2) and pipeline stages -- filled by gemm_skinny_shape
   int sk_rows_chunk, sk_rp, sk_nchunks, sk_stages, sk_small, sk_nk;
   int sk_tiles_m;          // > 0: the 128 x 128-tile mode of that kernel with this many row tiles (rows on the M side)
-  // CTA-pair form with a free row width (gemm_flex.cu): rows of a tile (a multiple of 32 up to 256), K blocks per
+  // CTA-pair form with a free row width (gemm_flex.cu): rows of a tile (a multiple of 16 up to 256), K blocks per
   // pipeline stage, stages
   int fx_nb, fx_nk, fx_stages;
   // EPI_PARTIAL (that form only): `splits` K ranges of whole stages, each one's sums [R][ld_out] fp32 (no bias) at

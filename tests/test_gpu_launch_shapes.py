@@ -99,6 +99,7 @@ def test_down_in_both_forms(fv, C, hw, B):
     (33, 64, 64, 32), (400, 192, 2048, 160), (400, 6144, 200, 224),     # half a feature tile, a remainder of one, K not whole blocks
     (255, 1920, 1920, 64), (257, 1920, 128, 256), (1, 256, 4096, 0),    # an odd number of 128-feature halves, one row past a tile
     (5000, 320, 136, 96), (2704, 1024, 1024, 0), (97, 8192, 2048, 0),   # several tiles a pair, the picked widths
+    (410, 8192, 2048, 0), (410, 6144, 2048, 0), (283, 6144, 2048, 0), (79, 8192, 2048, 0), (3000, 1920, 1920, 0),   # picked: multiples of 16 among them
 ])
 def test_gemm_free_width_pairs(fv, R, N, K, width):
     g = torch.Generator(device="cuda").manual_seed(R + N + K)

@@ -741,10 +741,9 @@ static cudaError_t launch_d(const CUtensorMap &tmQ, const CUtensorMap &tmK, cons
   attr[0].val.clusterDim.x = a.kv_splits;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  attr[1] = pdl_attribute();
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = one_predecessor(st) ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, attention_kernel<D, kRanges, false>, tmQ, tmK, tmV, a);
 }
 

@@ -464,14 +464,10 @@ __global__ void __launch_bounds__(kLnThreads) finish_parts_kernel(GemmParts part
 }
 
 cudaError_t launch_finish_parts(const GemmParts &parts, int E, int rows, int C, long long vec_stride, int bmul, int boff, float *out, RowMap omap,
-                                const int *scatter, bf16 *xsplit, int xsplit_mk, bool at_join, cudaStream_t st) {
+                                const int *scatter, bf16 *xsplit, int xsplit_mk, cudaStream_t st) {
   if (E * rows <= 0) return cudaSuccess;
   if (C % 8 != 0 || C > 2048 || parts.splits < 1 || parts.splits > kMaxParts || parts.stride % 4 != 0) return cudaErrorInvalidValue;
   auto go = [&](auto kern) {
-    if (at_join) {
-      kern<<<dim3(E * rows), dim3(kLnThreads), 0, st>>>(parts, rows, C, vec_stride, bmul, boff, out, omap, scatter, xsplit, xsplit_mk);
-      return cudaGetLastError();
-    }
     return launch_pdl(kern, dim3(E * rows), dim3(kLnThreads), 0, st, parts, rows, C, vec_stride, bmul, boff, out, omap, scatter, xsplit, xsplit_mk);
   };
   if (C <= 512) return go(finish_parts_kernel<1>);

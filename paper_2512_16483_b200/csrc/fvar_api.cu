@@ -1294,7 +1294,7 @@ static fvar_status scale_step_impl(fvar_ctx *ctx, const void *tokens, bool token
           if (last && (late || g + 1 == G || rank[g + 1] < M)) {
             FV_CUDA(ctx, join(), "join wait");
             ctx->prof_begin(FVAR_KCLASS_CONVERT, 0.0, 4.0 * R * C * (ranges + 2) + (ga.xsplit ? 4.0 * R * C : 0.0));
-            FV_CUDA(ctx, launch_finish_parts(parts, E, r, C, 6 * C, bmul, boff, ga.out_f32, ga.omap, ga.scatter, ga.xsplit, ga.xsplit_mk, to_group && forked, st), "fc2 sums");
+            FV_CUDA(ctx, launch_finish_parts(parts, E, r, C, 6 * C, bmul, boff, ga.out_f32, ga.omap, ga.scatter, ga.xsplit, ga.xsplit_mk, st), "fc2 sums");
             ctx->launched();
             parts.splits = 0;
           }

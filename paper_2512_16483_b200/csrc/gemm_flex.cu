@@ -301,10 +301,9 @@ static cudaError_t flex_launch_one(const CUtensorMap &tmA, const CUtensorMap &tm
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  attr[1] = pdl_attribute();
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = one_predecessor(st) ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, gemm_flex_kernel<EPI, PRE>, tmA, tmW, a);
 }
 

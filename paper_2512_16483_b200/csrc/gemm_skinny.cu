@@ -400,10 +400,9 @@ static cudaError_t skinny_launch_one(const CUtensorMap &tmA, const CUtensorMap &
   attr[0].val.clusterDim.x = S;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  attr[1] = pdl_attribute();
   cfg.attrs = attr;
-  cfg.numAttrs = a.w_early ? 2 : 1;      // the kernel requests weights before its wait: else it starts when its predecessor has ended
+  cfg.numAttrs = a.w_early && one_predecessor(st) ? 2 : 1;      // the kernel requests weights before its wait: else it starts when its predecessor has ended
   return cudaLaunchKernelEx(&cfg, gemm_skinny_kernel<EPI, ROWS>, tmA, tmW, a);
 }
 

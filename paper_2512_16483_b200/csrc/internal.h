@@ -183,7 +183,35 @@ void attention_plan(int B_eff, int H, int r, int L, int num_sms, int *tiles_per_
 cudaError_t launch_attention(const CUtensorMap &tmQ, const CUtensorMap &tmK, const CUtensorMap &tmV,
                              const AttnArgs &a, int num_sms, cudaStream_t st);
 
-// Launch with programmatic stream serialization (see pdl_wait in ptx.cuh).
+// Every launch allows programmatic stream serialization (see pdl_wait in ptx.cuh) except one at which branches of a capture
+// meet.  Capture gives a launch that allows it a programmatic edge from each kernel that it depends on (read back from the
+// step's graphs), and what is documented of an early start concerns one such kernel.  A launch that started when the first of
+// several lets it would hold, until the others have ended, SMs that the others may not have got yet, and that wait is not
+// bounded.  So with several dependencies the launch is an ordinary one, whose edges are full: it starts when all of them have
+// ended.  In the step these are, in every late group, the launch before which the branches meet and the first of the side branch
+// (whose stream still hangs on the side branch of the group before).  A step takes as long as with early starts there: 680 rows
+// of 1024 columns 975 us both ways, 2048 rows of 1920 columns 7418 and 7425 (0.5 % between runs), the table's ranks at 40 x 40 3411 and 3408; its first pass
+// takes 45 us a group of one block longer, and 30 a group of four, for instantiating the graph.  To hang the side branch on its fork alone, so that
+// it may start early, is slower: 1031 us, and 3430.
+inline bool one_predecessor(cudaStream_t st) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  cudaGraph_t graph = nullptr;
+  const cudaGraphNode_t *deps = nullptr;
+  const cudaGraphEdgeData *edges = nullptr;
+  size_t n = 0;
+  if (cudaStreamGetCaptureInfo_v3(st, &status, &id, &graph, &deps, &edges, &n) != cudaSuccess) {
+    cudaGetLastError();                      // the launch itself will say what is wrong
+    return true;
+  }
+  return status != cudaStreamCaptureStatusActive || n <= 1;
+}
+inline cudaLaunchAttribute pdl_attribute() {
+  cudaLaunchAttribute a = {};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  return a;
+}
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args) {
   cudaLaunchConfig_t cfg = {};
@@ -191,11 +219,9 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute attr = pdl_attribute();
+  cfg.attrs = &attr;
+  cfg.numAttrs = one_predecessor(st) ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
@@ -227,11 +253,9 @@ constexpr int kMaxParts = 4;
 cudaError_t launch_ln_parts(float *x, RowMap xmap, int E, int rows, int C, const GemmParts &parts, const float *shift, const float *scale,
                             long long vec_stride, int bmul, int boff, float eps, bf16 *y, cudaStream_t st);
 // No LayerNorm follows: row j of element e goes to row scatter[e][j] (j without scatter) of out, rows by omap, and as its
-// two-term bf16 split to xsplit (optional; see GemmArgs::xsplit).  at_join: two branches of a graph meet at this launch.  It then
-// starts only when both have ended: its blocks, started early, would hold the SMs that the other branch may still need, and
-// blocks that let their own successor go before their wait would have that one queued in front of it.
+// two-term bf16 split to xsplit (optional; see GemmArgs::xsplit).
 cudaError_t launch_finish_parts(const GemmParts &parts, int E, int rows, int C, long long vec_stride, int bmul, int boff, float *out, RowMap omap,
-                                const int *scatter, bf16 *xsplit, int xsplit_mk, bool at_join, cudaStream_t st);
+                                const int *scatter, bf16 *xsplit, int xsplit_mk, cudaStream_t st);
 // early: shift, scale and gamma are not written by any kernel that may still be in flight (they may then be read before
 // the preceding kernel has finished).
 cudaError_t launch_ln_modulate(const float *x, RowMap xmap, int E, int rows, int C, const float *shift,

@@ -160,3 +160,60 @@ def test_gemm_waits_for_a_weight_that_the_call_before_writes(fv, form, R, N, K):
         del W
         assert (out.double() - ref).abs().max() <= bound, s
     assert fv.kernel_poll_status() == fv.OK
+
+
+def _join_calls(fv):
+    """Every way the library launches a kernel, as calls on the current stream."""
+    g = torch.Generator(device="cuda").manual_seed(3)
+    def rnd(*shape): return torch.randn(shape, generator=g, device="cuda")
+    A, W = {R: rnd(R, 512).bfloat16() for R in (16, 200)}, rnd(256, 512).bfloat16()
+    x, vec, prev, pair = rnd(2, 64, 256), rnd(2, 256), rnd(2, 16, 256), rnd(2, 64, 256).bfloat16()
+    scores, out = rnd(2, 64), rnd(2, 64, 256)
+    def attn(r, L):
+        q, K, Vt = rnd(1, r, 128).bfloat16(), rnd(1, 1, L, 128).bfloat16(), rnd(1, 1, 128, L).bfloat16()
+        return lambda: fv.fvar_attention(q, K, Vt, L)
+    calls = {"form %s" % f: (lambda f=f, R=R: fv.fvar_gemm_bf16_form(A[R], W, None, getattr(fv, f), 0))
+             for f, R in (("GEMM_SINGLE", 200), ("GEMM_PAIR", 200), ("GEMM_SKINNY", 16), ("GEMM_KSPLIT", 200), ("GEMM_FLEX", 200))}
+    return dict(calls, attention=attn(64, 128), ranges=attn(16, 4096), scores=lambda: fv.fvar_row_scores(x), select=lambda: fv.fvar_select_topr(scores, 9)[0],
+                ln=lambda: fv.fvar_ln_modulate(x, vec, vec, 1e-6), fill=lambda: fv.fvar_rtr_fill(prev, (4, 4), (8, 8), None, out),
+                combine=lambda: fv.fvar_cfg_combine(pair, 2.0))
+
+
+def _edge_types(graph):
+    """{(from, to): type} of a captured graph; type 1 is a programmatic edge, 0 a full one."""
+    import ctypes as ct
+
+    class Edge(ct.Structure):
+        _fields_ = [("from_port", ct.c_ubyte), ("to_port", ct.c_ubyte), ("type", ct.c_ubyte), ("reserved", ct.c_ubyte * 5)]
+    ask, g, n = ct.CDLL("libcuda.so.1").cuGraphGetEdges_v2, ct.c_void_p(graph.raw_cuda_graph()), ct.c_size_t(0)
+    assert ask(g, None, None, None, ct.byref(n)) == 0
+    fr, to, data = (ct.c_void_p * n.value)(), (ct.c_void_p * n.value)(), (Edge * n.value)()
+    assert ask(g, fr, to, data, ct.byref(n)) == 0
+    return {(a, b): e.type for a, b, e in zip(fr, to, data)}
+
+
+def test_a_launch_where_branches_of_a_capture_meet_waits_for_all_of_them(fv):
+    """A kernel that depends on several others starts when they have ended; one that follows a single kernel may start
+    early.  The step's own graphs are captured through the same launches."""
+    x, pair = torch.randn(2, 64, 256, device="cuda"), torch.randn(2, 64, 256, device="cuda").bfloat16()
+    for name, call in _join_calls(fv).items():
+        ref = call().clone()
+        fv.fvar_row_scores(x), fv.fvar_cfg_combine(pair, 1.0)
+        main, side, graph = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.CUDAGraph(keep_graph=True)
+        with torch.cuda.graph(graph, stream=main):
+            keep = [fv.fvar_row_scores(x)]
+            side.wait_stream(main)
+            with torch.cuda.stream(side):
+                keep += [fv.fvar_cfg_combine(pair, 1.0)]
+            keep += [fv.fvar_cfg_combine(pair, 1.0)]
+            main.wait_stream(side)
+            got = call()
+        edges = _edge_types(graph)
+        last = [b for _, b in edges]
+        meet = [t for (_, b), t in edges.items() if last.count(b) > 1]
+        assert meet == [0, 0], (name, edges)
+        assert [t for (_, b), t in edges.items() if last.count(b) == 1] == [1, 1], (name, edges)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(got, ref), name
+    assert fv.kernel_poll_status() == fv.OK

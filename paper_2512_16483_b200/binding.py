@@ -7,6 +7,7 @@ built (python -m paper_2512_16483_b200.build) -- there is no fallback path.
 from __future__ import annotations
 
 import ctypes as ct
+import importlib
 import os
 from typing import Dict, List, Optional, Sequence
 
@@ -122,18 +123,24 @@ def load_library() -> ct.CDLL:
     for name, (res, args) in sigs.items():
         fn = getattr(lib, name)
         fn.restype, fn.argtypes = res, args
-    global _calls
-    try:
-        from . import _calls as calls
-    except ImportError as e:
-        raise FileNotFoundError("the library's call layer is not built: run `python -m paper_2512_16483_b200.build`") from e
-    _lib, _calls = lib, calls
+    _lib = lib
     return lib
 
 
 def _native():
+    """The call layer (_calls.so).  It is built against one torch; the library itself, which is not, loads without it."""
+    global _calls
     if _calls is None:
         load_library()
+        again = "run `python -m paper_2512_16483_b200.build`"
+        try:
+            _calls = importlib.import_module("._calls", __package__)
+        except ImportError as e:
+            from . import build
+            if not os.path.exists(build.CALLS):
+                raise FileNotFoundError("the library's call layer _calls.so is not built: " + again) from e
+            raise ImportError("the library's call layer _calls.so does not load (%s); it is a %s, this is torch %s: %s" % (
+                e, build.calls_built_for() or "call layer of an unknown torch", torch.__version__, again)) from e
     return _calls
 
 

@@ -20,6 +20,9 @@
 
 #include "../../include/fvar.h"
 
+// Read from the file by build.py: the symbols below are those of one torch and one Python.
+extern "C" __attribute__((used)) const char fvar_calls_built_for[] = FVAR_BUILT_FOR;
+
 namespace {
 
 bool modes_active() { return at::impl::torch_function_mode_enabled() || c10::impl::TorchDispatchModeTLS::any_modes_set(); }

@@ -30,6 +30,39 @@ def test_library_builds_loads_and_exports_every_declared_symbol():
     assert sorted(binding.EXPORTED) == names
 
 
+def test_library_loads_without_its_call_layer(monkeypatch):
+    """The call layer is built against torch.  Where it does not load, the error names the reason, and what needs no
+    tensors works."""
+    import sys
+    from paper_2512_16483_b200 import binding
+    fbuild.build()
+    monkeypatch.setattr(binding, "_lib", None)
+    monkeypatch.setattr(binding, "_calls", None)
+    monkeypatch.delattr("paper_2512_16483_b200._calls", raising=False)
+    monkeypatch.setitem(sys.modules, "paper_2512_16483_b200._calls", None)       # its import fails
+    assert schedule.rank_from_keep_ratio(169, 0.5) == 85
+    assert hasattr(binding.load_library(), "fvar_scale_step")
+    with pytest.raises(ImportError) as e:
+        binding._native()
+    assert str(e.value.__cause__) in str(e.value) and "torch" in str(e.value)
+    monkeypatch.setattr(fbuild, "CALLS", fbuild.CALLS + ".missing")
+    with pytest.raises(FileNotFoundError, match="not built"):
+        binding._native()
+
+
+def test_call_layer_of_another_torch_is_stale(monkeypatch):
+    """After torch or Python is replaced the sources are no newer than the call layer, which has to be built anew all the same."""
+    fbuild.build()
+    assert not fbuild._calls_stale() and not fbuild._lib_stale()
+    assert fbuild.calls_built_for() == fbuild._built_for()
+    built = []
+    monkeypatch.setattr(fbuild, "_built_for", lambda: "fvar call layer for torch 0.0, Python 0.0")
+    monkeypatch.setattr(fbuild, "_compile_calls", lambda: built.append("calls"))
+    monkeypatch.setattr(fbuild, "_build_lib", lambda: built.append("library"))
+    fbuild.build()
+    assert built == ["calls"]
+
+
 def test_workspace_bytes_and_bad_shapes_without_gpu():
     import ctypes as ct
     from paper_2512_16483_b200 import binding

@@ -398,11 +398,24 @@ GemmPlan gemm_plan(int R, int nbatch, int N, int K, int num_sms, int max_cluster
     }
   }
   // The free-width form has to be clearly ahead, as full tiles are level; up to 32 rows its narrowest tile is half padding.
+  // Widths: multiples of 32, each cut down to the multiple of 16 that its number of chunks still needs (up to 6 % of a launch:
+  // 400 x 8192 x 2048 208 rows a tile 15.3 us, 224 16.3), besides 208, the widest with six stages, and 176 for short sums.  Any
+  // other multiple of 16 makes more chunks than the next of 32 and loses or gains nothing: 648 x 2048 x 2048 80 rows a tile 10.8 us, 96 10.3; 1224 x 2048 x
+  // 8192 144 37.8, 160 36.8; a step of 2048 rows of 1920 columns with 240 7258, with the pairs of 256 that it fills 7187.
+  // Above 96 rows a stage is one K block instead of two, and 112 rows take what 128 do: 936 x 2048 x 8192 36.6 us, pairs of
+  // 128 features 28.9 (a step of 920 rows 6530 and 6230, of 944 rows of 1920 columns 4237 and 4035).
   if (flex && R > 32) {
-    for (int nb = 64; nb <= 256; nb += 16) {
-      const float t = 0.098f + 0.00077f * nb < 0.155f ? 0.155f : 0.098f + 0.00077f * nb;
-      const float c = 2.0f + 0.019f * nb + work(static_cast<long long>((N + 2 * kBlockM - 1) / (2 * kBlockM)) * ((R + nb - 1) / nb), t, 1.28f);
+    auto consider = [&](int nb) {
+      const int priced = nb > 96 && nb < 128 ? 128 : nb;
+      const float t = 0.098f + 0.00077f * priced < 0.155f ? 0.155f : 0.098f + 0.00077f * priced;
+      const float c = 2.0f + 0.019f * priced + work(static_cast<long long>((N + 2 * kBlockM - 1) / (2 * kBlockM)) * ((R + nb - 1) / nb), t, 1.28f);
       if (c < 0.97f * best) { best = c / 0.97f; plan = GemmPlan{kGemmFlex, nb, 1}; }
+    };
+    for (int nb = 64; nb <= 256; nb += 32) {
+      const int chunks = (R + nb - 1) / nb, w = ((R + chunks - 1) / chunks + 15) / 16 * 16;
+      consider(w > 64 ? w : 64);
+      if (nb == 160 && K <= 2048) consider(176);
+      if (nb == 192) consider(208);
     }
   }
   return plan;

@@ -1,4 +1,6 @@
 """Shared by the GPU tests: moving seeded numpy inputs to the device and comparing results."""
+import ctypes as ct
+
 import numpy as np
 import torch
 
@@ -48,3 +50,28 @@ def assert_out_close(got_bf16, ref, what="", max_rel=2e-2):
     _, c = rel_err(got, ref)
     assert excess.max() <= 0 and c >= 0.999, "%s: worst excess over the bound %.3e (RMS %.3e), cosine %.6f" % (
         what, excess.max(), rms, c)
+
+
+class _Plan(ct.Structure):
+    _fields_ = [("form", ct.c_int), ("block_n", ct.c_int), ("splits", ct.c_int)]
+
+
+PLAN_SINGLE, PLAN_PAIR, PLAN_FLEX = 0, 1, 2
+B200_SMS, B200_PAIRS = 148, 74
+
+
+def gemm_plan(R, N, K):
+    """(form, tile width) that the library's cost model picks for R x N x K on a B200 (fvar::gemm_plan)."""
+    from paper_2512_16483_b200 import binding
+    fn = binding.load_library()._ZN4fvar9gemm_planEiiiiiiimb
+    fn.restype, fn.argtypes = _Plan, [ct.c_int] * 7 + [ct.c_size_t, ct.c_bool]
+    p = fn(R, 1, N, K, B200_SMS, B200_PAIRS, 1, 0, N % 64 == 0)
+    return p.form, p.block_n
+
+
+def partial_ranges(R, N, K):
+    """K ranges in which the step leaves an R x N x K product for the next kernel to add up (fvar::gemm_partial_plan), 0: none."""
+    from paper_2512_16483_b200 import binding
+    fn, rows = binding.load_library()._ZN4fvar17gemm_partial_planEiiiiPi, ct.c_int(0)
+    fn.restype, fn.argtypes = ct.c_int, [ct.c_int] * 4 + [ct.POINTER(ct.c_int)]
+    return fn(R, N, K, B200_PAIRS, ct.byref(rows))

@@ -111,6 +111,24 @@ def test_kernel_calls_refuse_addresses_off_their_vector_grid(call, args, vary):
         assert fn(*args[:6], 6, *args[7:]) == binding.EINVAL
 
 
+@pytest.mark.parametrize("C,F", [(1024, 4096), (1920, 7680), (2048, 8192)])
+def test_free_width_tiles_make_no_more_chunks_than_they_have_to(C, F):
+    """A tile of 16 more rows than a multiple of 32 is taken where it makes no more chunks than the next multiple of 32;
+    208, the widest with six pipeline stages, and 176 over short sums may.  Pairs of 128 features are faster than 112 rows."""
+    from helpers import PLAN_FLEX, PLAN_PAIR, gemm_plan
+    for N, K in ((3 * C, C), (C, C), (F, C), (C, F)):
+        for R in list(range(33, 1100)) + list(range(1100, 8193, 7)) + [2048, 4096]:
+            form, w = gemm_plan(R, N, K)
+            if form == PLAN_FLEX:
+                assert w % 16 == 0 and 64 <= w <= 256
+                if w % 32 and not (w == 208 or (w == 176 and K <= 2048)):
+                    assert -(-R // w) == -(-R // (w + 16)), (R, N, K, w)
+                if w == 112:                         # where pairs of 128 features would need another round of the chip
+                    assert -(-R // 256) * -(-N // 128) > 74 >= -(-R // w) * -(-N // 256), (R, N, K)
+    for R in (2048, 4096):                           # full pairs of 256 rows
+        assert gemm_plan(R, 2048, 2048)[0] == PLAN_PAIR and gemm_plan(R, 2048, 8192)[0] == PLAN_PAIR
+
+
 def test_schedule_matches_printed_table():
     rows = []
     with open(os.path.join(ROOT, "tests", "golden", "rank_ratio_alpha096.txt")) as f:

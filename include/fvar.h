@@ -361,7 +361,7 @@ fvar_status fvar_gemm_bf16_wt(const void *A, const void *Wt, const void *bias, i
  * tests and tuning.  FVAR_GEMM_SKINNY: the weight-streaming form for R <= 512 (see FVAR_OPT_SKINNY_MAX_ROWS);
  * block_n is then the number of K ranges per 128-feature tile, 1 .. 8, or 0 to let the library pick.  FVAR_GEMM_KSPLIT:
  * 128 x 128 output tiles (rows on the M side, any R) whose K range is spread over a cluster in the same way.
- * FVAR_GEMM_FLEX: CTA pairs with 256 features on the M side and block_n rows (a multiple of 32 up to 256; 0: picked) on the
+ * FVAR_GEMM_FLEX: CTA pairs with 256 features on the M side and block_n rows (a multiple of 16 from 32 to 256; 0: picked) on the
  * N side; needs N % 64 == 0.
  * FVAR_EINVAL for a form / width the problem does not allow. */
 #define FVAR_GEMM_AUTO 0

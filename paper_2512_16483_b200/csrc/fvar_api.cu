@@ -1637,7 +1637,7 @@ fvar_status fvar_gemm_bf16_form(const void *A, const void *W, const void *bias, 
     if (block_n) plan.block_n = block_n;
   } else if (form == FVAR_GEMM_FLEX) {
     if (!flex_ok || max_clusters <= 0) return kfail(FVAR_EINVAL, "gemm: the free-width pair form needs N % 64 == 0 and a device that runs CTA pairs");
-    if (block_n != 0 && (block_n < 32 || block_n > 256 || block_n % 32)) return kfail(FVAR_EINVAL, "gemm: free-width block_n must be a multiple of 32 up to 256");
+    if (block_n != 0 && (block_n < 32 || block_n > 256 || block_n % 16)) return kfail(FVAR_EINVAL, "gemm: free-width block_n must be a multiple of 16 from 32 to 256");
     if (plan.form != kGemmFlex) plan = GemmPlan{kGemmFlex, R < 256 ? (R + 31) / 32 * 32 : 256, 1};
     if (block_n) plan.block_n = block_n;
   } else if (block_n != 0) {

@@ -4,7 +4,7 @@ import pytest
 import torch
 
 import synth_inputs as si
-from helpers import rel_err, to_bf16_cuda, weights_to_cuda
+from helpers import PLAN_FLEX, gemm_plan, partial_ranges, rel_err, to_bf16_cuda, weights_to_cuda
 
 pytestmark = pytest.mark.gpu
 
@@ -99,9 +99,16 @@ def test_down_in_both_forms(fv, C, hw, B):
     (33, 64, 64, 32), (400, 192, 2048, 160), (400, 6144, 200, 224),     # half a feature tile, a remainder of one, K not whole blocks
     (255, 1920, 1920, 64), (257, 1920, 128, 256), (1, 256, 4096, 0),    # an odd number of 128-feature halves, one row past a tile
     (5000, 320, 136, 96), (2704, 1024, 1024, 0), (97, 8192, 2048, 0),   # several tiles a pair, the picked widths
-    (410, 8192, 2048, 0), (410, 6144, 2048, 0), (283, 6144, 2048, 0), (79, 8192, 2048, 0), (3000, 1920, 1920, 0),   # picked: multiples of 16 among them
+    (79, 8192, 2048, 0), (283, 6144, 2048, 0), (3000, 1920, 1920, -176),
+    (410, 8192, 2048, -208), (410, 6144, 2048, -144), (283, 8192, 2048, -144),      # negative: picked, and known to be this
+    # odd multiples of 16, whose last 32 rows are half the next tile's: full tiles, last tiles of 1, 15, 16, 17, 31 and 47 rows
+    (96, 192, 264, 48), (81, 320, 2048, 80), (127, 1920, 200, 112), (160, 64, 1920, 144), (193, 8192, 128, 176),
+    (239, 1024, 4096, 208), (5087, 448, 136, 240), (5008, 256, 72, 112), (2704, 2048, 1024, 208),
 ])
 def test_gemm_free_width_pairs(fv, R, N, K, width):
+    if width < 0:
+        assert gemm_plan(R, N, K) == (PLAN_FLEX, -width)
+        width = 0
     g = torch.Generator(device="cuda").manual_seed(R + N + K)
     A = torch.randn((R, K), generator=g, device="cuda").bfloat16()
     W = torch.randn((N, K), generator=g, device="cuda").bfloat16()
@@ -113,32 +120,45 @@ def test_gemm_free_width_pairs(fv, R, N, K, width):
     assert (out.double() - ref).abs().max() <= bound
 
 
-@pytest.mark.parametrize("shape,B,k,blocks,bar", [("d16", 16, 8, 1, 2e-2), ("d16", 2, 7, 1, 2e-2), ("infinity", 1, 7, 1, 3e-2),
-                                                  ("infinity", 1, 7, 2, 3e-2), ("d16", 2, 8, 2, 2e-2), ("narrow", 1, 3, 3, 2e-2)])
-def test_step_epilogues_of_the_free_width_pairs(fv, shape, B, k, blocks, bar):
-    """Dense blocks at sizes where that form is taken for out-proj and fc2 (2704 rows of 1024 columns) and for QKV and fc1
-    (400 rows of 2048), every epilogue of it and the KV cache against the CPU oracle; at 200 rows of 1024 columns no GEMM
-    takes it.  With several blocks a group (400, 338 and 324 rows), fc2 of all but the last in K ranges that the next
-    block's LayerNorm adds up: four of them, or three where K / 64 = 66 is a multiple of 6 and not of 8."""
+@pytest.mark.parametrize("shape,B,k,blocks,per_group,bar,ranges", [
+    ("d16", 16, 8, 1, 1, 2e-2, 0), ("d16", 2, 7, 1, 1, 2e-2, 0), ("d16", 2, 8, 2, 2, 2e-2, 0), ("narrow", 1, 3, 3, 3, 2e-2, 0),
+    ("crossed", 14, 2, 1, 1, 2e-2, 0),                                      # 3584 rows: 208 a tile in every GEMM
+    ("infinity", 1, 7, 1, 1, 3e-2, 4), ("infinity", 1, 7, 2, 2, 3e-2, 4),   # a group's last fc2: added up by a pass of its own
+    ("infinity", 1, 7, 2, 1, 3e-2, 4),                                      # by the LayerNorm that writes a group's output, 2048 columns
+    ("d16", 6, 7, 3, 3, 2e-2, 4), ("wide", 1, 3, 3, 3, 3e-2, 3), ("wide", 1, 3, 2, 1, 3e-2, 3)])
+def test_step_epilogues_of_the_free_width_pairs(fv, shape, B, k, blocks, per_group, bar, ranges):
+    """Dense blocks at sizes where that form is taken for out-proj and fc2 (2704 rows of 1024 columns), for QKV and fc1 (400 rows
+    of 2048) and for every GEMM with a last chunk of 16 rows (3584 of 1024), every epilogue of it and the KV cache against
+    the CPU oracle; at 200 and 338 rows of 1024 columns and 324 of 512 fc2 is not split.  With `ranges`, fc2 leaves the sums of
+    that many K ranges, which the next block's LayerNorm adds up, within a group and from one dense group to the next, or
+    after the last block a kernel of its own: four, or three where K / 64 = 66 is a multiple of 6 and not of 8."""
     import numpy as np
     from oracle import fvar_oracle as orc
     from helpers import assert_close
-    shp = (si.shape_var_d16(n_blocks=blocks) if shape == "d16" else si.shape_infinity_2b(n_blocks=blocks, blocks_per_group=blocks) if shape == "infinity"
-           else si.shape_tiny(n_blocks=blocks, blocks_per_group=blocks, width=512, n_heads=8, head_dim=64, ffn_dim=4224, scales=(1, 2, 3, 18, 19)))
+    shp = {"d16": lambda: si.shape_var_d16(n_blocks=blocks, blocks_per_group=per_group),
+           "infinity": lambda: si.shape_infinity_2b(n_blocks=blocks, blocks_per_group=per_group),
+           "crossed": lambda: si.shape_tiny(n_blocks=blocks, blocks_per_group=per_group, width=1024, n_heads=16, head_dim=64, ffn_dim=4096, scales=(1, 2, 16, 16), cross=True),
+           "narrow": lambda: si.shape_tiny(n_blocks=blocks, blocks_per_group=per_group, width=512, n_heads=8, head_dim=64, ffn_dim=4224, scales=(1, 2, 3, 18, 19)),
+           "wide": lambda: si.shape_tiny(n_blocks=blocks, blocks_per_group=per_group, width=2048, n_heads=16, head_dim=128, ffn_dim=4224, scales=(1, 2, 3, 18, 19))}[shape]()
+    M, C, F = shp.tokens_per_scale()[k], shp.width, shp.ffn_dim
+    assert partial_ranges(B * M, C, F) == ranges
+    if shape == "crossed":
+        for N, K in ((3 * C, C), (C, C), (F, C), (C, F)):
+            assert gemm_plan(B * M, N, K) == (PLAN_FLEX, 208)
     w = si.make_weights(11, shp)
-    ctx = fv.Fvar(weights_to_cuda(w), blocks_per_group=blocks, n_heads=shp.n_heads, head_dim=shp.head_dim, ffn_dim=shp.ffn_dim, scale_hw=shp.hw(),
+    ctx = fv.Fvar(weights_to_cuda(w), blocks_per_group=per_group, n_heads=shp.n_heads, head_dim=shp.head_dim, ffn_dim=shp.ffn_dim, scale_hw=shp.hw(),
                   max_batch=B, ctx_len=shp.ctx_len, ctx_width=shp.ctx_width)
-    o = orc.Oracle(w, shp.n_heads, blocks, shp.hw(), shp.ln_eps)
+    o = orc.Oracle(w, shp.n_heads, per_group, shp.hw(), shp.ln_eps)
     cond = si.make_cond(12, B, shp.width)
     text = si.make_context(13, B, shp.ctx_len, shp.ctx_width) if shp.has_cross_attn else None
     ctx.set_cond(to_bf16_cuda(cond), to_bf16_cuda(text) if text is not None else None)
     o.set_cond(cond, text)
-    M = shp.tokens_per_scale()[k]
     for scale in (k, k):                # the second time over the keys and values the first one left in the cache
         toks = si.make_tokens(14, B, M, shp.width)
         ctx.scale_step(to_bf16_cuda(toks), scale)
         o.scale_step(toks, scale, orc.Policy("dense", "pair"))
-        assert_close(ctx.get_group_output(0, M).cpu().numpy(), np.stack([o.group_cache[0][b] for b in range(B)]), max_rel=bar, what=shape)
+        for g in range(shp.n_groups):
+            assert_close(ctx.get_group_output(g, M).cpu().numpy(), np.stack([o.group_cache[g][b] for b in range(B)]), max_rel=bar, what="%s, group %d" % (shape, g))
         ctx.kv_append(scale)
         o.kv_append(scale)
     assert ctx.poll_status() == fv.OK

@@ -575,8 +575,8 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     cluster_sync_all();                                            // nobody's ring is in use any more
     if (warp >= kSoftmaxWarp && final_ok) {
       tc_fence_after();
-      // a lone tile is shared by both warp-groups, half of the columns each (with the merge below: a step of 26 - 410 rows
-      // of 2048 columns 3470 -> 3449 us, of 16 rows 2550 -> 2529)
+      // A lone tile is shared by both warp-groups, half of the columns each.  Worth 0.4 % of a step of few rows with the merge below,
+      // which is then not waited for (16 rows of 2048 columns 2538 -> 2526 us, 64 rows 2798 -> 2790), nothing without it.
       const int wg = (warp - kSoftmaxWarp) >> 2, t = x.ntiles > 1 ? wg : 0, row = (warp & 3) * 32 + lane, rpr = t == 0 ? rpr0 : rpr1;
       const int half = x.ntiles > 1 ? D / 32 : D / 64, cc0 = x.ntiles > 1 ? 0 : wg * half;
       const uint32_t o_addr = tmem_base + 256 + t * D + (static_cast<uint32_t>((warp & 3) * 32) << 16);
@@ -614,8 +614,9 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         const uint32_t slot0 = static_cast<uint32_t>((tt == 0 ? 0 : splits * rpr0) + lrow);
         // A lane of the row's threads takes one range's maximum and sum; the weights are formed side by side and handed round
         // (eight ranges at most), and the sum is the same whatever the timing.  One range after another in every thread, in two
-        // passes, was a chain of 640 clocks a row.  Code that runs once a launch has to be short: two rows a round cost
-        // 1.2 us of a 21 us launch instead of gaining.
+        // passes, was a chain of 640 clocks a row (a step of 16 rows of 2048 columns 2544 -> 2538 us, of 64 rows 2818 -> 2798; 26 - 410
+        // rows, in two ranges, level).  Code that runs once a launch has to be short: two rows a round cost 1.2 us of a
+        // 21 us launch instead of gaining.
         const int l8 = st & 7;
         const float2 ml = l8 < splits ? ld_shared_f2(part_m + (slot0 + l8 * rpr) * 8u) : make_float2(-INFINITY, 0.f);
         float m_all = ml.x;

@@ -480,9 +480,9 @@ cudaError_t launch_finish_parts(const GemmParts &parts, int E, int rows, int C, 
 // (half-pixel centres, source coordinate clamped at 0, neighbours clamped at the edge).
 // One warp per output row; rows inside the index set are skipped.  Bound by latency and by the map's way to
 // memory.  In a late step it runs beside the QKV product, whose blocks leave 11 K registers of an SM: four rows a block of at most 64
-// registers a thread fit beside it, eight of 56 waited for it to end and then held the SMs that the attention needs whole (a step
-// of 408 rows of 1920 columns 2112 -> 1994 us, of 2048 rows 7560 -> 7433, of 1632 rows of 1024 columns 1566 -> 1544; 40 registers spill:
-// 2106, 7670, 1625).  By itself 5.2 -> 4.8 us for 16 x 128 rows of 1024 columns.
+// registers a thread fit beside it (8 bytes spill), eight of 56 waited for it to end and then held the SMs that the attention needs
+// whole: a step of 404 rows of 1920 columns 2393 -> 2301 us, of 2048 rows 7320 -> 7238, of 1616 or 680 rows of 1024 columns level.  At 40
+// registers 128 bytes spill: 2360, 7477.  By itself 5.2 -> 4.8 us for 16 x 128 rows of 1024 columns.
 constexpr int kFillThreads = 128;
 __global__ void __launch_bounds__(kFillThreads, 8) rtr_fill_kernel(const float *__restrict__ prev, float *__restrict__ out, int E,
                                                        int bmul, int boff, int h0, int w0, int h1, int w1, int C,

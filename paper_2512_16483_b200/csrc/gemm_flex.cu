@@ -267,8 +267,9 @@ void gemm_flex_shape(GemmArgs &a) {
 // can add up the ranges instead: the LayerNorm of the next block (400 x 2048 x 8192 with its gate and residual 25.9 us in the
 // chain of a step, now 17 and 1 in the LayerNorm), or after a group's last block, whose rows are scattered and split for a
 // projection, a pass of its own (26 us, now 17 and 3).
-// Taken where the ranges fill most of the pairs and are long division enough: three or four of them, 0.6 of the pairs at
-// work, two to four chunks of rows.  A step with ranges in every block and without (us):
+// Taken where the ranges fill most of the pairs: three or four of them, 0.6 of the pairs at work, two to four chunks of rows,
+// the fewest that hold them (more and smaller chunks would put more pairs to work; not measured).  A step with ranges in every
+// block and without (us):
 //   2048 columns, K = 8192, four ranges, 64 pairs: 257 rows 3659 and 3934, 400 rows 4061 and 4253, 512 rows 4344 and 4424;
 //   600 and 768 rows, where two ranges are all that fit: 5085 and 5039, 5554 and 5533 -- not taken;
 //   1920 columns, K = 7680: 340 rows (64 pairs) 2361 and 2548, 510 rows 3012 and 3153, 680 rows (three ranges, 72 pairs) 3350 and 3515;

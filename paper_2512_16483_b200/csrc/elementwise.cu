@@ -414,7 +414,7 @@ cudaError_t launch_ln_parts(float *x, RowMap xmap, int E, int rows, int C, const
 // GEMM and this launch take together against a GEMM that reduces by itself.
 template <int T>
 __global__ void __launch_bounds__(kLnThreads) finish_parts_kernel(GemmParts parts, int rows, int C, long long vec_stride, int bmul, int boff,
-                                                                  float *__restrict__ out, RowMap omap, const int *__restrict__ scatter,
+                                                                  float *out, RowMap omap, const int *__restrict__ scatter,
                                                                   bf16 *__restrict__ xsplit, int xsplit_mk) {
   const int e = blockIdx.x / rows, j = blockIdx.x - e * rows, n4 = C / 4, tid = threadIdx.x;
   float4 gate[T];

@@ -253,7 +253,7 @@ constexpr int kMaxParts = 4;
 cudaError_t launch_ln_parts(float *x, RowMap xmap, int E, int rows, int C, const GemmParts &parts, const float *shift, const float *scale,
                             long long vec_stride, int bmul, int boff, float eps, bf16 *y, cudaStream_t st);
 // No LayerNorm follows: row j of element e goes to row scatter[e][j] (j without scatter) of out, rows by omap, and as its
-// two-term bf16 split to xsplit (optional; see GemmArgs::xsplit).
+// two-term bf16 split to xsplit (optional; see GemmArgs::xsplit).  Without scatter out may be xin, with the same map.
 cudaError_t launch_finish_parts(const GemmParts &parts, int E, int rows, int C, long long vec_stride, int bmul, int boff, float *out, RowMap omap,
                                 const int *scatter, bf16 *xsplit, int xsplit_mk, cudaStream_t st);
 // early: shift, scale and gamma are not written by any kernel that may still be in flight (they may then be read before

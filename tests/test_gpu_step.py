@@ -8,7 +8,7 @@ import torch
 
 import synth_inputs as si
 from oracle import fvar_oracle as orc
-from helpers import assert_close, assert_out_close, bf16_to_numpy, rel_err, to_bf16_cuda, weights_to_cuda
+from helpers import assert_close, assert_out_close, bf16_to_numpy, partial_ranges, rel_err, to_bf16_cuda, weights_to_cuda
 
 pytestmark = pytest.mark.gpu
 
@@ -607,6 +607,25 @@ def test_lls_restoration_two_groups_and_limits(fv):
     with pytest.raises(fv.FvarError) as ei:
         p.gpu.scale_step(to_bf16_cuda(toks), 3, mode=fv.LOWRANK_RTR, rank_per_group=[200, 24], restore=fv.RESTORE_LLS)
     assert ei.value.status == fv.EUNSUPPORTED
+
+
+def test_lls_restoration_with_k_ranges(fv):
+    """680 block-output rows of 1024 columns: fc2 leaves K ranges after the group's last block too, and their sums go into the
+    residual stream in place, which the restoration reads."""
+    assert partial_ranges(8 * 85, 1024, 4096) == 4
+    shp = si.shape_var_d16(n_blocks=2, blocks_per_group=2)
+    B, k, M, r = 8, 8, 169, 85
+    p = Pair(fv, shp, seed=135, B=B)
+    p.prefill(k)
+    p.set_projections(k, [r])
+    toks = si.make_tokens(135, B, M, 1024, "spread")
+    ref = p.oracle.scale_step(toks, k, orc.Policy("lowrank_rtr", "pair", rank_per_group=[r], restore="lls"))
+    out = p.gpu.scale_step(to_bf16_cuda(toks), k, mode=fv.LOWRANK_RTR, rank_per_group=[r], restore=fv.RESTORE_LLS)
+    p.check_ok()
+    e, c = rel_err(p.gpu.get_group_output(0, M).cpu().numpy(), np.stack([p.oracle.group_cache[0][b] for b in range(B)]))
+    print("LLS in K ranges: max-abs/RMS %.3e cosine %.6f" % (e, c))
+    assert e <= 2e-2 and c >= 0.999, (e, c)
+    assert_out_close(bf16_to_numpy(out), ref, what="LLS step with K ranges")
 
 
 @pytest.mark.parametrize("B,k,blocks,ranks,kind,forced", [

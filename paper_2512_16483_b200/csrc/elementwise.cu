@@ -394,7 +394,8 @@ cudaError_t launch_ln_modulate(const float *x, RowMap xmap, int E, int rows, int
   return go(ln_modulate_kernel<16, false>);
 }
 
-// C <= 2048: gemm_partial_plan takes no wider output.
+// C <= 2048: gemm_partial_plan takes no wider output.  (512 columns and fewer have too few tiles for K ranges on a B200, so they have no
+// variant of their own.)
 cudaError_t launch_ln_parts(float *x, RowMap xmap, int E, int rows, int C, const GemmParts &parts, const float *shift, const float *scale,
                             long long vec_stride, int bmul, int boff, float eps, bf16 *y, cudaStream_t st) {
   if (E * rows <= 0) return cudaSuccess;
@@ -403,7 +404,6 @@ cudaError_t launch_ln_parts(float *x, RowMap xmap, int E, int rows, int C, const
     return launch_pdl(kern, dim3(E * rows), dim3(kLnThreads), 0, st, static_cast<const float *>(x), xmap, rows, C, shift, scale, vec_stride, bmul, boff,
                       static_cast<const bf16 *>(nullptr), eps, 1, y, parts);
   };
-  if (C <= 512) return go(ln_modulate_kernel<1, true>);
   if (C <= 1024) return go(ln_modulate_kernel<2, true>);
   return go(ln_modulate_kernel<4, true>);
 }
@@ -470,7 +470,6 @@ cudaError_t launch_finish_parts(const GemmParts &parts, int E, int rows, int C, 
   auto go = [&](auto kern) {
     return launch_pdl(kern, dim3(E * rows), dim3(kLnThreads), 0, st, parts, rows, C, vec_stride, bmul, boff, out, omap, scatter, xsplit, xsplit_mk);
   };
-  if (C <= 512) return go(finish_parts_kernel<1>);
   if (C <= 1024) return go(finish_parts_kernel<2>);
   return go(finish_parts_kernel<4>);
 }
